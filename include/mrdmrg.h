@@ -58,11 +58,16 @@ extern "C" {
                             /* the library; the handles of the failed call may be stale:  */
                             /* destroy them)                                              */
 
-#define MRD_PREC_FP64 0     /* complex128 operands, FP64 arithmetic                       */
+#define MRD_PREC_FP64 0     /* complex128 operands, FP64 accuracy: FP64 arithmetic, or for  */
+                            /* larger products 62-bit fixed point against the largest entry */
+                            /* of each row and column, exact sums and one rounding (digit   */
+                            /* products on the tensor cores; FP64 where an entry is not     */
+                            /* finite)                                                      */
 #define MRD_PREC_TF32 1     /* tcgen05 tensor cores, TF32 operands, FP32 accumulation     */
 #define MRD_PREC_BF16X3 2   /* tcgen05, split BF16 (hi*hi + hi*lo + lo*hi), FP32 accum.   */
 #define MRD_PREC_FF 3       /* complex128 operands split into float-float pairs (~48-bit  */
-                            /* products, TwoSum accumulation) on the FP32 pipes           */
+                            /* products, TwoSum accumulation) on the FP32 pipes, or for larger */
+                            /* products 55-bit fixed point as above                       */
 
 #define MRD_BASIS_MIXED 0   /* orbitals (x, k_m), charges (N, K mod Ly)                   */
 #define MRD_BASIS_REAL 1    /* orbitals (x, y), charge N only (modulus 1)                 */
@@ -149,8 +154,8 @@ int mrd_heff_sizes(const mrd_heff* h, int64_t* theta_len, int64_t* lenv_len, int
  * WR_{w'} = sum_{w''} W_{i+1}[w',w''] R_{w''}; the caller's buffers are not retained. */
 int mrd_heff_set_env(mrd_heff* h, const double* lenv_dev, const double* renv_dev);
 /* theta_out = H_eff theta_in (device pointers, complex128; must not overlap). prec:
- * MRD_PREC_FP64 runs FP64 grouped GEMMs, MRD_PREC_FF the same grouped GEMMs in float-float
- * arithmetic (~1e-13 relative); MRD_PREC_TF32 and MRD_PREC_BF16X3 run the same
+ * MRD_PREC_FP64 runs grouped GEMMs of FP64 accuracy, MRD_PREC_FF the same grouped GEMMs in
+ * float-float arithmetic (~1e-13 relative or better); MRD_PREC_TF32 and MRD_PREC_BF16X3 run the same
  * contraction on the tcgen05 tensor cores with FP32 accumulation (complex products as four
  * real ones), operands repacked into 128-byte swizzled tiles: the folded environments once
  * after each mrd_heff_set_env, theta on every call; the result is returned in complex128. */
@@ -178,7 +183,7 @@ int mrd_heff_timing(mrd_heff* h, int32_t on);
  *                           task order) and keeps the fastest for the context; later H_effs
  *                           of the class reuse it; 0: the default configuration. */
 /*   MRD_OPT_WAIT_LIMIT_US   1000000 (default): how long, in microseconds, a wait inside a
- *                           tensor-core GEMM (for a shared-memory stage, an accumulator or
+ *                           tensor-core GEMM of any precision (for a shared-memory stage, an accumulator or
  *                           the other warp roles) may last before the kernel gives up: it then
  *                           sets an error flag, waits for its own copies and MMAs in flight,
  *                           frees its tensor memory and returns. 0 gives up at the first wait,

@@ -23,7 +23,7 @@ std::vector<int2> ff_item_order(const int64_t* tasks, const int64_t* segs, int64
 cudaError_t to_ff(const double2* x, float4* y, int64_t n, cudaStream_t s);
 cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
                               const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s);
+                              int n_sm, cudaStream_t s, const int* run_if = nullptr);
 cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* rows, int64_t nrows,
                             const int64_t* env_map, int n_sec, const int32_t* perm, const int32_t* idx,
                             const double* val, int chan_field, cudaStream_t s);
@@ -428,22 +428,36 @@ int mrd_heff_sizes(const mrd_heff* h, int64_t* theta_len, int64_t* lenv_len, int
   return MRD_E_HOST;
 }
 
+}  // extern "C"
+
+// Fold the environments with the MPO; a null environment is skipped (its side must not be used
+// until it is folded; h->env_loaded is set only when both are there).
+int heff_fold(mrd_heff* h, const double2* lenv, const double2* renv) {
+  mrd_ctx* ctx = h->ctx;
+  Guard g(ctx->device);
+  cudaError_t e = cudaSuccess;
+  if (lenv)
+    e = launch_fold_env(lenv, h->lw, h->p.lw, h->counts[C_NLW], h->p.lmap, h->d.n_l, h->p.wi_perm, h->p.wi_idx,
+                        h->wi_val, 0, ctx->stream);
+  if (renv && e == cudaSuccess)
+    e = launch_fold_env(renv, h->wr, h->p.wr, h->counts[C_NWR], h->p.rmap, h->d.n_r, h->p.wj_perm, h->p.wj_idx,
+                        h->wj_val, 1, ctx->stream);
+  if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "mrd_heff_set_env");
+  h->env_loaded = (lenv || h->counts[C_LENV] == 0) && (renv || h->counts[C_RENV] == 0);
+  tc_env_changed(h);
+  dg_env_changed(h);
+  h->ff_dirty = true;
+  return MRD_OK;
+}
+
+extern "C" {
+
 int mrd_heff_set_env(mrd_heff* h, const double* lenv_dev, const double* renv_dev) try {
   if (!h) return MRD_E_ARG;
   mrd_ctx* ctx = h->ctx;
   if ((!lenv_dev && h->counts[C_LENV] > 0) || (!renv_dev && h->counts[C_RENV] > 0))
     return mrd_fail(ctx, MRD_E_ARG, "mrd_heff_set_env: null environment");
-  Guard g(ctx->device);
-  cudaError_t e = launch_fold_env((const double2*)lenv_dev, h->lw, h->p.lw, h->counts[C_NLW], h->p.lmap, h->d.n_l,
-                                  h->p.wi_perm, h->p.wi_idx, h->wi_val, 0, ctx->stream);
-  if (e == cudaSuccess)
-    e = launch_fold_env((const double2*)renv_dev, h->wr, h->p.wr, h->counts[C_NWR], h->p.rmap, h->d.n_r,
-                        h->p.wj_perm, h->p.wj_idx, h->wj_val, 1, ctx->stream);
-  if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "mrd_heff_set_env");
-  h->env_loaded = true;
-  tc_env_changed(h);
-  h->ff_dirty = true;
-  return MRD_OK;
+  return heff_fold(h, (const double2*)lenv_dev, (const double2*)renv_dev);
 } catch (...) {   // host memory or threads exhausted: no exception crosses the C ABI
   return MRD_E_HOST;
 }
@@ -489,6 +503,9 @@ static int heff_prepare(mrd_heff* h, int32_t prec) {
   mrd_ctx* ctx = h->ctx;
   cudaStream_t s = ctx->stream;
   if (prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3) return tc_prepare(h, prec);
+  // FP64 and float-float: digit-split products on the tensor cores where they are cheaper
+  int rc_dg = dg_prepare(h, prec, &h->dg_use);
+  if (rc_dg != MRD_OK || h->dg_use) return rc_dg;
   if (h->per_task) {
     int rc = ensure_per_task(h);
     if (rc != MRD_OK) return rc;
@@ -550,6 +567,10 @@ int mrd_heff_apply(mrd_heff* h, const double* theta_in_dev, double* theta_out_de
   if (h->timing && !apply_events(h, s, ev, &cap)) return mrd_fail(ctx, MRD_E_CUDA, "mrd_heff_apply: cudaEventCreate");
   const cudaEvent_t e0 = ev[0], e1 = ev[1], e2 = ev[2];
   cudaError_t e = cudaMemsetAsync(theta_out_dev, 0, (size_t)n * 16, s);
+  if (h->dg_use) {
+    if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "mrd_heff_apply");
+    return dg_apply(h, (const double2*)theta_in_dev, (double2*)theta_out_dev, prec, ev, cap);
+  }
   if (prec == MRD_PREC_FF) {
     float4* z_ff = (float4*)h->z;
     // real operands (MRD_OPT_REAL): one float-float product per multiply-add instead of three
@@ -733,7 +754,7 @@ int mrd_lanczos(mrd_heff* h, double* theta_dev, int32_t max_iter, double tol, in
   rc = lanczos_run(h->lz, ctx, apply_cb, &arg, (double2*)theta_dev, max_iter, tol, energy, &it, nullptr, key,
                    h->timing ? replay_timing_cb : nullptr);
   *iters = it;
-  if (rc == MRD_OK && (prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3)) rc = tc_status(h);
+  if (rc == MRD_OK) rc = prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3 ? tc_status(h) : dg_status(h);
   return rc;
 } catch (...) {   // host memory or threads exhausted: no exception crosses the C ABI
   return MRD_E_HOST;
@@ -748,7 +769,7 @@ int mrd_heff_rayleigh(mrd_heff* h, const double* theta_dev, int32_t prec, double
   if (rc != MRD_OK) return rc;
   double2* hv = lanczos_work(h->lz);   // the workspace's spare vector
   rc = mrd_heff_apply(h, theta_dev, (double*)hv, prec);
-  if (rc == MRD_OK && (prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3)) rc = tc_status(h);
+  if (rc == MRD_OK) rc = prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3 ? tc_status(h) : dg_status(h);
   if (rc != MRD_OK) return rc;
   double nn, ni, en, ei;
   if ((rc = vdot(h->lz, ctx, (const double2*)theta_dev, (const double2*)theta_dev, &nn, &ni)) != MRD_OK) return rc;
@@ -805,7 +826,9 @@ int mrd_heff_status(mrd_heff* h) try {
   if (!h) return MRD_E_ARG;
   Guard g(h->ctx->device);
   MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
-  return tc_status(h);
+  const int rc = tc_status(h);
+  const int rc2 = dg_status(h);   // both flags are read and cleared
+  return rc != MRD_OK ? rc : rc2;
 } catch (...) {   // host memory or threads exhausted: no exception crosses the C ABI
   return MRD_E_HOST;
 }
@@ -905,13 +928,6 @@ int mrd_heff_table(const mrd_heff* h, int32_t which, int64_t* rows, int64_t* cou
 }
 
 }  // extern "C"
-
-// Start the float-float conversion of LW / WR (asynchronous device work) ahead of a
-// float-float application, e.g. so that it runs while the host builds the tensor-core tables.
-int heff_prefetch_ff(mrd_heff* h) {
-  Guard g(h->ctx->device);
-  return heff_prepare(h, MRD_PREC_FF);
-}
 
 namespace mrd {
 

@@ -21,6 +21,7 @@
 #include <string>
 #include <vector>
 
+#include "digits.cuh"
 #include "heff_internal.h"
 
 namespace mrd {
@@ -35,7 +36,7 @@ std::vector<int2> ff_item_order(const int64_t* tasks, const int64_t* segs, int64
 cudaError_t to_ff(const double2* x, float4* y, int64_t n, cudaStream_t s);
 cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
                               const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s);
+                              int n_sm, cudaStream_t s, const int* run_if = nullptr);
 cudaError_t svd_load(const double2* theta, const int64_t* blk, const int64_t* src_off, int nblk, double2* work,
                      double* fro2, cudaStream_t s);
 int64_t svd_bround_smem(int W, int64_t p, int64_t r_v, bool f32);
@@ -347,7 +348,7 @@ struct mrd_dmrg {
   std::vector<EnvT> L, R;
   Buf gtask, gseg, gpref, gitems, ctask, theta, theta2, svd_blk, svd_src, svd_pref, svd_work, svd_u, svd_vh, svd_s,
       svd_ss, svd_ord, svd_flat, svd_keep, svd_info, svd_w32, svd_x2, svd_fro, svd_last, svd_ctr, tbuf,
-      zeros, svd_perm;
+      svd_perm;
   // columns entering the final Jacobi sweeps and columns of all blocks, last block SVD
   double svd_cols[2] = {0, 0};
   // environments stored in complex64 (MRD_DMRG_OPT_ENV_FP32); envx: complex128 working copies
@@ -378,6 +379,9 @@ struct mrd_dmrg {
   std::vector<double> schmidt_val;
   Buf schmidt_tab, schmidt_out;
   Buf ff_a, ff_b;   // float-float copies of the operands of a grouped GEMM
+  // digit-split grouped GEMMs: tables, panels, exponents and words of the last one
+  Buf dg_tab, dg_panel[2], dg_expo, dg_partial, dg_words;
+  bool dg_ran = false;   // since the last dg_check
   int last_iters = 0, last_refine = 0;
   bool timing = false;
   double kms[4] = {0, 0, 0, 0};   // accumulated GEMM ms: tensor-core step 1, step 2, FP64 step 1, step 2
@@ -387,13 +391,81 @@ struct mrd_dmrg {
 
 namespace {
 
+// The grouped GEMM as digit-split tensor-core products (digits.cuh); *done = false when the
+// CUDA-core kernels are cheaper (small problems) or the panels find no memory.
+int run_gemm_digits(mrd_dmrg* D, const GemmList& g, int64_t nt, const double2* Aop, const double2* Bop, double2* C,
+                    DgStack how, bool* done) {
+  mrd_ctx* ctx = D->ctx;
+  cudaStream_t s = ctx->stream;
+  const bool real = D->real && D->gemm_ff;
+  const int beta = D->gemm_ff ? 7 : 8;
+  const double cores = dg_cost_cores(g.t.data(), g.s.data(), nt, D->gemm_ff, real, D->n_sm);
+  // planning, uploading and the digit passes' launches take ~60 us even for a small product
+  constexpr double kSetup = 110000.0;
+  if (cores < kSetup) return MRD_OK;
+  DgPlan p;
+  dg_plan(p, g.t.data(), g.s.data(), nt, how, nullptr, real, beta, D->n_sm);
+  // the exponent and digit passes and their launches
+  const double pass = (double)(p.bytes[0] + p.bytes[1]) * 2.0 / 5.0e12 * 1.9e9 + kSetup;
+  if (p.items.empty() || p.cost + pass >= cores) return MRD_OK;
+  const int64_t nt8 = 8 * (int64_t)p.splits.size();
+  const size_t tb = dg_table_bytes(p), nx = (size_t)(p.rows[0] + p.rows[1] + nt8) * 4;
+  const size_t need[5] = {dg_device_table_bytes(p), (size_t)p.bytes[0], (size_t)p.bytes[1], nx, (size_t)(p.slots * kDgSlotBytes)};
+  Buf* bufs[5] = {&D->dg_tab, &D->dg_panel[0], &D->dg_panel[1], &D->dg_expo, &D->dg_partial};
+  for (int k = 0; k < 5; ++k) {
+    const cudaError_t e = bufs[k]->need(need[k]);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      return MRD_OK;
+    }
+    if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "grouped GEMM: panels");
+  }
+  std::vector<uint8_t> host(tb);
+  DgDev d;
+  dg_tables(p, host.data(), D->dg_tab.as<uint8_t>(), d);
+  MRD_CUDA(ctx, cudaMemcpyAsync(D->dg_tab.p, host.data(), tb, cudaMemcpyHostToDevice, s));   // pageable: consumed on return
+  MRD_CUDA(ctx, dg_expand(d, s));
+  MRD_CUDA(ctx, D->dg_words.need(DG_WORDS * 4));
+  int* words = D->dg_words.as<int>();
+  d.panel[0] = D->dg_panel[0].as<uint8_t>();
+  d.panel[1] = D->dg_panel[1].as<uint8_t>();
+  d.partial = D->dg_partial.as<uint8_t>();
+  d.expo[0] = D->dg_expo.as<int>();
+  d.expo[1] = d.expo[0] + p.rows[0];
+  d.tickets = d.expo[1] + p.rows[1];
+  // the error flag (word DG_ERR) stays until dg_check reads it
+  if (!D->dg_ran) MRD_CUDA(ctx, cudaMemsetAsync(words, 0, DG_WORDS * 4, s));
+  MRD_CUDA(ctx, cudaMemsetAsync(d.expo[0], 0, nx, s));
+  D->dg_ran = true;
+  MRD_CUDA(ctx, dg_pack(d, 0, Aop, beta, words, DG_BAD, s));
+  MRD_CUDA(ctx, dg_pack(d, 1, Bop, beta, words, DG_BAD, s));
+  MRD_CUDA(ctx, dg_gemm(d, C, beta, words, D->n_sm, 1000000000ull, s));
+  *done = true;
+  return MRD_OK;
+}
+
+// Reports a wait that gave up in the digit-split GEMMs run since the last check.
+int dg_check(mrd_dmrg* D) {
+  if (!D->dg_ran) return MRD_OK;
+  D->dg_ran = false;
+  int herr = 0;
+  MRD_CUDA(D->ctx, cudaMemcpyAsync(&herr, D->dg_words.as<int>() + DG_ERR, 4, cudaMemcpyDeviceToHost, D->ctx->stream));
+  MRD_CUDA(D->ctx, cudaStreamSynchronize(D->ctx->stream));
+  if (herr)
+    return mrd_fail(D->ctx, MRD_E_TIMEOUT, "digit-split GEMM: a bounded wait gave up (code " + std::to_string(herr) + ")");
+  return MRD_OK;
+}
+
 // Grouped GEMM C += sum over segments A . B on the context stream, FP64 or float-float
-// (D->gemm_ff). a_ff / b_ff: the operands already split into float-float (e.g. the H_eff's
-// own copies of LW / WR), used instead of converting Aop / Bop again. Asynchronous: the task
-// tables are copied from pageable host memory (consumed when the copy call returns) into
-// device buffers that later calls reuse in stream order.
+// (D->gemm_ff); `how`: which tasks share panels in the digit-split form. a_ff / b_ff: the
+// operands already split into float-float (e.g. the H_eff's own copies of LW / WR), c_ff: a
+// float-float result, all for the CUDA-core float-float kernel only: *in_f64 tells that the
+// digit-split form ran and C holds the FP64 result. Asynchronous: the task tables are copied
+// from pageable host memory (consumed when the copy call returns) into device buffers that
+// later calls reuse in stream order.
 int run_gemm(mrd_dmrg* D, GemmList& g, const double2* Aop, int64_t alen, const double2* Bop, int64_t blen, double2* C,
-             int64_t clen, const float4* a_ff = nullptr, const float4* b_ff = nullptr, float4* c_ff = nullptr) {
+             int64_t clen, const float4* a_ff = nullptr, const float4* b_ff = nullptr, float4* c_ff = nullptr,
+             DgStack how = DG_BY_B, bool* in_f64 = nullptr, bool digits = true) {
   mrd_ctx* ctx = D->ctx;
   g.drop_empty_last();
   const int64_t nt = (int64_t)g.t.size() / TF;
@@ -415,6 +487,13 @@ int run_gemm(mrd_dmrg* D, GemmList& g, const double2* Aop, int64_t alen, const d
     }
     pref[i + 1] = pref[i] + ((r[0] + kTile - 1) / kTile) * ((r[1] + kTile - 1) / kTile);
   }
+  bool done = false;
+  if (digits) {
+    const int rc = run_gemm_digits(D, g, nt, Aop, Bop, C, how, &done);
+    if (rc != MRD_OK) return rc;
+  }
+  if (in_f64) *in_f64 = done;
+  if (done) return MRD_OK;
   cudaStream_t s = ctx->stream;
   MRD_CUDA(ctx, D->gtask.need(g.t.size() * 8));
   MRD_CUDA(ctx, D->gseg.need(std::max<size_t>(g.s.size(), 1) * 8));
@@ -515,8 +594,8 @@ int env_store(mrd_dmrg* D, EnvT& E, const double2* src) {
   return MRD_OK;
 }
 
-// Build the H_eff handle for sites (i, i+1) from the current bonds; env pointers may be the
-// zero buffer when a side is only needed for its fold with the MPO.
+// Build the H_eff handle for sites (i, i+1) from the current bonds; an env pointer may be null
+// when only the other side's fold with the MPO is needed.
 int make_heff(mrd_dmrg* D, int i, const double2* lenv, const double2* renv, mrd_heff** out) {
   const SiteT& X = D->A[i];
   const SiteT& Y = D->A[i + 1];
@@ -539,14 +618,7 @@ int make_heff(mrd_dmrg* D, int i, const double2* lenv, const double2* renv, mrd_
   int rc = mrd_heff_create(D->ctx, &d, out);
   if (rc != MRD_OK) return rc;
   mrd_heff* h = *out;
-  // zero stand-ins for absent environments
-  const int64_t need = std::max(h->counts[C_LENV], h->counts[C_RENV]);
-  if (!lenv || !renv) {
-    MRD_CUDA(D->ctx, D->zeros.need((size_t)std::max<int64_t>(need, 1) * 16));
-    MRD_CUDA(D->ctx, cudaMemsetAsync(D->zeros.p, 0, (size_t)std::max<int64_t>(need, 1) * 16, D->ctx->stream));
-  }
-  rc = mrd_heff_set_env(h, (const double*)(lenv ? lenv : D->zeros.as<double2>()),
-                        (const double*)(renv ? renv : D->zeros.as<double2>()));
+  rc = heff_fold(h, lenv, renv);   // an absent environment is not folded (nothing reads that side)
   if (rc != MRD_OK) { mrd_heff_free(h); *out = nullptr; }
   return rc;
 }
@@ -582,8 +654,11 @@ int form_theta(mrd_dmrg* D, mrd_heff* h, const SiteT& X, const SiteT& Y, double2
       }
     }
   }
-  // X and Y live in different buffers: run as two operands
-  return run_gemm(D, g, X.data.as<double2>(), X.size, Y.data.as<double2>(), Y.size, theta, n);
+  // X and Y live in different buffers: run as two operands. The update's own small products (theta,
+  // the SVD's and the projection) stay on the CUDA-core kernels: they take under 2% of an update,
+  // and a reduced-precision Lanczos turns any change of their rounding into one of its own size.
+  return run_gemm(D, g, X.data.as<double2>(), X.size, Y.data.as<double2>(), Y.size, theta, n, nullptr, nullptr, nullptr,
+                  DG_BY_B, nullptr, false);
 }
 
 // Block SVD of the blocks `blk` (SVF rows) of `src`; returns kept counts per block and info.
@@ -796,7 +871,7 @@ int block_svd(mrd_dmrg* D, std::vector<int64_t>& blk, const std::vector<int64_t>
       g.seg(d[5], r, d[4], p, r, 0);
     }
     rc = run_gemm(D, g, D->svd_work.as<double2>(), work, D->svd_work.as<double2>(), work, D->svd_x2.as<double2>(),
-                  xlen);
+                  xlen, nullptr, nullptr, nullptr, DG_BY_B, nullptr, false);
     if (rc != MRD_OK) return rc;
   }
   // Columns set aside before the final sweeps. After the pre-sweeps the columns of X = M V32
@@ -876,8 +951,9 @@ int block_svd(mrd_dmrg* D, std::vector<int64_t>& blk, const std::vector<int64_t>
   return MRD_OK;
 }
 
-// L[i+1] = A^+ (L[i] W_i) A with A = D->A[i] (mode 0) and the LW fold of h (sites i, i+1).
-int env_left(mrd_dmrg* D, mrd_heff* h, int i) {
+// L[i+1] = A^+ (L[i] W_i) A with A = D->A[i] (mode 0) and the LW fold of h (sites i, i+1). digits:
+// the digit-split products may be used.
+int env_left(mrd_dmrg* D, mrd_heff* h, int i, bool digits) {
   mrd_ctx* ctx = D->ctx;
   const SiteT& A = D->A[i];
   const Secs& ls = A.left;   // bond i
@@ -893,27 +969,44 @@ int env_left(mrd_dmrg* D, mrd_heff* h, int i) {
       return mrd_fail(ctx, MRD_E_STATE, "internal: LW block outside the bond's channels or sectors");
     lw[(size_t)(((r[0] * 2 + r[1]) * 2 + r[2]) * nls + r[3])] = r[7];
   }
+  // sector lookups of the lists below, once per charge: c + c_w' for every (w', c), the left sector
+  // of (c, s), and A's sub-blocks (a, s)
+  std::vector<int> img((size_t)(nw * ncs)), from((size_t)(ncs * 2));
+  struct Sub { int64_t off, ld; int c; };
+  std::vector<Sub> sub((size_t)(nls * 2), Sub{0, 0, -1});
+  for (int64_t w = 0; w < nw; ++w)
+    for (int64_t c = 0; c < ncs; ++c)
+      img[(size_t)(w * ncs + c)] = find_sec(cs, cs[c].N + cm[w][0], kmod(cs[c].K + cm[w][1], mod));
+  for (int64_t c = 0; c < ncs; ++c)
+    for (int s = 0; s < 2; ++s) from[(size_t)(c * 2 + s)] = find_sec(ls, cs[c].N - s, kmod(cs[c].K - s * m1, mod));
+  for (int64_t a = 0; a < nls; ++a)
+    for (int s = 0; s < 2; ++s) {
+      Sub& q = sub[(size_t)(a * 2 + s)];
+      if (!A.subblock((int)a, s, &q.off, &q.ld, &q.c)) q.c = -1;
+    }
   // step 1: T(w', c, s') = sum_s LW(w', s', s, a) A(a, s -> c)
   GemmList g1;
+  g1.t.reserve((size_t)(nw * ncs * 2 * TF));
+  g1.s.reserve((size_t)(nw * ncs * 4 * SF));
   struct TB { int64_t off, rows; };
   std::vector<TB> tblk((size_t)(nw * ncs * 2), TB{-1, 0});   // (w', c, s') -> block of T
   int64_t tlen = 0;
   for (int w = 0; w < (int)cm.size(); ++w)
     for (int c = 0; c < (int)cs.size(); ++c) {
-      const int cp = find_sec(cs, cs[c].N + cm[w][0], kmod(cs[c].K + cm[w][1], mod));
+      const int cp = img[(size_t)(w * ncs + c)];
       if (cp < 0) continue;
       for (int sp = 0; sp < 2; ++sp) {
-        const int ap = find_sec(ls, cs[cp].N - sp, kmod(cs[cp].K - sp * m1, mod));
+        const int ap = from[(size_t)(cp * 2 + sp)];
         if (ap < 0) continue;
         bool started = false;
         for (int s = 0; s < 2; ++s) {
-          const int a = find_sec(ls, cs[c].N - s, kmod(cs[c].K - s * m1, mod));
+          const int a = from[(size_t)(c * 2 + s)];
           if (a < 0) continue;
           const int64_t lwo = lw[(size_t)((((int64_t)w * 2 + sp) * 2 + s) * nls + a)];
           if (lwo < 0) continue;
-          int64_t ao, ald;
-          int rr;
-          if (!A.subblock(a, s, &ao, &ald, &rr) || rr != c) continue;
+          const Sub& q = sub[(size_t)(a * 2 + s)];
+          if (q.c != c) continue;
+          const int64_t ao = q.off, ald = q.ld;
           if (!started) {
             tblk[(size_t)(((int64_t)w * ncs + c) * 2 + sp)] = {tlen, ls[ap].d};
             g1.task(ls[ap].d, cs[c].d, tlen, cs[c].d);
@@ -927,8 +1020,9 @@ int env_left(mrd_dmrg* D, mrd_heff* h, int i) {
   MRD_CUDA(ctx, D->tbuf.need((size_t)std::max<int64_t>(tlen, 1) * 16));
   // with float-float GEMMs T stays in float-float (the same 16 bytes per element) for step 2
   float4* t_ff = D->gemm_ff ? D->tbuf.as<float4>() : nullptr;
+  bool t64 = false;   // T written in FP64 (digit-split product)
   int rc = run_gemm(D, g1, h->lw, h->counts[C_LWLEN], A.data.as<double2>(), A.size, D->tbuf.as<double2>(), tlen,
-                    heff_ff_lw(h), nullptr, t_ff);
+                    heff_ff_lw(h), nullptr, t_ff, DG_BY_B, &t64, digits);
   if (rc != MRD_OK) return rc;
   // step 2: L'(w', c) = sum_s' A(a', s' -> c')^+ T(w', c, s')
   EnvT& E = D->L[i + 1];
@@ -944,28 +1038,30 @@ int env_left(mrd_dmrg* D, mrd_heff* h, int i) {
     for (int c = 0; c < (int)cs.size(); ++c) {
       const int64_t off = E.off[(size_t)w * cs.size() + c];
       if (off < 0) continue;
-      const int cp = find_sec(cs, cs[c].N + cm[w][0], kmod(cs[c].K + cm[w][1], mod));
+      const int cp = img[(size_t)(w * ncs + c)];
       bool started = false;
       for (int sp = 0; sp < 2; ++sp) {
         const TB& tb = tblk[(size_t)(((int64_t)w * ncs + c) * 2 + sp)];
         if (tb.off < 0) continue;
-        const int ap = find_sec(ls, cs[cp].N - sp, kmod(cs[cp].K - sp * m1, mod));
-        int64_t ao, ald;
-        int rr;
-        if (!A.subblock(ap, sp, &ao, &ald, &rr) || rr != cp) continue;
+        const int ap = from[(size_t)(cp * 2 + sp)];
+        const Sub& q = sub[(size_t)(ap * 2 + sp)];
+        if (q.c != cp) continue;
+        const int64_t ao = q.off, ald = q.ld;
         if (!started) { g2.task(cs[cp].d, cs[c].d, off, cs[c].d); started = true; }
         // A-op: conj-transpose of the d_a' x d_c' sub-block
         g2.seg(ao, ald, tb.off, cs[c].d, ls[ap].d, 1);
       }
     }
+  // blocks of one A(c') are stacked over (w', c): the transposed product with T's columns tall. A
+  // float-float T keeps the float-float kernel.
   rc = run_gemm(D, g2, A.data.as<double2>(), A.size, D->tbuf.as<double2>(), tlen, eout.as<double2>(), E.size, nullptr,
-                t_ff);
+                t64 ? nullptr : t_ff, nullptr, DG_BY_A, nullptr, digits && (t64 || !t_ff));
   if (rc != MRD_OK) return rc;
   return env_store(D, E, eout.as<double2>());
 }
 
 // R[i+1] = B (W_{i+1} R[i+2]) B^+ with B = D->A[i+1] (mode 1) and the WR fold of h.
-int env_right(mrd_dmrg* D, mrd_heff* h, int i) {
+int env_right(mrd_dmrg* D, mrd_heff* h, int i, bool digits) {
   mrd_ctx* ctx = D->ctx;
   const SiteT& B = D->A[i + 1];
   const Secs& cs = B.left;   // bond i+1
@@ -981,23 +1077,40 @@ int env_right(mrd_dmrg* D, mrd_heff* h, int i) {
       return mrd_fail(ctx, MRD_E_STATE, "internal: WR block outside the bond's channels or sectors");
     wr[(size_t)(((r[0] * 2 + r[1]) * 2 + r[2]) * nbs + r[3])] = r[7];
   }
+  // sector lookups of the lists below, once per charge: c + c_w' for every (w', c), the right
+  // sector of (c, s), and B's sub-blocks (c, s)
+  std::vector<int> img((size_t)(nw * ncs)), to((size_t)(ncs * 2));
+  struct Sub { int64_t off, ld; int b; };
+  std::vector<Sub> sub((size_t)(ncs * 2), Sub{0, 0, -1});
+  for (int64_t w = 0; w < nw; ++w)
+    for (int64_t c = 0; c < ncs; ++c)
+      img[(size_t)(w * ncs + c)] = find_sec(cs, cs[c].N + cm[w][0], kmod(cs[c].K + cm[w][1], mod));
+  for (int64_t c = 0; c < ncs; ++c)
+    for (int s = 0; s < 2; ++s) {
+      to[(size_t)(c * 2 + s)] = find_sec(bs, cs[c].N + s, kmod(cs[c].K + s * m2, mod));
+      Sub& q = sub[(size_t)(c * 2 + s)];
+      if (!B.subblock((int)c, s, &q.off, &q.ld, &q.b)) q.b = -1;
+    }
   // step 1: T(w', c, s') = sum_s B(c, s -> b) WR(w', s, s', b)
   GemmList g1;
+  g1.t.reserve((size_t)(nw * ncs * 2 * TF));
+  g1.s.reserve((size_t)(nw * ncs * 4 * SF));
   struct TB { int64_t off, cols; };
   std::vector<TB> tblk((size_t)(nw * ncs * 2), TB{-1, 0});   // (w', c, s') -> block of T
   int64_t tlen = 0;
   for (int w = 0; w < (int)cm.size(); ++w)
     for (int c = 0; c < (int)cs.size(); ++c) {
-      const int cp = find_sec(cs, cs[c].N + cm[w][0], kmod(cs[c].K + cm[w][1], mod));
+      const int cp = img[(size_t)(w * ncs + c)];
       if (cp < 0) continue;
       for (int sp = 0; sp < 2; ++sp) {
-        const int bp = find_sec(bs, cs[cp].N + sp, kmod(cs[cp].K + sp * m2, mod));
+        const int bp = to[(size_t)(cp * 2 + sp)];
         if (bp < 0) continue;
         bool started = false;
         for (int s = 0; s < 2; ++s) {
-          int64_t bo, bld;
-          int b;
-          if (!B.subblock(c, s, &bo, &bld, &b)) continue;
+          const Sub& q = sub[(size_t)(c * 2 + s)];
+          if (q.b < 0) continue;
+          const int64_t bo = q.off, bld = q.ld;
+          const int b = q.b;
           const int64_t wro = wr[(size_t)((((int64_t)w * 2 + s) * 2 + sp) * nbs + b)];
           if (wro < 0) continue;
           if (!started) {
@@ -1012,8 +1125,9 @@ int env_right(mrd_dmrg* D, mrd_heff* h, int i) {
     }
   MRD_CUDA(ctx, D->tbuf.need((size_t)std::max<int64_t>(tlen, 1) * 16));
   float4* t_ff = D->gemm_ff ? D->tbuf.as<float4>() : nullptr;   // T in float-float for step 2
+  bool t64 = false;   // T written in FP64 (digit-split product)
   int rc = run_gemm(D, g1, B.data.as<double2>(), B.size, h->wr, h->counts[C_WRLEN], D->tbuf.as<double2>(), tlen,
-                    nullptr, heff_ff_wr(h), t_ff);
+                    nullptr, heff_ff_wr(h), t_ff, DG_BY_A, &t64, digits);
   if (rc != MRD_OK) return rc;
   EnvT& E = D->R[i + 1];
   E.sec = cs;
@@ -1028,20 +1142,22 @@ int env_right(mrd_dmrg* D, mrd_heff* h, int i) {
     for (int c = 0; c < (int)cs.size(); ++c) {
       const int64_t off = E.off[(size_t)w * cs.size() + c];
       if (off < 0) continue;
-      const int cp = find_sec(cs, cs[c].N + cm[w][0], kmod(cs[c].K + cm[w][1], mod));
+      const int cp = img[(size_t)(w * ncs + c)];
       bool started = false;
       for (int sp = 0; sp < 2; ++sp) {
         const TB& tb = tblk[(size_t)(((int64_t)w * ncs + c) * 2 + sp)];
         if (tb.off < 0) continue;
-        int64_t bo, bld;
-        int bp;
-        if (!B.subblock(cp, sp, &bo, &bld, &bp)) continue;
+        const Sub& q = sub[(size_t)(cp * 2 + sp)];
+        if (q.b < 0) continue;
+        const int64_t bo = q.off, bld = q.ld;
+        const int bp = q.b;
         if (!started) { g2.task(cs[c].d, cs[cp].d, off, cs[cp].d); started = true; }
         // B-op: conj-transpose of the d_c' x d_b' sub-block
         g2.seg(tb.off, tb.cols, bo, bld, bs[bp].d, 2);
       }
     }
-  rc = run_gemm(D, g2, D->tbuf.as<double2>(), tlen, B.data.as<double2>(), B.size, eout.as<double2>(), E.size, t_ff);
+  rc = run_gemm(D, g2, D->tbuf.as<double2>(), tlen, B.data.as<double2>(), B.size, eout.as<double2>(), E.size,
+                t64 ? nullptr : t_ff, nullptr, nullptr, DG_BY_B, nullptr, digits && (t64 || !t_ff));
   if (rc != MRD_OK) return rc;
   return env_store(D, E, eout.as<double2>());
 }
@@ -1101,7 +1217,9 @@ int orthonormalise(mrd_dmrg* D, SiteT& T) {
 
 // Orthonormalise every tensor but the centre's (left of it left-canonical, right of it
 // right-canonical) and build the left environments up to the centre and the right ones down to
-// centre + 2 (the initial state of mrd_dmrg_create, or its real-valued version).
+// centre + 2 (the initial state of mrd_dmrg_create, or its real-valued version). The environments
+// come from the CUDA-core kernels, so that a seed names the same state bit for bit whichever
+// products its updates run on.
 int canonicalise_and_build_envs(mrd_dmrg* D, int center) {
   const int n = D->n;
   int rcd = MRD_OK;
@@ -1114,7 +1232,7 @@ int canonicalise_and_build_envs(mrd_dmrg* D, int center) {
     const double2* lj = nullptr;
     rcd = env_fp64(D, D->L[j], 0, &lj);
     if (rcd == MRD_OK) rcd = make_heff(D, j, lj, nullptr, &h);
-    if (rcd == MRD_OK) rcd = env_left(D, h, j);
+    if (rcd == MRD_OK) rcd = env_left(D, h, j, false);
     if (h) mrd_heff_free(h);
   }
   for (int j = n - 1; j >= center + 2 && rcd == MRD_OK; --j) {
@@ -1122,7 +1240,7 @@ int canonicalise_and_build_envs(mrd_dmrg* D, int center) {
     const double2* rj = nullptr;
     rcd = env_fp64(D, D->R[j + 1], 1, &rj);
     if (rcd == MRD_OK) rcd = make_heff(D, j - 1, nullptr, rj, &h);
-    if (rcd == MRD_OK) rcd = env_right(D, h, j - 1);
+    if (rcd == MRD_OK) rcd = env_right(D, h, j - 1, false);
     if (h) mrd_heff_free(h);
   }
   return rcd;
@@ -1321,6 +1439,9 @@ int mrd_two_site_update(mrd_dmrg* D, int32_t i, int32_t direction, const mrd_dmr
   // the device folds the environments, forms theta and converts the refinement's operands
   const bool tc = p->prec == MRD_PREC_TF32 || p->prec == MRD_PREC_BF16X3;
   if (tc) tc_prebuild(h, p->prec);
+  // likewise the plans of the FP64 / float-float products (the refinement's run beside the Lanczos)
+  h->dg_uses = tc ? p->refine_iter : p->lanczos_max_iter;
+  if (!tc || p->refine_iter > 0) dg_prebuild(h, tc ? p->refine_prec : p->prec);
   auto collect = [&](int which) {
     if (!D->timing) return;
     double a = 0, b = 0;
@@ -1338,7 +1459,6 @@ int mrd_two_site_update(mrd_dmrg* D, int32_t i, int32_t direction, const mrd_dmr
   lap(1);
   double e = 0.0;
   int32_t it = 0;
-  if (tc && p->refine_iter > 0 && p->refine_prec == MRD_PREC_FF && (rc = heff_prefetch_ff(h)) != MRD_OK) return rc;
   if ((rc = mrd_lanczos(h, (double*)theta, p->lanczos_max_iter, p->lanczos_tol, p->prec, &e, &it)) != MRD_OK) return rc;
   D->last_iters = it;
   for (int r = 0; r < p->lanczos_restarts && it == p->lanczos_max_iter; ++r) {
@@ -1417,9 +1537,11 @@ int mrd_two_site_update(mrd_dmrg* D, int32_t i, int32_t direction, const mrd_dmr
     return rc;
   const int64_t svd_ulen = D->svd_u.bytes / 16, svd_vlen = D->svd_vh.bytes / 16;
   if (direction > 0)
-    rc = run_gemm(D, proj, D->svd_u.as<double2>(), svd_ulen, theta, n, centre.data.as<double2>(), centre.size);
+    rc = run_gemm(D, proj, D->svd_u.as<double2>(), svd_ulen, theta, n, centre.data.as<double2>(), centre.size, nullptr,
+                  nullptr, nullptr, DG_BY_B, nullptr, false);
   else
-    rc = run_gemm(D, proj, theta, n, D->svd_vh.as<double2>(), svd_vlen, centre.data.as<double2>(), centre.size);
+    rc = run_gemm(D, proj, theta, n, D->svd_vh.as<double2>(), svd_vlen, centre.data.as<double2>(), centre.size, nullptr,
+                  nullptr, nullptr, DG_BY_B, nullptr, false);
   if (rc != MRD_OK) return rc;
   if (centre.size > 0) {
     MRD_CUDA(ctx, D->svd_x2.need((size_t)kNormParts * 8));
@@ -1466,9 +1588,9 @@ int mrd_two_site_update(mrd_dmrg* D, int32_t i, int32_t direction, const mrd_dmr
     D->schmidt_bond = i + 1;
   }
   lap(4);
-  if (direction > 0) rc = env_left(D, h, i);
-  else rc = env_right(D, h, i);
-  if (rc != MRD_OK) return rc;
+  if (direction > 0) rc = env_left(D, h, i, true);
+  else rc = env_right(D, h, i, true);
+  if (rc != MRD_OK || (rc = dg_check(D)) != MRD_OK) return rc;
   lap(5);
   D->last_energy = e;
   D->last_trunc = info[1];
@@ -1516,7 +1638,8 @@ int mrd_env_update(mrd_dmrg* D, int32_t site, int32_t direction, int32_t prec) t
   if (rc == MRD_OK)
     rc = direction > 0 ? make_heff(D, i, ein, nullptr, &h) : make_heff(D, i, nullptr, ein, &h);
   if (rc != MRD_OK) return rc;
-  rc = direction > 0 ? env_left(D, h, i) : env_right(D, h, i);
+  rc = direction > 0 ? env_left(D, h, i, true) : env_right(D, h, i, true);
+  if (rc == MRD_OK) rc = dg_check(D);
   mrd_heff_free(h);
   return rc;
 } catch (...) {   // host memory or threads exhausted: no exception crosses the C ABI

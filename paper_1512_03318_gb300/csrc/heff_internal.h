@@ -21,7 +21,14 @@ int tc_config(const mrd_heff* h, int32_t* cfg4);
 int autotune(mrd_heff* h, int prec);
 void tc_env_changed(mrd_heff* h);
 int tc_status(mrd_heff* h);
-int heff_prefetch_ff(mrd_heff* h);
+int heff_fold(mrd_heff* h, const double2* lenv, const double2* renv);
+struct DgHeff;
+void dg_heff_free(DgHeff* g);
+void dg_prebuild(mrd_heff* h, int32_t prec);
+int dg_prepare(mrd_heff* h, int32_t prec, bool* use);
+int dg_apply(mrd_heff* h, const double2* in, double2* out, int32_t prec, const cudaEvent_t ev[3], bool cap);
+void dg_env_changed(mrd_heff* h);
+int dg_status(mrd_heff* h);
 using mrd::Lanczos;
 using mrd::lanczos_free;
 using mrd::PlanDims;
@@ -104,6 +111,10 @@ struct mrd_heff {
   // tensor-core path state (tc_host.cu)
   struct Tc* tc = nullptr;
   struct TcPre* tc_pre = nullptr;   // panel tables being built on a host thread (tc_prebuild)
+  // digit-split products of the FP64 and float-float precisions (digits_host.cu)
+  DgHeff* dg = nullptr;
+  double dg_uses = 50.0;            // FP64 / float-float applications expected per environment load
+  bool dg_use = false;              // the last prepared FP64 / float-float application runs on them
   // float-float path: LW, WR in float-float layout (prepared after each environment load) and
   // theta staging
   Arena ff_mem;
@@ -125,6 +136,7 @@ struct mrd_heff {
   std::vector<int64_t> pt_tiles1, pt_tiles2;
   ~mrd_heff() {
     tc_pre_free(tc_pre);   // joins the thread, which reads the host tables
+    dg_heff_free(dg);      // the same
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
     for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : gev)
