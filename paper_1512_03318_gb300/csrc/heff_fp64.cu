@@ -126,26 +126,131 @@ __global__ void __launch_bounds__(256) k_cgemm_fp64(const double2* __restrict__ 
 // rows: LW or WR table (10 int64 per row); env_map: [channel][sector] -> env offset;
 // perm/idx/val: sorted MPO entries; chan_field: index of the env channel in an entry
 // (0 = w for W_i, 1 = w'' for W_{i+1}); sec_field: row field holding the env sector.
+//
+// The blocks lie one after another in `out`, and a CTA takes kFoldChunk consecutive elements of it,
+// whichever blocks they belong to, so that the few large blocks spread over the GPU like the many
+// small ones; the search for the first block and a block's entry tables (a chain of dependent
+// loads) are paid once per CTA and block. Most entries are real, and most blocks one entry of
+// value 1 (a channel that passes through): those take 2 and 0 of the 6 FP64 operations of a general
+// complex entry (the FP64 pipe has 2 lanes per SM), with the same rounding. Ly = 10, chi = 3200
+// (LW, WR: 0.82 GB written each): 0.49 + 0.40 ms; one CTA per block with every entry taken as
+// complex needed 1.4 + 0.9. (Testing every element for infinities inside its own branch instead
+// of four at once: 0.83 + 0.93.)
+constexpr int kFoldChunk = 8192, kFoldPer = 4, kFoldSub = kFoldPer * 256, kFoldTerms = 32;
+
+// An infinity or NaN takes the full product, zero times it included.
+__device__ __forceinline__ bool fold_odd(double2 x) {
+  constexpr int kExp = 0x7ff00000;
+  const int a = __double2hiint(x.x) & kExp, b = __double2hiint(x.y) & kExp;
+  return (a > b ? a : b) == kExp;
+}
+
+__device__ __forceinline__ void fold_full(double2& acc, double2 x, double2 v) {
+  acc.x += v.x * x.x - v.y * x.y;
+  acc.y += v.x * x.y + v.y * x.x;
+}
+
+__device__ __forceinline__ void fold_real(double2& acc, double2 x, double v, bool first) {
+  if (v == -1.0) x = make_double2(-x.x, -x.y);
+  else if (v != 1.0) x = make_double2(__dmul_rn(v, x.x), __dmul_rn(v, x.y));
+  acc = first ? x : make_double2(__dadd_rn(acc.x, x.x), __dadd_rn(acc.y, x.y));
+}
+
 __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ env, double2* __restrict__ out,
-                                                  const int64_t* __restrict__ rows, int64_t nrows,
+                                                  const int64_t* __restrict__ rows, int nrows, int64_t len,
                                                   const int64_t* __restrict__ env_map, int n_sec,
                                                   const int32_t* __restrict__ perm, const int32_t* __restrict__ idx,
                                                   const double* __restrict__ val, int chan_field) {
-  for (int64_t r = blockIdx.x; r < nrows; r += gridDim.x) {
-    const int64_t* row = rows + LWF * r;
-    const int64_t sec = row[3], n = row[5] * row[6], off = row[7], cb = row[8], ce = row[9];
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
+  __shared__ int64_t s_off[257];
+  __shared__ const double2* s_src[kFoldTerms];
+  __shared__ double2 s_val[kFoldTerms];
+  const int tid = threadIdx.x;
+  const int64_t base = (int64_t)blockIdx.x * kFoldChunk;
+  // the last block that starts at or before the chunk, by 256-way search
+  int lo = 0, hi = nrows;
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 255) / 256, i = lo + tid * step;
+    const int k = __syncthreads_count(i < hi && rows[(int64_t)LWF * i + 7] <= base);
+    lo += (k - 1) * step;
+    hi = hi < lo + step ? hi : lo + step;
+  }
+  for (int i = tid; i < 257; i += 256) s_off[i] = lo + i < nrows ? rows[(int64_t)LWF * (lo + i) + 7] : len;
+  __syncthreads();
+  int cur = -1;          // block whose terms are staged
+  int terms = 0;
+  int64_t cur_off = 0, cur_n = 0;
+  for (int64_t e0 = base; e0 < base + kFoldChunk && e0 < len; e0 += kFoldSub) {
+    int r = 0, top = 257;                // the last staged block that starts at or before e0
+    while (top - r > 1) {
+      const int m = (r + top) >> 1;
+      if (s_off[m] <= e0) r = m; else top = m;
+    }
+    const int64_t end = e0 + kFoldSub < len ? e0 + kFoldSub : len;
+    if (r < 256 && s_off[r + 1] >= end) {   // one block
+      if (r != cur) {
+        const int64_t* row = rows + (int64_t)LWF * (lo + r);
+        const int64_t cb = row[8];
+        __syncthreads();                    // the staged terms have been used
+        terms = (int)(row[9] - cb);
+        cur_off = row[7];
+        cur_n = row[5] * row[6];
+        cur = r;
+        if (tid < terms && tid < kFoldTerms) {
+          const int ent = perm[cb + tid];
+          s_src[tid] = env + env_map[(int64_t)idx[4 * ent + chan_field] * n_sec + row[3]];
+          s_val[tid] = make_double2(val[2 * ent], val[2 * ent + 1]);
+        }
+        __syncthreads();
+      }
+      if (terms <= kFoldTerms) {
+        const int64_t f = e0 - cur_off + tid;
+        double2 acc[kFoldPer];
+#pragma unroll
+        for (int q = 0; q < kFoldPer; ++q) acc[q] = make_double2(0.0, 0.0);
+        for (int c = 0; c < terms; ++c) {
+          const double2* src = s_src[c];
+          const double2 v = s_val[c];
+          double2 x[kFoldPer];
+#pragma unroll
+          for (int q = 0; q < kFoldPer; ++q) x[q] = f + q * 256 < cur_n ? src[f + q * 256] : make_double2(0.0, 0.0);
+          bool full = v.y != 0.0;
+#pragma unroll
+          for (int q = 0; q < kFoldPer; ++q) full |= fold_odd(x[q]);
+          if (full) {
+#pragma unroll
+            for (int q = 0; q < kFoldPer; ++q) fold_full(acc[q], x[q], v);
+          } else {
+#pragma unroll
+            for (int q = 0; q < kFoldPer; ++q) fold_real(acc[q], x[q], v.x, c == 0);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kFoldPer; ++q)
+          if (f + q * 256 < cur_n) out[cur_off + f + q * 256] = acc[q];
+        continue;
+      }
+    }
+    for (int64_t e = e0 + tid; e < end; e += 256) {   // several blocks: every element finds its own
+      int b = 0;
+      top = 257;
+      while (top - b > 1) {
+        const int m = (b + top) >> 1;
+        if (s_off[m] <= e) b = m; else top = m;
+      }
+      b += lo;
+      while (b + 1 < nrows && rows[(int64_t)LWF * (b + 1) + 7] <= e) ++b;   // beyond the staged ones
+      const int64_t* row = rows + (int64_t)LWF * b;
+      const int64_t off = row[7], sec = row[3], cb = row[8], ce = row[9];
+      if (e - off >= row[5] * row[6]) continue;
       double2 acc = make_double2(0.0, 0.0);
       for (int64_t c = cb; c < ce; ++c) {
         const int ent = perm[c];
-        const int ch = idx[4 * ent + chan_field];
-        const int64_t src = env_map[(int64_t)ch * n_sec + sec];
-        const double vr = val[2 * ent], vi = val[2 * ent + 1];
-        const double2 x = env[src + e];
-        acc.x += vr * x.x - vi * x.y;
-        acc.y += vr * x.y + vi * x.x;
+        const double2* src = env + env_map[(int64_t)idx[4 * ent + chan_field] * n_sec + sec];
+        const double2 x = src[e - off], v = make_double2(val[2 * ent], val[2 * ent + 1]);
+        if (v.y != 0.0 || fold_odd(x)) fold_full(acc, x, v);
+        else fold_real(acc, x, v.x, c == cb);
       }
-      out[off + e] = acc;
+      out[e] = acc;
     }
   }
 }
@@ -163,10 +268,10 @@ cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, co
 
 cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* rows, int64_t nrows,
                             const int64_t* env_map, int n_sec, const int32_t* perm, const int32_t* idx,
-                            const double* val, int chan_field, cudaStream_t s) {
-  if (nrows <= 0) return cudaSuccess;
-  int64_t grid = nrows < 65535 ? nrows : 65535;
-  k_fold_env<<<(unsigned)grid, 256, 0, s>>>(env, out, rows, nrows, env_map, n_sec, perm, idx, val, chan_field);
+                            const double* val, int chan_field, int64_t len, cudaStream_t s) {
+  if (nrows <= 0 || len <= 0) return cudaSuccess;
+  k_fold_env<<<(unsigned)((len + kFoldChunk - 1) / kFoldChunk), 256, 0, s>>>(env, out, rows, (int)nrows, len, env_map, n_sec,
+                                                                             perm, idx, val, chan_field);
   mrd::count_launch();
   return cudaGetLastError();
 }
