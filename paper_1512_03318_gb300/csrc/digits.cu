@@ -137,7 +137,10 @@ __device__ __forceinline__ int64_t panel_pos(bool tall, int prows, int nks, int 
 // threads along K, one 4-byte store per plane (a row's 32-byte segment per 8 threads);
 // row-contiguous pieces: units (chunk of 8 K values, row), consecutive threads along the rows,
 // one 16-byte store per plane. K positions beyond the block are written as zeros.
-// 16 bytes read and 32 written per complex element; the digits take ~50 instructions per real.
+// 16 bytes read and 32 written per complex element; the digits take ~45 instructions per real.
+// Ly = 10, chi = 3200: LW (51 M elements) 0.52 ms, WR 0.76, Z (78 M) 0.81, 0.4-0.7 of the copy
+// bandwidth. Units of 4 K values (8-byte stores) and of a whole panel step (32-byte stores) hold
+// twice the registers: 0.52, 0.85 and 0.76 ms there, but 120 against 93 us for Z at chi = 1024.
 template <int BETA, bool REAL>
 __global__ void __launch_bounds__(256) k_dg_pack(const double2* __restrict__ src, uint8_t* __restrict__ dst,
                                                  const DgJob* __restrict__ jobs, const int2* __restrict__ pieces,
@@ -289,40 +292,56 @@ __device__ __forceinline__ void tmem_ld4(uint32_t* v, uint32_t taddr) {
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr));
 }
 
-// Results outside the normal range: r 2^e, r < 2^54.
-__device__ __noinline__ double scaled_slow(unsigned long long r, int e) { return ldexp((double)(long long)r, e); }
-
-// (hi 2^(4 BETA) + lo) 2^ex as a double, rounded to nearest, in integer arithmetic; lo in
-// [0, 2^(4 BETA)). Not inlined: the epilogue converts 32 numbers per thread, and as unrolled
-// copies of this the kernel ran out of the instruction caches (2.7 of ~10 stall cycles per
-// instruction were instruction misses).
+// (hi 2^(4 BETA) + lo) 2^ex as a double, rounded to nearest, in integer arithmetic (the FP64 pipe
+// would take 4 operations per number at 2 lanes per SM); lo in [0, 2^(4 BETA)). Without branches,
+// so that the 32 conversions of a thread overlap: with the rare cases inside, a tile's conversions
+// and stores took 12,000 cycles. `odd` is set when the result is outside the normal range (the value
+// returned is then meaningless).
 template <int BETA>
-__device__ __noinline__ double to_double(long long hi, uint32_t lo, int ex) {
-  const uint32_t sg = (uint32_t)(hi >> 63);   // 0 or all ones
+__device__ __forceinline__ void leading_bits(long long hi, uint32_t lo, int ex, uint32_t& sg, unsigned long long& r, int& e2) {
+  sg = (uint32_t)(hi >> 63);                  // 0 or all ones
   uint32_t c = lo << (32 - 4 * BETA);         // value = (a b c) 2^(ex + 4 BETA - 32) as 96 bits
   uint32_t b = (uint32_t)hi, a = (uint32_t)((unsigned long long)hi >> 32);
-  {   // absolute value
-    const unsigned long long low = (((unsigned long long)b << 32 | c) ^ ((unsigned long long)sg << 32 | sg)) + (sg & 1);
-    a = (a ^ sg) + ((sg & 1) && low == 0 ? 1u : 0u);
-    b = (uint32_t)(low >> 32);
-    c = (uint32_t)low;
-  }
-  int e2 = ex + 4 * BETA - 32 + 95;           // exponent of bit 95
-  if (a == 0) {
-    a = b; b = c; c = 0; e2 -= 32;
-    if (a == 0) { a = b; b = 0; e2 -= 32; }
-    if (a == 0) return 0.0;
+  const unsigned long long low = (((unsigned long long)b << 32 | c) ^ ((unsigned long long)sg << 32 | sg)) + (sg & 1);
+  a = (a ^ sg) + (low == 0 ? (sg & 1) : 0u);
+  b = (uint32_t)(low >> 32);
+  c = (uint32_t)low;
+  e2 = ex + 4 * BETA - 32 + 95;               // exponent of bit 95
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const bool z = a == 0;
+    a = z ? b : a;
+    b = z ? c : b;
+    c = z ? 0 : c;
+    e2 -= z ? 32 : 0;
   }
   const int lz = __clz((int)a);
   const uint32_t m1 = __funnelshift_l(b, a, lz), m0 = __funnelshift_l(c, b, lz);
   e2 -= lz;
   const unsigned long long m = (unsigned long long)m1 << 32 | m0;
-  const unsigned long long r = (m >> 11) + ((m >> 10) & 1);
-  double v;
-  if (e2 >= -1022 && e2 < 1023)
-    v = __longlong_as_double((long long)(((unsigned long long)(e2 + 1022) << 52) + r));
-  else
-    v = scaled_slow(r, e2 - 52);
+  r = (m >> 11) + ((m >> 10) & 1);
+}
+
+template <int BETA>
+__device__ __forceinline__ double to_double(long long hi, uint32_t lo, int ex, bool& odd) {
+  uint32_t sg;
+  unsigned long long r;
+  int e2;
+  leading_bits<BETA>(hi, lo, ex, sg, r, e2);
+  const bool zero = (hi | (long long)lo) == 0;
+  odd = odd || (!zero && (unsigned)(e2 + 1022) >= 2045u);
+  const unsigned long long bits = ((unsigned long long)(uint32_t)(e2 + 1022) << 52) + r + ((unsigned long long)(sg & 1) << 63);
+  return __longlong_as_double(zero ? 0ll : (long long)bits);
+}
+
+template <int BETA>
+__device__ __noinline__ double to_double_slow(long long hi, uint32_t lo, int ex) {
+  if (hi == 0 && lo == 0) return 0.0;
+  uint32_t sg;
+  unsigned long long r;
+  int e2;
+  leading_bits<BETA>(hi, lo, ex, sg, r, e2);
+  const double v = ldexp((double)(long long)r, e2 - 52);
   return sg ? -v : v;
 }
 
@@ -527,7 +546,7 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
       // while the MMAs run
       const int* ea = q.tall_op ? g.eb : g.ea;
       const int* eb = q.tall_op ? g.ea : g.eb;
-      const bool by_row = q.cm_rows != 0;
+      const bool by_row = q.cm_rows;
       int er = 0, ec = 0;
       longlong2 map = {0, 0};
       if (row < R) er = ea[q.ea + row];
@@ -611,17 +630,29 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
         }
       }
       const int exr = er - 2 * 1022 + (BETA == 8 ? -68 : -61);
+      bool odd = false;   // a result outside the normal range, or a row or column that is not finite
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
         const int eg = __shfl_sync(0xffffffffu, ec, c);
-        long long at = by_row ? map.x + (long long)(col0 + c) * map.y
-                              : __shfl_sync(0xffffffffu, map.x, c) + (long long)row * __shfl_sync(0xffffffffu, map.y, c);
-        if (row < R && c < w && col0 + c < N) {
-          double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], exr + eg),
-                                   REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg));
-          if (er == 2047 || eg == 2047)   // an infinity or NaN in the row or column
-            o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);
-          g.c[at] = o;
+        const long long at = by_row ? map.x + (long long)(col0 + c) * map.y
+                                    : __shfl_sync(0xffffffffu, map.x, c) + (long long)row * __shfl_sync(0xffffffffu, map.y, c);
+        const double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], exr + eg, odd),
+                                       REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg, odd));
+        odd = odd || eg == 2047;
+        if (row < R && c < w && col0 + c < N) g.c[at] = o;
+      }
+      if (__any_sync(0xffffffffu, (odd || er == 2047) && row < R)) {   // rare: convert again, with care
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const int eg = __shfl_sync(0xffffffffu, ec, c);
+          const long long at = by_row ? map.x + (long long)(col0 + c) * map.y
+                                      : __shfl_sync(0xffffffffu, map.x, c) + (long long)row * __shfl_sync(0xffffffffu, map.y, c);
+          if (row < R && c < w && col0 + c < N) {
+            double2 o = make_double2(to_double_slow<BETA>(hi[0][c], lo[0][c], exr + eg),
+                                     REAL ? 0.0 : to_double_slow<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg));
+            if (er == 2047 || eg == 2047) o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);
+            g.c[at] = o;
+          }
         }
       }
     }

@@ -235,21 +235,18 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
     const int tm = (d.R + kDgRows - 1) / kDgRows, tn = (d.N + kDgCols - 1) / kDgCols;
     if (group_major)
       while ((int32_t)p.item0.size() <= c.group) p.item0.push_back((int64_t)p.items.size());
-    for (int r = 0; r < tm; ++r)
-      for (int ct = c.ct0; ct < c.ct1; ++ct) {
-        const int tile = r * tn + ct;
-        if (c.parts == 1) {
-          p.items.push_back({c.group, tile, d.nks << 16, -1});
-          continue;
-        }
-        const int sid = (int)p.splits.size();
-        p.splits.push_back(make_int2((int)p.slots, c.parts));
-        p.slots += c.parts;
-        for (int q = 0; q < c.parts; ++q) {
-          const int k0 = (int)((int64_t)d.nks * q / c.parts), k1 = (int)((int64_t)d.nks * (q + 1) / c.parts);
-          p.items.push_back({c.group, tile, k0 | k1 << 16, sid * 64 + q});
-        }
-      }
+    // the tiles of one K range follow each other: CTAs that run together then read the same rows and
+    // columns of the panels, which come from DRAM once
+    const int sid = (int)p.splits.size(), wide = c.ct1 - c.ct0;
+    if (c.parts > 1)
+      for (int q = 0; q < tm * wide; ++q, p.slots += c.parts) p.splits.push_back(make_int2((int)p.slots, c.parts));
+    for (int q = 0; q < c.parts; ++q) {
+      const int k0 = (int)((int64_t)d.nks * q / c.parts), k1 = (int)((int64_t)d.nks * (q + 1) / c.parts);
+      for (int r = 0; r < tm; ++r)
+        for (int ct = c.ct0; ct < c.ct1; ++ct)
+          p.items.push_back({c.group, r * tn + ct, k0 | k1 << 16,
+                             c.parts > 1 ? (sid + r * wide + ct - c.ct0) * 64 + q : -1});
+    }
   }
   if (group_major) p.item0.push_back((int64_t)p.items.size());
   p.cost = total / n_sm + 0.5 * longest + 12000.0;
