@@ -157,7 +157,7 @@ int mrd_heff_set_env(mrd_heff* h, const double* lenv_dev, const double* renv_dev
  * MRD_PREC_FP64 runs grouped GEMMs of FP64 accuracy, MRD_PREC_FF the same grouped GEMMs in
  * float-float arithmetic (~1e-13 relative or better); MRD_PREC_TF32 and MRD_PREC_BF16X3 run the same
  * contraction on the tcgen05 tensor cores with FP32 accumulation (complex products as four
- * real ones), operands repacked into 128-byte swizzled tiles: the folded environments once
+ * real ones), operands repacked into swizzled tiles of 32-byte rows: the folded environments once
  * after each mrd_heff_set_env, theta on every call; the result is returned in complex128. */
 int mrd_heff_apply(mrd_heff* h, const double* theta_in_dev, double* theta_out_dev, int32_t prec);
 /* Real flops of one H_eff application (8 per complex multiply-add), written to flops4:
@@ -207,8 +207,8 @@ int mrd_heff_set_option(mrd_heff* h, int32_t option, int64_t value);
 /* Wait for the context stream and report a device-side wait of a tensor-core GEMM that gave
  * up since the last check: MRD_E_TIMEOUT (the flag is then cleared), else 0. */
 int mrd_heff_status(mrd_heff* h);
-/* Tensor-core tile configuration in use: cfg4 = {columns per tile, pipeline stages, task
- * order (0: charge order, 1: largest work first), source (0: default, 1: tuned on this
+/* Tensor-core tile configuration in use: cfg4 = {columns per tile (step 2 may take fewer), pipeline
+ * depth in tiles of 128 bytes of K, task order (0: charge order, 1: largest work first), source (0: default, 1: tuned on this
  * H_eff, 2: tuned earlier on the context)}; all -1 before the first tensor-core application. */
 int mrd_heff_tc_config(const mrd_heff* h, int32_t* cfg4);
 int mrd_heff_timing_collect(mrd_heff* h, double* ms_step1, double* ms_step2, int32_t* n_calls);

@@ -4,7 +4,6 @@
 #include <algorithm>
 #include <map>
 #include <new>
-#include <queue>
 #include <thread>
 #include <vector>
 
@@ -12,13 +11,13 @@
 #include "tc.cuh"
 
 namespace mrd {
-cudaError_t tc_pack(const double2* src, uint8_t* dst, const int64_t* jobs, int njobs, int64_t npieces, int prec,
-                    cudaStream_t s);
+cudaError_t tc_pack(const double2* src, uint8_t* dst, const int64_t* jobs, int njobs, int64_t npieces, int prec, int* ctr,
+                    int* bad, cudaStream_t s);
 cudaError_t tc_gemm_init();
-cudaError_t tc_gemm(const uint8_t* a_base, const uint8_t* b_base, const int64_t* tasks, const int64_t* segs,
-                    const int64_t* prefix, const int2* items, const int32_t* cta_off, const int64_t* rowmap,
-                    int64_t n_tasks, int64_t total_tiles, uint8_t* z_out, double2* f_out, int prec, TcCfg cfg,
-                    int* err, int n_sm, uint64_t wait_ns, cudaStream_t s);
+cudaError_t tc_gemm(const uint8_t* a_base, const uint8_t* b_base, const TcItem* items, int count, const TcItem* alt,
+                    int alt_count, const int* bad, const TcSeg* segs,
+                    const int64_t* rowmap, uint8_t* z_out, double2* f_out, int prec, TcCfg cfg, int ntile, int* ctr, int* err, int n_sm,
+                    uint64_t wait_ns, cudaStream_t s);
 }  // namespace mrd
 
 struct Tc {
@@ -28,19 +27,20 @@ struct Tc {
   bool env_dirty = true;
   Arena mem;
   uint8_t *lw = nullptr, *wr = nullptr, *th = nullptr, *z = nullptr;
-  int64_t lw_bytes = 0, wr_bytes = 0, th_bytes = 0, z_bytes = 0;
-  int64_t *t1 = nullptr, *s1 = nullptr, *p1 = nullptr, *t2 = nullptr, *s2 = nullptr, *p2 = nullptr;
-  int64_t n1 = 0, ntiles1 = 0, n2 = 0, ntiles2 = 0;
+  TcItem *it1 = nullptr, *it2 = nullptr;   // tiles of the two steps, longest first
+  TcSeg *s1 = nullptr, *s2 = nullptr;
+  int n_it1 = 0, n_it2 = 0, ntile2 = 0;
+  TcItem* alt2 = nullptr;                  // step-2 tiles that keep each row to its own K segments
+  int n_alt2 = 0;
+  std::vector<int32_t> task1, task2, taska; // first tile of every task, + total (per-task launches)
+  int64_t* rmap1 = nullptr;                // step-1 row map (tc_rowmap)
   int64_t *j_lw = nullptr, *j_wr = nullptr, *j_th = nullptr;
   int n_lw = 0, n_wr = 0, n_th = 0;
-  int64_t pc_lw = 0, pc_wr = 0, pc_th = 0;   // pack pieces of each job list
-  // per-task launches: [0, tiles of task t] pairs (device) and tiles per task (host)
-  int64_t *pt1 = nullptr, *pt2 = nullptr;
-  std::vector<int64_t> tiles1, tiles2;
-  int2 *it1 = nullptr, *it2 = nullptr;   // item tables of the grouped launches
-  int32_t *co1 = nullptr, *co2 = nullptr; // first item of each CTA in them (grid + 1 entries)
-  int64_t* rmap1 = nullptr;               // step-1 row map: (Z panel byte offset << 16) | row in panel
-  int* err = nullptr;
+  int64_t pc_lw = 0, pc_wr = 0, pc_th = 0; // pack pieces of each job list
+  bool zero_out = true;                    // some output blocks receive no product
+  int* words = nullptr;                    // tile counters of the two steps, error flag, WR not finite
+  int* err() const { return words + 2; }
+  int* bad() const { return words + 3; }
 };
 
 void tc_free(Tc* t) { delete t; }
@@ -57,7 +57,7 @@ namespace {
 int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
 struct Panel {
-  int64_t off, nkt;
+  int64_t off, nks;
 };
 
 // Panels keyed by the FP64 element offset of their block: appended in build order, sorted once
@@ -80,9 +80,12 @@ struct PanelIndex {
   }
 };
 
-// bytes of an A panel (128-row tiles) or a B panel (ntile-row tiles, rows padded to 16)
-int64_t a_bytes(int64_t rows, int64_t nkt, int planes) { return round_up(rows, 128) * nkt * planes * 128; }
-int64_t b_bytes(int64_t rows, int64_t nkt, int planes) { return round_up(rows, 16) * nkt * planes * 128; }
+// bytes of an A panel (128-row tiles) or a B panel (ntile-row tiles)
+int64_t a_bytes(int64_t rows, int64_t nks, int prec) { return tc_apad(rows) * nks * tc_aplanes(prec) * 32; }
+int64_t b_bytes(int64_t rows, int64_t nks, int prec, int ntile) {
+  const int64_t full = rows / ntile, rest = tc_bpad(rows - full * ntile);
+  return (full * ntile * tc_bplanes(prec, ntile) + rest * tc_bplanes(prec, (int)rest)) * nks * 32;
+}
 
 // Host tables of the tensor-core path for one precision and tile configuration: panel
 // layouts, pack jobs, tasks, segments, row map and the per-CTA item deal. Built without any
@@ -91,19 +94,121 @@ struct TcTables {
   int prec = 0;
   TcCfg cfg{0, 0, 0};
   int n_sm = 0;
-  std::vector<int64_t> j_lw, j_wr, j_th, t1, s1, p1, t2, s2, p2, q1, q2, rowmap;
-  std::vector<int2> i1, i2;
-  std::vector<int32_t> co1, co2;
+  std::vector<int64_t> j_lw, j_wr, j_th, rowmap;
+  std::vector<TcSeg> s1, s2;
+  int ntile2 = 0;              // columns per tile of step 2 (WR panels), at most cfg.ntile
+  std::vector<TcItem> i1, i2, ia;
+  std::vector<int32_t> task1, task2, taska;
   int64_t lw_b = 0, wr_b = 0, th_b = 0, z_b = 0, pc_lw = 0, pc_wr = 0, pc_th = 0;
+  bool zero_z = false, zero_out = false;   // rows of Z that are read but not written; blocks of the output
   const char* err = nullptr;   // why the tables could not be built
 };
+
+// A stacked product: M x N outputs, K segments seg0 .. seg0 + nseg - 1 of nks steps in all. Rows from
+// `cut` on may have other segments than the ones before (part 0 and 1: psg0, pseg, pnks; their union is the
+// task's): 0 if all rows have the same.
+struct TcTask {
+  int64_t M, N, out, ld;   // out, ld: TcItem (of the task's first tile)
+  int32_t seg0, nseg;
+  int64_t nks;
+  int64_t cut;
+  int32_t psg0[2], pseg[2];
+  int64_t pnks[2];
+};
+
+// Tiles of the tasks, tasks by decreasing K steps (equal ones in task order, or, for order 1, by
+// decreasing work), which is the order in which the CTAs take them. alt: the tiles that compute the
+// same outputs with every row's own segments only.
+void cut_tiles(std::vector<TcTask>& tasks, int ntile, int order, bool z_out, const std::vector<TcSeg>& segs, std::vector<TcItem>& items,
+               std::vector<int32_t>& first, std::vector<TcItem>* alt = nullptr, std::vector<int32_t>* afirst = nullptr) {
+  const int64_t nt = ntile;
+  auto tiles = [&](const TcTask& t) { return ((t.M + 127) / 128) * ((t.N + nt - 1) / nt); };
+  if (order == 1)
+    std::stable_sort(tasks.begin(), tasks.end(),
+                     [&](const TcTask& a, const TcTask& b) { return tiles(a) * a.nks > tiles(b) * b.nks; });
+  std::stable_sort(tasks.begin(), tasks.end(), [](const TcTask& a, const TcTask& b) { return a.nks > b.nks; });
+  int64_t n = 0;
+  for (const TcTask& t : tasks) n += tiles(t);
+  items.reserve((size_t)n);
+  auto cut = [&](std::vector<TcItem>& v, const TcTask& t, int64_t lo, int64_t hi, int32_t seg0, int32_t nseg, int64_t nks) {
+    if (nseg == 0) return;
+    for (int64_t r = lo / 128 * 128; r < hi; r += 128)
+      for (int64_t c = 0; c < t.N; c += nt) {
+        const int64_t rows = std::min<int64_t>(hi - r, 128), cols = std::min<int64_t>(t.N - c, nt);
+        v.push_back({(int32_t)tc_bpad(cols), (int32_t)tc_apad(std::min<int64_t>(t.M - r, 128)), (int32_t)rows, (int32_t)cols,
+                     seg0, nseg, (int32_t)(r / 128), (int32_t)(c / nt), z_out ? t.out + r : t.out + r * t.ld + c, t.ld,
+                     (int32_t)std::max<int64_t>(lo - r, 0), (int32_t)nks, 0,
+                     {segs[(size_t)seg0], segs[(size_t)(nseg > 1 ? seg0 + 1 : seg0)]}});
+      }
+  };
+  for (const TcTask& t : tasks) {
+    first.push_back((int32_t)items.size());
+    cut(items, t, 0, t.M, t.seg0, t.nseg, t.nks);
+    if (!alt) continue;
+    afirst->push_back((int32_t)alt->size());
+    if (t.cut == 0) {
+      cut(*alt, t, 0, t.M, t.seg0, t.nseg, t.nks);
+    } else {
+      cut(*alt, t, 0, t.cut, t.psg0[0], t.pseg[0], t.pnks[0]);
+      cut(*alt, t, t.cut, t.M, t.psg0[1], t.pseg[1], t.pnks[1]);
+    }
+  }
+  first.push_back((int32_t)items.size());
+  if (alt) afirst->push_back((int32_t)alt->size());
+}
+
+// Columns per tile of step 2. Its tiles have long and unequal K (every channel of an output sector),
+// and K is not cut (the FP32 sums keep their order), so with few sectors the longest tile sets the
+// time: narrower tiles finish it sooner, and cost more in all (the 128 rows of A are multiplied for
+// fewer columns). Estimated cycles: per K step of a tile its MMAs (max(48, N / 2) each) and a share of
+// the slots' hand-over; the choice minimises the larger of the longest tile and the average load of a
+// CTA, plus half of the latter for the uneven rest. Measured us of step 2 (16 / 32 / 48 / 64 columns):
+// BF16X3 Ly = 8, chi = 1024 68 / 60 / 65 / 64, Ly = 10, chi = 3200 632 / 348 / 317 / 292; TF32 Ly = 8,
+// chi = 2049 222 / 146 / 111 / 115; real BF16X3 Ly = 6, chi = 777 32.8 / 32.8 / 34.6 / 34.9 (128: 37.0).
+int step2_columns(const mrd_heff* h, int prec, int ntile) {
+  auto cost = [&](int64_t n) {   // cycles per K step of a tile of n columns (padded to 16)
+    const double wide = std::max(48.0, tc_aplanes(prec) * n / 2.0), half = std::max(48.0, tc_aplanes(prec) * n / 4.0);
+    const int ap = tc_aplanes(prec);
+    const double m = tc_is_real(prec) || tc_neg_planes(prec, (int)n) ? ap * wide : ap / 2 * wide + ap * half;
+    return m + 600.0 / tc_group(prec);
+  };
+  const int kst = tc_kstep(prec);
+  int best = ntile;
+  double best_t = -1.0;
+  for (int n = ntile; n >= 16; n = n > 64 ? 64 : n - 16) {
+    double longest = 0.0, total = 0.0;
+    for (int64_t m = 0; m < h->counts[C_NMID]; ++m) {
+      const int64_t* rout = &h->mid_host[MIDF * m];
+      for (int s2p = 0; s2p < 2; ++s2p) {
+        if (rout[8 + s2p] < 0) continue;
+        int64_t ks = 0;
+        for (int s1p = 0; s1p < 2; ++s1p) {   // (about the union of the two lists)
+          const int64_t* t = &h->t2_host[TF * ((m * 2 + s1p) * 2 + s2p)];
+          int64_t k = 0;
+          for (int64_t q = 0; q < t[5]; ++q) k += (h->s2_host[SF * (t[4] + q) + 4] + kst - 1) / kst;
+          ks = std::max(ks, k);
+        }
+        const int64_t N = h->right[3 * rout[8 + s2p] + 2], rows = (rout[2] + 127) / 128;
+        const int64_t rest = tc_bpad(N % n);
+        total += rows * ks * ((N / n) * cost(n) + (rest ? cost(rest) : 0.0));
+        longest = std::max(longest, ks * cost(std::min<int64_t>(n, tc_bpad(N))));
+      }
+    }
+    const double load = total / std::max(h->n_sm, 1), t = std::max(longest, load) + 0.5 * load;
+    if (best_t < 0.0 || t < best_t) { best_t = t; best = n; }
+  }
+  return best;
+}
 
 bool tables(const mrd_heff* h, int prec, TcCfg cfg, TcTables& o) {
   auto fail = [&](const char* m) { o.err = m; return false; };
   o.prec = prec;
   o.cfg = cfg;
   o.n_sm = h->n_sm;
-  const int aplanes = tc_aplanes(prec), bplanes = tc_bplanes(prec), kpt = tc_kpt(prec), ntile = cfg.ntile;
+  if (!tc_cfg_ok(prec, cfg)) return fail("tc: tile configuration does not fit");
+  const int kst = tc_kstep(prec), ntile = cfg.ntile, ntile2 = step2_columns(h, prec, cfg.ntile);
+  o.ntile2 = ntile2;
+  auto steps = [&](int64_t K) { return (K + kst - 1) / kst; };
   const int64_t* c = h->counts;
   PanelIndex wr_map, th_map, z_map;
   wr_map.v.reserve(c[C_NWR]);
@@ -111,12 +216,13 @@ bool tables(const mrd_heff* h, int prec, TcCfg cfg, TcTables& o) {
   int64_t &lw_b = o.lw_b, &wr_b = o.wr_b, &th_b = o.th_b, &z_b = o.z_b;
   // (the folded left operand LW is packed below, stacked by input middle sector)
   // folded right operand WR(w', s2, s2', b): B panel of its transpose, rows d_b', K d_b
+  j_wr.reserve((size_t)c[C_NWR] * TCJ);
   for (int64_t k = 0; k < c[C_NWR]; ++k) {
     const int64_t* r = &h->wr_host[WRF * k];
-    const int64_t K = r[5], rows = r[6], nkt = (K + kpt - 1) / kpt;
-    wr_map.add(r[7], {wr_b, nkt});
-    j_wr.insert(j_wr.end(), {r[7], rows, 1, rows, K, wr_b, ntile, nkt, round_up(rows, 16), 0, 1, 0, 0});
-    wr_b += b_bytes(rows, nkt, bplanes);
+    const int64_t K = r[5], rows = r[6], nks = steps(K);
+    wr_map.add(r[7], {wr_b, nks});
+    j_wr.insert(j_wr.end(), {r[7], rows, 1, rows, K, wr_b, ntile2, nks, rows, 0, 0});
+    wr_b += b_bytes(rows, nks, prec, ntile2);
   }
   // theta block (s1, a) x (s2, b) of every middle sector: B panel of its transpose, rows d_b, K d_a
   const std::vector<int64_t>& mid = h->mid_host;
@@ -124,65 +230,102 @@ bool tables(const mrd_heff* h, int prec, TcCfg cfg, TcTables& o) {
     const int64_t* r = &mid[MIDF * m];
     for (int s1 = 0; s1 < 2; ++s1) {
       if (r[5 + s1] < 0) continue;
-      const int64_t K = h->left[3 * r[5 + s1] + 2], nkt = (K + kpt - 1) / kpt;
+      const int64_t K = h->left[3 * r[5 + s1] + 2], nks = steps(K);
       for (int s2 = 0; s2 < 2; ++s2) {
         if (r[8 + s2] < 0) continue;
         const int64_t rows = h->right[3 * r[8 + s2] + 2];
         const int64_t src = r[4] + (s1 ? r[7] : 0) * r[3] + (s2 ? r[10] : 0);
-        th_map.add(src, {th_b, nkt});
-        j_th.insert(j_th.end(), {src, r[3], 1, rows, K, th_b, ntile, nkt, round_up(rows, 16), 0, 1, 0, 0});
-        th_b += b_bytes(rows, nkt, bplanes);
+        th_map.add(src, {th_b, nks});
+        j_th.insert(j_th.end(), {src, r[3], 1, rows, K, th_b, ntile, nks, rows, 0, 0});
+        th_b += b_bytes(rows, nks, prec, ntile);
       }
     }
   }
-  // Z(w', m_in) rows (s1') x columns (s2): A panels keyed by their FP64 element offset
+  // Z(w', m_in), columns s2: A panels with the rows of both s1' under each other, keyed by their FP64
+  // element offset (row 0). Rows that no LW block feeds (s1mask) are zeros.
   const std::vector<int64_t>& z = h->z_host;   // downloaded with the other tables at creation
   if ((int64_t)z.size() < ZF * c[C_NZ]) return fail("tc: Z table missing");
   const int64_t nmid = c[C_NMID];
+  z_map.v.reserve((size_t)c[C_NZ] * 2);
   for (int64_t k = 0; k < c[C_NZ]; ++k) {
     const int64_t* zr = &z[ZF * k];
-    const int64_t wp = zr[0], mi = zr[1], mo = zr[2];
-    const int64_t* rin = &mid[MIDF * mi];
-    const int64_t* rout = &mid[MIDF * mo];
-    for (int s1p = 0; s1p < 2; ++s1p) {
-      const int64_t ti = (wp * nmid + mi) * 2 + s1p;
-      if (h->t1_host[TF * ti + 5] == 0) continue;   // no rows of this part written
-      const int64_t rows = h->left[3 * rout[5 + s1p] + 2];
-      for (int s2 = 0; s2 < 2; ++s2) {
-        if (rin[8 + s2] < 0) continue;
-        const int64_t K = h->right[3 * rin[8 + s2] + 2], nkt = (K + kpt - 1) / kpt;
-        const int64_t key = zr[5] + (s1p ? rout[7] : 0) * rin[3] + (s2 ? rin[10] : 0);
-        z_map.add(key, {z_b, nkt});
-        z_b += a_bytes(rows, nkt, aplanes);
-      }
+    const int64_t* rin = &mid[MIDF * zr[1]];
+    const int64_t* rout = &mid[MIDF * zr[2]];
+    for (int s1p = 0; s1p < 2; ++s1p)
+      if (rout[5 + s1p] >= 0 && h->t1_host[TF * ((zr[0] * nmid + zr[1]) * 2 + s1p) + 5] == 0) o.zero_z = true;
+    for (int s2 = 0; s2 < 2; ++s2) {
+      if (rin[8 + s2] < 0) continue;
+      const int64_t nks = steps(h->right[3 * rin[8 + s2] + 2]);
+      z_map.add(zr[5] + (s2 ? rin[10] : 0), {z_b, nks});
+      z_b += a_bytes(zr[3], nks, prec);
     }
   }
   wr_map.finish();
   th_map.finish();
   z_map.finish();
-  std::vector<int64_t>&t1 = o.t1, &s1 = o.s1, &p1 = o.p1, &t2 = o.t2, &s2 = o.s2, &p2 = o.p2;
-  p1.assign(1, 0);
-  p2.assign(1, 0);
+  for (const PanelIndex* m : {&wr_map, &th_map, &z_map})
+    for (const auto& e : m->v)
+      if (e.second.nks > 0xffff) return fail("tc: sector dimension too large");
+  auto seg = [](const Panel& a, const Panel& b) { return TcSeg{a.off, b.off / 256 << 16 | b.nks}; };
   // step-2 tasks (theta' = sum Z WR), built on a second host thread while this one builds the
-  // step-1 tasks: the two loops share only the finished (read-only) panel indexes
+  // step-1 tasks: the two loops share only the finished (read-only) panel indexes. A task is an
+  // output block column (m_out, s2') with the rows of both s1' (twice the rows per tile for the same
+  // WR): its segments are those of either, in the tables' order (w', s2), which both lists have;
+  // rows that lack one meet zeros of Z there. Zero times an infinity or NaN of WR would not be
+  // nothing: when WR holds one, the kernel runs the tiles of the two lists by themselves.
   bool step2_ok = true;
+  std::vector<TcTask> tasks1, tasks2;
   auto build_step2 = [&] {
-    for (int64_t i = 0; i < c[C_NT2]; ++i) {
-      const int64_t* t = &h->t2_host[TF * i];
-      if (t[5] == 0 || t[0] == 0 || t[1] == 0) continue;
-      const int64_t seg0 = (int64_t)s2.size() / TCS;
-      for (int64_t k = 0; k < t[5]; ++k) {
-        const int64_t* sg = &h->s2_host[SF * (t[4] + k)];
-        const Panel* a = z_map.find(sg[0]);
-        const Panel* b = wr_map.find(sg[2]);
-        if (!a || !b || a->nkt != b->nkt) {
-          step2_ok = false;
-          return;
+    std::vector<TcSeg> part[2];
+    for (int64_t m = 0; m < nmid; ++m) {
+      const int64_t* rout = &mid[MIDF * m];
+      for (int s2p = 0; s2p < 2; ++s2p) {
+        if (rout[8 + s2p] < 0) continue;
+        const int64_t *t[2], *sg[2];
+        int64_t n[2];
+        for (int s1p = 0; s1p < 2; ++s1p) {
+          t[s1p] = &h->t2_host[TF * ((m * 2 + s1p) * 2 + s2p)];
+          n[s1p] = t[s1p][0] && t[s1p][1] ? t[s1p][5] : 0;
+          sg[s1p] = h->s2_host.data() + SF * t[s1p][4];
+          part[s1p].clear();
         }
-        s2.insert(s2.end(), {a->off, b->off, a->nkt, 0});
+        const int64_t N = h->right[3 * rout[8 + s2p] + 2];
+        TcTask k{rout[2], N, rout[4] + (s2p ? rout[10] : 0), rout[3], (int32_t)o.s2.size(), 0, 0, 0, {0, 0}, {0, 0}, {0, 0}};
+        int64_t last = -1, i[2] = {0, 0};
+        while (i[0] < n[0] || i[1] < n[1]) {
+          int64_t key[2] = {INT64_MAX, INT64_MAX};   // Z panel of either list's next segment
+          for (int q = 0; q < 2; ++q)
+            if (i[q] < n[q]) key[q] = sg[q][SF * i[q]] - (q ? rout[7] : 0) * sg[q][SF * i[q] + 1];
+          const int64_t next = std::min(key[0], key[1]), wr = sg[key[0] == next ? 0 : 1][SF * i[key[0] == next ? 0 : 1] + 2];
+          const Panel* a = z_map.find(next);
+          const Panel* b = wr_map.find(wr);
+          if (!a || !b || a->nks != b->nks || next <= last) { step2_ok = false; return; }
+          last = next;
+          for (int q = 0; q < 2; ++q) {
+            if (key[q] != next) continue;
+            if (sg[q][SF * i[q] + 2] != wr) { step2_ok = false; return; }
+            if (a->nks > 0) part[q].push_back(seg(*a, *b));
+            ++i[q];
+          }
+          if (a->nks == 0) continue;
+          o.s2.push_back(seg(*a, *b));
+          ++k.nseg;
+          k.nks += a->nks;
+        }
+        const bool lo = rout[5] >= 0 && rout[7] > 0, hi = rout[6] >= 0 && rout[7] < k.M;   // rows of either s1'
+        if (lo && hi && (part[0].size() != (size_t)k.nseg || part[1].size() != (size_t)k.nseg)) {
+          k.cut = rout[7];
+          for (int q = 0; q < 2; ++q) {
+            k.psg0[q] = (int32_t)o.s2.size();
+            k.pseg[q] = (int32_t)part[q].size();
+            for (const TcSeg& e : part[q]) k.pnks[q] += e.b & 0xffff;
+            o.s2.insert(o.s2.end(), part[q].begin(), part[q].end());
+            if (part[q].empty()) o.zero_out = true;   // (only the separate lists leave these rows out)
+          }
+        }
+        if (k.nks > 0 && k.M > 0 && k.N > 0) tasks2.push_back(k);
+        else if (k.M > 0 && k.N > 0) o.zero_out = true;
       }
-      t2.insert(t2.end(), {t[0], t[1], t[2], t[3], 0, seg0, t[5], 1, 0, 0});
-      p2.push_back(p2.back() + ((t[0] + 127) / 128) * ((t[1] + ntile - 1) / ntile));
     }
   };
   std::thread step2;
@@ -207,7 +350,7 @@ bool tables(const mrd_heff* h, int prec, TcCfg cfg, TcTables& o) {
   // three classes by the LW blocks that feed them (s1 = 0 only, s1 = 1 only, both), each
   // class a task of its own with the K segments it needs, so no zero block is multiplied.
   // The stacked LW of a class and K segment s1 is one A panel; each output row is scattered to
-  // its Z panel through a row map (mode 2).
+  // its Z panel through a row map.
   std::vector<int64_t>& rowmap = o.rowmap;
   {
     std::vector<int64_t> zrow_of((size_t)c[C_NMID] > 0 ? (size_t)h->d.d_m * nmid : 0, -1);
@@ -242,178 +385,70 @@ bool tables(const mrd_heff* h, int prec, TcCfg cfg, TcTables& o) {
           if (k != 2 && k != q1) continue;
           if (rin[5 + q1] < 0) return fail("tc: LW block without its theta rows");
           const int64_t K = h->left[3 * rin[5 + q1] + 2];
-          ank[q1] = (K + kpt - 1) / kpt;
+          ank[q1] = steps(K);
           aoff[q1] = lw_b;
           for (const Member& mb : cls[k])
-            j_lw.insert(j_lw.end(), {mb.lw[q1], K, 0, mb.rows, K, lw_b, 128, ank[q1], round_up(R, 128), 0, 0, mb.row0, 0});
-          lw_b += a_bytes(R, ank[q1], aplanes);
+            j_lw.insert(j_lw.end(), {mb.lw[q1], K, 0, mb.rows, K, lw_b, 0, ank[q1], R, 0, mb.row0});
+          lw_b += a_bytes(R, ank[q1], prec);
         }
         for (int s2p = 0; s2p < 2; ++s2p) {
           if (rin[8 + s2p] < 0) continue;
-          const int64_t N = h->right[3 * rin[8 + s2p] + 2], coff = s2p ? rin[10] : 0;
+          const int64_t N = h->right[3 * rin[8 + s2p] + 2], coff = s2p ? rin[10] : 0, nks_z = steps(N);
           if (N == 0) continue;
-          const int64_t seg0 = (int64_t)s1.size() / TCS, map0 = (int64_t)rowmap.size();
-          int64_t nseg = 0;
+          TcTask task{R, N, (int64_t)rowmap.size(), nks_z, (int32_t)o.s1.size(), 0, 0, 0, {0, 0}, {0, 0}, {0, 0}};
           for (int q1 = 0; q1 < 2; ++q1) {
             if (aoff[q1] < 0) continue;
             const Panel* b = th_map.find(rin[4] + (q1 ? rin[7] : 0) * rin[3] + coff);
-            if (!b || b->nkt != ank[q1]) return fail("tc: step-1 operand not packed");
-            s1.insert(s1.end(), {aoff[q1], b->off, ank[q1], 0});
-            ++nseg;
+            if (!b || b->nks != ank[q1]) return fail("tc: step-1 operand not packed");
+            if (ank[q1] == 0) continue;
+            o.s1.push_back(seg({aoff[q1], ank[q1]}, *b));
+            ++task.nseg;
+            task.nks += ank[q1];
           }
-          const int64_t nkt_z = (N + kpt - 1) / kpt;
+          if (task.nks == 0) { o.zero_z = true; continue; }
           for (const Member& mb : cls[k]) {
             const int64_t zk = zrow_of[(size_t)(mb.wp * nmid + mi)];
             if (zk < 0) return fail("tc: step-1 output block missing");
             const int64_t* zr = &z[ZF * zk];
             const int64_t* rout = &mid[MIDF * zr[2]];
-            const Panel* q = z_map.find(zr[5] + (mb.s1p ? rout[7] : 0) * rin[3] + coff);
-            if (!q || q->nkt != nkt_z) return fail("tc: step-1 output panel missing");
-            for (int64_t r = 0; r < mb.rows; ++r) rowmap.push_back(q->off << 16 | r);
+            const Panel* q = z_map.find(zr[5] + coff);
+            if (!q || q->nks != nks_z) return fail("tc: step-1 output panel missing");
+            const int64_t row0 = mb.s1p ? rout[7] : 0;
+            if (row0 + mb.rows > zr[3]) return fail("tc: step-1 output rows outside their panel");
+            for (int64_t r = row0; r < row0 + mb.rows; ++r) {
+              const int64_t rt = r / 128, mrow = tc_apad(std::min<int64_t>(zr[3] - rt * 128, 128));
+              rowmap.push_back(tc_rowmap(q->off + rt * a_bytes(128, nks_z, prec), mrow, r % 128));
+            }
           }
-          t1.insert(t1.end(), {R, N, map0, 0, 0, seg0, nseg, 2, nkt_z, 0});
-          p1.push_back(p1.back() + ((R + 127) / 128) * ((N + ntile - 1) / ntile));
+          tasks1.push_back(task);
         }
       }
     }
   }
   if (step2.joinable()) step2.join();
   if (!step2_ok) return fail("tc: step-2 operand not packed");
-  // block schedule: tiles are dealt to the persistent CTAs in task order; order 1 puts the
-  // tasks with the most work (tiles x K tiles) first so that the long ones start early
-  if (cfg.order == 1) {
-    auto reorder = [&](std::vector<int64_t>& tk, const std::vector<int64_t>& sg, std::vector<int64_t>& pf) {
-      const size_t nt = tk.size() / TCT;
-      std::vector<int64_t> work(nt), idx(nt);
-      for (size_t i = 0; i < nt; ++i) {
-        int64_t kt = 0;
-        for (int64_t k = 0; k < tk[TCT * i + 6]; ++k) kt += sg[TCS * (tk[TCT * i + 5] + k) + 2];
-        work[i] = (pf[i + 1] - pf[i]) * kt;
-        idx[i] = (int64_t)i;
-      }
-      std::stable_sort(idx.begin(), idx.end(), [&](int64_t a, int64_t b) { return work[a] > work[b]; });
-      std::vector<int64_t> t2v(tk.size()), p2v(nt + 1, 0);
-      for (size_t i = 0; i < nt; ++i) {
-        std::copy(tk.begin() + TCT * idx[i], tk.begin() + TCT * (idx[i] + 1), t2v.begin() + TCT * i);
-        p2v[i + 1] = p2v[i] + (pf[idx[i] + 1] - pf[idx[i]]);
-      }
-      tk.swap(t2v);
-      pf.swap(p2v);
-    };
-    reorder(t1, s1, p1);
-    reorder(t2, s2, p2);
-  }
-  // every tile the kernel reads or writes must lie inside its buffer
+  // every tile the kernel reads must lie inside its buffer (the Z rows it writes: checked above)
   {
-    auto chk = [&](const std::vector<int64_t>& tk, const std::vector<int64_t>& sg, int64_t alen, int64_t blen,
-                   bool zout) {
-      for (size_t i = 0; i < tk.size(); i += TCT) {
-        const int64_t M = tk[i], N = tk[i + 1];
-        for (int64_t k = 0; k < tk[i + 6]; ++k) {
-          const int64_t* q = &sg[TCS * (tk[i + 5] + k)];
-          if (q[0] < 0 || q[0] + a_bytes(M, q[2], aplanes) > alen) return false;
-          if (q[1] < 0 || q[1] + b_bytes(N, q[2], bplanes) > blen) return false;
+    auto chk = [&](const std::vector<TcTask>& tk, const std::vector<TcSeg>& sg, int64_t alen, int64_t blen, int nt) {
+      for (const TcTask& t : tk)
+        for (int64_t k = 0; k < t.nseg; ++k) {   // (the parts' segments are among them)
+          const TcSeg& q = sg[(size_t)(t.seg0 + k)];
+          const int64_t nks = q.b & 0xffff, b = (q.b >> 16) * 256;
+          if (nks < 1 || q.a < 0 || q.a % 256 || q.a + a_bytes(t.M, nks, prec) > alen) return false;
+          if (b < 0 || b + b_bytes(t.N, nks, prec, nt) > blen) return false;
         }
-        if (zout) {   // every mapped row lies in a Z panel of this task's K-tile count
-          if (tk[i + 2] < 0 || tk[i + 2] + M > (int64_t)rowmap.size() || tk[i + 8] * kpt < N) return false;
-          for (int64_t r = 0; r < M; ++r) {
-            const int64_t off = rowmap[tk[i + 2] + r] >> 16, zr = rowmap[tk[i + 2] + r] & 0xffff;
-            if (off < 0 || off + (zr / 128 + 1) * tk[i + 8] * aplanes * 128 * 128 > z_b) return false;
-          }
-        }
-      }
       return true;
     };
-    if (!chk(t1, s1, lw_b, th_b, true) || !chk(t2, s2, z_b, wr_b, false))
-      return fail("tc: internal panel table check failed");
-    if (!tc_cfg_ok(prec, cfg)) return fail("tc: tile configuration does not fit");
+    if (!chk(tasks1, o.s1, lw_b, th_b, ntile) || !chk(tasks2, o.s2, z_b, wr_b, ntile2)) return fail("tc: internal panel table check failed");
   }
-  std::vector<int64_t>&q1 = o.q1, &q2 = o.q2;
-  q1.assign(2 * std::max<size_t>(p1.size() - 1, 1), 0);
-  q2.assign(2 * std::max<size_t>(p2.size() - 1, 1), 0);
-  for (size_t t = 0; t + 1 < p1.size(); ++t) q1[2 * t + 1] = p1[t + 1] - p1[t];
-  for (size_t t = 0; t + 1 < p2.size(); ++t) q2[2 * t + 1] = p2[t + 1] - p2[t];
-  // Item tables: (task, tile within task) of every tile, dealt to the persistent CTAs by
-  // longest-processing-time-first: items by decreasing cost (the task's K tiles plus two for the
-  // pipeline fill and the epilogue; equal costs in task order), each to the CTA with the least
-  // work so far (the lowest-numbered of those). Each CTA's items are stored together,
-  // co[c] .. co[c + 1]. A static deal in item order left step 2's SMs between 25% and 91% busy
-  // (ncu) because the tiles' K lengths differ by orders of magnitude.
-  // Tasks are ordered by a counting sort of their costs, and the least-loaded CTA is found in a
-  // bucket queue: bit sets of the CTAs per amount of work, in a ring of cmax + 1 buckets (every
-  // CTA's work lies within cmax of the least), so tens of thousands of items cost no sort and
-  // no heap operations.
-  const int grid_sm = std::max(h->n_sm, 1);
-  auto deal = [&](const std::vector<int64_t>& tk, const std::vector<int64_t>& sg, const std::vector<int64_t>& pf,
-                  std::vector<int2>& items, std::vector<int32_t>& co) {
-    const size_t nt = tk.size() / TCT;
-    const int64_t total = pf.back();
-    const int G = (int)std::min<int64_t>(total, grid_sm);
-    co.assign((size_t)G + 1, 0);
-    if (total <= 0) return;
-    std::vector<int64_t> cost(nt, 0);
-    int64_t cmax = 0;
-    for (size_t t = 0; t < nt; ++t) {
-      if (pf[t + 1] == pf[t]) continue;   // no tiles
-      int64_t kt = 0;
-      for (int64_t k = 0; k < tk[TCT * t + 6]; ++k) kt += sg[TCS * (tk[TCT * t + 5] + k) + 2];
-      cost[t] = kt + 2;
-      cmax = std::max(cmax, cost[t]);
-    }
-    std::vector<int64_t> first((size_t)cmax + 1, 0);   // first slot of each cost, decreasing costs
-    for (size_t t = 0; t < nt; ++t)
-      if (pf[t + 1] > pf[t]) ++first[(size_t)cost[t]];
-    for (int64_t c = cmax, acc = 0; c >= 0; --c) {
-      const int64_t n = first[(size_t)c];
-      first[(size_t)c] = acc;
-      acc += n;
-    }
-    size_t n_ord = 0;   // tasks with tiles
-    for (size_t t = 0; t < nt; ++t)
-      if (pf[t + 1] > pf[t]) ++n_ord;
-    std::vector<int32_t> ord(n_ord);
-    for (size_t t = 0; t < nt; ++t)
-      if (pf[t + 1] > pf[t]) ord[(size_t)first[(size_t)cost[t]]++] = (int32_t)t;
-    const int W = (G + 63) / 64;
-    const int64_t R = cmax + 1;
-    std::vector<uint64_t> bits((size_t)(R * W), 0);   // bucket (work mod R): the CTAs with that work
-    for (int c = 0; c < G; ++c) bits[(size_t)(c >> 6)] |= 1ull << (c & 63);
-    int64_t lo = 0;   // least work of any CTA
-    std::vector<int32_t> owner((size_t)total), count((size_t)G, 0);
-    size_t i = 0;
-    for (const int32_t t : ord) {
-      const int64_t add = cost[(size_t)t];
-      for (int64_t l = pf[(size_t)t]; l < pf[(size_t)t + 1]; ++l, ++i) {
-        int c = -1;
-        for (;; ++lo) {
-          const uint64_t* bk = &bits[(size_t)((lo % R) * W)];
-          for (int w = 0; w < W && c < 0; ++w)
-            if (bk[w]) c = w * 64 + __builtin_ctzll(bk[w]);
-          if (c >= 0) break;
-        }
-        bits[(size_t)((lo % R) * W + (c >> 6))] &= ~(1ull << (c & 63));
-        bits[(size_t)(((lo + add) % R) * W + (c >> 6))] |= 1ull << (c & 63);
-        owner[i] = c;
-        ++count[(size_t)c];
-      }
-    }
-    for (int c = 0; c < G; ++c) co[(size_t)c + 1] = co[(size_t)c] + count[(size_t)c];
-    items.assign((size_t)total, make_int2(0, 0));
-    std::vector<int32_t> fill(co.begin(), co.end() - 1);
-    i = 0;
-    for (const int32_t t : ord)
-      for (int64_t l = 0; l < pf[(size_t)t + 1] - pf[(size_t)t]; ++l, ++i)
-        items[(size_t)fill[(size_t)owner[i]]++] = make_int2(t, (int)l);
-  };
-  deal(t1, s1, p1, o.i1, o.co1);
-  deal(t2, s2, p2, o.i2, o.co2);
+  cut_tiles(tasks1, ntile, cfg.order, true, o.s1, o.i1, o.task1);
+  cut_tiles(tasks2, o.ntile2, cfg.order, false, o.s2, o.i2, o.task2, &o.ia, &o.taska);
   // first piece of every pack job (field 9) and the pieces of each list
-  const int kc = tc_is_tf32(prec) ? 4 : 8;
   auto pieces = [&](std::vector<int64_t>& j) {
     int64_t n = 0;
     for (size_t k = 0; k < j.size(); k += TCJ) {
       j[k + 9] = n;
-      n += (j[k + 3] * ((j[k + 4] + kc - 1) / kc) + kPackPiece - 1) / kPackPiece;
+      n += (j[k + 3] * j[k + 7] * (j[k + 2] ? 2 : kst / 2) + kPackPiece - 1) / kPackPiece;
     }
     return n;
   };
@@ -423,56 +458,49 @@ bool tables(const mrd_heff* h, int prec, TcCfg cfg, TcTables& o) {
   return true;
 }
 
-// Device buffers of the tables in `o` (which must have been built for this H_eff): allocation,
-// upload and zeroed panels; replaces the H_eff's tensor-core state. Synchronises the stream.
+// Device buffers of the tables in `o` (which must have been built for this H_eff): allocation
+// and upload; replaces the H_eff's tensor-core state. Synchronises the stream.
 int upload(mrd_heff* h, const TcTables& o) {
   mrd_ctx* ctx = h->ctx;
   delete h->tc;
   Tc* T = h->tc = new Tc();
   T->prec = o.prec;
   T->cfg = o.cfg;
+  T->ntile2 = o.ntile2;
   Arena& A = T->mem;
   A.stream = ctx->stream;
   cudaError_t e = cudaSuccess;
 #define TALLOC(ptr, n) if (e == cudaSuccess) e = A.alloc(&(ptr), (size_t)std::max<int64_t>((n), 1))
   TALLOC(T->lw, o.lw_b); TALLOC(T->wr, o.wr_b); TALLOC(T->th, o.th_b); TALLOC(T->z, o.z_b);
-  TALLOC(T->t1, o.t1.size()); TALLOC(T->s1, o.s1.size()); TALLOC(T->p1, o.p1.size());
-  TALLOC(T->t2, o.t2.size()); TALLOC(T->s2, o.s2.size()); TALLOC(T->p2, o.p2.size());
-  TALLOC(T->j_lw, o.j_lw.size()); TALLOC(T->j_wr, o.j_wr.size()); TALLOC(T->j_th, o.j_th.size());
-  TALLOC(T->err, 1);
-  TALLOC(T->pt1, o.q1.size()); TALLOC(T->pt2, o.q2.size());
-  TALLOC(T->it1, o.i1.size()); TALLOC(T->it2, o.i2.size());
-  TALLOC(T->co1, o.co1.size()); TALLOC(T->co2, o.co2.size());
+  TALLOC(T->it1, o.i1.size()); TALLOC(T->it2, o.i2.size()); TALLOC(T->alt2, o.ia.size());
+  TALLOC(T->s1, o.s1.size()); TALLOC(T->s2, o.s2.size());
   TALLOC(T->rmap1, o.rowmap.size());
+  TALLOC(T->j_lw, o.j_lw.size()); TALLOC(T->j_wr, o.j_wr.size()); TALLOC(T->j_th, o.j_th.size());
+  TALLOC(T->words, 4);
 #undef TALLOC
   if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "tc: device buffers");
-  T->lw_bytes = o.lw_b; T->wr_bytes = o.wr_b; T->th_bytes = o.th_b; T->z_bytes = o.z_b;
-  T->n1 = (int64_t)o.t1.size() / TCT; T->ntiles1 = o.p1.back();
-  T->n2 = (int64_t)o.t2.size() / TCT; T->ntiles2 = o.p2.back();
+  T->n_it1 = (int)o.i1.size(); T->n_it2 = (int)o.i2.size();
+  T->n_alt2 = (int)o.ia.size();
+  T->task1 = o.task1; T->task2 = o.task2; T->taska = o.taska;
   T->n_lw = (int)(o.j_lw.size() / TCJ); T->n_wr = (int)(o.j_wr.size() / TCJ); T->n_th = (int)(o.j_th.size() / TCJ);
   T->pc_lw = o.pc_lw; T->pc_wr = o.pc_wr; T->pc_th = o.pc_th;
+  T->zero_out = o.zero_out;
   cudaStream_t s = ctx->stream;
   auto up = [&](void* d, const void* v, size_t bytes) {
     if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(d, v, bytes, cudaMemcpyHostToDevice, s);
   };
-  for (auto pr : {std::make_pair(T->t1, &o.t1), std::make_pair(T->s1, &o.s1), std::make_pair(T->p1, &o.p1),
-                  std::make_pair(T->t2, &o.t2), std::make_pair(T->s2, &o.s2), std::make_pair(T->p2, &o.p2),
-                  std::make_pair(T->j_lw, &o.j_lw), std::make_pair(T->j_wr, &o.j_wr), std::make_pair(T->j_th, &o.j_th),
-                  std::make_pair(T->pt1, &o.q1), std::make_pair(T->pt2, &o.q2), std::make_pair(T->rmap1, &o.rowmap)})
+  for (auto pr : {std::make_pair(T->j_lw, &o.j_lw), std::make_pair(T->j_wr, &o.j_wr), std::make_pair(T->j_th, &o.j_th),
+                  std::make_pair(T->rmap1, &o.rowmap)})
     up(pr.first, pr.second->data(), pr.second->size() * 8);
-  up(T->it1, o.i1.data(), o.i1.size() * 8);
-  up(T->it2, o.i2.data(), o.i2.size() * 8);
-  up(T->co1, o.co1.data(), o.co1.size() * 4);
-  up(T->co2, o.co2.data(), o.co2.size() * 4);
-  T->tiles1.resize(o.p1.size() - 1);
-  T->tiles2.resize(o.p2.size() - 1);
-  for (size_t t = 0; t < T->tiles1.size(); ++t) T->tiles1[t] = o.q1[2 * t + 1];
-  for (size_t t = 0; t < T->tiles2.size(); ++t) T->tiles2[t] = o.q2[2 * t + 1];
-  // zero padding everywhere (packing and the Z epilogue only write valid elements)
-  for (auto pr : {std::make_pair(T->lw, o.lw_b), std::make_pair(T->wr, o.wr_b), std::make_pair(T->th, o.th_b),
-                  std::make_pair(T->z, o.z_b)})
-    if (e == cudaSuccess && pr.second) e = cudaMemsetAsync(pr.first, 0, (size_t)pr.second, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(T->err, 0, 4, s);
+  up(T->it1, o.i1.data(), o.i1.size() * sizeof(TcItem));
+  up(T->it2, o.i2.data(), o.i2.size() * sizeof(TcItem));
+  up(T->alt2, o.ia.data(), o.ia.size() * sizeof(TcItem));
+  up(T->s1, o.s1.data(), o.s1.size() * sizeof(TcSeg));
+  up(T->s2, o.s2.data(), o.s2.size() * sizeof(TcSeg));
+  // Packing and the Z epilogue write whole K steps; rows that only pad a tile reach only outputs that
+  // are not stored. Only Z rows that no product feeds have to be zeros.
+  if (e == cudaSuccess && o.zero_z && T->z) e = cudaMemsetAsync(T->z, 0, (size_t)o.z_b, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(T->words, 0, 16, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host tables may be released after this
   if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "tc: upload");
   return MRD_OK;
@@ -490,9 +518,10 @@ namespace {
 
 // Candidate tile configurations per precision (all fit the 227 KB of shared memory).
 std::vector<TcCfg> candidates(int prec) {
-  if (prec == TC_TF32) return {{128, 2, 0}, {64, 4, 0}, {128, 2, 1}, {64, 4, 1}};
+  if (prec == TC_TF32) return {{128, 3, 0}, {64, 4, 0}, {128, 3, 1}, {64, 4, 1}};
   if (prec == TC_BF16X3) return {{64, 2, 0}, {48, 2, 0}, {64, 2, 1}, {48, 2, 1}};
-  return {{128, 3, 0}, {64, 4, 0}, {128, 3, 1}, {64, 4, 1}};   // real operands: 1 or 2 planes
+  if (prec == TC_TF32_REAL) return {{128, 6, 0}, {64, 8, 0}, {128, 6, 1}, {64, 8, 1}};
+  return {{128, 3, 0}, {64, 4, 0}, {128, 3, 1}, {64, 4, 1}};
 }
 
 // Problem class of an H_eff for the tuning cache: precision, size of theta (powers of two)
@@ -500,6 +529,18 @@ std::vector<TcCfg> candidates(int prec) {
 uint64_t tune_key(const mrd_heff* h, int prec) {
   auto lg = [](int64_t v) { uint64_t b = 0; while (v > 1) { v >>= 1; ++b; } return b; };
   return (uint64_t)prec << 56 | lg(h->counts[C_THETA]) << 40 | lg(h->counts[C_NT2]) << 24 | (uint64_t)h->n_sm;
+}
+
+// The two grouped products on the packed operands (the tile counters are zero).
+cudaError_t products(const mrd_heff* h, double2* out, cudaStream_t s, cudaEvent_t between = nullptr, bool cap = false) {
+  const Tc* T = h->tc;
+  cudaError_t e = tc_gemm(T->lw, T->th, T->it1, T->n_it1, nullptr, 0, nullptr, T->s1, T->rmap1, T->z, nullptr, T->prec, T->cfg, T->cfg.ntile, T->words, T->err(),
+                          h->n_sm, h->wait_ns, s);
+  if (e == cudaSuccess && between) e = record_event(between, s, cap);
+  if (e == cudaSuccess)
+    e = tc_gemm(T->z, T->wr, T->it2, T->n_it2, T->alt2, T->n_alt2, T->bad(), T->s2, nullptr, nullptr, out, T->prec, T->cfg, T->ntile2, T->words + 1, T->err(), h->n_sm,
+                h->wait_ns, s);
+  return e;
 }
 
 // Kernel time (ms) of steps 1 and 2 with the built configuration, on the packed operands
@@ -516,12 +557,8 @@ int time_cfg(mrd_heff* h, double* ms) {
   e = cache_alloc((void**)&out, (size_t)std::max<int64_t>(h->counts[C_THETA], 1) * 16, s);
   for (int r = 0; r < 4 && e == cudaSuccess; ++r) {
     if (r == 1) e = cudaEventRecord(a, s);
-    if (e == cudaSuccess)
-      e = tc_gemm(T->lw, T->th, T->t1, T->s1, T->p1, T->it1, T->co1, T->rmap1, T->n1, T->ntiles1, T->z, nullptr, T->prec, T->cfg, T->err,
-                  h->n_sm, h->wait_ns, s);
-    if (e == cudaSuccess)
-      e = tc_gemm(T->z, T->wr, T->t2, T->s2, T->p2, T->it2, T->co2, nullptr, T->n2, T->ntiles2, nullptr, out, T->prec, T->cfg, T->err, h->n_sm,
-                  h->wait_ns, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(T->words, 0, 8, s);
+    if (e == cudaSuccess) e = products(h, out, s);
   }
   float f = 0.f;
   if (e == cudaSuccess) e = cudaEventRecord(b, s);
@@ -631,8 +668,8 @@ int autotune(mrd_heff* h, int prec) {
     int rc = build(h, prec, c);
     if (rc != MRD_OK) return rc;
     Tc* T = h->tc;
-    MRD_CUDA(ctx, tc_pack(h->lw, T->lw, T->j_lw, T->n_lw, T->pc_lw, prec, ctx->stream));
-    MRD_CUDA(ctx, tc_pack(h->wr, T->wr, T->j_wr, T->n_wr, T->pc_wr, prec, ctx->stream));
+    MRD_CUDA(ctx, tc_pack(h->lw, T->lw, T->j_lw, T->n_lw, T->pc_lw, prec, nullptr, nullptr, ctx->stream));
+    MRD_CUDA(ctx, tc_pack(h->wr, T->wr, T->j_wr, T->n_wr, T->pc_wr, prec, nullptr, T->bad(), ctx->stream));
     double ms = 0.0;
     if ((rc = time_cfg(h, &ms)) != MRD_OK) return rc;
     if (ms < best_ms) { best_ms = ms; best = c; }
@@ -655,10 +692,10 @@ void tc_env_changed(mrd_heff* h) {
 int tc_status(mrd_heff* h) {
   if (!h->tc) return MRD_OK;
   int herr = 0;
-  MRD_CUDA(h->ctx, cudaMemcpyAsync(&herr, h->tc->err, 4, cudaMemcpyDeviceToHost, h->ctx->stream));
+  MRD_CUDA(h->ctx, cudaMemcpyAsync(&herr, h->tc->err(), 4, cudaMemcpyDeviceToHost, h->ctx->stream));
   MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
   if (herr) {   // reported once: the flag is cleared for the next launches
-    MRD_CUDA(h->ctx, cudaMemsetAsync(h->tc->err, 0, 4, h->ctx->stream));
+    MRD_CUDA(h->ctx, cudaMemsetAsync(h->tc->err(), 0, 4, h->ctx->stream));
     MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
     return mrd_fail(h->ctx, MRD_E_TIMEOUT, "tensor-core GEMM: a bounded wait gave up (code " + std::to_string(herr) + ")");
   }
@@ -680,8 +717,9 @@ int tc_prepare(mrd_heff* h, int32_t prec) {
   Tc* T = h->tc;
   cudaStream_t s = ctx->stream;
   if (T->env_dirty) {
-    MRD_CUDA(ctx, tc_pack(h->lw, T->lw, T->j_lw, T->n_lw, T->pc_lw, tp, s));
-    MRD_CUDA(ctx, tc_pack(h->wr, T->wr, T->j_wr, T->n_wr, T->pc_wr, tp, s));
+    MRD_CUDA(ctx, cudaMemsetAsync(T->bad(), 0, 4, s));
+    MRD_CUDA(ctx, tc_pack(h->lw, T->lw, T->j_lw, T->n_lw, T->pc_lw, tp, nullptr, nullptr, s));
+    MRD_CUDA(ctx, tc_pack(h->wr, T->wr, T->j_wr, T->n_wr, T->pc_wr, tp, nullptr, T->bad(), s));
     T->env_dirty = false;
   }
   return MRD_OK;
@@ -710,23 +748,19 @@ int tc_apply(mrd_heff* h, const double* in, double* out, int32_t prec) {
   bool cap = false;
   if (h->timing && !apply_events(h, s, ev, &cap)) return mrd_fail(ctx, MRD_E_CUDA, "mrd_heff_apply: cudaEventCreate");
   const cudaEvent_t e0 = ev[0], e1 = ev[1], e2 = ev[2];
-  MRD_CUDA(ctx, cudaMemsetAsync(out, 0, (size_t)h->counts[C_THETA] * 16, s));
-  MRD_CUDA(ctx, tc_pack((const double2*)in, T->th, T->j_th, T->n_th, T->pc_th, tp, s));
+  if (T->zero_out) MRD_CUDA(ctx, cudaMemsetAsync(out, 0, (size_t)h->counts[C_THETA] * 16, s));
+  MRD_CUDA(ctx, tc_pack((const double2*)in, T->th, T->j_th, T->n_th, T->pc_th, tp, T->words, nullptr, s));
   MRD_CUDA(ctx, record_event(e0, s, cap));
   if (!h->per_task) {
-    MRD_CUDA(ctx, tc_gemm(T->lw, T->th, T->t1, T->s1, T->p1, T->it1, T->co1, T->rmap1, T->n1, T->ntiles1, T->z, nullptr, tp, T->cfg, T->err,
-                          h->n_sm, h->wait_ns, s));
-    MRD_CUDA(ctx, record_event(e1, s, cap));
-    MRD_CUDA(ctx, tc_gemm(T->z, T->wr, T->t2, T->s2, T->p2, T->it2, T->co2, nullptr, T->n2, T->ntiles2, nullptr, (double2*)out, tp, T->cfg,
-                          T->err, h->n_sm, h->wait_ns, s));
+    MRD_CUDA(ctx, products(h, (double2*)out, s, e1, cap));
   } else {   // one launch per task: the per-block baseline of the grouped persistent launch
-    for (int64_t t = 0; t < T->n1; ++t)
-      MRD_CUDA(ctx, tc_gemm(T->lw, T->th, T->t1 + TCT * t, T->s1, T->pt1 + 2 * t, nullptr, nullptr, T->rmap1, 1, T->tiles1[t], T->z, nullptr, tp,
-                            T->cfg, T->err, h->n_sm, h->wait_ns, s));
+    for (size_t t = 0; t + 1 < T->task1.size(); ++t)
+      MRD_CUDA(ctx, tc_gemm(T->lw, T->th, T->it1 + T->task1[t], T->task1[t + 1] - T->task1[t], nullptr, 0, nullptr, T->s1, T->rmap1, T->z, nullptr, tp, T->cfg,
+                            T->cfg.ntile, nullptr, T->err(), h->n_sm, h->wait_ns, s));
     MRD_CUDA(ctx, record_event(e1, s, cap));
-    for (int64_t t = 0; t < T->n2; ++t)
-      MRD_CUDA(ctx, tc_gemm(T->z, T->wr, T->t2 + TCT * t, T->s2, T->pt2 + 2 * t, nullptr, nullptr, nullptr, 1, T->tiles2[t], nullptr,
-                            (double2*)out, tp, T->cfg, T->err, h->n_sm, h->wait_ns, s));
+    for (size_t t = 0; t + 1 < T->task2.size(); ++t)
+      MRD_CUDA(ctx, tc_gemm(T->z, T->wr, T->it2 + T->task2[t], T->task2[t + 1] - T->task2[t], T->alt2 + T->taska[t],
+                            T->taska[t + 1] - T->taska[t], T->bad(), T->s2, nullptr, nullptr, (double2*)out, tp, T->cfg, T->ntile2, nullptr, T->err(), h->n_sm, h->wait_ns, s));
   }
   MRD_CUDA(ctx, record_event(e2, s, cap));
   return MRD_OK;
