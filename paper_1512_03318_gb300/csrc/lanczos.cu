@@ -11,9 +11,11 @@
 // max_iter; the ground vector is V y, normalised.
 //
 // All vector arithmetic runs in FP64 on the device with fixed-shape reductions (partial sums
-// per CTA, then one CTA), so results are bit-reproducible run to run. The tridiagonal
-// eigenproblem is solved on the device by one warp: Sturm-count multisection for the lowest
-// eigenvalue, inverse iteration with a pivoted tridiagonal LU for its vector.
+// per CTA, then the last CTA to finish sums them in a fixed order), so results are bit-reproducible
+// run to run. The tridiagonal eigenproblem is solved on the device by one warp: Sturm-count
+// multisection for the lowest eigenvalue at every step, inverse iteration with a pivoted tridiagonal LU
+// for its vector at the end. A step is launch bound at small sizes: eight kernels besides the
+// operator's.
 #include <cmath>
 #include <vector>
 
@@ -32,6 +34,17 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums of re and im over the warp: in lanes 0 .. 15 that of re, in 16 .. 31 that of im. The same tree as
+// two warp_sum calls (pairs 16, 8, 4, 2, 1 lanes apart; only the order within a pair differs, which a
+// sum does not see) with half of their FP64 additions, at 16 cycles each.
+__device__ __forceinline__ double warp_sum2(double re, double im, int lane) {
+  const bool hi = lane & 16;
+  double v = (hi ? im : re) + __shfl_xor_sync(0xffffffffu, hi ? re : im, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // Device state of one Lanczos run. j is the current step: the kernels of a step read it,
 // so that one captured CUDA graph of a step serves every step.
 struct LzState {
@@ -46,7 +59,6 @@ struct LzState {
   int j;
 };
 
-// number of vectors of a reduction: nv >= 0 as given, nv < 0 means v_0 .. v_j of the state
 // Vectors of a reduction or combination: nv >= 0: v_0 .. v_{nv-1}; nv = -1: v_0 .. v_j (all);
 // nv = -2: v_{j-1}, v_j (the two the three-term recurrence involves; v_0 alone at j = 0).
 __device__ __forceinline__ int eff_nv(int nv, const LzState* st) {
@@ -56,11 +68,56 @@ __device__ __forceinline__ int first_v(int nv, const LzState* st) { return nv ==
 
 constexpr int kJB = 4;   // vectors per pass of k_multidot (w is read once per pass)
 
-// partial[b * nv + j] = sum over this CTA's share of conj(V_j) . w, j < nv (re, im interleaved)
+// The CTA that is the last of its launch to get here (the ticket counts them and is zeroed again
+// by it); the others' earlier writes are visible to it.
+__device__ __forceinline__ bool last_cta(int* ticket) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  if (threadIdx.x == 0) *ticket = 0;
+  return true;
+}
+
+// out[j] = sum_b partial[b * nv + j] by the calling CTA; one warp per j, fixed order (lane-strided sums,
+// then a shuffle tree).
+__device__ __forceinline__ void finish_dots(const double2* partial, int nblocks, int nv, double2* out) {
+  const int lane = threadIdx.x & 31;
+  for (int j = threadIdx.x >> 5; j < nv; j += (int)blockDim.x >> 5) {
+    double a = 0.0, c = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < nblocks; b += 32) {
+      const double2 p = __ldcg(partial + (int64_t)b * nv + j);
+      a += p.x;
+      c += p.y;
+    }
+    const double v = warp_sum2(a, c, lane);
+    if ((lane & 15) == 0) ((double*)(out + j))[lane >> 4] = v;
+  }
+}
+
+// Lanczos bookkeeping after the Gram-Schmidt passes of step j, with |w|^2: alpha_j = Re(c1_j) + Re(c2_j)
+// (c1: coefficients of the local pass, v_{j-1} and v_j; c2: of the full pass, v_0 .. v_j), beta_j = |w|.
+__device__ __forceinline__ void record_step(LzState* st, const double2* c1, const double2* c2, double nrm2) {
+  const int j = st->j;
+  st->alpha[j] = c1[j > 0 ? 1 : 0].x + c2[j].x;
+  st->beta[j] = sqrt(nrm2);
+  st->beta_last = st->beta[j];
+  st->inv_beta = nrm2 > 0.0 ? 1.0 / st->beta[j] : 0.0;
+}
+
+// out[j] = conj(V_j) . w, j < nv: partial[b * nv + j] over each CTA's share (re, im interleaved), summed
+// by the last CTA (out null: by k_finish_dots). Bound by the FP64 pipe where the vectors are short (16
+// cycles per warp instruction): rows of threads without elements and vectors beyond nv are skipped.
+// MULTIDOT_US. record (with c1, c2): the dot is |w|^2 of a step, which is recorded.
 __global__ void __launch_bounds__(kRedThreads) k_multidot(const double2* __restrict__ V, int64_t ldv, int nv_arg,
-                                                          const LzState* __restrict__ st,
-                                                          const double2* __restrict__ w, int64_t n,
-                                                          double2* __restrict__ partial) {
+                                                          LzState* st, const double2* __restrict__ w, int64_t n,
+                                                          double2* partial, int* ticket, double2* out, bool record,
+                                                          const double2* __restrict__ c1,
+                                                          const double2* __restrict__ c2) {
   __shared__ double sre[kJB][kRedThreads / 32], sim[kJB][kRedThreads / 32];
   const int nv = eff_nv(nv_arg, st);
   V += (int64_t)first_v(nv_arg, st) * ldv;
@@ -73,6 +130,7 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot(const double2* __restr
 #pragma unroll
     for (int q = 0; q < kJB; ++q) re[q] = im[q] = 0.0;
     for (int64_t i0 = b + threadIdx.x; i0 < e; i0 += (int64_t)kE * blockDim.x) {
+      const int rows = (int)((e - (i0 - threadIdx.x) + blockDim.x - 1) / blockDim.x);   // with any element left
       double2 y[kE];
 #pragma unroll
       for (int u = 0; u < kE; ++u) {
@@ -90,6 +148,7 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot(const double2* __restr
           }
 #pragma unroll
           for (int u = 0; u < kE; ++u) {
+            if (u >= rows) break;
             re[q] = fma(x[u].x, y[u].x, re[q]);
             re[q] = fma(x[u].y, y[u].y, re[q]);
             im[q] = fma(x[u].x, y[u].y, im[q]);
@@ -100,12 +159,10 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot(const double2* __restr
     }
 #pragma unroll
     for (int q = 0; q < kJB; ++q) {
-      re[q] = warp_sum(re[q]);
-      im[q] = warp_sum(im[q]);
-      if ((threadIdx.x & 31) == 0) {
-        sre[q][threadIdx.x >> 5] = re[q];
-        sim[q][threadIdx.x >> 5] = im[q];
-      }
+      if (j0 + q >= nv) break;
+      const int lane = threadIdx.x & 31;
+      const double v = warp_sum2(re[q], im[q], lane);
+      if ((lane & 15) == 0) (lane ? sim : sre)[q][threadIdx.x >> 5] = v;
     }
     __syncthreads();
     if (threadIdx.x < kJB && j0 + (int)threadIdx.x < nv) {
@@ -119,30 +176,33 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot(const double2* __restr
     }
     __syncthreads();
   }
+  if (!out || !last_cta(ticket)) return;
+  finish_dots(partial, (int)gridDim.x, nv, out);
+  if (record && threadIdx.x == 0) record_step(st, c1, c2, out[0].x);   // (this thread wrote out[0])
 }
 
-// out[j] = sum_b partial[b * nv + j]; one warp per j, fixed order (lane-strided sums, then
-// a shuffle tree).
-__global__ void k_finish_dots(const double2* __restrict__ partial, int nblocks, int nv_arg,
-                              const LzState* __restrict__ st, double2* __restrict__ out) {
-  const int nv = eff_nv(nv_arg, st);
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (j >= nv) return;
+// The same sums for the full Gram-Schmidt pass, whose partials (one per CTA and vector: 2500 x 20 at chi =
+// 3200) are too many for one SM.
+__global__ void __launch_bounds__(128) k_finish_dots(const double2* __restrict__ partial, int nblocks,
+                                                     const LzState* __restrict__ st, double2* __restrict__ out) {
+  const int nv = st->j + 1, j0 = blockIdx.x * 4, nj = nv - j0 < 4 ? nv - j0 : 4;
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  if (q >= nj) return;
   double a = 0.0, c = 0.0;
+#pragma unroll 4
   for (int b = lane; b < nblocks; b += 32) {
-    const double2 p = partial[(int64_t)b * nv + j];
+    const double2 p = partial[(int64_t)b * nv + j0 + q];
     a += p.x;
     c += p.y;
   }
-  a = warp_sum(a);
-  c = warp_sum(c);
-  if (lane == 0) out[j] = make_double2(a, c);
+  const double v = warp_sum2(a, c, lane);
+  if ((lane & 15) == 0) ((double*)(out + j0 + q))[lane >> 4] = v;
 }
 
-// w -= sum_j c[j] V_j
+// w -= sum_j c[j] V_j (and its FP32 copy into w32 when given)
 __global__ void k_sub_combination(const double2* __restrict__ V, int64_t ldv, int nv_arg,
                                   const LzState* __restrict__ st, const double2* __restrict__ c,
-                                  double2* __restrict__ w, int64_t n) {
+                                  double2* __restrict__ w, int64_t n, float2* __restrict__ w32) {
   const int nv = eff_nv(nv_arg, st);
   V += (int64_t)first_v(nv_arg, st) * ldv;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -153,6 +213,7 @@ __global__ void k_sub_combination(const double2* __restrict__ V, int64_t ldv, in
       acc.y -= cj.x * v.y + cj.y * v.x;
     }
     w[i] = acc;
+    if (w32) w32[i] = make_float2(__double2float_rn(acc.x), __double2float_rn(acc.y));
   }
 }
 
@@ -167,18 +228,11 @@ __global__ void k_sub_combination(const double2* __restrict__ V, int64_t ldv, in
 constexpr int kMD32Chunk = 1024;   // elements of w per CTA of k_multidot32
 inline int64_t md32_blocks(int64_t n) { return n > 0 ? (n + kMD32Chunk - 1) / kMD32Chunk : 1; }
 
-__global__ void k_to_f32(const double2* __restrict__ x, float2* __restrict__ y, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = x[i];
-    y[i] = make_float2(__double2float_rn(v.x), __double2float_rn(v.y));
-  }
-}
-
 // partial[b * nv + j] = conj(V32_j) . w32 over the b-th chunk of kMD32Chunk elements, j <= st->j:
 // a skinny GEMV. The CTA stages its chunk of w32 in shared memory; its warps take the basis
 // vectors in turn and stream that chunk of each with 8 independent loads per lane. Products
 // and sums in FP32 (a warp's sum covers one chunk), stored as FP64 for the cross-chunk sum.
-__global__ void __launch_bounds__(256) k_multidot32(const float2* __restrict__ V32, int64_t ldv,
+__global__ void __launch_bounds__(512) k_multidot32(const float2* __restrict__ V32, int64_t ldv,
                                                     const LzState* __restrict__ st,
                                                     const float2* __restrict__ w32, int64_t n,
                                                     double2* __restrict__ partial) {
@@ -265,9 +319,10 @@ __global__ void k_combination_real(const double2* __restrict__ V, int64_t ldv, i
 }
 
 // dst = src * (1 / sqrt(norm2)), norm2 read from device memory (real part of *nrm)
-// (and its FP32 copy into dst32 when given)
+// (and a second copy into vin, an FP32 copy into dst32, and step 0 into the state, when given)
 __global__ void k_scale_by_invnorm(const double2* __restrict__ src, double2* __restrict__ dst, int64_t n,
-                                   const double2* __restrict__ nrm2, float2* __restrict__ dst32) {
+                                   const double2* __restrict__ nrm2, double2* __restrict__ vin,
+                                   float2* __restrict__ dst32, LzState* st) {
   __shared__ double s_sh;   // one FP64 square root and division per CTA, not per thread
   if (threadIdx.x == 0) s_sh = nrm2->x > 0.0 ? 1.0 / sqrt(nrm2->x) : 0.0;
   __syncthreads();
@@ -276,46 +331,24 @@ __global__ void k_scale_by_invnorm(const double2* __restrict__ src, double2* __r
     const double2 v = src[i];
     const double2 o = make_double2(v.x * s, v.y * s);
     dst[i] = o;
+    if (vin) vin[i] = o;
     if (dst32) dst32[i] = make_float2(__double2float_rn(o.x), __double2float_rn(o.y));
   }
+  if (st && blockIdx.x == 0 && threadIdx.x == 0) st->j = 0;
 }
 
-// Lanczos bookkeeping after the local and the full Gram-Schmidt pass of step j (single thread):
-// alpha_j = Re(c1_j) + Re(c2_j).
-// c1: coefficients of the local pass (v_{j-1}, v_j), c2: of the full pass (v_0 .. v_j)
-__global__ void k_record_alpha(LzState* st, const double2* __restrict__ c1, const double2* __restrict__ c2) {
-  const int j = st->j;
-  st->alpha[j] = c1[j > 0 ? 1 : 0].x + c2[j].x;
-}
-
-__global__ void k_record_beta(LzState* st, const double2* __restrict__ nrm2) {
-  const int j = st->j;
-  st->beta[j] = sqrt(nrm2->x);
-  st->beta_last = st->beta[j];
-  st->inv_beta = nrm2->x > 0.0 ? 1.0 / st->beta[j] : 0.0;
-}
-
-__global__ void k_set_step(LzState* st, int j) { st->j = j; }
-__global__ void k_next_step(LzState* st) { st->j += 1; }
-
-// vin = v_j (j read from the state: one captured iteration serves every j)
-__global__ void k_copy_vj(const double2* __restrict__ V, int64_t n, const LzState* __restrict__ st,
-                          double2* __restrict__ vin) {
-  const double2* v = V + (int64_t)st->j * n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    vin[i] = v[i];
-}
-
-// v_{j+1} = w / |w|
+// v_{j+1} = w / |w|, also staged in vin as the next step's operand (a fixed address: one captured step
+// serves every j)
 __global__ void k_scale_next(const double2* __restrict__ w, double2* __restrict__ V, int64_t n,
-                             const LzState* __restrict__ st, float2* __restrict__ V32) {
-  const double sc = st->inv_beta;   // formed once by k_record_beta
+                             const LzState* __restrict__ st, double2* __restrict__ vin, float2* __restrict__ V32) {
+  const double sc = st->inv_beta;   // formed once by record_step
   double2* dst = V + (int64_t)(st->j + 1) * n;
   float2* dst32 = V32 ? V32 + (int64_t)(st->j + 1) * n : nullptr;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = w[i];
     const double2 o = make_double2(v.x * sc, v.y * sc);
     dst[i] = o;
+    vin[i] = o;
     if (dst32) dst32[i] = make_float2(__double2float_rn(o.x), __double2float_rn(o.y));
   }
 }
@@ -329,22 +362,40 @@ __global__ void k_scale_next(const double2* __restrict__ w, double2* __restrict_
 // pivot). A row then changes the minors' scale by at most ~2^50 (the guard) and otherwise by
 // |a_i - x| + b_{i-1}^2, so every 8 rows both are rescaled by 2^-+500 when p_i has left
 // [2^-500, 2^500], and neither leaves the FP64 range in between.
+// Signs, zeros and magnitudes are read off the bits: a comparison of doubles would run on the FP64 pipe
+// (2 lanes per SM, 16 cycles for a warp) like the three operations of the recurrence itself.
+__device__ __forceinline__ int top_word(double p) { return __double2hiint(p); }
+__device__ __forceinline__ bool is_zero(double p) { return ((top_word(p) & 0x7fffffff) | __double2loint(p)) == 0; }
+
+// Eight rows at a time: their coefficients are loaded and shifted ahead of the serial chain, which is
+// then one multiply-add per row.
 __device__ int sturm_count(const double* a, const double* b2, int k, double x) {
   double pm = 1.0, p = a[0] - x;
-  if (p == 0.0) p = 0x1p-50;
-  int cnt = p < 0.0;
-  for (int i = 1; i < k; ++i) {
-    double pn = fma(a[i] - x, p, -b2[i - 1] * pm);
-    if (pn == 0.0) pn = p * 0x1p-50;
-    cnt += (pn < 0.0) != (p < 0.0);
-    pm = p;
-    p = pn;
-    if ((i & 7) == 0) {
-      const double m = fabs(p);
-      if (m > 0x1p500) {
+  if (is_zero(p)) p = 0x1p-50;
+  int cnt = (int)((unsigned)top_word(p) >> 31);
+  for (int i = 1; i < k; i += 8) {
+    double d[8], c[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int r = i + q < k ? i + q : k - 1;
+      d[q] = a[r] - x;
+      c[q] = b2[r - 1];
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (i + q >= k) break;
+      double pn = fma(d[q], p, -c[q] * pm);
+      if (__builtin_expect(is_zero(pn), 0)) pn = p * 0x1p-50;
+      cnt += (int)((unsigned)(top_word(pn) ^ top_word(p)) >> 31);
+      pm = p;
+      p = pn;
+    }
+    if (i + 7 < k) {
+      const int m = top_word(p) & 0x7fffffff;   // exponent and leading bits of |p|
+      if (m >= (1023 + 500) << 20) {
         p *= 0x1p-500;
         pm *= 0x1p-500;
-      } else if (m < 0x1p-500) {
+      } else if (m < (1023 - 500) << 20) {
         p *= 0x1p500;
         pm *= 0x1p500;
       }
@@ -449,10 +500,22 @@ __device__ void tridiag_inverse_iteration(const double* a_s, const double* b_s, 
   }
 }
 
-// Lowest eigenpair of the k x k tridiagonal Lanczos matrix, k = j + 1; one warp. The Ritz value
-// is FP64 (it decides convergence); the vector comes from FP64 inverse iteration, or FP32
-// (vec32) when the Lanczos matvecs are reduced-precision.
-__global__ void k_tridiag_lowest(LzState* st, int vec32) {
+// x / 33, rounded to nearest: the product with the rounded reciprocal and one correction of its remainder
+// (Markstein, IBM J. Res. Dev. 34, 1990), three FP64 operations instead of a division's sequence.
+// Where the quotient could be subnormal or infinite, the division.
+__device__ __forceinline__ double div33(double x) {
+  constexpr double r = 1.0 / 33.0;
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  if (e < 80 || e > 2000) return x / 33.0;
+  const double q = x * r;
+  return fma(fma(-33.0, q, x), r, q);
+}
+
+// Lowest eigenvalue of the k x k tridiagonal Lanczos matrix, k = j + 1, in FP64 (it decides convergence);
+// one warp. Ends the step: j + 1. Serial: ~10 Sturm counts of k rows of 3 FP64 operations each; with
+// comparisons on the FP64 pipe and the eigenvector in every step it took 35 us at k = 10 and 98 us at
+// k = 20 (of 310 us for a BF16X3 step at chi = 1024), now TRIDIAG_US.
+__global__ void k_tridiag_lowest(LzState* st) {
   const int k = st->j + 1;
   const int lane = threadIdx.x;
   __shared__ double a_s[MRD_LANCZOS_MAX_ITER + 1], b_s[MRD_LANCZOS_MAX_ITER + 1], b2_s[MRD_LANCZOS_MAX_ITER + 1];
@@ -501,26 +564,36 @@ __global__ void k_tridiag_lowest(LzState* st, int vec32) {
   for (int it = 0; it < 40; ++it) {
     if (!(hi - lo > 1e-14 * fmax(fabs(lo), fabs(hi))) || hi - lo == prev_w) break;
     prev_w = hi - lo;
-    const double x = lo + (hi - lo) * (lane + 1) / 33.0;
+    const double x = lo + div33((hi - lo) * (lane + 1));
     const int c = sturm_count(a_s, b2_s, k, x);
     const unsigned m = __ballot_sync(0xffffffffu, c >= 1);
-    if (m == 0) {
-      lo = lo + (hi - lo) * 32.0 / 33.0;
-    } else {
-      const int f = __ffs(m) - 1;  // first point with at least one eigenvalue below
-      const double nlo = f > 0 ? lo + (hi - lo) * f / 33.0 : lo;
-      hi = lo + (hi - lo) * (f + 1) / 33.0;
-      lo = nlo;
-    }
+    const int f = m ? __ffs(m) - 1 : 32;  // first point with at least one eigenvalue below
+    const double below = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0), above = __shfl_sync(0xffffffffu, x, f & 31);
+    if (f > 0) lo = below;
+    if (f < 32) hi = above;
   }
   if (lane != 0) return;
   const double lam = 0.5 * (lo + hi);
   st->energy = lam;
   st->ritz[k - 1] = lam;
+  st->j = k;
+}
+
+// Eigenvector at the lowest Ritz value of the last step, for the ground vector (once per run): FP64
+// inverse iteration, or FP32 (vec32) when the Lanczos matvecs are reduced-precision.
+__global__ void k_tridiag_vector(LzState* st, int vec32) {
+  const int k = st->j;
+  __shared__ double a_s[MRD_LANCZOS_MAX_ITER + 1], b_s[MRD_LANCZOS_MAX_ITER + 1];
+  for (int i = threadIdx.x; i < k; i += 32) {
+    a_s[i] = st->alpha[i];
+    b_s[i] = st->beta[i];
+  }
+  __syncwarp();
+  if (threadIdx.x != 0) return;
   if (vec32)
-    tridiag_inverse_iteration<float>(a_s, b_s, k, lam, 3, st->y);
+    tridiag_inverse_iteration<float>(a_s, b_s, k, st->energy, 3, st->y);
   else
-    tridiag_inverse_iteration<double>(a_s, b_s, k, lam, 3, st->y);
+    tridiag_inverse_iteration<double>(a_s, b_s, k, st->energy, 3, st->y);
 }
 
 }  // namespace
@@ -539,6 +612,7 @@ struct Lanczos {
   float2* w32 = nullptr;
   bool fp32_full = false;      // full Gram-Schmidt pass in FP32 (reduced-precision matvecs)
   LzState* st = nullptr;
+  int* ticket = nullptr;       // CTAs of a reduction that have finished; zero between launches
   LzState* st_host = nullptr;  // pinned
   cudaStream_t stream = nullptr;   // stream of the memory cache the buffers return to
   // captured Lanczos step: valid while the operator's key is unchanged
@@ -551,7 +625,7 @@ struct Lanczos {
 void lanczos_free(Lanczos* L) {
   if (!L) return;
   for (void* p : {(void*)L->V, (void*)L->w, (void*)L->vin, (void*)L->partial, (void*)L->c1, (void*)L->c2,
-                  (void*)L->scal, (void*)L->st, (void*)L->V32, (void*)L->w32, (void*)L->partial32})
+                  (void*)L->scal, (void*)L->st, (void*)L->ticket, (void*)L->V32, (void*)L->w32, (void*)L->partial32})
     cache_free(p, L->stream);
   if (L->st_host) cache_free_host(L->st_host);
   if (L->step_exec) cudaGraphExecDestroy(L->step_exec);
@@ -573,6 +647,8 @@ cudaError_t lanczos_alloc(Lanczos** out, int64_t n, cudaStream_t stream) {
   if (e == cudaSuccess) e = dev(&L->c2, kv * 16);
   if (e == cudaSuccess) e = dev(&L->scal, 4 * 16);
   if (e == cudaSuccess) e = dev(&L->st, sizeof(LzState));
+  if (e == cudaSuccess) e = dev(&L->ticket, 16);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L->ticket, 0, 16, stream);
   if (e == cudaSuccess) e = cache_alloc_host((void**)&L->st_host, sizeof(LzState));
   if (e != cudaSuccess) {
     lanczos_free(L);
@@ -605,11 +681,9 @@ cudaError_t lanczos_set_fp32_full(Lanczos* L, bool on) {
 }
 
 // nv >= 0: dots of v_0 .. v_{nv-1}; nv < 0: of v_0 .. v_j (j from the device state)
-static cudaError_t dots(Lanczos* L, const double2* V, int nv, const double2* w, double2* out, cudaStream_t s) {
-  k_multidot<<<kRedBlocks, kRedThreads, 0, s>>>(V, L->n, nv, L->st, w, L->n, L->partial);
-  mrd::count_launch();
-  const int nmax = nv >= 0 ? nv : MRD_LANCZOS_MAX_ITER + 1;
-  k_finish_dots<<<(nmax + 3) / 4, 128, 0, s>>>(L->partial, kRedBlocks, nv, L->st, out);
+static cudaError_t dots(Lanczos* L, const double2* V, int nv, const double2* w, double2* out, cudaStream_t s,
+                        bool record = false) {
+  k_multidot<<<kRedBlocks, kRedThreads, 0, s>>>(V, L->n, nv, L->st, w, L->n, L->partial, L->ticket, out, record, L->c1, L->c2);
   mrd::count_launch();
   return cudaGetLastError();
 }
@@ -626,39 +700,29 @@ static unsigned grid_for(int64_t n) {
 static int lanczos_step(Lanczos* L, mrd_ctx* ctx, int (*apply)(void*, const double2*, double2*), void* op) {
   cudaStream_t s = ctx->stream;
   const int64_t n = L->n;
-  k_copy_vj<<<grid_for(n), 256, 0, s>>>(L->V, n, L->st, L->vin);
-  mrd::count_launch();
   int rc = apply(op, L->vin, L->w);
   if (rc != MRD_OK) return rc;
   s = ctx->stream;
   // local pass against v_{j-1}, v_j (the three-term recurrence), then one full classical
   // Gram-Schmidt pass against v_0 .. v_j that removes what rounding left
   MRD_CUDA(ctx, dots(L, L->V, -2, L->w, L->c1, s));
-  k_sub_combination<<<grid_for(n), 256, 0, s>>>(L->V, n, -2, L->st, L->c1, L->w, n);
+  k_sub_combination<<<grid_for(n), 256, 0, s>>>(L->V, n, -2, L->st, L->c1, L->w, n, L->fp32_full ? L->w32 : nullptr);
   mrd::count_launch();
   if (L->fp32_full) {
-    k_to_f32<<<grid_for(n), 256, 0, s>>>(L->w, L->w32, n);
-    k_multidot32<<<(unsigned)md32_blocks(n), 256, 0, s>>>(L->V32, n, L->st, L->w32, n, L->partial32);
-    k_finish_dots<<<(MRD_LANCZOS_MAX_ITER + 1 + 3) / 4, 128, 0, s>>>(L->partial32, (int)md32_blocks(n), -1, L->st,
-                                                                      L->c2);
+    k_multidot32<<<(unsigned)md32_blocks(n), md32_blocks(n) < 304 ? 512 : 256, 0, s>>>(L->V32, n, L->st, L->w32, n, L->partial32);
+    k_finish_dots<<<(MRD_LANCZOS_MAX_ITER + 1 + 3) / 4, 128, 0, s>>>(L->partial32, (int)md32_blocks(n), L->st, L->c2);
     k_sub_combination32<<<grid_for(n), 256, 0, s>>>(L->V32, n, L->st, L->c2, L->w, n);
-    mrd::count_launches(4);
+    mrd::count_launches(3);
   } else {
-    MRD_CUDA(ctx, dots(L, L->V, -1, L->w, L->c2, s));
-    k_sub_combination<<<grid_for(n), 256, 0, s>>>(L->V, n, -1, L->st, L->c2, L->w, n);
-    mrd::count_launch();
+    MRD_CUDA(ctx, dots(L, L->V, -1, L->w, nullptr, s));
+    k_finish_dots<<<(MRD_LANCZOS_MAX_ITER + 1 + 3) / 4, 128, 0, s>>>(L->partial, kRedBlocks, L->st, L->c2);
+    k_sub_combination<<<grid_for(n), 256, 0, s>>>(L->V, n, -1, L->st, L->c2, L->w, n, nullptr);
+    mrd::count_launches(2);
   }
-  k_record_alpha<<<1, 1, 0, s>>>(L->st, L->c1, L->c2);
-  mrd::count_launch();
-  MRD_CUDA(ctx, dots(L, L->w, 1, L->w, L->scal, s));
-  k_record_beta<<<1, 1, 0, s>>>(L->st, L->scal);
-  mrd::count_launch();
-  k_tridiag_lowest<<<1, 32, 0, s>>>(L->st, L->fp32_full ? 1 : 0);
-  mrd::count_launch();
-  k_scale_next<<<grid_for(n), 256, 0, s>>>(L->w, L->V, n, L->st, L->fp32_full ? L->V32 : nullptr);
-  mrd::count_launch();
-  k_next_step<<<1, 1, 0, s>>>(L->st);
-  mrd::count_launch();
+  MRD_CUDA(ctx, dots(L, L->w, 1, L->w, L->scal, s, true));
+  k_scale_next<<<grid_for(n), 256, 0, s>>>(L->w, L->V, n, L->st, L->vin, L->fp32_full ? L->V32 : nullptr);
+  k_tridiag_lowest<<<1, 32, 0, s>>>(L->st);
+  mrd::count_launches(2);
   MRD_CUDA(ctx, cudaGetLastError());
   MRD_CUDA(ctx, cudaMemcpyAsync(L->st_host, L->st, sizeof(LzState), cudaMemcpyDeviceToHost, s));
   return MRD_OK;
@@ -724,9 +788,7 @@ int lanczos_run(Lanczos* L, mrd_ctx* ctx, int (*apply)(void*, const double2*, do
     return mrd_fail(ctx, MRD_E_ARG, "mrd_lanczos: max_iter out of range");
   // v_0 = theta / |theta|
   MRD_CUDA(ctx, dots(L, theta, 1, theta, L->scal, s));
-  k_scale_by_invnorm<<<grid_for(n), 256, 0, s>>>(theta, L->V, n, L->scal, L->fp32_full ? L->V32 : nullptr);
-  mrd::count_launch();
-  k_set_step<<<1, 1, 0, s>>>(L->st, 0);
+  k_scale_by_invnorm<<<grid_for(n), 256, 0, s>>>(theta, L->V, n, L->scal, L->vin, L->fp32_full ? L->V32 : nullptr, L->st);
   mrd::count_launch();
   MRD_CUDA(ctx, cudaGetLastError());
   bool graph = graph_key != 0 && (L->step_exec && L->step_key == graph_key);
@@ -756,10 +818,12 @@ int lanczos_run(Lanczos* L, mrd_ctx* ctx, int (*apply)(void*, const double2*, do
     e_prev = e;
   }
   // ground vector = V y, normalised
+  k_tridiag_vector<<<1, 32, 0, s>>>(L->st, L->fp32_full ? 1 : 0);
+  mrd::count_launch();
   k_combination_real<<<grid_for(n), 256, 0, s>>>(L->V, n, k, L->st->y, L->w, n);
   mrd::count_launch();
   MRD_CUDA(ctx, dots(L, L->w, 1, L->w, L->scal, s));
-  k_scale_by_invnorm<<<grid_for(n), 256, 0, s>>>(L->w, theta, n, L->scal, nullptr);
+  k_scale_by_invnorm<<<grid_for(n), 256, 0, s>>>(L->w, theta, n, L->scal, nullptr, nullptr, nullptr);
   mrd::count_launch();
   MRD_CUDA(ctx, cudaGetLastError());
   MRD_CUDA(ctx, cudaStreamSynchronize(s));
