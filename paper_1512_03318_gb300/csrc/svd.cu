@@ -153,6 +153,116 @@ __device__ __forceinline__ bool jacobi_pair(T2* xi, T2* xj, int p, T2* vi, T2* v
   return true;
 }
 
+// FP64 version of jacobi_pair, with the columns' squared norms na, nb kept by the caller. An FP64
+// warp instruction occupies its quarter of an SM for 64 cycles whatever its lanes do (measured; a
+// division is 23 of them, a square root 13), and the first form spent more of them on the scalars of a
+// pair (3 divisions, 4 square roots, 20 shuffle additions: ~140) than on its elements (at p = 128, 80).
+// So square roots come from an FP32 seed and one third-order step, tests compare bits or squares,
+// the two sums share one shuffle tree, and the norms follow from the rotation: ~35 instructions. One sweep
+// at Ly = 6, chi = 512: 0.96 -> 0.57 ms, the update 18.5 -> 12.5.
+__device__ __forceinline__ bool bits_less_equal(double a, double b) {   // of non-negative numbers
+  return __double_as_longlong(a) <= __double_as_longlong(b);
+}
+
+// A float close to |x| (truncated mantissa; |x| within the FP32 exponent range), and a double from a normal
+// float, without the FP64 pipe.
+__device__ __forceinline__ float mag_f32(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  return __int_as_float(((hi >> 20) - 1023 + 127) << 23 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double from_f32(float x) {
+  const int i = __float_as_int(x);
+  return __hiloint2double((i & 0x80000000) | (((i >> 3) & 0x0fffffff) + ((1023 - 127) << 20)), i << 29);
+}
+
+// 1 / sqrt(x), x > 0 normal, to ~1 ulp: an FP32 seed y (error e = 1 - x y^2 ~ 2^-21) and y (1 + e / 2 + 3 e^2 / 8).
+__device__ __forceinline__ double rsqrt_fp64(double x) {
+  const int hi = __double2hiint(x);
+  const int k = ((hi >> 20) - 1023) & ~1;                                    // x = m 2^k, m in [1, 4)
+  const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
+  const double y = from_f32(rsqrtf(mag_f32(m)));
+  const double e = fma(-(m * y), y, 1.0);
+  const double r = fma(y * e, fma(0.375, e, 0.5), y);
+  return __hiloint2double(__double2hiint(r) - ((k / 2) << 20), __double2loint(r));
+}
+
+template <bool REAL>
+__device__ __forceinline__ double norm2_fp64(const double2* x, int p, int lane) {
+  double s = 0.0;
+  for (int t = lane; t < p; t += 32) {
+    const double2 u = x[t];
+    s = REAL ? fma(u.x, u.x, s) : fma(u.x, u.x, fma(u.y, u.y, s));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+template <bool REAL>
+__device__ __forceinline__ bool jacobi_pair_fp64(double2* xi, double2* xj, int p, double tol2, double floor2, double& na,
+                                                 double& nb, int lane) {
+  const double a = na, b = nb;
+  if (bits_less_equal(a, floor2) || bits_less_equal(b, floor2)) return false;
+  double gr = 0.0, gi = 0.0;
+  for (int t = lane; t < p; t += 32) {
+    const double2 u = xi[t], v = xj[t];
+    if (REAL) {
+      gr = fma(u.x, v.x, gr);
+    } else {
+      gr = fma(u.x, v.x, fma(u.y, v.y, gr));     // Re(conj(u) v)
+      gi = fma(u.x, v.y, fma(-u.y, v.x, gi));    // Im(conj(u) v)
+    }
+  }
+  {   // lanes 0 .. 15 end up with the sum of gr, 16 .. 31 with that of gi
+    const bool up = !REAL && (lane & 16);
+    double s = REAL ? gr + __shfl_xor_sync(0xffffffffu, gr, 16) : (up ? gi : gr) + __shfl_xor_sync(0xffffffffu, up ? gr : gi, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    gr = __shfl_sync(0xffffffffu, s, 0);
+    gi = REAL ? 0.0 : __shfl_sync(0xffffffffu, s, 16);
+  }
+  const double g2 = REAL ? gr * gr : fma(gr, gr, gi * gi);
+  // |g| > tol sqrt(a b); a NaN or an overflow does not rotate
+  if (bits_less_equal(g2, tol2 * a * b) || __double2hiint(g2) >= 0x7ff00000 || __double2hiint(g2) < 0x00200000) return false;
+  // phase-free real rotation on (x_i, e^{-i phi} x_j), phi = arg(gamma)
+  const double ig = rsqrt_fp64(g2);
+  const double ph_r = gr * ig, ph_i = -gi * ig;
+  const double zeta = (b - a) * (0.5 * ig);
+  double tt;
+  {   // t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)): in FP32, then one Newton step for t^2 + 2 zeta t = 1
+    const int ex = ((__double2hiint(zeta) >> 20) & 0x7ff) - 1023;
+    const bool neg = __double2hiint(zeta) < 0;
+    if (ex > 120) return false;                   // no representable rotation
+    const float z = ex < -60 ? 0.f : mag_f32(zeta);
+    const float t0 = z > 1e9f ? 0.5f / z : 1.f / (z + sqrtf(1.f + z * z));
+    const float r0 = 0.5f / (t0 + z);             // 1 / f'
+    const double t1 = from_f32(t0), zz = neg ? -zeta : zeta;
+    tt = fma(-fma(t1, fma(2.0, zz, t1), -1.0), from_f32(r0), t1);
+    tt = neg ? -tt : tt;
+  }
+  const double c = rsqrt_fp64(fma(tt, tt, 1.0)), sn = c * tt;
+  for (int k = lane; k < p; k += 32) {
+    const double2 u = xi[k], v0 = xj[k];
+    if (REAL) {
+      const double vx = v0.x * ph_r;
+      xi[k] = make_double2(c * u.x - sn * vx, 0.0);
+      xj[k] = make_double2(sn * u.x + c * vx, 0.0);
+    } else {
+      const double vx = v0.x * ph_r - v0.y * ph_i, vy = v0.x * ph_i + v0.y * ph_r;
+      xi[k] = make_double2(c * u.x - sn * vx, c * u.y - sn * vy);
+      xj[k] = make_double2(sn * u.x + c * vx, sn * u.y + c * vy);
+    }
+  }
+  // |x_i'|^2 = a - t |g|, |x_j'|^2 = b + t |g|; summed anew where that cancels
+  const double tg = tt * (g2 * ig);
+  na = a - tg;
+  nb = b + tg;
+  __syncwarp();
+  if (!bits_less_equal(0.125 * a, na) || __double2hiint(na) < 0) na = norm2_fp64<REAL>(xi, p, lane);
+  if (!bits_less_equal(0.125 * b, nb) || __double2hiint(nb) < 0) nb = norm2_fp64<REAL>(xj, p, lane);
+  return true;
+}
+
 // Float-float version of jacobi_pair: columns of complex float-float values (float4 =
 // re.hi, im.hi, re.lo, im.lo) on the FP32 pipes. Dot products are accumulated and reduced
 // in float-float (~48 bits, so the orthogonality test resolves 5e-13); the rotation
@@ -308,6 +418,7 @@ __global__ void __launch_bounds__(512) k_svd_bround(T2* __restrict__ work, const
   __shared__ unsigned long long n_tested, n_rotated;   // element-pairs tested / rotated
   __shared__ int s_last[32];   // sweep in which each staged column last rotated
   __shared__ FF s_norm[32];    // float-float column norms (MODE 2)
+  __shared__ double s_norm2[32];   // FP64 squared column norms (MODE 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
   const int64_t cta = blockIdx.x;
   int lo = 0, hi = nblk - 1;   // largest k with grp_prefix[k] <= cta; the CTAs run over the
@@ -392,6 +503,14 @@ __global__ void __launch_bounds__(512) k_svd_bround(T2* __restrict__ work, const
     }
     __syncthreads();
   }
+  if constexpr (MODE == 1) {
+    for (int cc = warp; cc < nI + nJ; cc += nwarp) {
+      const int lc = cc < nI ? cc : W + cc - nI;
+      const double s = norm2_fp64<REAL>((const double2*)sx + (int64_t)lc * p, p, lane);
+      if (lane == 0) s_norm2[lc] = s;
+    }
+    __syncthreads();
+  }
   const double floor2 = zero_rel * fro2[b];
   // A pair found orthogonal in the previous sweep stays orthogonal while neither column
   // rotates: pairs whose columns last rotated before the previous sweep are skipped (the
@@ -406,6 +525,13 @@ __global__ void __launch_bounds__(512) k_svd_bround(T2* __restrict__ work, const
       if (rot && lane == 0) {
         s_norm[i] = na;
         s_norm[j] = nb;
+      }
+    } else if constexpr (MODE == 1) {
+      double na = s_norm2[i], nb = s_norm2[j];
+      rot = jacobi_pair_fp64<REAL>(sx + (int64_t)i * p, sx + (int64_t)j * p, p, (double)tol * (double)tol, floor2, na, nb, lane);
+      if (rot && lane == 0) {
+        s_norm2[i] = na;
+        s_norm2[j] = nb;
       }
     } else {
       rot = jacobi_pair<T, T2, REAL>(sx + (int64_t)i * p, sx + (int64_t)j * p, p, V ? sv + (int64_t)i * r : nullptr,
