@@ -12,7 +12,7 @@
 //
 // All vector arithmetic runs in FP64 on the device with fixed-shape reductions (partial sums
 // per CTA, then the last CTA to finish sums them in a fixed order), so results are bit-reproducible
-// run to run. The tridiagonal eigenproblem is solved on the device by one warp: Sturm-count
+// run to run. The tridiagonal eigenproblem is solved on the device by one CTA: Sturm-count
 // multisection for the lowest eigenvalue at every step, inverse iteration with a pivoted tridiagonal LU
 // for its vector at the end. A step is launch bound at small sizes: eight kernels besides the
 // operator's.
@@ -112,7 +112,7 @@ __device__ __forceinline__ void record_step(LzState* st, const double2* c1, cons
 // out[j] = conj(V_j) . w, j < nv: partial[b * nv + j] over each CTA's share (re, im interleaved), summed
 // by the last CTA (out null: by k_finish_dots). Bound by the FP64 pipe where the vectors are short (16
 // cycles per warp instruction): rows of threads without elements and vectors beyond nv are skipped.
-// MULTIDOT_US. record (with c1, c2): the dot is |w|^2 of a step, which is recorded.
+// 17.5 -> 11 us at n = 84,000 with two vectors. record (with c1, c2): the dot is |w|^2 of a step, which is recorded.
 __global__ void __launch_bounds__(kRedThreads) k_multidot(const double2* __restrict__ V, int64_t ldv, int nv_arg,
                                                           LzState* st, const double2* __restrict__ w, int64_t n,
                                                           double2* partial, int* ticket, double2* out, bool record,
@@ -362,8 +362,8 @@ __global__ void k_scale_next(const double2* __restrict__ w, double2* __restrict_
 // pivot). A row then changes the minors' scale by at most ~2^50 (the guard) and otherwise by
 // |a_i - x| + b_{i-1}^2, so every 8 rows both are rescaled by 2^-+500 when p_i has left
 // [2^-500, 2^500], and neither leaves the FP64 range in between.
-// Signs, zeros and magnitudes are read off the bits: a comparison of doubles would run on the FP64 pipe
-// (2 lanes per SM, 16 cycles for a warp) like the three operations of the recurrence itself.
+// Signs, zeros and magnitudes are read off the bits: every FP64 warp instruction, a comparison too, takes
+// its quarter of the SM for 64 cycles (measured), like the three operations of the recurrence itself.
 __device__ __forceinline__ int top_word(double p) { return __double2hiint(p); }
 __device__ __forceinline__ bool is_zero(double p) { return ((top_word(p) & 0x7fffffff) | __double2loint(p)) == 0; }
 
@@ -385,7 +385,7 @@ __device__ int sturm_count(const double* a, const double* b2, int k, double x) {
     for (int q = 0; q < 8; ++q) {
       if (i + q >= k) break;
       double pn = fma(d[q], p, -c[q] * pm);
-      if (__builtin_expect(is_zero(pn), 0)) pn = p * 0x1p-50;
+      if (is_zero(pn)) pn = __hiloint2double(top_word(p) - (50 << 20), __double2loint(p));   // (p is normal)
       cnt += (int)((unsigned)(top_word(pn) ^ top_word(p)) >> 31);
       pm = p;
       p = pn;
@@ -500,33 +500,41 @@ __device__ void tridiag_inverse_iteration(const double* a_s, const double* b_s, 
   }
 }
 
-// x / 33, rounded to nearest: the product with the rounded reciprocal and one correction of its remainder
-// (Markstein, IBM J. Res. Dev. 34, 1990), three FP64 operations instead of a division's sequence.
-// Where the quotient could be subnormal or infinite, the division.
-__device__ __forceinline__ double div33(double x) {
-  constexpr double r = 1.0 / 33.0;
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  if (e < 80 || e > 2000) return x / 33.0;
-  const double q = x * r;
-  return fma(fma(-33.0, q, x), r, q);
+// The same count in FP32, in the form that cannot overflow (pivots q_i = a_i - x - b_{i-1}^2 / q_{i-1}).
+__device__ int sturm_count32(const float* a, const float* b2, int k, float x) {
+  float q = a[0] - x;
+  int cnt = q < 0.f;
+  for (int i = 1; i < k; ++i) {
+    if (fabsf(q) < 1e-30f) q = 1e-30f;
+    q = a[i] - x - __fdividef(b2[i - 1], q);
+    cnt += q < 0.f;
+  }
+  return cnt;
 }
 
 // Lowest eigenvalue of the k x k tridiagonal Lanczos matrix, k = j + 1, in FP64 (it decides convergence);
-// one warp. Ends the step: j + 1. Serial: ~10 Sturm counts of k rows of 3 FP64 operations each; with
-// comparisons on the FP64 pipe and the eigenvector in every step it took 35 us at k = 10 and 98 us at
-// k = 20 (of 310 us for a BF16X3 step at chi = 1024), now TRIDIAG_US.
-__global__ void k_tridiag_lowest(LzState* st) {
+// four warps, one per quarter of the SM. Ends the step: j + 1. Sturm counts at 128 points cut a bracket to
+// 1/127 of its width; its time is the FP64 instructions of k rows (192 cycles each), so the first digits
+// come from FP32 counts (scaled to the bracket, right to ~1e-6 of it), checked by the first FP64 counts.
+// One warp with 33 sections from the start, FP64 comparisons and the eigenvector in every step: 35 us at
+// k = 10, 98 us at k = 20; without the vector 42 at k = 20; now 23.
+constexpr int kTriPoints = 128;
+
+__global__ void __launch_bounds__(kTriPoints) k_tridiag_lowest(LzState* st) {
   const int k = st->j + 1;
-  const int lane = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ double a_s[MRD_LANCZOS_MAX_ITER + 1], b_s[MRD_LANCZOS_MAX_ITER + 1], b2_s[MRD_LANCZOS_MAX_ITER + 1];
-  for (int i = lane; i < k; i += 32) {
-    a_s[i] = st->alpha[i];
-    b_s[i] = st->beta[i];
-    b2_s[i] = st->beta[i] * st->beta[i];
+  __shared__ float a32[MRD_LANCZOS_MAX_ITER + 1], b32[MRD_LANCZOS_MAX_ITER + 1];
+  __shared__ double x_s[kTriPoints];
+  __shared__ int first_s[kTriPoints / 32];
+  if (tid < k) {
+    a_s[tid] = st->alpha[tid];
+    b_s[tid] = st->beta[tid];
+    b2_s[tid] = st->beta[tid] * st->beta[tid];
   }
-  __syncwarp();
+  __syncthreads();
   // the lowest eigenvalue lies between the lowest Gershgorin bound and the smallest diagonal
-  // element (a Rayleigh quotient of a unit vector); every lane holds the same bracket
+  // element (a Rayleigh quotient of a unit vector); every thread holds the same bracket
   double lo = 1e300, hi = 1e300;
   for (int i = lane; i < k; i += 32) {
     const double r = (i > 0 ? fabs(b_s[i - 1]) : 0.0) + (i + 1 < k ? fabs(b_s[i]) : 0.0);
@@ -538,42 +546,81 @@ __global__ void k_tridiag_lowest(LzState* st) {
     lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
     hi = fmin(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
-  const double pad = 1e-12 * fmax(fabs(lo), fabs(hi)) + 1e-300;
+  const double big = fmax(fabs(lo), fabs(hi)), pad = 1e-12 * big + 1e-300;
   lo -= pad;
   hi += pad;
-  // warm start: by interlacing the lowest eigenvalue of T_k is at most that of T_{k-1}; late
-  // in a run it moves little, so try [E_{k-1} - 4|E_{k-1} - E_{k-2}|, E_{k-1}], padded, and
-  // keep it where Sturm counts confirm it (no eigenvalue below, at least one below the top),
-  // the two counts on lanes 0 and 1; otherwise the Gershgorin bracket
+  // index of the first point with an eigenvalue below it (kTriPoints if none)
+  auto first_above = [&](bool above) {
+    const unsigned m = __ballot_sync(0xffffffffu, above);
+    if (lane == 0) first_s[warp] = m ? warp * 32 + __ffs(m) - 1 : kTriPoints;
+    __syncthreads();
+    int f = kTriPoints;
+    for (int w = 0; w < kTriPoints / 32; ++w) f = min(f, first_s[w]);
+    __syncthreads();
+    return f;
+  };
+  // Narrower bracket to try first. Warm start: by interlacing the lowest eigenvalue of T_k is at most
+  // that of T_{k-1}, and late in a run it moves little: [E_{k-1} - 4 |E_{k-1} - E_{k-2}|, E_{k-1}],
+  // padded. Else FP32 counts on (T - lo) / (hi - lo), whose lowest eigenvalue lies in [0, 1].
+  double tlo = lo, thi = hi;
+  bool tried = false;
   if (k >= 3) {
     const double e1 = st->ritz[k - 2], e2 = st->ritz[k - 3];
     const double tol = 1e-13 * fmax(fabs(e1), 1.0);
     const double wlo = e1 - 4.0 * fabs(e1 - e2) - tol, whi = e1 + tol;
-    if (wlo > lo && whi < hi) {
-      const int c = lane < 2 ? sturm_count(a_s, b2_s, k, lane == 0 ? wlo : whi) : 0;
-      const int c_lo = __shfl_sync(0xffffffffu, c, 0), c_hi = __shfl_sync(0xffffffffu, c, 1);
-      if (c_lo == 0 && c_hi >= 1) {
-        lo = wlo;
-        hi = whi;
-      }
+    if (wlo > lo && whi < hi && whi - wlo < 1e-4 * (hi - lo)) {
+      tlo = wlo;
+      thi = whi;
+      tried = true;
     }
   }
+  if (!tried && k >= 2) {
+    const double w = hi - lo, iw = 1.0 / w;
+    if (tid < k) {
+      a32[tid] = __double2float_rn((a_s[tid] - lo) * iw);
+      const float b = __double2float_rn(b_s[tid] * iw);
+      b32[tid] = b * b;
+    }
+    __syncthreads();
+    float flo = 0.f, fhi = 1.f;
+    for (int it = 0; it < 3; ++it) {
+      const float x = flo + (fhi - flo) * ((float)tid / (kTriPoints - 1));
+      const int f = first_above(sturm_count32(a32, b32, k, x) >= 1);
+      const float nlo = f > 0 ? flo + (fhi - flo) * ((float)(f - 1) / (kTriPoints - 1)) : flo;
+      if (f < kTriPoints) fhi = flo + (fhi - flo) * ((float)f / (kTriPoints - 1));
+      flo = nlo;
+    }
+    // the counts err by a few FP32 roundings of the largest entries, which |a - lo| <= 2 w bounds
+    tlo = lo + w * (double)(flo - 4e-6f);
+    thi = lo + w * (double)(fhi + 4e-6f);
+    tried = true;
+  }
   // multisection to 1e-14 relative width (the Ritz value is compared to 1e-10 and refined
-  // afterwards), or until a subdivision no longer shrinks the interval in FP64
+  // afterwards), or until a subdivision no longer shrinks the interval in FP64. The points include both
+  // ends of the bracket, so a trial bracket that does not hold the eigenvalue shows itself.
   double prev_w = 0.0;
   for (int it = 0; it < 40; ++it) {
-    if (!(hi - lo > 1e-14 * fmax(fabs(lo), fabs(hi))) || hi - lo == prev_w) break;
-    prev_w = hi - lo;
-    const double x = lo + div33((hi - lo) * (lane + 1));
-    const int c = sturm_count(a_s, b2_s, k, x);
-    const unsigned m = __ballot_sync(0xffffffffu, c >= 1);
-    const int f = m ? __ffs(m) - 1 : 32;  // first point with at least one eigenvalue below
-    const double below = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0), above = __shfl_sync(0xffffffffu, x, f & 31);
-    if (f > 0) lo = below;
-    if (f < 32) hi = above;
+    if (!tried) {
+      tlo = lo;
+      thi = hi;
+    }
+    if (!tried && (!(thi - tlo > 1e-14 * fmax(fabs(tlo), fabs(thi))) || thi - tlo == prev_w)) break;
+    const double x = tid == kTriPoints - 1 ? thi : tlo + (thi - tlo) * ((double)tid * (1.0 / (kTriPoints - 1)));
+    x_s[tid] = x;
+    const int f = first_above(sturm_count(a_s, b2_s, k, x) >= 1);
+    if (tried && (f == 0 || f == kTriPoints)) {   // not in the trial bracket
+      tried = false;
+      prev_w = 0.0;
+      continue;
+    }
+    prev_w = thi - tlo;
+    hi = f < kTriPoints ? x_s[f] : thi;
+    lo = f > 0 ? x_s[f - 1] : tlo;
+    tried = false;
+    __syncthreads();
   }
-  if (lane != 0) return;
-  const double lam = 0.5 * (lo + hi);
+  if (tid != 0) return;
+  const double lam = 0.5 * (tlo + thi);
   st->energy = lam;
   st->ritz[k - 1] = lam;
   st->j = k;
@@ -721,7 +768,7 @@ static int lanczos_step(Lanczos* L, mrd_ctx* ctx, int (*apply)(void*, const doub
   }
   MRD_CUDA(ctx, dots(L, L->w, 1, L->w, L->scal, s, true));
   k_scale_next<<<grid_for(n), 256, 0, s>>>(L->w, L->V, n, L->st, L->vin, L->fp32_full ? L->V32 : nullptr);
-  k_tridiag_lowest<<<1, 32, 0, s>>>(L->st);
+  k_tridiag_lowest<<<1, kTriPoints, 0, s>>>(L->st);
   mrd::count_launches(2);
   MRD_CUDA(ctx, cudaGetLastError());
   MRD_CUDA(ctx, cudaMemcpyAsync(L->st_host, L->st, sizeof(LzState), cudaMemcpyDeviceToHost, s));
