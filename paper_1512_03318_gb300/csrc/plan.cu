@@ -25,20 +25,17 @@ constexpr int kTile = 32;
 
 __device__ int64_t block_scan(int64_t* v, int64_t n, int64_t* smem) {
   // exclusive prefix sum in place over v[0..n); returns the total. All threads call it; the
-  // CTA has a multiple of 32 threads, at most 1024. Each thread sums a contiguous chunk; the
-  // chunk sums are scanned by shuffles within each warp and then over the warps' totals.
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-  const int64_t chunk = (n + nt - 1) / nt;
-  const int64_t b = tid * chunk;
-  const int64_t e = b + chunk < n ? b + chunk : n;
+  // CTA has a multiple of 32 threads, at most 1024. A warp takes a contiguous part, 32 consecutive
+  // elements at a time: first the sums of the parts (independent loads), then the prefixes.
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int64_t part = ((n + nw - 1) / nw + 31) / 32 * 32;
+  const int64_t b = wid * part < n ? wid * part : n, e = b + part < n ? b + part : n;
   int64_t s = 0;
-  for (int64_t i = b; i < e; ++i) s += v[i];
-  int64_t x = s;   // inclusive prefix of the chunk sums within the warp
-  for (int o = 1; o < 32; o <<= 1) {
-    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) smem[wid] = x;
+#pragma unroll 8
+  for (int64_t i = b + lane; i < e; i += 32) s += v[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) smem[wid] = s;
   __syncthreads();
   if (wid == 0) {   // inclusive prefix of the warps' totals
     int64_t t = lane < nw ? smem[lane] : 0;
@@ -49,12 +46,23 @@ __device__ int64_t block_scan(int64_t* v, int64_t n, int64_t* smem) {
     smem[32 + lane] = t;
   }
   __syncthreads();
-  int64_t acc = (wid > 0 ? smem[32 + wid - 1] : 0) + x - s;
+  int64_t acc = wid > 0 ? smem[32 + wid - 1] : 0;
   const int64_t total = smem[32 + nw - 1];
-  for (int64_t i = b; i < e; ++i) {
-    const int64_t y = v[i];
-    v[i] = acc;
-    acc += y;
+  constexpr int kT = 4;   // tiles whose loads are in flight together
+  for (int64_t i0 = b; i0 < e; i0 += 32 * kT) {
+    int64_t y[kT];
+#pragma unroll
+    for (int q = 0; q < kT; ++q) y[q] = i0 + 32 * q + lane < e ? v[i0 + 32 * q + lane] : 0;
+#pragma unroll
+    for (int q = 0; q < kT; ++q) {
+      int64_t x = y[q];   // inclusive prefix of the tile
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t z = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += z;
+      }
+      if (i0 + 32 * q + lane < e) v[i0 + 32 * q + lane] = acc + x - y[q];
+      acc += __shfl_sync(0xffffffffu, x, 31);
+    }
   }
   __syncthreads();
   return total;
@@ -114,29 +122,32 @@ __global__ void __launch_bounds__(1024) k_plan(PlanDims d, PlanPtrs p) {
   const int32_t *L = p.left, *Rs = p.right;
 
   // ---- P1: sort MPO entries by (w', s1', s1, w) and (w', s2, s2', w''); triple ranges
-  for (int i = tid; i < d.nnz_i; i += nt) {
+  // (each entry's rank is the number of smaller keys; the keys of up to kMidKeys entries in shared memory)
+  auto sort_entries = [&](int nnz, int32_t* perm, auto key_of) {
+    const bool staged = nnz <= kMidKeys;
+    if (staged)
+      for (int i = tid; i < nnz; i += nt) mkey[i] = key_of(i);
+    __syncthreads();
+    for (int i = tid; i < nnz; i += nt) {
+      const int64_t ki = staged ? mkey[i] : key_of(i);
+      int r = 0;
+#pragma unroll 4
+      for (int j = 0; j < nnz; ++j) {
+        const int64_t kj = staged ? mkey[j] : key_of(j);
+        r += (kj < ki) || (kj == ki && j < i);
+      }
+      perm[r] = i;
+    }
+    __syncthreads();
+  };
+  sort_entries(d.nnz_i, p.wi_perm, [&](int i) {   // entry (w, w', s1', s1): key (w', s1', s1, w)
     const int32_t* e = p.wi_idx + 4 * i;
-    int64_t ki = (((int64_t)e[1] * 2 + e[2]) * 2 + e[3]) * d.d_l + e[0];
-    int r = 0;
-    for (int j = 0; j < d.nnz_i; ++j) {
-      const int32_t* f = p.wi_idx + 4 * j;
-      int64_t kj = (((int64_t)f[1] * 2 + f[2]) * 2 + f[3]) * d.d_l + f[0];
-      r += (kj < ki) || (kj == ki && j < i);
-    }
-    p.wi_perm[r] = i;
-  }
-  for (int i = tid; i < d.nnz_j; i += nt) {
+    return (((int64_t)e[1] * 2 + e[2]) * 2 + e[3]) * d.d_l + e[0];
+  });
+  sort_entries(d.nnz_j, p.wj_perm, [&](int i) {   // entry (w', w'', s2', s2): key (w', s2, s2', w'')
     const int32_t* e = p.wj_idx + 4 * i;
-    // entry (w', w'', s2', s2): key (w', s2, s2', w'')
-    int64_t ki = (((int64_t)e[0] * 2 + e[3]) * 2 + e[2]) * d.d_r + e[1];
-    int r = 0;
-    for (int j = 0; j < d.nnz_j; ++j) {
-      const int32_t* f = p.wj_idx + 4 * j;
-      int64_t kj = (((int64_t)f[0] * 2 + f[3]) * 2 + f[2]) * d.d_r + f[1];
-      r += (kj < ki) || (kj == ki && j < i);
-    }
-    p.wj_perm[r] = i;
-  }
+    return (((int64_t)e[0] * 2 + e[3]) * 2 + e[2]) * d.d_r + e[1];
+  });
   for (int i = tid; i < d.d_m * 4; i += nt) {
     p.trip_i[2 * i] = p.trip_i[2 * i + 1] = 0;
     p.trip_j[2 * i] = p.trip_j[2 * i + 1] = 0;
@@ -420,50 +431,74 @@ __global__ void __launch_bounds__(1024) k_plan(PlanDims d, PlanPtrs p) {
   const int64_t flops1 = block_scan(p.scr_b, n_t1, smem);
 
   // ---- P7: step-2 tasks, items (m_out, s1', s2'): theta'[s1', s2'] = sum_{w', s2} Z WR
+  // one warp per task: its lanes look up 32 channels w' at a time (a chain of dependent loads each), and
+  // the segments found are numbered by a prefix over the lanes, in the order (w', s2)
   const int64_t n_t2 = nmid * 4;
-  for (int64_t i = tid; i < n_t2; i += nt) {
-    int mo = (int)(i >> 2), s1p = (int)((i >> 1) & 1), s2p = (int)(i & 1);
+  const int lane = tid & 31;
+  for (int64_t i = tid >> 5; i < n_t2; i += nt >> 5) {
+    const int mo = (int)(i >> 2), s1p = (int)((i >> 1) & 1), s2p = (int)(i & 1);
     const int64_t* mout = p.mid + MIDF * mo;
     int64_t* task = p.t2 + TF * i;
     int cnt = 0;
-    int64_t Mrows = 0, Ncols = 0, flops = 0;
-    int64_t ap = mout[5 + s1p], bp = mout[8 + s2p];
+    int64_t Mrows = 0, Ncols = 0, flops = 0, c_off = 0, ldc = 0;
+    const int64_t ap = mout[5 + s1p], bp = mout[8 + s2p];
     if (ap >= 0 && bp >= 0) {
       Mrows = L[3 * ap + 2];
       Ncols = Rs[3 * bp + 2];
-      int64_t rowoff_out = s1p ? mout[7] : 0;
-      int64_t coloff_out = s2p ? mout[10] : 0;
-      task[2] = mout[4] + rowoff_out * mout[3] + coloff_out;
-      task[3] = mout[3];
-      for (int wp = 0; wp < d.d_m; ++wp) {
-        int mi = mid_of((int)mout[0] - p.cm[2 * wp], kmod((int)mout[1] - p.cm[2 * wp + 1], M));
-        if (mi < 0) continue;
-        int64_t zi = (int64_t)wp * nmid + mi;
-        int64_t zid = p.zmap[zi];
-        if (zid < 0 || !(p.s1mask[zi] >> s1p & 1)) continue;
-        const int64_t* min_ = p.mid + MIDF * mi;
-        for (int s2 = 0; s2 < 2; ++s2) {
-          int64_t b = min_[8 + s2];
-          if (b < 0) continue;
-          int64_t wrid = p.wrmap[(((int64_t)wp * 2 + s2) * 2 + s2p) * d.n_r + b];
-          if (wrid < 0) continue;
-          int64_t* seg = p.seg2 + SF * (i * d.seg2_stride + cnt);
-          int64_t K = Rs[3 * b + 2];
-          seg[0] = p.z[ZF * zid + 5] + rowoff_out * min_[3] + (s2 ? min_[10] : 0);
-          seg[1] = min_[3];
-          seg[2] = p.wr[WRF * wrid + 7];
-          seg[3] = Ncols;
-          seg[4] = K;
-          seg[5] = 0;
-          flops += 8 * Mrows * Ncols * K;
-          ++cnt;
+      const int64_t rowoff_out = s1p ? mout[7] : 0;
+      c_off = mout[4] + rowoff_out * mout[3] + (s2p ? mout[10] : 0);
+      ldc = mout[3];
+      for (int w0 = 0; w0 < d.d_m; w0 += 32) {
+        const int wp = w0 + lane;
+        int64_t sg[2][5];
+        int n = 0;
+        if (wp < d.d_m) {
+          const int mi = mid_of((int)mout[0] - p.cm[2 * wp], kmod((int)mout[1] - p.cm[2 * wp + 1], M));
+          const int64_t zi = (int64_t)wp * nmid + mi;
+          const int64_t zid = mi < 0 ? -1 : p.zmap[zi];
+          if (zid >= 0 && (p.s1mask[zi] >> s1p & 1)) {
+            const int64_t* min_ = p.mid + MIDF * mi;
+            const int64_t z_off = p.z[ZF * zid + 5] + rowoff_out * min_[3];
+#pragma unroll
+            for (int s2 = 0; s2 < 2; ++s2) {
+              const int64_t b = min_[8 + s2];
+              if (b < 0) continue;
+              const int64_t wrid = p.wrmap[(((int64_t)wp * 2 + s2) * 2 + s2p) * d.n_r + b];
+              if (wrid < 0) continue;
+              int64_t* q = sg[n++];
+              q[0] = z_off + (s2 ? min_[10] : 0);
+              q[1] = min_[3];
+              q[2] = p.wr[WRF * wrid + 7];
+              q[3] = Ncols;
+              q[4] = Rs[3 * b + 2];
+              flops += 8 * Mrows * Ncols * q[4];
+            }
+          }
         }
+        int at = n;   // inclusive prefix over the lanes
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, at, o);
+          if (lane >= o) at += y;
+        }
+        int64_t* seg = p.seg2 + SF * (i * d.seg2_stride + cnt + at - n);
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+          if (s < n) {
+#pragma unroll
+            for (int f = 0; f < 5; ++f) seg[SF * s + f] = sg[s][f];
+            seg[SF * s + 5] = 0;
+          }
+        cnt += __shfl_sync(0xffffffffu, at, 31);
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) flops += __shfl_xor_sync(0xffffffffu, flops, o);
     }
-    if (cnt == 0) { Mrows = 0; Ncols = 0; task[2] = 0; task[3] = 0; }
-    task[0] = Mrows; task[1] = Ncols; task[4] = i * d.seg2_stride; task[5] = cnt;
-    p.tile2[i] = ceil_div(Mrows, kTile) * ceil_div(Ncols, kTile);
-    p.scr_b[i] = flops;
+    if (cnt == 0) { Mrows = 0; Ncols = 0; c_off = 0; ldc = 0; }
+    if (lane == 0) {
+      task[0] = Mrows; task[1] = Ncols; task[2] = c_off; task[3] = ldc; task[4] = i * d.seg2_stride; task[5] = cnt;
+      p.tile2[i] = ceil_div(Mrows, kTile) * ceil_div(Ncols, kTile);
+      p.scr_b[i] = flops;
+    }
   }
   __syncthreads();
   const int64_t tiles2 = block_scan(p.tile2, n_t2, smem);
