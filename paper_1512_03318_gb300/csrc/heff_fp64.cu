@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256) k_cgemm_fp64(const double2* __restrict__ 
 // perm/idx/val: sorted MPO entries; chan_field: index of the env channel in an entry
 // (0 = w for W_i, 1 = w'' for W_{i+1}); sec_field: row field holding the env sector.
 //
-// The blocks lie one after another in `out`, and a CTA takes kFoldChunk consecutive elements of it,
+// The blocks lie one after another in `out`, and a CTA takes a chunk of consecutive elements of it,
 // whichever blocks they belong to, so that the few large blocks spread over the GPU like the many
 // small ones; the search for the first block and a block's entry tables (a chain of dependent
 // loads) are paid once per CTA and block. Most entries are real, and most blocks one entry of
@@ -136,7 +136,12 @@ __global__ void __launch_bounds__(256) k_cgemm_fp64(const double2* __restrict__ 
 // (LW, WR: 0.82 GB written each): 0.49 + 0.40 ms; one CTA per block with every entry taken as
 // complex needed 1.4 + 0.9. (Testing every element for infinities inside its own branch instead
 // of four at once: 0.83 + 0.93.)
-constexpr int kFoldChunk = 8192, kFoldPer = 4, kFoldSub = kFoldPer * 256, kFoldTerms = 32;
+constexpr int kFoldPer = 4, kFoldSub = kFoldPer * 256, kFoldTerms = 32;
+// Elements per CTA: 8192 where that gives four CTAs per SM, else fewer (down to one per thread).
+inline int64_t fold_chunk(int64_t len) {
+  const int64_t c = (len / 608 + 255) / 256 * 256;
+  return c < 256 ? 256 : c > 8192 ? 8192 : c;
+}
 
 // An infinity or NaN takes the full product, zero times it included.
 __device__ __forceinline__ bool fold_odd(double2 x) {
@@ -156,16 +161,41 @@ __device__ __forceinline__ void fold_real(double2& acc, double2 x, double v, boo
   acc = first ? x : make_double2(__dadd_rn(acc.x, x.x), __dadd_rn(acc.y, x.y));
 }
 
+// Blocks of a few elements: one CTA each, so that its chain of dependent loads is paid once
+// per block, side by side with those of the other blocks. At Ly = 5, chi = 61 the flat form in chunks of
+// 8192 elements took ~100 us, in chunks of 256 10, this one 9 and 6 (LW, WR).
+constexpr int64_t kFoldSmall = 128;   // mean elements per block up to which this form runs
+
+__global__ void __launch_bounds__(256) k_fold_small(const double2* __restrict__ env, double2* __restrict__ out,
+                                                   const int64_t* __restrict__ rows, int nrows,
+                                                   const int64_t* __restrict__ env_map, int n_sec,
+                                                   const int32_t* __restrict__ perm, const int32_t* __restrict__ idx,
+                                                   const double* __restrict__ val, int chan_field) {
+  for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
+    const int64_t* row = rows + (int64_t)LWF * r;
+    const int64_t sec = row[3], n = row[5] * row[6], off = row[7], cb = row[8], ce = row[9];
+    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
+      double2 acc = make_double2(0.0, 0.0);
+      for (int64_t c = cb; c < ce; ++c) {
+        const int ent = perm[c];
+        const double2 x = env[env_map[(int64_t)idx[4 * ent + chan_field] * n_sec + sec] + e];
+        fold_full(acc, x, make_double2(val[2 * ent], val[2 * ent + 1]));
+      }
+      out[off + e] = acc;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ env, double2* __restrict__ out,
                                                   const int64_t* __restrict__ rows, int nrows, int64_t len,
                                                   const int64_t* __restrict__ env_map, int n_sec,
                                                   const int32_t* __restrict__ perm, const int32_t* __restrict__ idx,
-                                                  const double* __restrict__ val, int chan_field) {
+                                                  const double* __restrict__ val, int chan_field, int chunk) {
   __shared__ int64_t s_off[257];
   __shared__ const double2* s_src[kFoldTerms];
   __shared__ double2 s_val[kFoldTerms];
   const int tid = threadIdx.x;
-  const int64_t base = (int64_t)blockIdx.x * kFoldChunk;
+  const int64_t base = (int64_t)blockIdx.x * chunk, stop = base + chunk < len ? base + chunk : len;
   // the last block that starts at or before the chunk, by 256-way search
   int lo = 0, hi = nrows;
   while (hi - lo > 1) {
@@ -179,13 +209,13 @@ __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ en
   int cur = -1;          // block whose terms are staged
   int terms = 0;
   int64_t cur_off = 0, cur_n = 0;
-  for (int64_t e0 = base; e0 < base + kFoldChunk && e0 < len; e0 += kFoldSub) {
+  for (int64_t e0 = base; e0 < stop; e0 += kFoldSub) {
     int r = 0, top = 257;                // the last staged block that starts at or before e0
     while (top - r > 1) {
       const int m = (r + top) >> 1;
       if (s_off[m] <= e0) r = m; else top = m;
     }
-    const int64_t end = e0 + kFoldSub < len ? e0 + kFoldSub : len;
+    const int64_t end = e0 + kFoldSub < stop ? e0 + kFoldSub : stop;
     if (r < 256 && s_off[r + 1] >= end) {   // one block
       if (r != cur) {
         const int64_t* row = rows + (int64_t)LWF * (lo + r);
@@ -203,7 +233,7 @@ __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ en
         __syncthreads();
       }
       if (terms <= kFoldTerms) {
-        const int64_t f = e0 - cur_off + tid;
+        const int64_t f = e0 - cur_off + tid, n = end - cur_off < cur_n ? end - cur_off : cur_n;
         double2 acc[kFoldPer];
 #pragma unroll
         for (int q = 0; q < kFoldPer; ++q) acc[q] = make_double2(0.0, 0.0);
@@ -212,7 +242,7 @@ __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ en
           const double2 v = s_val[c];
           double2 x[kFoldPer];
 #pragma unroll
-          for (int q = 0; q < kFoldPer; ++q) x[q] = f + q * 256 < cur_n ? src[f + q * 256] : make_double2(0.0, 0.0);
+          for (int q = 0; q < kFoldPer; ++q) x[q] = f + q * 256 < n ? src[f + q * 256] : make_double2(0.0, 0.0);
           bool full = v.y != 0.0;
 #pragma unroll
           for (int q = 0; q < kFoldPer; ++q) full |= fold_odd(x[q]);
@@ -226,7 +256,7 @@ __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ en
         }
 #pragma unroll
         for (int q = 0; q < kFoldPer; ++q)
-          if (f + q * 256 < cur_n) out[cur_off + f + q * 256] = acc[q];
+          if (f + q * 256 < n) out[cur_off + f + q * 256] = acc[q];
         continue;
       }
     }
@@ -270,8 +300,15 @@ cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* row
                             const int64_t* env_map, int n_sec, const int32_t* perm, const int32_t* idx,
                             const double* val, int chan_field, int64_t len, cudaStream_t s) {
   if (nrows <= 0 || len <= 0) return cudaSuccess;
-  k_fold_env<<<(unsigned)((len + kFoldChunk - 1) / kFoldChunk), 256, 0, s>>>(env, out, rows, (int)nrows, len, env_map, n_sec,
-                                                                             perm, idx, val, chan_field);
+  if (len <= kFoldSmall * nrows) {
+    k_fold_small<<<(unsigned)(nrows < 65535 ? nrows : 65535), 256, 0, s>>>(env, out, rows, (int)nrows, env_map, n_sec, perm, idx, val,
+                                                                       chan_field);
+    mrd::count_launch();
+    return cudaGetLastError();
+  }
+  const int64_t chunk = fold_chunk(len);
+  k_fold_env<<<(unsigned)((len + chunk - 1) / chunk), 256, 0, s>>>(env, out, rows, (int)nrows, len, env_map, n_sec, perm, idx, val,
+                                                                   chan_field, (int)chunk);
   mrd::count_launch();
   return cudaGetLastError();
 }
