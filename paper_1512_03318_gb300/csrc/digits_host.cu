@@ -372,6 +372,28 @@ double cores_cost(const mrd_heff* h, bool ff, bool real) {
          dg_cost_cores(h->t2_host.data(), h->s2_host.data(), h->counts[C_NT2], ff, real, h->n_sm);
 }
 
+// K of the segments, padded to the 16 of one MMA, over K.
+double k_padding(const mrd_heff* h) {
+  double padded = 0.0, k = 0.0;
+  auto add = [&](const std::vector<int64_t>& t, const std::vector<int64_t>& sg, int64_t n) {
+    for (int64_t i = 0; i < n; ++i)
+      for (int64_t q = 0; q < t[(size_t)(TF * i + 5)]; ++q) {
+        const int64_t K = sg[(size_t)(SF * (t[(size_t)(TF * i + 4)] + q) + 4)];
+        k += (double)K;
+        padded += (double)((K + 15) / 16 * 16);
+      }
+  };
+  add(h->t1_host, h->s1_host, h->counts[C_NT1]);
+  add(h->t2_host, h->s2_host, h->counts[C_NT2]);
+  return k > 0.0 ? padded / k : 1.0;
+}
+
+// Float-float products whose segments are mostly padding stay on the CUDA cores, which take their K as
+// it is (FP64 ones do not: that pipe is 12 times slower). Setting environments and one application,
+// us with digits / without: padding 4.3 (Ly = 10, chi = 100) 280 / 209, 3.4 (Ly = 5, chi = 61) 141 / 107,
+// 1.9 (Ly = 6, chi = 173) 231 / 240, 1.6 (Ly = 10, chi = 400) 550 / 635.
+constexpr double kMaxPadding = 2.2;
+
 // Plans of both products for a precision, and whether they are the cheaper way (the same
 // decision for grouped and per-task launches, which give the same bits).
 void plan_both(const mrd_heff* h, DgHeff* g, int32_t prec, bool real, bool major) {
@@ -385,6 +407,7 @@ void plan_both(const mrd_heff* h, DgHeff* g, int32_t prec, bool real, bool major
   g->planned = true;
   const double cores = cores_cost(h, ff, real);
   if (cores * h->dg_uses < kSetupCycles) return;   // not worth planning
+  if (ff && k_padding(h) > kMaxPadding) return;
   std::vector<int32_t> ids((size_t)n2);   // step 2: the two row parts s1' of an output sector
   for (int64_t i = 0; i < n2; ++i) ids[(size_t)i] = (int32_t)(i >> 2 << 1 | (i & 1));   // share (nearly) all WR blocks
   auto both = [&](bool gm) {
