@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
       const int* ea = q.tall_op ? g.eb : g.ea;
       const int* eb = q.tall_op ? g.ea : g.eb;
       const bool by_row = q.cm_rows;
-      int er = 0, ec = 0;
+      int er = 0, ec = -1;   // (-1: a padding column)
       longlong2 map = {0, 0};
       if (row < R) er = ea[q.ea + row];
       if (lane < w && col0 + lane < N) ec = eb[q.eb + col0 + lane];
@@ -636,8 +636,10 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
         const int eg = __shfl_sync(0xffffffffu, ec, c);
         const long long at = by_row ? map.x + (long long)(col0 + c) * map.y
                                     : __shfl_sync(0xffffffffu, map.x, c) + (long long)row * __shfl_sync(0xffffffffu, map.y, c);
-        const double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], exr + eg, odd),
-                                       REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg, odd));
+        // (the panels' padding is never written: whatever its columns' sums are, they are within range)
+        const int ex = eg < 0 ? 0 : exr + eg;
+        const double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], ex, odd),
+                                       REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], ex, odd));
         odd = odd || eg == 2047;
         if (row < R && c < w && col0 + c < N) g.c[at] = o;
       }
