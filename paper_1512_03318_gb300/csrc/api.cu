@@ -23,7 +23,7 @@ std::vector<int2> ff_item_order(const int64_t* tasks, const int64_t* segs, int64
 cudaError_t to_ff(const double2* x, float4* y, int64_t n, cudaStream_t s);
 cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
                               const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s, const int* run_if = nullptr);
+                              int n_sm, cudaStream_t s);
 cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* rows, int64_t nrows,
                             const int64_t* env_map, int n_sec, const int32_t* perm, const int32_t* idx,
                             const double* val, int chan_field, int64_t len, cudaStream_t s);
@@ -569,7 +569,7 @@ int mrd_heff_apply(mrd_heff* h, const double* theta_in_dev, double* theta_out_de
   cudaError_t e = cudaMemsetAsync(theta_out_dev, 0, (size_t)n * 16, s);
   if (h->dg_use) {
     if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "mrd_heff_apply");
-    return dg_apply(h, (const double2*)theta_in_dev, (double2*)theta_out_dev, prec, ev, cap);
+    return dg_apply(h, (const double2*)theta_in_dev, (double2*)theta_out_dev, ev, cap);
   }
   if (prec == MRD_PREC_FF) {
     float4* z_ff = (float4*)h->z;

@@ -73,8 +73,7 @@ __device__ __forceinline__ void digit_pairs(long long Ta, long long Tb, uint32_t
 // rows, 8 lanes per row along K; row-contiguous pieces: 32 values of K, lanes along the rows.
 // Memory bound: 16 bytes read per element.
 __global__ void __launch_bounds__(256) k_dg_expo(const double2* __restrict__ src, const DgJob* __restrict__ jobs,
-                                                 const int2* __restrict__ pieces, int n_pieces, int* __restrict__ expo,
-                                                 int* __restrict__ bad_flag) {
+                                                 const int2* __restrict__ pieces, int n_pieces, int* __restrict__ expo) {
   for (int pc = blockIdx.x; pc < n_pieces; pc += gridDim.x) {
     const int2 pi = pieces[pc];
     const DgJob& j = jobs[pi.x];
@@ -83,7 +82,6 @@ __global__ void __launch_bounds__(256) k_dg_expo(const double2* __restrict__ src
     const int64_t ld = j.ld;
     const double2* x = src + j.off;
     int* out = expo + j.exp0;
-    bool bad = false;
     if (j.flags & DGJ_KCONTIG) {
       const int sub = threadIdx.x >> 3, lane = threadIdx.x & 7;
       for (int r = pi.y + sub; r < rows && r < pi.y + kDgMaxRows; r += 32) {
@@ -97,7 +95,6 @@ __global__ void __launch_bounds__(256) k_dg_expo(const double2* __restrict__ src
         e = max(e, __shfl_xor_sync(m, e, 4));
         e = max(e, __shfl_xor_sync(m, e, 2));
         e = max(e, __shfl_xor_sync(m, e, 1));
-        bad = bad || e == 2047;
         if (lane == 0 && e > 0) atomicMax(out + r, e);
       }
     } else {
@@ -112,11 +109,9 @@ __global__ void __launch_bounds__(256) k_dg_expo(const double2* __restrict__ src
             const double2 v = x[k * ld + r];
             e = max(e, max(expo_field(v.x), expo_field(v.y)));
           }
-          bad = bad || e == 2047;
           if (e > 0) atomicMax(out + r, e);
         }
     }
-    if (bad) *bad_flag = 1;
   }
 }
 
@@ -296,17 +291,17 @@ __device__ __forceinline__ void tmem_ld4(uint32_t* v, uint32_t taddr) {
 // would take 4 operations per number at 2 lanes per SM); lo in [0, 2^(4 BETA)). Without branches,
 // so that the 32 conversions of a thread overlap: with the rare cases inside, a tile's conversions
 // and stores took 12,000 cycles. `odd` is set when the result is outside the normal range (the value
-// returned is then meaningless).
+// returned is then meaningless; the task is computed again in FP64).
 template <int BETA>
-__device__ __forceinline__ void leading_bits(long long hi, uint32_t lo, int ex, uint32_t& sg, unsigned long long& r, int& e2) {
-  sg = (uint32_t)(hi >> 63);                  // 0 or all ones
+__device__ __forceinline__ double to_double(long long hi, uint32_t lo, int ex, bool& odd) {
+  const uint32_t sg = (uint32_t)(hi >> 63);   // 0 or all ones
   uint32_t c = lo << (32 - 4 * BETA);         // value = (a b c) 2^(ex + 4 BETA - 32) as 96 bits
   uint32_t b = (uint32_t)hi, a = (uint32_t)((unsigned long long)hi >> 32);
   const unsigned long long low = (((unsigned long long)b << 32 | c) ^ ((unsigned long long)sg << 32 | sg)) + (sg & 1);
   a = (a ^ sg) + (low == 0 ? (sg & 1) : 0u);
   b = (uint32_t)(low >> 32);
   c = (uint32_t)low;
-  e2 = ex + 4 * BETA - 32 + 95;               // exponent of bit 95
+  int e2 = ex + 4 * BETA - 32 + 95;           // exponent of bit 95
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const bool z = a == 0;
@@ -318,31 +313,11 @@ __device__ __forceinline__ void leading_bits(long long hi, uint32_t lo, int ex, 
   const int lz = __clz((int)a);
   const uint32_t m1 = __funnelshift_l(b, a, lz), m0 = __funnelshift_l(c, b, lz);
   e2 -= lz;
-  const unsigned long long m = (unsigned long long)m1 << 32 | m0;
-  r = (m >> 11) + ((m >> 10) & 1);
-}
-
-template <int BETA>
-__device__ __forceinline__ double to_double(long long hi, uint32_t lo, int ex, bool& odd) {
-  uint32_t sg;
-  unsigned long long r;
-  int e2;
-  leading_bits<BETA>(hi, lo, ex, sg, r, e2);
+  const unsigned long long m = (unsigned long long)m1 << 32 | m0, r = (m >> 11) + ((m >> 10) & 1);
   const bool zero = (hi | (long long)lo) == 0;
   odd = odd || (!zero && (unsigned)(e2 + 1022) >= 2045u);
   const unsigned long long bits = ((unsigned long long)(uint32_t)(e2 + 1022) << 52) + r + ((unsigned long long)(sg & 1) << 63);
   return __longlong_as_double(zero ? 0ll : (long long)bits);
-}
-
-template <int BETA>
-__device__ __noinline__ double to_double_slow(long long hi, uint32_t lo, int ex) {
-  if (hi == 0 && lo == 0) return 0.0;
-  uint32_t sg;
-  unsigned long long r;
-  int e2;
-  leading_bits<BETA>(hi, lo, ex, sg, r, e2);
-  const double v = ldexp((double)(long long)r, e2 - 52);
-  return sg ? -v : v;
 }
 
 }  // namespace
@@ -358,7 +333,7 @@ struct DgArgs {
   const int *ea, *eb;        // exponents of operand buffers 0 and 1
   const int2* splits;
   uint8_t* partial;
-  int* tickets;
+  int *tickets, *res;
   double2* c;
   int* words;
   uint64_t wait_ns;
@@ -547,7 +522,7 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
       const int* ea = q.tall_op ? g.eb : g.ea;
       const int* eb = q.tall_op ? g.ea : g.eb;
       const bool by_row = q.cm_rows;
-      int er = 0, ec = -1;   // (-1: a padding column)
+      int er = 0, ec = 0;
       longlong2 map = {0, 0};
       if (row < R) er = ea[q.ea + row];
       if (lane < w && col0 + lane < N) ec = eb[q.eb + col0 + lane];
@@ -630,41 +605,171 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
         }
       }
       const int exr = er - 2 * 1022 + (BETA == 8 ? -68 : -61);
-      bool odd = false;   // a result outside the normal range, or a row or column that is not finite
+      int top[16];   // exponent field of the larger part of each result; 2047 outside the normal range
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
         const int eg = __shfl_sync(0xffffffffu, ec, c);
         const long long at = by_row ? map.x + (long long)(col0 + c) * map.y
                                     : __shfl_sync(0xffffffffu, map.x, c) + (long long)row * __shfl_sync(0xffffffffu, map.y, c);
-        // (the panels' padding is never written: whatever its columns' sums are, they are within range)
-        const int ex = eg < 0 ? 0 : exr + eg;
-        const double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], ex, odd),
-                                       REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], ex, odd));
-        odd = odd || eg == 2047;
-        if (row < R && c < w && col0 + c < N) g.c[at] = o;
+        bool odd = false;
+        const double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], exr + eg, odd),
+                                       REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg, odd));
+        const bool valid = row < R && c < w && col0 + c < N;
+        top[c] = !valid ? 0 : odd ? 2047 : max(expo_field(o.x), expo_field(o.y));
+        if (valid) g.c[at] = o;
       }
-      if (__any_sync(0xffffffffu, (odd || er == 2047) && row < R)) {   // rare: convert again, with care
+      // the largest of this lane's row, or (lanes 0 .. 15) column, of the C map
+      int most = 0;
+      if (by_row) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c) most = max(most, top[c]);
+      } else {
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-          const int eg = __shfl_sync(0xffffffffu, ec, c);
-          const long long at = by_row ? map.x + (long long)(col0 + c) * map.y
-                                      : __shfl_sync(0xffffffffu, map.x, c) + (long long)row * __shfl_sync(0xffffffffu, map.y, c);
-          if (row < R && c < w && col0 + c < N) {
-            double2 o = make_double2(to_double_slow<BETA>(hi[0][c], lo[0][c], exr + eg),
-                                     REAL ? 0.0 : to_double_slow<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg));
-            if (er == 2047 || eg == 2047) o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);
-            g.c[at] = o;
-          }
+          const int v = __reduce_max_sync(0xffffffffu, top[c]);
+          if (lane == c) most = v;
         }
       }
+      if (most > 0) atomicMax(g.res + q.cm + (by_row ? row : col0 + lane), most);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (k_dg_check waits for this grid's results)
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
   }
+}
+
+// ---------------------------------------------------------------- products that are computed again
+
+// One warp per task: its tiles join the list when a row or column of its operands is not finite (exponent
+// field 2047) or a result is outside the normal range (marked likewise). Not after a wait gave up, when nothing is valid.
+__global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members, int n,
+                                                  const int* __restrict__ e0, const int* __restrict__ e1,
+                                                  const int* __restrict__ res, int* __restrict__ count, int2* __restrict__ list,
+                                                  const int* __restrict__ err) {
+  const int lane = threadIdx.x & 31;
+  int i = (blockIdx.x * 256 + threadIdx.x) >> 5;
+  DgMember m = members[min(i, n - 1)];
+  DgGroup g = groups[m.group];
+  // launched as a programmatic dependent of the product: above are tables, below its results
+  asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
+  if (*err) return;
+  for (; i < n; i += gridDim.x * 8, m = members[min(i, n - 1)], g = groups[m.group]) {
+    const int *tall = g.tall_op ? e1 : e0, *flat = g.tall_op ? e0 : e1;
+    const int* stacked = (g.cm_rows ? tall + g.ea : flat + g.eb) + (m.first - g.cm);
+    const int* shared = g.cm_rows ? flat + g.eb : tall + g.ea;
+    const int ns = g.cm_rows ? g.N : g.R;
+    int a = 0, b = 0, o = 0;
+    for (int r = lane; r < m.rows; r += 32) {
+      a = max(a, stacked[r]);
+      o = max(o, res[m.first + r]);
+    }
+    for (int c = lane; c < ns; c += 32) b = max(b, shared[c]);
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
+    o = __reduce_max_sync(0xffffffffu, o);
+    if (a < 2047 && b < 2047 && o < 2047) continue;
+    const int tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32);
+    int at = 0;
+    if (lane == 0) at = atomicAdd(count, tiles);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    for (int t = lane; t < tiles; t += 32) list[at + t] = make_int2(i, t);
+  }
+}
+
+// The listed tiles (32 stacked rows x 32 of the shared side) in FP64 FMAs, K in chunks of 16, blocks
+// in the order of the job lists; REAL: imaginary parts taken and returned as zeros. Usually the list is
+// empty and the launch returns at once.
+template <bool REAL>
+__global__ void __launch_bounds__(256) k_dg_redo(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members,
+                                                 const DgJob* __restrict__ sjobs, const DgJob* __restrict__ ujobs,
+                                                 const double2* __restrict__ ssrc, const double2* __restrict__ usrc,
+                                                 double2* __restrict__ C, const int* __restrict__ count,
+                                                 const int2* __restrict__ list) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // (dependent of k_dg_check)
+  const int total = *count;
+  if ((int)blockIdx.x >= total) return;
+  __shared__ double2 As[32][17], Bs[16][33];
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  for (int item = blockIdx.x; item < total; item += gridDim.x) {
+    const int2 it = list[item];
+    const DgMember m = members[it.x];
+    const DgGroup& g = groups[m.group];
+    const int ns = g.cm_rows ? g.N : g.R, tn = (ns + 31) / 32;
+    const int r0 = it.y / tn * 32, c0 = it.y % tn * 32;
+    double2 acc[2][2] = {};
+    for (int f = 0; f < g.n_jobs; ++f) {
+      const DgJob &sj = sjobs[m.job + f], &uj = ujobs[g.job + f];
+      if (sj.off < 0) continue;                            // a block this task does not multiply
+      const int K = uj.K;
+      const bool sk = sj.flags & DGJ_KCONTIG, uk = uj.flags & DGJ_KCONTIG;
+      const double ss = sj.flags & DGJ_CONJ ? -1.0 : 1.0, us = uj.flags & DGJ_CONJ ? -1.0 : 1.0;
+      for (int k0 = 0; k0 < K; k0 += 16) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int e = tid + q * 256;
+          const int sr = sk ? e >> 4 : e & 31, sc = sk ? e & 15 : e >> 5;
+          double2 v = make_double2(0.0, 0.0);
+          if (r0 + sr < m.rows && k0 + sc < K)
+            v = ssrc[sj.off + (sk ? (r0 + sr) * sj.ld + k0 + sc : (k0 + sc) * sj.ld + r0 + sr)];
+          As[sr][sc] = make_double2(v.x, REAL ? 0.0 : v.y * ss);
+          const int ur = uk ? e >> 4 : e & 31, uc = uk ? e & 15 : e >> 5;
+          v = make_double2(0.0, 0.0);
+          if (c0 + ur < ns && k0 + uc < K)
+            v = usrc[uj.off + (uk ? (c0 + ur) * uj.ld + k0 + uc : (k0 + uc) * uj.ld + c0 + ur)];
+          Bs[uc][ur] = make_double2(v.x, REAL ? 0.0 : v.y * us);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const double2 a = As[2 * ty + i][k], b = Bs[k][2 * tx + j];
+              acc[i][j].x = fma(-a.y, b.y, fma(a.x, b.x, acc[i][j].x));
+              acc[i][j].y = fma(a.y, b.x, fma(a.x, b.y, acc[i][j].y));
+            }
+        __syncthreads();
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int r = r0 + 2 * ty + i, c = c0 + 2 * tx + j;
+        if (r < m.rows && c < ns) C[m.off + r * m.step + c * m.other] = make_double2(acc[i][j].x, REAL ? 0.0 : acc[i][j].y);
+      }
+  }
+}
+
+cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, const int* words, int n_sm, cudaStream_t s) {
+  if (d.n_members <= 0) return cudaSuccess;
+  const int grid = (d.n_members + 7) / 8, u = 1 - d.sop;
+  // both as programmatic dependents of the launch before them, so that they cost little when there is
+  // nothing to do: 4 us per product less than in plain stream order
+  cudaLaunchAttribute pdl;
+  pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid < 2048 ? grid : 2048);
+  lc.blockDim = dim3(256);
+  lc.stream = s;
+  lc.attrs = &pdl;
+  lc.numAttrs = 1;
+  const int* err = words + DG_ERR;
+  cudaError_t e = cudaLaunchKernelEx(&lc, k_dg_check, (const DgGroup*)d.groups, (const DgMember*)d.members, d.n_members,
+                                     (const int*)d.expo[0], (const int*)d.expo[1], (const int*)d.res, d.redo_count, d.redo, err);
+  if (e != cudaSuccess) return e;
+  lc.gridDim = dim3(2 * n_sm);
+  e = cudaLaunchKernelEx(&lc, d.real ? k_dg_redo<true> : k_dg_redo<false>, (const DgGroup*)d.groups, (const DgMember*)d.members,
+                         (const DgJob*)d.jobs[d.sop], (const DgJob*)d.jobs[u], d.sop ? b : a, d.sop ? a : b, C,
+                         (const int*)d.redo_count, (const int2*)d.redo);
+  count_launches(2);
+  return e;
 }
 
 cudaError_t dg_init() {
@@ -686,10 +791,10 @@ cudaError_t dg_expand(const DgDev& d, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t dg_pack(const DgDev& d, int op, const double2* src, int beta, int* words, int bad, cudaStream_t s) {
+cudaError_t dg_pack(const DgDev& d, int op, const double2* src, int beta, int* words, cudaStream_t s) {
   if (d.n_mpieces[op] > 0) {
     k_dg_expo<<<d.n_mpieces[op] < 16384 ? d.n_mpieces[op] : 16384, 256, 0, s>>>(src, d.jobs[op], d.mpieces[op],
-                                                                               d.n_mpieces[op], d.expo[op], words + bad);
+                                                                               d.n_mpieces[op], d.expo[op]);
     count_launch();
   }
   if (d.n_pieces[op] > 0) {
@@ -709,7 +814,7 @@ cudaError_t dg_gemm(const DgDev& d, double2* C, int beta, int* words, int n_sm, 
   cudaError_t e = dg_init();
   if (e != cudaSuccess) return e;
   DgArgs g{d.panel[0], d.panel[1], d.groups, d.items, first, count, d.cmap, d.expo[0], d.expo[1],
-           d.splits, d.partial, d.tickets, C, words, wait_ns};
+           d.splits, d.partial, d.tickets, d.res, C, words, wait_ns};
   auto k = beta == 8 ? (d.real ? k_dg_gemm<8, true> : k_dg_gemm<8, false>)
                      : (d.real ? k_dg_gemm<7, true> : k_dg_gemm<7, false>);
   k<<<count < n_sm ? count : n_sm, 320, kDgSmem, s>>>(g);

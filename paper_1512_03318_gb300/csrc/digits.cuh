@@ -61,12 +61,15 @@ struct DgGroup {
   int32_t R, N, nks, ea, eb;   // ea, eb: first row's / column's exponent
   int32_t tall_op;
   int32_t cm, cm_rows;         // C map: first entry; indexed by rows (1) or by columns (0)
+  int32_t job, n_jobs;         // the shared operand's blocks in its job list
 };
 // C map entries of one task: entry r is (off + r step, other), the C offset of its r-th stacked
-// row (column) and the stride along the shared side.
+// row (column) and the stride along the shared side. job: its first block in the stacked operand's
+// job list (one per block of the group, in the same order).
 struct DgMember {
   int64_t off, step, other;
   int32_t first, rows;
+  int32_t group, job;
 };
 // K steps ks0 .. ks1 - 1 of a tile; split >= 0: one part of a tile cut along K (split * 64 + part).
 struct DgItem {
@@ -87,6 +90,8 @@ struct DgPlan {
   int64_t bytes[2] = {0, 0};         // panels
   int64_t rows[2] = {0, 0};          // exponents
   int64_t slots = 0;                 // partial sums of split tiles
+  int64_t redo = 0;                  // 32 x 32 tiles of all tasks
+  int sop = 0;                       // the stacked operand
   double cost = 0.0;                 // estimated cycles of the product
   bool real = false;
 };
@@ -122,6 +127,10 @@ struct DgDev {
   int64_t rows[2] = {0, 0};
   uint8_t* partial = nullptr;        // dg_partial_bytes
   int* tickets = nullptr;            // 8 per split tile, zeroed before each product
+  int* res = nullptr;                // largest exponent field of each stacked row's results; zeroed likewise
+  int* redo_count = nullptr;         // tiles to be computed again, zeroed likewise
+  int2* redo = nullptr;              // (task, tile)
+  int sop = 0;
   bool real = false;
 };
 // Partial sums of a split tile: 128 x 32 complex numbers of 12-byte sums, per part.
@@ -134,21 +143,29 @@ size_t dg_device_table_bytes(const DgPlan& p);
 // upload dg_expand forms the C map.
 void dg_tables(const DgPlan& p, uint8_t* host, uint8_t* dev, DgDev& d);
 cudaError_t dg_expand(const DgDev& d, cudaStream_t s);
-// Scratch words of a product (device ints): item counter, error flag, and whether an infinity or
-// NaN was met in operands that are packed once (environments) or per product.
-enum { DG_CTR = 0, DG_ERR = 1, DG_BAD_ENV = 2, DG_BAD = 3, DG_WORDS = 4 };
+// Zeroed words of a product besides its exponents: tickets, result exponents, count of tiles to redo.
+inline int64_t dg_state_words(const DgPlan& p) { return 8 * (int64_t)p.splits.size() + p.cmap + 1; }
+inline void dg_state(const DgPlan& p, int* words, DgDev& d) {
+  d.tickets = words;
+  d.res = words + 8 * p.splits.size();
+  d.redo_count = d.res + p.cmap;
+}
+// Scratch words shared by the products of a handle (device ints): item counter, error flag.
+enum { DG_CTR = 0, DG_ERR = 1, DG_WORDS = 4 };
 // Units of a pack / exponent piece (see the kernels).
 constexpr int kDgPairPiece = 2048;   // kcontig pack: (row, pair of K) units
 constexpr int kDgChunkPiece = 512;   // row-contiguous pack: (chunk of 8 K, row) units
 constexpr int kDgMaxRows = 64;       // kcontig exponents: rows
 constexpr int kDgMaxK = 32;          // row-contiguous exponents: K
 // Exponents and digits of operand buffer `op` (0: tasks' A, 1: tasks' B) from `src`; the caller has
-// zeroed expo[op], words[bad] (DG_BAD_ENV or DG_BAD) and the tickets. Resets the item counter
-// for the next dg_gemm.
-cudaError_t dg_pack(const DgDev& d, int op, const double2* src, int beta, int* words, int bad, cudaStream_t s);
+// zeroed expo[op] and the product's state. Resets the item counter for the next dg_gemm.
+cudaError_t dg_pack(const DgDev& d, int op, const double2* src, int beta, int* words, cudaStream_t s);
 // The product; first / count: a sub-range of the items (per-group launches), count < 0: all.
 cudaError_t dg_gemm(const DgDev& d, double2* C, int beta, int* words, int n_sm, uint64_t wait_ns, cudaStream_t s,
                     int first = 0, int count = -1);
+// After the product: the tasks whose operands or results have an infinity or NaN, which has no
+// fixed-point form, are computed again in FP64 from the operands themselves (buffers 0 and 1).
+cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, const int* words, int n_sm, cudaStream_t s);
 cudaError_t dg_init();
 
 }  // namespace mrd

@@ -34,6 +34,7 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
   p.real = real;
   // the stacked operand (members one under the other) and the shared one
   const int sop = how == DG_BY_A ? 1 : 0, uop = 1 - sop;
+  p.sop = sop;
   const int sf = sop ? 2 : 0, uf = uop ? 2 : 0;        // first segment field of their blocks (off, ld)
   const int64_t sbit = sop ? 2 : 1, ubit = uop ? 2 : 1;   // their flag bits (conjugate-transposed)
   struct Entry {   // a shared block of a group
@@ -164,6 +165,8 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
     d.tall_op = s_tall ? sop : uop;
     d.cm = (int32_t)p.cmap;
     d.cm_rows = s_tall ? 1 : 0;
+    d.job = (int32_t)p.jobs[uop].size();
+    d.n_jobs = (int32_t)g.e.size();
     const int32_t s_flag = s_tall ? DGJ_TALL : 0, u_flag = s_tall ? 0 : DGJ_TALL;
     auto kind = [](int op, bool ct) { return ((op ? ct : !ct) ? DGJ_KCONTIG : 0) | (ct ? DGJ_CONJ : 0); };
     for (const Entry& e : g.e)
@@ -171,6 +174,7 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
     for (const Member& m : g.m) {
       const int64_t* t = tasks + 6 * m.task;
       const int64_t* sg = segs + 6 * t[4];
+      const int32_t job0 = (int32_t)p.jobs[sop].size();
       int64_t k = 0;
       for (size_t f = 0; f < g.e.size(); ++f) {
         const Entry& e = g.e[f];
@@ -192,7 +196,8 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
         p.jobs[sop].push_back({hit >= 0 ? s[sf] : -1, s[sf + 1], os, m.rows, e.K, e.kpad, m.row0, e.k0, g.R, nks,
                                es + m.row0, kind(sop, ct) | s_flag, 0});
       }
-      p.members.push_back({t[2], sop ? 1 : t[3], sop ? t[3] : 1, (int32_t)p.cmap + m.row0, m.rows});
+      p.members.push_back({t[2], sop ? 1 : t[3], sop ? t[3] : 1, (int32_t)p.cmap + m.row0, m.rows, (int32_t)p.groups.size(), job0});
+      p.redo += up(m.rows, 32) / 32 * (up(g.N, 32) / 32);
     }
     p.cmap += g.R;
     p.bytes[sop] += up(g.R, s_tall ? 8 : 16) * nks * pb;
@@ -326,12 +331,9 @@ void dg_tables(const DgPlan& p, uint8_t* host, uint8_t* dev, DgDev& d) {
   d.n_items = (int)p.items.size();
   d.n_splits = (int)p.splits.size();
   d.tab_bytes = off;
+  d.sop = p.sop;
   d.real = p.real;
 }
-
-cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
-                              const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s, const int* run_if = nullptr);
 
 }  // namespace mrd
 
@@ -344,7 +346,7 @@ struct DgHeff {
   int beta = 0;
   DgPlan p1, p2;
   DgDev d1, d2;
-  int* words = nullptr;   // DG_WORDS, then the exponents of theta and Z and the tickets (zeroed
+  int* words = nullptr;   // DG_WORDS, then the exponents of theta and Z and the products' states (zeroed
   size_t zero_bytes = 0;  // together before each application)
   Arena mem;
   std::thread th;
@@ -472,11 +474,13 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
     uint8_t* tab = nullptr;
     int* env_expo = nullptr;
     uint8_t* partial = nullptr;
-    const int64_t ne = g->p1.rows[0] + g->p2.rows[1], nt1 = 8 * (int64_t)g->p1.splits.size();
-    const int64_t nz = g->p1.rows[1] + g->p2.rows[0] + nt1 + 8 * (int64_t)g->p2.splits.size();
+    const int64_t ne = g->p1.rows[0] + g->p2.rows[1], ns1 = dg_state_words(g->p1);
+    const int64_t nz = g->p1.rows[1] + g->p2.rows[0] + ns1 + dg_state_words(g->p2);
+    int2* redo = nullptr;
     cudaError_t e = A.alloc(&tab, d1 + dg_device_table_bytes(g->p2) + 16);
     if (e == cudaSuccess) e = A.alloc(&g->words, (size_t)(DG_WORDS + nz));
     if (e == cudaSuccess) e = A.alloc(&env_expo, (size_t)std::max<int64_t>(ne, 1));
+    if (e == cudaSuccess) e = A.alloc(&redo, (size_t)std::max(g->p1.redo, g->p2.redo));
     if (e == cudaSuccess) e = A.alloc(&partial, (size_t)(std::max<int64_t>({g->p1.slots, g->p2.slots, 1}) * kDgSlotBytes));
     if (e == cudaSuccess) e = A.alloc(&g->d1.panel[0], (size_t)g->p1.bytes[0]);
     if (e == cudaSuccess) e = A.alloc(&g->d1.panel[1], (size_t)g->p1.bytes[1]);
@@ -492,9 +496,10 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
     g->zero_bytes = (size_t)(DG_WORDS + nz) * 4;
     g->d1.expo[1] = g->words + DG_WORDS;
     g->d2.expo[0] = g->d1.expo[1] + g->p1.rows[1];
-    g->d1.tickets = g->d2.expo[0] + g->p2.rows[0];
-    g->d2.tickets = g->d1.tickets + nt1;
+    dg_state(g->p1, g->d2.expo[0] + g->p2.rows[0], g->d1);
+    dg_state(g->p2, g->d1.tickets + ns1, g->d2);
     g->d1.partial = g->d2.partial = partial;   // step 2 starts after step 1 has read its sums
+    g->d1.redo = g->d2.redo = redo;            // (and its list)
     g->d1.expo[0] = env_expo;
     g->d2.expo[1] = env_expo + g->p1.rows[0];
     std::vector<uint8_t> host(std::max(b1, b2) + 16);
@@ -511,10 +516,9 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
     ++h->gen;
   }
   if (g->env_dirty) {
-    MRD_CUDA(ctx, cudaMemsetAsync(g->words + DG_BAD_ENV, 0, 4, s));
     MRD_CUDA(ctx, cudaMemsetAsync(g->d1.expo[0], 0, (size_t)(g->p1.rows[0] + g->p2.rows[1]) * 4, s));
-    MRD_CUDA(ctx, dg_pack(g->d1, 0, h->lw, beta, g->words, DG_BAD_ENV, s));
-    MRD_CUDA(ctx, dg_pack(g->d2, 1, h->wr, beta, g->words, DG_BAD_ENV, s));
+    MRD_CUDA(ctx, dg_pack(g->d1, 0, h->lw, beta, g->words, s));
+    MRD_CUDA(ctx, dg_pack(g->d2, 1, h->wr, beta, g->words, s));
     g->env_dirty = false;
   }
   return MRD_OK;
@@ -526,15 +530,14 @@ void dg_env_changed(mrd_heff* h) {
 
 // theta_out = H_eff theta_in; ev: timing events (or null) before step 1, between the steps and
 // after step 2. `out` has been cleared.
-int dg_apply(mrd_heff* h, const double2* in, double2* out, int32_t prec, const cudaEvent_t ev[3], bool cap) {
+int dg_apply(mrd_heff* h, const double2* in, double2* out, const cudaEvent_t ev[3], bool cap) {
   mrd_ctx* ctx = h->ctx;
   cudaStream_t s = ctx->stream;
   DgHeff* g = h->dg;
   const int beta = g->beta;
-  const int* bad = prec == MRD_PREC_FP64 ? g->words + DG_BAD_ENV : nullptr;   // and DG_BAD after it
-  // the error flag and the environments' flag outlive a product; the exponents and tickets do not
-  MRD_CUDA(ctx, cudaMemsetAsync(g->words + DG_BAD, 0, g->zero_bytes - DG_BAD * 4, s));
-  MRD_CUDA(ctx, dg_pack(g->d1, 1, in, beta, g->words, DG_BAD, s));
+  // the error flag outlives a product; the exponents and the products' states do not
+  MRD_CUDA(ctx, cudaMemsetAsync(g->words + DG_WORDS, 0, g->zero_bytes - DG_WORDS * 4, s));
+  MRD_CUDA(ctx, dg_pack(g->d1, 1, in, beta, g->words, s));
   MRD_CUDA(ctx, record_event(ev[0], s, cap));
   auto product = [&](const DgPlan& p, const DgDev& d, double2* C) -> int {
     if (!h->per_task) {
@@ -550,16 +553,11 @@ int dg_apply(mrd_heff* h, const double2* in, double2* out, int32_t prec, const c
   };
   int rc = product(g->p1, g->d1, h->z);
   if (rc != MRD_OK) return rc;
-  // infinities and NaN have no fixed-point form: the FP64 kernel redoes the product then
-  if (bad)
-    MRD_CUDA(ctx, launch_cgemm_fp64(h->lw, in, h->z, h->p.t1, h->p.seg1, h->p.tile1, h->counts[C_NT1],
-                                    h->counts[C_TILES1], h->n_sm, s, bad));
+  MRD_CUDA(ctx, dg_redo(g->d1, h->lw, in, h->z, g->words, h->n_sm, s));
   MRD_CUDA(ctx, record_event(ev[1], s, cap));
-  MRD_CUDA(ctx, dg_pack(g->d2, 0, h->z, beta, g->words, DG_BAD, s));
+  MRD_CUDA(ctx, dg_pack(g->d2, 0, h->z, beta, g->words, s));
   if ((rc = product(g->p2, g->d2, out)) != MRD_OK) return rc;
-  if (bad)
-    MRD_CUDA(ctx, launch_cgemm_fp64(h->z, h->wr, out, h->p.t2, h->p.seg2, h->p.tile2, h->counts[C_NT2],
-                                    h->counts[C_TILES2], h->n_sm, s, bad));
+  MRD_CUDA(ctx, dg_redo(g->d2, h->z, h->wr, out, g->words, h->n_sm, s));
   MRD_CUDA(ctx, record_event(ev[2], s, cap));
   return MRD_OK;
 }

@@ -36,7 +36,7 @@ std::vector<int2> ff_item_order(const int64_t* tasks, const int64_t* segs, int64
 cudaError_t to_ff(const double2* x, float4* y, int64_t n, cudaStream_t s);
 cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
                               const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s, const int* run_if = nullptr);
+                              int n_sm, cudaStream_t s);
 cudaError_t svd_load(const double2* theta, const int64_t* blk, const int64_t* src_off, int nblk, double2* work,
                      double* fro2, cudaStream_t s);
 int64_t svd_bround_smem(int W, int64_t p, int64_t r_v, bool f32);
@@ -380,7 +380,7 @@ struct mrd_dmrg {
   Buf schmidt_tab, schmidt_out;
   Buf ff_a, ff_b;   // float-float copies of the operands of a grouped GEMM
   // digit-split grouped GEMMs: tables, panels, exponents and words of the last one
-  Buf dg_tab, dg_panel[2], dg_expo, dg_partial, dg_words;
+  Buf dg_tab, dg_panel[2], dg_expo, dg_partial, dg_redo, dg_words;
   bool dg_ran = false;   // since the last dg_check
   int last_iters = 0, last_refine = 0;
   bool timing = false;
@@ -408,11 +408,11 @@ int run_gemm_digits(mrd_dmrg* D, const GemmList& g, int64_t nt, const double2* A
   // the exponent and digit passes and their launches
   const double pass = (double)(p.bytes[0] + p.bytes[1]) * 2.0 / 5.0e12 * 1.9e9 + kSetup;
   if (p.items.empty() || p.cost + pass >= cores) return MRD_OK;
-  const int64_t nt8 = 8 * (int64_t)p.splits.size();
-  const size_t tb = dg_table_bytes(p), nx = (size_t)(p.rows[0] + p.rows[1] + nt8) * 4;
-  const size_t need[5] = {dg_device_table_bytes(p), (size_t)p.bytes[0], (size_t)p.bytes[1], nx, (size_t)(p.slots * kDgSlotBytes)};
-  Buf* bufs[5] = {&D->dg_tab, &D->dg_panel[0], &D->dg_panel[1], &D->dg_expo, &D->dg_partial};
-  for (int k = 0; k < 5; ++k) {
+  const size_t tb = dg_table_bytes(p), nx = (size_t)(p.rows[0] + p.rows[1] + dg_state_words(p)) * 4;
+  const size_t need[6] = {dg_device_table_bytes(p), (size_t)p.bytes[0], (size_t)p.bytes[1], nx, (size_t)(p.slots * kDgSlotBytes),
+                          (size_t)p.redo * sizeof(int2)};
+  Buf* bufs[6] = {&D->dg_tab, &D->dg_panel[0], &D->dg_panel[1], &D->dg_expo, &D->dg_partial, &D->dg_redo};
+  for (int k = 0; k < 6; ++k) {
     const cudaError_t e = bufs[k]->need(need[k]);
     if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
@@ -432,14 +432,16 @@ int run_gemm_digits(mrd_dmrg* D, const GemmList& g, int64_t nt, const double2* A
   d.partial = D->dg_partial.as<uint8_t>();
   d.expo[0] = D->dg_expo.as<int>();
   d.expo[1] = d.expo[0] + p.rows[0];
-  d.tickets = d.expo[1] + p.rows[1];
+  dg_state(p, d.expo[1] + p.rows[1], d);
+  d.redo = D->dg_redo.as<int2>();
   // the error flag (word DG_ERR) stays until dg_check reads it
   if (!D->dg_ran) MRD_CUDA(ctx, cudaMemsetAsync(words, 0, DG_WORDS * 4, s));
   MRD_CUDA(ctx, cudaMemsetAsync(d.expo[0], 0, nx, s));
   D->dg_ran = true;
-  MRD_CUDA(ctx, dg_pack(d, 0, Aop, beta, words, DG_BAD, s));
-  MRD_CUDA(ctx, dg_pack(d, 1, Bop, beta, words, DG_BAD, s));
+  MRD_CUDA(ctx, dg_pack(d, 0, Aop, beta, words, s));
+  MRD_CUDA(ctx, dg_pack(d, 1, Bop, beta, words, s));
   MRD_CUDA(ctx, dg_gemm(d, C, beta, words, D->n_sm, 1000000000ull, s));
+  MRD_CUDA(ctx, dg_redo(d, Aop, Bop, C, words, D->n_sm, s));
   *done = true;
   return MRD_OK;
 }

@@ -42,14 +42,10 @@ __device__ __forceinline__ void cmac(double2& c, const double2 a, const double2 
 
 }  // namespace
 
-// run_if (or null): two device flags; the kernel returns at once when both are zero (the second
-// attempt of a digit-split product that met an infinity or NaN).
 __global__ void __launch_bounds__(256) k_cgemm_fp64(const double2* __restrict__ A, const double2* __restrict__ B,
                                                     double2* __restrict__ C, const int64_t* __restrict__ tasks,
                                                     const int64_t* __restrict__ segs,
-                                                    const int64_t* __restrict__ prefix, int64_t n_tasks,
-                                                    const int* __restrict__ run_if) {
-  if (run_if != nullptr && run_if[0] == 0 && run_if[1] == 0) return;
+                                                    const int64_t* __restrict__ prefix, int64_t n_tasks) {
   __shared__ double2 As[kT][kK + 1];
   __shared__ double2 Bs[kK][kT + 1];
   const int tid = threadIdx.x;
@@ -287,11 +283,11 @@ __global__ void __launch_bounds__(256) k_fold_env(const double2* __restrict__ en
 
 cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
                               const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s, const int* run_if) {
+                              int n_sm, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
-  int64_t grid = (int64_t)n_sm * (run_if ? 2 : 8);
+  int64_t grid = (int64_t)n_sm * 8;
   if (grid > total_tiles) grid = total_tiles;
-  k_cgemm_fp64<<<(unsigned)grid, 256, 0, s>>>(A, B, C, tasks, segs, prefix, n_tasks, run_if);
+  k_cgemm_fp64<<<(unsigned)grid, 256, 0, s>>>(A, B, C, tasks, segs, prefix, n_tasks);
   mrd::count_launch();
   return cudaGetLastError();
 }

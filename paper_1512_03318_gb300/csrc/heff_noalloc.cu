@@ -19,7 +19,7 @@
 namespace mrd {
 cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, const int64_t* tasks,
                               const int64_t* segs, const int64_t* prefix, int64_t n_tasks, int64_t total_tiles,
-                              int n_sm, cudaStream_t s, const int* run_if = nullptr);
+                              int n_sm, cudaStream_t s);
 }  // namespace mrd
 
 namespace {

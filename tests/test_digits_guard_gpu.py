@@ -1,0 +1,112 @@
+"""What digit-split products cannot represent is computed again in FP64: infinities and NaN."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import synth  # noqa: E402
+from oracle import blocksparse as B  # noqa: E402
+from tests import gpu_cases as G  # noqa: E402
+from tests import test_env_gpu as E  # noqa: E402
+from tests.test_heff_gpu import _dev  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+TOL = {0: 1e-12, 3: 1e-11}
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_1512_03318_gb300 as P
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return P.Context(0, torch.cuda.current_stream())
+
+
+def _oracle(case):
+    return B.heff_apply(case["left"], case["right"], case["m1"], case["m2"], case["mod"], case["cl"], case["cm"],
+                        case["cr"], case["wi"], case["wj"], case["lflat"], case["rflat"], case["tflat"])
+
+
+def _spin_channels(seed, dl, dr, channels, own):
+    """Modulus 1, diagonal entries. With `own`, channel x is fed by spin s1 = x mod 2 only and
+    becomes channel x of the right environment, so the two row parts of an output block
+    multiply different right blocks."""
+    left = B.BondSectors([((5, 0), dl), ((6, 0), dl)])
+    right = B.BondSectors([((5, 0), dr), ((6, 0), dr), ((7, 0), dr)])
+    c = [(0, 0)] * channels
+    u = synth.uniform_pm1(synth.substream(seed, 3), 4 * channels * channels)
+    wi = [(w, x, s, s, complex(u[2 * (w * channels + x)], u[2 * (w * channels + x) + 1]))
+          for w in range(channels) for x in range(channels) for s in (0, 1) if not own or x % 2 == s]
+    wj = [(x, x, s, s, complex(1.0, -0.5)) for x in range(channels) for s in (0, 1)] if own else wi
+    return G.finish_case(seed, left, right, 0, 0, 1, c, c, c, wi, wj)
+
+
+@pytest.mark.parametrize("prec", [0, 3])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_non_finite_right_block_stays_with_its_part(ctx, prec, bad):
+    """An infinity or NaN in a right block that one spin part multiplies leaves the other part's outputs
+    finite and right, and that part's own non-finite where the plain product is."""
+    import paper_1512_03318_gb300 as P
+    case = dict(_spin_channels(79, 120, 96, 12, True))
+    good = _oracle(case)
+    r = case["rflat"].copy()
+    off, d0, d1 = next(row[3:] for row in case["rl"] if row[:2] == (3, 1))
+    r[off + (d0 // 2) * d1 + d1 // 3] = bad          # a block of channel 3: spin part 1 only
+    case["rflat"] = r
+    with np.errstate(all="ignore"):
+        ref = _oracle(case)
+    fine = np.isfinite(ref)
+    assert np.any(~fine) and np.any(fine)
+    h = P.Heff(ctx, **G.heff_args(case))
+    h.set_env(_dev(case["lflat"]), _dev(r))
+    T = _dev(case["tflat"])
+    out = torch.empty_like(T)
+    h.apply(T, out, prec)
+    h.status()
+    got = out.cpu().numpy()
+    assert np.all(np.isfinite(got[fine]))
+    assert np.all(~np.isfinite(got[~fine]))
+    assert np.max(np.abs(got[fine] - ref[fine])) <= TOL[prec] * np.max(np.abs(good))
+    h.close()
+
+
+def _raw_env(d, bond, side):
+    """Environment as real numbers (an infinite imaginary part must not touch the real one)."""
+    import ctypes
+    import paper_1512_03318_gb300 as P
+    n = ctypes.c_int64()
+    x = np.zeros(2 * d.env_len(bond, side))
+    d.ctx.check(P.lib().mrd_dmrg_env(d.h, bond, side, ctypes.byref(n), x.ctypes.data_as(ctypes.POINTER(ctypes.c_double))))
+    return x
+
+
+@pytest.mark.parametrize("direction", [+1, -1])
+@pytest.mark.parametrize("prec", [0, 3])
+def test_env_update_non_finite(ctx, direction, prec):
+    """Environment update from a site tensor with one infinite entry: non-finite exactly where the plain
+    sums are, the rest right."""
+    import paper_1512_03318_gb300 as P
+    ly, chi = 4, 400
+    mpo = P.MPO(None, 6, ly, 1, 4, 1.0, 1.0, P.MRD_BASIS_MIXED)
+    d = P.DMRG(ctx, mpo, 12, 0, chi, seed=3, center=12)
+    j = 10 if direction > 0 else 14
+    _, t = d.site(j)
+    x = t.copy()
+    x[len(x) // 2] = np.inf
+    host = np.ascontiguousarray(x)
+    d.set_site(j, host.ctypes.data)
+    d.env_update(j, direction, prec)
+    with np.errstate(all="ignore"):
+        pairs = E.oracle_left(d, mpo, j, d.env(j, 0)) if direction > 0 else E.oracle_right(d, mpo, j, d.env(j + 1, 1))
+    flat = _raw_env(d, j + 1, 0) if direction > 0 else _raw_env(d, j, 1)
+    n_bad = 0
+    for (w, xi, xpi, off, d0, d1), blk in pairs:
+        got = flat[2 * off:2 * (off + d0 * d1)]
+        ref = np.ascontiguousarray(blk).reshape(-1).view(np.float64)
+        n_bad += int(np.sum(~np.isfinite(ref)))
+        assert np.array_equal(np.isfinite(got), np.isfinite(ref))
+        f = np.isfinite(ref)
+        assert np.max(np.abs(got[f] - ref[f]), initial=0.0) <= TOL[prec]
+    assert n_bad > 0
+    d.close()
