@@ -61,14 +61,16 @@ extern "C" {
 #define MRD_PREC_FP64 0     /* complex128 operands, FP64 accuracy: FP64 arithmetic, or for  */
                             /* larger products 62-bit fixed point against the largest entry */
                             /* of each row and column, exact sums and one rounding (digit   */
-                            /* products on the tensor cores; FP64 arithmetic for the output */
-                            /* blocks that an entry that is not finite enters)              */
+                            /* products on the tensor cores; FP64 arithmetic again for the  */
+                            /* output blocks that an entry that is not finite enters, and   */
+                            /* for those whose terms are all far below the largest row times */
+                            /* the largest column of their operands)                        */
 #define MRD_PREC_TF32 1     /* tcgen05 tensor cores, TF32 operands, FP32 accumulation     */
 #define MRD_PREC_BF16X3 2   /* tcgen05, split BF16 (hi*hi + hi*lo + lo*hi), FP32 accum.   */
 #define MRD_PREC_FF 3       /* complex128 operands split into float-float pairs (~48-bit  */
                             /* products, TwoSum accumulation) on the FP32 pipes, or for larger */
-                            /* products 55-bit fixed point as above (output blocks that an */
-                            /* entry that is not finite enters: FP64)                      */
+                            /* products 55-bit fixed point as above, with the same blocks   */
+                            /* computed again in FP64 or float-float arithmetic            */
 
 #define MRD_BASIS_MIXED 0   /* orbitals (x, k_m), charges (N, K mod Ly)                   */
 #define MRD_BASIS_REAL 1    /* orbitals (x, y), charge N only (modulus 1)                 */

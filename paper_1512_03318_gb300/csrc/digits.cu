@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 
 #include "digits.cuh"
+#include "ff.cuh"
 
 namespace mrd {
 
@@ -605,7 +606,7 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
         }
       }
       const int exr = er - 2 * 1022 + (BETA == 8 ? -68 : -61);
-      int top[16];   // exponent field of the larger part of each result; 2047 outside the normal range
+      int top[16];   // upper word of the larger part of each result; the largest number outside the normal range
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
         const int eg = __shfl_sync(0xffffffffu, ec, c);
@@ -615,7 +616,7 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
         const double2 o = make_double2(to_double<BETA>(hi[0][c], lo[0][c], exr + eg, odd),
                                        REAL ? 0.0 : to_double<BETA>(hi[PARTS - 1][c], lo[PARTS - 1][c], exr + eg, odd));
         const bool valid = row < R && c < w && col0 + c < N;
-        top[c] = !valid ? 0 : odd ? 2047 : max(expo_field(o.x), expo_field(o.y));
+        top[c] = !valid ? 0 : odd ? 0x7fffffff : max(__double2hiint(o.x) & 0x7fffffff, __double2hiint(o.y) & 0x7fffffff);
         if (valid) g.c[at] = o;
       }
       // the largest of this lane's row, or (lanes 0 .. 15) column, of the C map
@@ -630,7 +631,7 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
           if (lane == c) most = v;
         }
       }
-      if (most > 0) atomicMax(g.res + q.cm + (by_row ? row : col0 + lane), most);
+      if (most > 0) atomicMax(g.res + q.cm + (by_row ? row : col0 + lane), most >> 20);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
@@ -644,12 +645,44 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
 
 // ---------------------------------------------------------------- products that are computed again
 
+constexpr int kDgFF = 1 << 30;   // mark of a listed tile that float-float arithmetic can do
+
+// log2 of sum_k |s_rk| |u_ck| over the bounds of row r and column c, in the part (real or imaginary) where
+// it is larger; one warp, 8 lanes per block, the lanes along K.
+__device__ __forceinline__ double terms_log2(const DgJob* sj, const DgJob* uj, int n, const double2* ssrc, const double2* usrc, int r,
+                                             int c, int er, int ec, int lane) {
+  const double sr = ldexp(1.0, 1022 - er), sc = ldexp(1.0, 1022 - ec);
+  double re = 0.0, im = 0.0;
+  for (int f = lane >> 3; f < n; f += 4) {
+    const DgJob &x = sj[f], &y = uj[f];
+    if (x.off < 0) continue;
+    const int64_t x0 = x.off + (x.flags & DGJ_KCONTIG ? r * x.ld : r), xs = x.flags & DGJ_KCONTIG ? 1 : x.ld;
+    const int64_t y0 = y.off + (y.flags & DGJ_KCONTIG ? c * y.ld : c), ys = y.flags & DGJ_KCONTIG ? 1 : y.ld;
+    for (int k = lane & 7; k < y.K; k += 8) {
+      const double2 p = ssrc[x0 + k * xs], q = usrc[y0 + k * ys];
+      const double px = fabs(p.x * sr), py = fabs(p.y * sr), qx = fabs(q.x * sc), qy = fabs(q.y * sc);
+      re = fma(px, qx, fma(py, qy, re));
+      im = fma(px, qy, fma(py, qx, im));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, o);
+    im += __shfl_xor_sync(0xffffffffu, im, o);
+  }
+  return log2(fmax(re, im));
+}
+
 // One warp per task: its tiles join the list when a row or column of its operands is not finite (exponent
-// field 2047) or a result is outside the normal range (marked likewise). Not after a wait gave up, when nothing is valid.
+// field 2047), a result is outside the normal range (marked likewise), or the fixed point was too coarse:
+// no result within 2^kDgSpread of the largest row times the largest column, and not for want of large
+// terms (sums that cancel are as inexact in FMAs): the terms of the largest row and column tell.
 __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members, int n,
+                                                  const DgJob* __restrict__ sjobs, const DgJob* __restrict__ ujobs,
+                                                  const double2* __restrict__ ssrc, const double2* __restrict__ usrc,
                                                   const int* __restrict__ e0, const int* __restrict__ e1,
                                                   const int* __restrict__ res, int* __restrict__ count, int2* __restrict__ list,
-                                                  const int* __restrict__ err) {
+                                                  const int* __restrict__ err, bool ff) {
   const int lane = threadIdx.x & 31;
   int i = (blockIdx.x * 256 + threadIdx.x) >> 5;
   DgMember m = members[min(i, n - 1)];
@@ -662,28 +695,127 @@ __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ gr
     const int* stacked = (g.cm_rows ? tall + g.ea : flat + g.eb) + (m.first - g.cm);
     const int* shared = g.cm_rows ? flat + g.eb : tall + g.ea;
     const int ns = g.cm_rows ? g.N : g.R;
-    int a = 0, b = 0, o = 0;
+    int a = 0, b = 0, o = 0, ra = 0, cb = 0;   // largest exponents, and a row and a column that have them
     for (int r = lane; r < m.rows; r += 32) {
-      a = max(a, stacked[r]);
+      const int e = stacked[r];
+      if (e > a) { a = e; ra = r; }
       o = max(o, res[m.first + r]);
     }
-    for (int c = lane; c < ns; c += 32) b = max(b, shared[c]);
-    a = __reduce_max_sync(0xffffffffu, a);
-    b = __reduce_max_sync(0xffffffffu, b);
+    for (int c = lane; c < ns; c += 32) {
+      const int e = shared[c];
+      if (e > b) { b = e; cb = c; }
+    }
+    const int am = __reduce_max_sync(0xffffffffu, a), bm = __reduce_max_sync(0xffffffffu, b);
     o = __reduce_max_sync(0xffffffffu, o);
-    if (a < 2047 && b < 2047 && o < 2047) continue;
+    if (am < 2047 && bm < 2047 && o < 2047) {
+      // bounds of rows and columns 2^(field - 1022), result >= 2^(field - 1023)
+      if (am == 0 || bm == 0 || am + bm - o <= 1021 + kDgSpread) continue;
+      const int r = __shfl_sync(0xffffffffu, ra, __ffs(__ballot_sync(0xffffffffu, a == am)) - 1);
+      const int c = __shfl_sync(0xffffffffu, cb, __ffs(__ballot_sync(0xffffffffu, b == bm)) - 1);
+      if (terms_log2(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane) >= -(double)kDgSpread) continue;
+    }
+    // float-float products take operands within the FP32 range only
+    const int mark = ff && abs(am - 1022) <= 30 && abs(bm - 1022) <= 30 && o < 2047 ? kDgFF : 0;
     const int tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32);
     int at = 0;
     if (lane == 0) at = atomicAdd(count, tiles);
     at = __shfl_sync(0xffffffffu, at, 0);
-    for (int t = lane; t < tiles; t += 32) list[at + t] = make_int2(i, t);
+    for (int t = lane; t < tiles; t += 32) list[at + t] = make_int2(i, t | mark);
   }
 }
 
-// The listed tiles (32 stacked rows x 32 of the shared side) in FP64 FMAs, K in chunks of 16, blocks
-// in the order of the job lists; REAL: imaginary parts taken and returned as zeros. Usually the list is
-// empty and the launch returns at once.
-template <bool REAL>
+// One listed tile: 32 stacked rows x 32 of the shared side, K in chunks of 16, blocks in the order of the job
+// lists. FP64 FMAs, or float-float (four times as fast: the FP64 pipe has 2 lanes per SM); REAL: imaginary
+// parts taken and returned as zeros.
+template <bool FFM, bool REAL>
+__device__ __forceinline__ void redo_tile(const DgGroup& g, const DgMember& m, int tile, const DgJob* __restrict__ sjobs,
+                                          const DgJob* __restrict__ ujobs, const double2* __restrict__ ssrc,
+                                          const double2* __restrict__ usrc, double2* __restrict__ C, void* sa, void* sb, float2* sas,
+                                          float2* sbs) {
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int ns = g.cm_rows ? g.N : g.R, tn = (ns + 31) / 32;
+  const int r0 = tile / tn * 32, c0 = tile % tn * 32;
+  auto put = [&](void* s, float2* sum, int at, double2 v, bool conj) {   // stage one element
+    if (conj) v.y = -v.y;
+    if (REAL) v.y = 0.0;
+    if constexpr (FFM) {
+      const float4 x = cff_from(v);
+      ((float4*)s)[at] = x;
+      if (!REAL) sum[at] = cff_sum(x);
+    } else {
+      ((double2*)s)[at] = v;
+    }
+  };
+  double2 acc[2][2] = {};
+  CAcc fac[2][2] = {};
+  for (int f = 0; f < g.n_jobs; ++f) {
+    const DgJob &sj = sjobs[m.job + f], &uj = ujobs[g.job + f];
+    if (sj.off < 0) continue;                            // a block this task does not multiply
+    const int K = uj.K;
+    const bool sk = sj.flags & DGJ_KCONTIG, uk = uj.flags & DGJ_KCONTIG;
+    for (int k0 = 0; k0 < K; k0 += 16) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int e = tid + q * 256;
+        const int sr = sk ? e >> 4 : e & 31, sc = sk ? e & 15 : e >> 5;
+        double2 v = make_double2(0.0, 0.0);
+        if (r0 + sr < m.rows && k0 + sc < K)
+          v = ssrc[sj.off + (sk ? (r0 + sr) * sj.ld + k0 + sc : (k0 + sc) * sj.ld + r0 + sr)];
+        put(sa, sas, sr * 17 + sc, v, sj.flags & DGJ_CONJ);
+        const int ur = uk ? e >> 4 : e & 31, uc = uk ? e & 15 : e >> 5;
+        v = make_double2(0.0, 0.0);
+        if (c0 + ur < ns && k0 + uc < K)
+          v = usrc[uj.off + (uk ? (c0 + ur) * uj.ld + k0 + uc : (k0 + uc) * uj.ld + c0 + ur)];
+        put(sb, sbs, uc * 33 + ur, v, uj.flags & DGJ_CONJ);
+      }
+      __syncthreads();
+      const int kn = K - k0 < 16 ? K - k0 : 16;
+      for (int k = 0; k < kn; ++k)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int p = (2 * ty + i) * 17 + k, q = k * 33 + 2 * tx + j;
+            if constexpr (FFM) {
+              const float4 a = ((const float4*)sa)[p], b = ((const float4*)sb)[q];
+              if (REAL) ff_mac(fac[i][j].rr, FF{a.x, a.z}, FF{b.x, b.z});
+              else cff_mac(fac[i][j], a, sas[p], b, sbs[q]);
+            } else {
+              const double2 a = ((const double2*)sa)[p], b = ((const double2*)sb)[q];
+              acc[i][j].x = fma(-a.y, b.y, fma(a.x, b.x, acc[i][j].x));
+              acc[i][j].y = fma(a.y, b.x, fma(a.x, b.y, acc[i][j].y));
+            }
+          }
+      if constexpr (FFM) {   // as the float-float GEMM: errors collected over 16 products at most
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            CAcc& x = fac[i][j];
+            x.rr = ff_renorm(x.rr);
+            if (!REAL) { x.ii = ff_renorm(x.ii); x.ss = ff_renorm(x.ss); }
+          }
+      }
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int r = r0 + 2 * ty + i, c = c0 + 2 * tx + j;
+      double2 v = acc[i][j];
+      if constexpr (FFM) {
+        FF re = ff_norm(fac[i][j].rr), im = {0.f, 0.f};
+        if (!REAL) cff_result(fac[i][j], re, im);
+        v = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
+      }
+      if (r < m.rows && c < ns) C[m.off + r * m.step + c * m.other] = make_double2(v.x, REAL ? 0.0 : v.y);
+    }
+}
+
+// The listed tiles. Usually the list is empty and the launch returns at once.
+template <bool FFM, bool REAL>
 __global__ void __launch_bounds__(256) k_dg_redo(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members,
                                                  const DgJob* __restrict__ sjobs, const DgJob* __restrict__ ujobs,
                                                  const double2* __restrict__ ssrc, const double2* __restrict__ usrc,
@@ -691,62 +823,18 @@ __global__ void __launch_bounds__(256) k_dg_redo(const DgGroup* __restrict__ gro
                                                  const int2* __restrict__ list) {
   asm volatile("griddepcontrol.wait;" ::: "memory");   // (dependent of k_dg_check)
   const int total = *count;
-  if ((int)blockIdx.x >= total) return;
-  __shared__ double2 As[32][17], Bs[16][33];
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  __shared__ __align__(16) uint8_t sa[32 * 17 * 16], sb[16 * 33 * 16];
+  __shared__ float2 sas[FFM && !REAL ? 32 * 17 : 1], sbs[FFM && !REAL ? 16 * 33 : 1];
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int2 it = list[item];
     const DgMember m = members[it.x];
-    const DgGroup& g = groups[m.group];
-    const int ns = g.cm_rows ? g.N : g.R, tn = (ns + 31) / 32;
-    const int r0 = it.y / tn * 32, c0 = it.y % tn * 32;
-    double2 acc[2][2] = {};
-    for (int f = 0; f < g.n_jobs; ++f) {
-      const DgJob &sj = sjobs[m.job + f], &uj = ujobs[g.job + f];
-      if (sj.off < 0) continue;                            // a block this task does not multiply
-      const int K = uj.K;
-      const bool sk = sj.flags & DGJ_KCONTIG, uk = uj.flags & DGJ_KCONTIG;
-      const double ss = sj.flags & DGJ_CONJ ? -1.0 : 1.0, us = uj.flags & DGJ_CONJ ? -1.0 : 1.0;
-      for (int k0 = 0; k0 < K; k0 += 16) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int e = tid + q * 256;
-          const int sr = sk ? e >> 4 : e & 31, sc = sk ? e & 15 : e >> 5;
-          double2 v = make_double2(0.0, 0.0);
-          if (r0 + sr < m.rows && k0 + sc < K)
-            v = ssrc[sj.off + (sk ? (r0 + sr) * sj.ld + k0 + sc : (k0 + sc) * sj.ld + r0 + sr)];
-          As[sr][sc] = make_double2(v.x, REAL ? 0.0 : v.y * ss);
-          const int ur = uk ? e >> 4 : e & 31, uc = uk ? e & 15 : e >> 5;
-          v = make_double2(0.0, 0.0);
-          if (c0 + ur < ns && k0 + uc < K)
-            v = usrc[uj.off + (uk ? (c0 + ur) * uj.ld + k0 + uc : (k0 + uc) * uj.ld + c0 + ur)];
-          Bs[uc][ur] = make_double2(v.x, REAL ? 0.0 : v.y * us);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-#pragma unroll
-          for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-              const double2 a = As[2 * ty + i][k], b = Bs[k][2 * tx + j];
-              acc[i][j].x = fma(-a.y, b.y, fma(a.x, b.x, acc[i][j].x));
-              acc[i][j].y = fma(a.y, b.x, fma(a.x, b.y, acc[i][j].y));
-            }
-        __syncthreads();
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int r = r0 + 2 * ty + i, c = c0 + 2 * tx + j;
-        if (r < m.rows && c < ns) C[m.off + r * m.step + c * m.other] = make_double2(acc[i][j].x, REAL ? 0.0 : acc[i][j].y);
-      }
+    const DgGroup g = groups[m.group];
+    if (FFM && (it.y & kDgFF)) redo_tile<FFM, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sa, sb, sas, sbs);
+    else redo_tile<false, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sa, sb, sas, sbs);
   }
 }
 
-cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, const int* words, int n_sm, cudaStream_t s) {
+cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, int beta, const int* words, int n_sm, cudaStream_t s) {
   if (d.n_members <= 0) return cudaSuccess;
   const int grid = (d.n_members + 7) / 8, u = 1 - d.sop;
   // both as programmatic dependents of the launch before them, so that they cost little when there is
@@ -762,10 +850,13 @@ cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2*
   lc.numAttrs = 1;
   const int* err = words + DG_ERR;
   cudaError_t e = cudaLaunchKernelEx(&lc, k_dg_check, (const DgGroup*)d.groups, (const DgMember*)d.members, d.n_members,
-                                     (const int*)d.expo[0], (const int*)d.expo[1], (const int*)d.res, d.redo_count, d.redo, err);
+                                     (const DgJob*)d.jobs[d.sop], (const DgJob*)d.jobs[u], d.sop ? b : a, d.sop ? a : b,
+                                     (const int*)d.expo[0], (const int*)d.expo[1], (const int*)d.res, d.redo_count, d.redo, err,
+                                     beta != 8);
   if (e != cudaSuccess) return e;
   lc.gridDim = dim3(2 * n_sm);
-  e = cudaLaunchKernelEx(&lc, d.real ? k_dg_redo<true> : k_dg_redo<false>, (const DgGroup*)d.groups, (const DgMember*)d.members,
+  auto k = beta == 8 ? k_dg_redo<false, false> : d.real ? k_dg_redo<true, true> : k_dg_redo<true, false>;
+  e = cudaLaunchKernelEx(&lc, k, (const DgGroup*)d.groups, (const DgMember*)d.members,
                          (const DgJob*)d.jobs[d.sop], (const DgJob*)d.jobs[u], d.sop ? b : a, d.sop ? a : b, C,
                          (const int*)d.redo_count, (const int2*)d.redo);
   count_launches(2);

@@ -17,7 +17,16 @@
 //   beta = 7 (t = 55, the float-float products): fewer flushes; 4e-16 and 2-4e-15 (the float-float
 //     CUDA-core kernel: 2-4e-14, 0.6-1.4e-14).
 // Entries far below the largest of their row or column keep fewer bits than a floating-point
-// product would give them: the error is relative to the row's and column's scale.
+// product would give them: a term is off by at most 2^-58 (FP64; 2^-51.8 float-float) of its row's
+// times its column's bound: two roundings of 2^-63 (2^-56), seven dropped digit pairs of 2^-62 (2^-56)
+// on the first level, and twice that in a complex product. K FMAs in FP64 may be off by
+// 2 K 2^-53 (float-float: 2 K 2^-46) of the sum of the terms' magnitudes, so a result block is kept when
+// that sum reaches 2^-kDgSpread of the largest row times the largest column somewhere in it: the error is
+// then below what FMAs may be off in the block. The largest result is a lower bound of the sum and costs
+// nothing; where it is too small, the terms of the largest row and column are added up. The other blocks
+// (operands graded against each other along K) are computed again in FP64, or in float-float for the
+// float-float products. On states of the cylinders
+// under 1% of the blocks fail the first test, and of those most pass the second.
 //
 // Measured on H_eff applications (Hofstadter cylinder, mid-ring sites, random operands): FP64 at
 // Ly = 8, chi = 1024 0.49 ms (CUDA cores 11.2 ms); loading environments and one float-float
@@ -37,6 +46,7 @@ constexpr int kDgRows = 128;      // rows of a left (tall) tile
 constexpr int kDgCols = 32;       // columns of a tile: 8 levels x 32 x (re, im) = 512 TMEM columns
 constexpr int kDgDigits = 8;
 constexpr int kDgStep = 16;       // K of one MMA, one panel step
+constexpr int kDgSpread = 6;      // bits a block's largest result may lie below its operands' bounds
 __host__ __device__ inline int dg_planes(bool real) { return real ? kDgDigits : 2 * kDgDigits; }
 __host__ __device__ inline int dg_tbits(int beta) { return beta == 8 ? 62 : 55; }
 // K steps between flushes. Level l sums 2 (l + 1) digit products of at most 2^(2 beta - 2) per
@@ -164,8 +174,9 @@ cudaError_t dg_pack(const DgDev& d, int op, const double2* src, int beta, int* w
 cudaError_t dg_gemm(const DgDev& d, double2* C, int beta, int* words, int n_sm, uint64_t wait_ns, cudaStream_t s,
                     int first = 0, int count = -1);
 // After the product: the tasks whose operands or results have an infinity or NaN, which has no
-// fixed-point form, are computed again in FP64 from the operands themselves (buffers 0 and 1).
-cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, const int* words, int n_sm, cudaStream_t s);
+// fixed-point form, or for which the fixed point was too coarse, are computed again in FP64 (float-float
+// where the product is and their range allows it) from the operands themselves (buffers 0 and 1).
+cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, int beta, const int* words, int n_sm, cudaStream_t s);
 cudaError_t dg_init();
 
 }  // namespace mrd

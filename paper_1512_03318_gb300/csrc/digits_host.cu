@@ -553,11 +553,11 @@ int dg_apply(mrd_heff* h, const double2* in, double2* out, const cudaEvent_t ev[
   };
   int rc = product(g->p1, g->d1, h->z);
   if (rc != MRD_OK) return rc;
-  MRD_CUDA(ctx, dg_redo(g->d1, h->lw, in, h->z, g->words, h->n_sm, s));
+  MRD_CUDA(ctx, dg_redo(g->d1, h->lw, in, h->z, beta, g->words, h->n_sm, s));
   MRD_CUDA(ctx, record_event(ev[1], s, cap));
   MRD_CUDA(ctx, dg_pack(g->d2, 0, h->z, beta, g->words, s));
   if ((rc = product(g->p2, g->d2, out)) != MRD_OK) return rc;
-  MRD_CUDA(ctx, dg_redo(g->d2, h->z, h->wr, out, g->words, h->n_sm, s));
+  MRD_CUDA(ctx, dg_redo(g->d2, h->z, h->wr, out, beta, g->words, h->n_sm, s));
   MRD_CUDA(ctx, record_event(ev[2], s, cap));
   return MRD_OK;
 }

@@ -441,7 +441,7 @@ int run_gemm_digits(mrd_dmrg* D, const GemmList& g, int64_t nt, const double2* A
   MRD_CUDA(ctx, dg_pack(d, 0, Aop, beta, words, s));
   MRD_CUDA(ctx, dg_pack(d, 1, Bop, beta, words, s));
   MRD_CUDA(ctx, dg_gemm(d, C, beta, words, D->n_sm, 1000000000ull, s));
-  MRD_CUDA(ctx, dg_redo(d, Aop, Bop, C, words, D->n_sm, s));
+  MRD_CUDA(ctx, dg_redo(d, Aop, Bop, C, beta, words, D->n_sm, s));
   *done = true;
   return MRD_OK;
 }

@@ -1,4 +1,5 @@
-"""What digit-split products cannot represent is computed again in FP64: infinities and NaN."""
+"""What digit-split products cannot represent is computed again in FP64: infinities, NaN, and operands
+graded against each other along K."""
 import numpy as np
 import pytest
 
@@ -110,3 +111,52 @@ def test_env_update_non_finite(ctx, direction, prec):
         assert np.max(np.abs(got[f] - ref[f]), initial=0.0) <= TOL[prec]
     assert n_bad > 0
     d.close()
+
+
+@pytest.mark.parametrize("prec", [0, 3])
+@pytest.mark.parametrize("decades", [0, 3, 6, 10, 16, 150])
+def test_graded_along_k(ctx, prec, decades):
+    """Both products with their operands graded against each other along K: every term counts alike, but the
+    largest row times the largest column is 10^decades of it. With n terms in all (a fold, a product over dl
+    and one over channels * dr, each complex), FP64 sums are off by at most n 2^-53 of the sum of the terms'
+    magnitudes, the oracle's too, and float-float ones by n 2^-46; the bounds are twice the sum of both,
+    relative to the largest such sum of the output block."""
+    import paper_1512_03318_gb300 as P
+    dl, dr, channels = 120, 96, 4
+    case = dict(_spin_channels(83, dl, dr, channels, False))
+    up = 10.0 ** (decades * np.arange(dl) / (dl - 1) - decades / 2.0)
+    vp = 10.0 ** (decades * np.arange(dr) / (dr - 1) - decades / 2.0)
+    l, r, t = case["lflat"].copy(), case["rflat"].copy(), case["tflat"].copy()
+    for row in case["ll"]:
+        off, d0, d1 = row[3:]
+        l[off:off + d0 * d1].reshape(d0, d1)[:] *= up[None, :]
+    for row in case["rl"]:
+        off, d0, d1 = row[3:]
+        r[off:off + d0 * d1].reshape(d0, d1)[:] *= (1.0 / vp)[:, None]
+    for m in case["lay"]:
+        blk = t[m["offset"]: m["offset"] + m["rowdim"] * m["coldim"]].reshape(m["rowdim"], m["coldim"])
+        for _, _, da, ro in m["rows"]:
+            blk[ro:ro + da] /= up[:, None]
+        for _, _, db, co in m["cols"]:
+            blk[:, co:co + db] *= vp[None, :]
+    case.update(lflat=l, rflat=r, tflat=t)
+    ref = _oracle(case)
+    mag = dict(case, lflat=np.abs(l), rflat=np.abs(r), tflat=np.abs(t),
+               wi=[(*e[:4], abs(e[4])) for e in case["wi"]], wj=[(*e[:4], abs(e[4])) for e in case["wj"]])
+    bound = np.abs(_oracle(mag))
+    n = 4 * (dl + channels + channels * dr)
+    tol = 2.0 * n * (2.0 ** -53 + (2.0 ** -53 if prec == 0 else 2.0 ** -46))
+    h = P.Heff(ctx, **G.heff_args(case))
+    h.set_env(_dev(l), _dev(r))
+    T = _dev(t)
+    out = torch.empty_like(T)
+    h.apply(T, out, prec)
+    h.status()
+    got = out.cpu().numpy()
+    for m in case["lay"]:
+        view = lambda x: x[m["offset"]: m["offset"] + m["rowdim"] * m["coldim"]].reshape(m["rowdim"], m["coldim"])
+        for _, _, da, ro in m["rows"]:
+            for _, _, db, co in m["cols"]:
+                e = np.abs(view(got) - view(ref))[ro:ro + da, co:co + db]
+                assert np.max(e) <= tol * np.max(view(bound)[ro:ro + da, co:co + db])
+    h.close()
