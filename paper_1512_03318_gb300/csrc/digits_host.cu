@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <thread>
 
 #include "digits.cuh"
@@ -339,29 +340,45 @@ void dg_tables(const DgPlan& p, uint8_t* host, uint8_t* dev, DgDev& d) {
 
 // ---------------------------------------------------------------- H_eff
 
-// Digit-split state of an H_eff: the plans of its two products and their device buffers. The
-// plans may be built on a host thread (dg_prebuild) while the device works.
-struct DgHeff {
-  bool planned = false, use = false, built = false, real = false, major = false, env_dirty = true;
+// The two products of an H_eff in one form: a precision, with or without imaginary parts, grouped or
+// one launch per stacked block. Plans, device buffers and packed environments stay until the handle is
+// freed, so that a program that changes precisions on it plans and packs once for each.
+struct DgForm {
+  int32_t prec = 0;
   int beta = 0;
+  bool real = false, major = false;
+  bool planned = false, use = false, built = false, env_dirty = true;
   DgPlan p1, p2;
   DgDev d1, d2;
   int* words = nullptr;   // DG_WORDS, then the exponents of theta and Z and the products' states (zeroed
   size_t zero_bytes = 0;  // together before each application)
   Arena mem;
+};
+// Digit-split state of an H_eff. A form's plans may be built on a host thread (dg_prebuild) while the
+// device works.
+struct DgHeff {
+  std::vector<std::unique_ptr<DgForm>> forms;
+  DgForm* cur = nullptr;   // of the last prepared application
   std::thread th;
   ~DgHeff() {
     if (th.joinable()) th.join();
+  }
+  DgForm* form(int32_t prec, bool real, bool major) {
+    for (auto& f : forms)
+      if (f->prec == prec && f->real == real && f->major == major) return f.get();
+    forms.push_back(std::make_unique<DgForm>());
+    DgForm* f = forms.back().get();
+    f->prec = prec;
+    f->beta = prec == MRD_PREC_FP64 ? 8 : 7;
+    f->real = real;
+    f->major = major;
+    return f;
   }
 };
 
 void dg_heff_free(DgHeff* g) { delete g; }
 
 namespace {
-
-// beta per precision: FP64 products keep 62 bits of every entry below the row's or column's
-// largest, float-float ones 55 (their own format has 48)
-int beta_of(int32_t prec) { return prec == MRD_PREC_FP64 ? 8 : 7; }
 
 // Cycles of planning, uploading and packing the environments of a small H_eff (~50 us: what the
 // applications of one environment load must save together; the other way needs next to no
@@ -396,16 +413,13 @@ double k_padding(const mrd_heff* h) {
 // 1.9 (Ly = 6, chi = 173) 231 / 240, 1.6 (Ly = 10, chi = 400) 550 / 635.
 constexpr double kMaxPadding = 2.2;
 
-// Plans of both products for a precision, and whether they are the cheaper way (the same
-// decision for grouped and per-task launches, which give the same bits).
-void plan_both(const mrd_heff* h, DgHeff* g, int32_t prec, bool real, bool major) {
+// Plans of both products of a form, and whether they are the cheaper way (the same decision for
+// grouped and per-task launches, which give the same bits).
+void plan_both(const mrd_heff* h, DgForm* g) {
   const int64_t n1 = h->counts[C_NT1], n2 = h->counts[C_NT2];
-  const int beta = beta_of(prec);
-  const bool ff = prec == MRD_PREC_FF;
+  const bool ff = g->prec == MRD_PREC_FF, real = g->real;
+  const int beta = g->beta;
   g->use = false;
-  g->real = real;
-  g->major = major;
-  g->beta = beta;
   g->planned = true;
   const double cores = cores_cost(h, ff, real);
   if (cores * h->dg_uses < kSetupCycles) return;   // not worth planning
@@ -423,7 +437,7 @@ void plan_both(const mrd_heff* h, DgHeff* g, int32_t prec, bool real, bool major
   const double pass = (double)(h->counts[C_THETA] + h->counts[C_ZLEN]) * 80.0 / 5.0e12 * 1.9e9 + 25000.0;
   const double mine = g->p1.cost + g->p2.cost + pass;
   g->use = !g->p1.items.empty() && !g->p2.items.empty() && mine * h->dg_uses + kSetupCycles < cores * h->dg_uses;
-  if (g->use && major) both(true);
+  if (g->use && g->major) both(true);
 }
 
 }  // namespace
@@ -431,17 +445,18 @@ void plan_both(const mrd_heff* h, DgHeff* g, int32_t prec, bool real, bool major
 // Start planning on a host thread (the host tables of h must not change until dg_prepare or
 // until h is freed); does nothing when no thread can be had.
 void dg_prebuild(mrd_heff* h, int32_t prec) {
-  if (h->dg || cores_cost(h, prec == MRD_PREC_FF, h->real && prec == MRD_PREC_FF) * h->dg_uses < 2 * kSetupCycles)
+  const bool ff = prec == MRD_PREC_FF;
+  if (h->dg || cores_cost(h, ff, h->real && ff) * h->dg_uses < 2 * kSetupCycles)
     return;   // planned on demand (or not at all) where that is a matter of microseconds
   DgHeff* g = new DgHeff();
-  const bool real = h->real && prec == MRD_PREC_FF, major = h->per_task;
   h->dg = g;
+  DgForm* f = g->form(prec, h->real && ff, h->per_task);
   try {
-    g->th = std::thread([h, g, prec, real, major] {
+    g->th = std::thread([h, f] {
       try {
-        plan_both(h, g, prec, real, major);
+        plan_both(h, f);
       } catch (...) {   // out of host memory: planned on demand instead
-        g->planned = false;
+        f->planned = false;
       }
     });
   } catch (...) {
@@ -454,15 +469,12 @@ void dg_prebuild(mrd_heff* h, int32_t prec) {
 int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
   mrd_ctx* ctx = h->ctx;
   cudaStream_t s = ctx->stream;
-  const int beta = beta_of(prec);
-  const bool real = h->real && prec == MRD_PREC_FF;
   if (!h->dg) h->dg = new DgHeff();
-  DgHeff* g = h->dg;
-  if (g->th.joinable()) g->th.join();
-  if (!g->planned || g->real != real || g->beta != beta || g->major != h->per_task) {
-    if (g->built) g->mem.release();   // panels of the other form
-    g->built = false;
-    plan_both(h, g, prec, real, h->per_task);
+  if (h->dg->th.joinable()) h->dg->th.join();
+  DgForm* g = h->dg->cur = h->dg->form(prec, h->real && prec == MRD_PREC_FF, h->per_task);
+  const int beta = g->beta;
+  if (!g->planned) {
+    plan_both(h, g);
     ++h->gen;
   }
   *use = g->use;
@@ -525,7 +537,8 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
 }
 
 void dg_env_changed(mrd_heff* h) {
-  if (h->dg) h->dg->env_dirty = true;
+  if (h->dg)
+    for (auto& f : h->dg->forms) f->env_dirty = true;
 }
 
 // theta_out = H_eff theta_in; ev: timing events (or null) before step 1, between the steps and
@@ -533,7 +546,7 @@ void dg_env_changed(mrd_heff* h) {
 int dg_apply(mrd_heff* h, const double2* in, double2* out, const cudaEvent_t ev[3], bool cap) {
   mrd_ctx* ctx = h->ctx;
   cudaStream_t s = ctx->stream;
-  DgHeff* g = h->dg;
+  DgForm* g = h->dg->cur;
   const int beta = g->beta;
   // the error flag outlives a product; the exponents and the products' states do not
   MRD_CUDA(ctx, cudaMemsetAsync(g->words + DG_WORDS, 0, g->zero_bytes - DG_WORDS * 4, s));
@@ -564,13 +577,17 @@ int dg_apply(mrd_heff* h, const double2* in, double2* out, const cudaEvent_t ev[
 
 // A wait of the digit-split products that gave up since the last check (MRD_E_TIMEOUT, then cleared).
 int dg_status(mrd_heff* h) {
-  DgHeff* g = h->dg;
-  if (!g || !g->built) return MRD_OK;
-  int herr = 0;
-  MRD_CUDA(h->ctx, cudaMemcpyAsync(&herr, g->words + DG_ERR, 4, cudaMemcpyDeviceToHost, h->ctx->stream));
-  MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
-  if (!herr) return MRD_OK;
-  MRD_CUDA(h->ctx, cudaMemsetAsync(g->words + DG_ERR, 0, 4, h->ctx->stream));
-  MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
-  return mrd_fail(h->ctx, MRD_E_TIMEOUT, "digit-split GEMM: a bounded wait gave up (code " + std::to_string(herr) + ")");
+  if (!h->dg) return MRD_OK;
+  int rc = MRD_OK;
+  for (auto& f : h->dg->forms) {
+    if (!f->built) continue;
+    int herr = 0;
+    MRD_CUDA(h->ctx, cudaMemcpyAsync(&herr, f->words + DG_ERR, 4, cudaMemcpyDeviceToHost, h->ctx->stream));
+    MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
+    if (!herr) continue;
+    MRD_CUDA(h->ctx, cudaMemsetAsync(f->words + DG_ERR, 0, 4, h->ctx->stream));
+    MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));
+    rc = mrd_fail(h->ctx, MRD_E_TIMEOUT, "digit-split GEMM: a bounded wait gave up (code " + std::to_string(herr) + ")");
+  }
+  return rc;
 }
