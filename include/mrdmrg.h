@@ -161,7 +161,11 @@ int mrd_heff_set_env(mrd_heff* h, const double* lenv_dev, const double* renv_dev
  * float-float arithmetic (~1e-13 relative or better); MRD_PREC_TF32 and MRD_PREC_BF16X3 run the same
  * contraction on the tcgen05 tensor cores with FP32 accumulation (complex products as four
  * real ones), operands repacked into swizzled tiles of 32-byte rows: the folded environments once
- * after each mrd_heff_set_env, theta on every call; the result is returned in complex128. */
+ * after each mrd_heff_set_env, theta on every call; the result is returned in complex128.
+ * In a caller's stream capture MRD_PREC_FP64 needs no earlier call and a replay multiplies the
+ * environments loaded last (by the FP64 kernel, whatever the size). The other precisions must have been
+ * applied once outside a capture, and a replay multiplies the environments that the last
+ * application outside a capture, or the capture itself, has repacked. */
 int mrd_heff_apply(mrd_heff* h, const double* theta_in_dev, double* theta_out_dev, int32_t prec);
 /* Real flops of one H_eff application (8 per complex multiply-add), written to flops4:
  * [0] in the order of the definition (L step, W step, R step); [1] as executed by the

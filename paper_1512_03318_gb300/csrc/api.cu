@@ -444,6 +444,7 @@ int heff_fold(mrd_heff* h, const double2* lenv, const double2* renv) {
                         h->wj_val, 1, h->counts[C_WRLEN], ctx->stream);
   if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "mrd_heff_set_env");
   h->env_loaded = (lenv || h->counts[C_LENV] == 0) && (renv || h->counts[C_RENV] == 0);
+  h->env_captured = h->env_captured || stream_capturing(ctx->stream);
   tc_env_changed(h);
   dg_env_changed(h);
   h->ff_dirty = true;
@@ -751,6 +752,11 @@ int mrd_lanczos(mrd_heff* h, double* theta_dev, int32_t max_iter, double tol, in
   MRD_CUDA(ctx, lanczos_set_fp32_full(h->lz, prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3));
   const uint64_t key =
       h->use_graph ? ((uint64_t)h->gen << 8 | (h->timing ? 0x80u : 0u) | (uint64_t)(prec + 1)) : 0;
+  struct Run {   // every step's application is prepared
+    bool& f;
+    explicit Run(bool& x) : f(x) { f = true; }
+    ~Run() { f = false; }
+  } run(h->in_lanczos);
   rc = lanczos_run(h->lz, ctx, apply_cb, &arg, (double2*)theta_dev, max_iter, tol, energy, &it, nullptr, key,
                    h->timing ? replay_timing_cb : nullptr);
   *iters = it;

@@ -469,10 +469,17 @@ void dg_prebuild(mrd_heff* h, int32_t prec) {
 int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
   mrd_ctx* ctx = h->ctx;
   cudaStream_t s = ctx->stream;
+  // In a caller's capture nothing can be allocated, and what is packed now would be old when the graph is
+  // replayed after another environment load. The FP64 kernel needs no preparation and reads LW and WR
+  // themselves; float-float products run in the form that an earlier application has built.
+  const bool cap = !h->in_lanczos && stream_capturing(s);
+  *use = false;
+  if (cap && prec == MRD_PREC_FP64) return MRD_OK;
   if (!h->dg) h->dg = new DgHeff();
   if (h->dg->th.joinable()) h->dg->th.join();
   DgForm* g = h->dg->cur = h->dg->form(prec, h->real && prec == MRD_PREC_FF, h->per_task);
   const int beta = g->beta;
+  if (cap && !g->built) return MRD_OK;
   if (!g->planned) {
     plan_both(h, g);
     ++h->gen;
@@ -527,11 +534,11 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
     g->env_dirty = true;
     ++h->gen;
   }
-  if (g->env_dirty) {
+  if (g->env_dirty || (h->env_captured && !h->in_lanczos)) {
     MRD_CUDA(ctx, cudaMemsetAsync(g->d1.expo[0], 0, (size_t)(g->p1.rows[0] + g->p2.rows[1]) * 4, s));
     MRD_CUDA(ctx, dg_pack(g->d1, 0, h->lw, beta, g->words, s));
     MRD_CUDA(ctx, dg_pack(g->d2, 1, h->wr, beta, g->words, s));
-    g->env_dirty = false;
+    g->env_dirty = cap;   // (packed by the replays, not now)
   }
   return MRD_OK;
 }

@@ -115,6 +115,8 @@ struct mrd_heff {
   DgHeff* dg = nullptr;
   double dg_uses = 50.0;            // FP64 / float-float applications expected per environment load
   bool dg_use = false;              // the last prepared FP64 / float-float application runs on them
+  bool in_lanczos = false;          // applications come from mrd_lanczos, which has prepared them
+  bool env_captured = false;        // an environment load was captured: a replay may change LW and WR at any time
   // float-float path: LW, WR in float-float layout (prepared after each environment load) and
   // theta staging
   Arena ff_mem;
@@ -151,6 +153,11 @@ struct mrd_heff {
 inline const float4* heff_ff_lw(const mrd_heff* h) { return h->lw_ff && !h->ff_dirty ? h->lw_ff : nullptr; }
 inline const float4* heff_ff_wr(const mrd_heff* h) { return h->wr_ff && !h->ff_dirty ? h->wr_ff : nullptr; }
 
+inline bool stream_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusActive;
+}
+
 inline cudaError_t record_event(cudaEvent_t e, cudaStream_t s, bool captured) {
   if (!e) return cudaSuccess;
   return captured ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
@@ -172,8 +179,7 @@ inline cudaEvent_t take_event(mrd_heff* h) {
 // captured into the Lanczos step graph, the graph's own three (external event nodes, so that
 // each replay records them). *captured tells which.
 inline bool apply_events(mrd_heff* h, cudaStream_t s, cudaEvent_t ev[3], bool* captured) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  *captured = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusActive;
+  *captured = stream_capturing(s);
   if (!*captured) {
     for (int k = 0; k < 3; ++k)
       if (!(ev[k] = take_event(h))) return false;
