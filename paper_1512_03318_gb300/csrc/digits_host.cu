@@ -210,9 +210,12 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
     total += tm * (tn - 1) * tile_cost(nks, 32) + tm * tile_cost(nks, d.N - (tn - 1) * kDgCols);
   }
   // Items. A tile longer than a third of an SM's share is cut along K into parts (their integer
-  // sums add exactly), so that a few long tiles neither leave SMs idle nor end the launch
-  // alone; parts of less than 3 steps cost more than they spread.
-  const double cap = std::max(total / (3.0 * n_sm), 9000.0);
+  // sums add exactly), so that a few long tiles neither leave SMs idle nor end the launch alone. A part
+  // writes its 96-bit sums and the last one reads those of all others, one after another (~20,000
+  // cycles for each), so parts stay above 100,000 cycles or 1.6 shares where the shares are short. us of
+  // step 2 (parts from a third of a share or 9,000 cycles on / these): float-float Ly = 5, chi = 301
+  // 128 / 70, Ly = 8, chi = 1024 418 / 333, Ly = 10, chi = 400 303 / 125; FP64 85 / 67, 338 / 331, 155 / 110.
+  const double share = total / n_sm, cap = std::max({9000.0, std::min(1.6 * share, 100000.0), share / 3.0});
   struct Cls {   // tiles of a group with the same number of columns
     double cost;
     int32_t group, parts, ct0, ct1;
