@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <thread>
 
@@ -51,6 +52,7 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
     int32_t N, R, kp;   // shared and stacked extents, padded K
     std::vector<Entry> e;
     std::vector<Member> m;
+    bool rising;        // the blocks' offsets rise from one to the next, here and in every member's list
   };
   std::vector<Group> gs;
   gs.reserve((size_t)std::min<int64_t>(n_tasks, 1024));
@@ -98,17 +100,30 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
         break;
       }
     }
-    if (gi == (int32_t)gs.size()) gs.push_back(Group{N, 0, 0, {}, {}});
+    if (gi == (int32_t)gs.size()) gs.push_back(Group{N, 0, 0, {}, {}, true});
     Group& g = gs[(size_t)gi];
     if (g.m.empty() || how == DG_BY_ID) {   // collect the shared blocks (members list them in one order)
       size_t cur = 0;
+      int64_t before = -1;
+      if (g.m.empty()) g.e.reserve((size_t)ns);
       for (int64_t k = 0; k < ns; ++k) {
         const int64_t off = sg[6 * k + uf];
         const size_t n = g.e.size();
-        size_t q = 0, f = n;   // the entries from the cursor on, around to it
-        for (; q < n && f == n; ++q)
-          if (g.e[(cur + q) % n].off == off) f = (cur + q) % n;
-        if (f == n) g.e.push_back({off, sg[6 * k + uf + 1], (int32_t)sg[6 * k + 4], 0, 0, (sg[6 * k + 5] & ubit) != 0});
+        g.rising = g.rising && off > before;
+        before = off;
+        size_t f = n;
+        if (cur < n && g.e[cur].off == off) {
+          f = cur;
+        } else if (!g.rising || (n > 0 && off <= g.e[n - 1].off)) {   // from the cursor on, around to it
+          for (size_t q = 0; q < n && f == n; ++q) {
+            const size_t at = cur + q < n ? cur + q : cur + q - n;
+            if (g.e[at].off == off) f = at;
+          }
+        }
+        if (f == n) {
+          g.rising = g.rising && (n == 0 || off > g.e[n - 1].off);
+          g.e.push_back({off, sg[6 * k + uf + 1], (int32_t)sg[6 * k + 4], 0, 0, (sg[6 * k + 5] & ubit) != 0});
+        }
         cur = f + 1;
       }
     }
@@ -184,7 +199,7 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
         int64_t hit = -1;
         if (k < t[5] && sg[6 * k + uf] == e.off) {
           hit = k++;
-        } else if (how == DG_BY_ID) {
+        } else if (how == DG_BY_ID && !(g.rising && (k == t[5] || sg[6 * k + uf] > e.off))) {
           for (int64_t q = 0; q < t[5]; ++q)
             if (sg[6 * q + uf] == e.off) {
               hit = q;
@@ -429,11 +444,39 @@ void plan_both(const mrd_heff* h, DgForm* g) {
   if (ff && k_padding(h) > kMaxPadding) return;
   std::vector<int32_t> ids((size_t)n2);   // step 2: the two row parts s1' of an output sector
   for (int64_t i = 0; i < n2; ++i) ids[(size_t)i] = (int32_t)(i >> 2 << 1 | (i & 1));   // share (nearly) all WR blocks
+  // the two plans are independent: the second on a host thread of its own where that pays for starting
+  // one (~60 us with its first use of the tables; a plan takes ~40 ns per segment)
+  int64_t segs2 = 0;
+  for (int64_t i = 0; i < n2; ++i) segs2 += h->t2_host[(size_t)(TF * i + 5)];
   auto both = [&](bool gm) {
     g->p1 = DgPlan();
     g->p2 = DgPlan();
+    auto second = [&] {
+      dg_plan(g->p2, h->t2_host.data(), h->s2_host.data(), n2, DG_BY_ID, ids.data(), real, beta, h->n_sm, gm);
+    };
+    std::exception_ptr failed;
+    std::thread th;
+    if (segs2 > 2500) {
+      try {
+        th = std::thread([&] {
+          try {
+            second();
+          } catch (...) {
+            failed = std::current_exception();
+          }
+        });
+      } catch (...) {   // no thread to be had
+      }
+    }
+    struct Join {
+      std::thread& t;
+      ~Join() { if (t.joinable()) t.join(); }
+    } join{th};
+    const bool split = th.joinable();
     dg_plan(g->p1, h->t1_host.data(), h->s1_host.data(), n1, DG_BY_B, nullptr, real, beta, h->n_sm, gm);
-    dg_plan(g->p2, h->t2_host.data(), h->s2_host.data(), n2, DG_BY_ID, ids.data(), real, beta, h->n_sm, gm);
+    if (!split) return second();
+    th.join();
+    if (failed) std::rethrow_exception(failed);
   };
   both(false);
   // the exponent and digit passes move ~80 bytes per element of theta and Z
