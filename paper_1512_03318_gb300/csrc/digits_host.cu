@@ -409,7 +409,7 @@ double cores_cost(const mrd_heff* h, bool ff, bool real) {
          dg_cost_cores(h->t2_host.data(), h->s2_host.data(), h->counts[C_NT2], ff, real, h->n_sm);
 }
 
-// K of the segments, padded to the 16 of one MMA, over K.
+// K of the segments over their K in the panels: dg_plan pads each to 8 (and a group's total to 16).
 double k_padding(const mrd_heff* h) {
   double padded = 0.0, k = 0.0;
   auto add = [&](const std::vector<int64_t>& t, const std::vector<int64_t>& sg, int64_t n) {
@@ -417,7 +417,7 @@ double k_padding(const mrd_heff* h) {
       for (int64_t q = 0; q < t[(size_t)(TF * i + 5)]; ++q) {
         const int64_t K = sg[(size_t)(SF * (t[(size_t)(TF * i + 4)] + q) + 4)];
         k += (double)K;
-        padded += (double)((K + 15) / 16 * 16);
+        padded += (double)up(K, 8);
       }
   };
   add(h->t1_host, h->s1_host, h->counts[C_NT1]);
@@ -425,11 +425,13 @@ double k_padding(const mrd_heff* h) {
   return k > 0.0 ? padded / k : 1.0;
 }
 
-// Float-float products whose segments are mostly padding stay on the CUDA cores, which take their K as
-// it is (FP64 ones do not: that pipe is 12 times slower). Setting environments and one application,
-// us with digits / without: padding 4.3 (Ly = 10, chi = 100) 280 / 209, 3.4 (Ly = 5, chi = 61) 141 / 107,
-// 1.9 (Ly = 6, chi = 173) 231 / 240, 1.6 (Ly = 10, chi = 400) 550 / 635.
-constexpr double kMaxPadding = 2.2;
+// Float-float products whose segments are mostly padding stay on the CUDA cores, which take their K as it
+// is: dg_cost_cores counts whole chunks of 16 there and would call them too dear (FP64 ones do not, that
+// pipe is 12 times slower). First application on a new handle / every further one, us, digits | CUDA cores:
+// padding 2.3 (Ly = 10, chi = 100) 916 / 116 | 340 / 165, 2.2 (Ly = 4, chi = 40) 239 / 85 | 117 / 58, 2.1 (Ly = 6, chi
+// = 64) 390 / 96 | 178 / 91, 1.9 (Ly = 5, chi = 61) 278 / 90 | 141 / 79; 1.4 (Ly = 5, chi = 301) 500 / 123 |
+// 280 / 191, 1.2 (Ly = 10, chi = 400) 717 / 183 | 699 / 520.
+constexpr double kMaxPadding = 1.55;
 
 // Plans of both products of a form, and whether they are the cheaper way (the same decision for
 // grouped and per-task launches, which give the same bits).
