@@ -673,10 +673,41 @@ __device__ __forceinline__ double terms_log2(const DgJob* sj, const DgJob* uj, i
   return log2(fmax(re, im));
 }
 
-// One warp per task: its tiles join the list when a row or column of its operands is not finite (exponent
-// field 2047), a result is outside the normal range (marked likewise), or the fixed point was too coarse:
-// no result within 2^kDgSpread of the largest row times the largest column, and not for want of large
-// terms (sums that cancel are as inexact in FMAs): the terms of the largest row and column tell.
+// Whether a task has to be computed again (0: no, 1: in FP64, 2: in float-float): a row or column of its
+// operands is not finite (exponent field 2047), a result is outside the normal range (marked likewise), or
+// the fixed point was too coarse: no result within 2^kDgSpread of the largest row times the largest
+// column, and not for want of large terms (sums that cancel are as inexact in FMAs): the terms of the
+// largest row and column tell. One warp.
+__device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, const DgJob* sjobs, const DgJob* ujobs, const double2* ssrc,
+                                         const double2* usrc, const int* e0, const int* e1, const int* res, bool ff, int lane) {
+  const int *tall = g.tall_op ? e1 : e0, *flat = g.tall_op ? e0 : e1;
+  const int* stacked = (g.cm_rows ? tall + g.ea : flat + g.eb) + (m.first - g.cm);
+  const int* shared = g.cm_rows ? flat + g.eb : tall + g.ea;
+  const int ns = g.cm_rows ? g.N : g.R;
+  int a = 0, b = 0, o = 0, ra = 0, cb = 0;   // largest exponents, and a row and a column that have them
+  for (int r = lane; r < m.rows; r += 32) {
+    const int e = stacked[r];
+    if (e > a) { a = e; ra = r; }
+    o = max(o, res[m.first + r]);
+  }
+  for (int c = lane; c < ns; c += 32) {
+    const int e = shared[c];
+    if (e > b) { b = e; cb = c; }
+  }
+  const int am = __reduce_max_sync(0xffffffffu, a), bm = __reduce_max_sync(0xffffffffu, b);
+  o = __reduce_max_sync(0xffffffffu, o);
+  if (am == 2047 || bm == 2047 || o == 2047) return 1;
+  // bounds of rows and columns 2^(field - 1022), result >= 2^(field - 1023)
+  if (am == 0 || bm == 0 || am + bm - o <= 1021 + kDgSpread) return 0;
+  const int r = __shfl_sync(0xffffffffu, ra, __ffs(__ballot_sync(0xffffffffu, a == am)) - 1);
+  const int c = __shfl_sync(0xffffffffu, cb, __ffs(__ballot_sync(0xffffffffu, b == bm)) - 1);
+  if (terms_log2(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane) >= -(double)kDgSpread) return 0;
+  // float-float products take operands within the FP32 range only
+  return ff && abs(am - 1022) <= 30 && abs(bm - 1022) <= 30 ? 2 : 1;
+}
+
+// One warp per task: the tiles of those to be computed again join the list. Not after a wait gave up, when
+// nothing is valid.
 __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members, int n,
                                                   const DgJob* __restrict__ sjobs, const DgJob* __restrict__ ujobs,
                                                   const double2* __restrict__ ssrc, const double2* __restrict__ usrc,
@@ -691,32 +722,9 @@ __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ gr
   asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
   if (*err) return;
   for (; i < n; i += gridDim.x * 8, m = members[min(i, n - 1)], g = groups[m.group]) {
-    const int *tall = g.tall_op ? e1 : e0, *flat = g.tall_op ? e0 : e1;
-    const int* stacked = (g.cm_rows ? tall + g.ea : flat + g.eb) + (m.first - g.cm);
-    const int* shared = g.cm_rows ? flat + g.eb : tall + g.ea;
-    const int ns = g.cm_rows ? g.N : g.R;
-    int a = 0, b = 0, o = 0, ra = 0, cb = 0;   // largest exponents, and a row and a column that have them
-    for (int r = lane; r < m.rows; r += 32) {
-      const int e = stacked[r];
-      if (e > a) { a = e; ra = r; }
-      o = max(o, res[m.first + r]);
-    }
-    for (int c = lane; c < ns; c += 32) {
-      const int e = shared[c];
-      if (e > b) { b = e; cb = c; }
-    }
-    const int am = __reduce_max_sync(0xffffffffu, a), bm = __reduce_max_sync(0xffffffffu, b);
-    o = __reduce_max_sync(0xffffffffu, o);
-    if (am < 2047 && bm < 2047 && o < 2047) {
-      // bounds of rows and columns 2^(field - 1022), result >= 2^(field - 1023)
-      if (am == 0 || bm == 0 || am + bm - o <= 1021 + kDgSpread) continue;
-      const int r = __shfl_sync(0xffffffffu, ra, __ffs(__ballot_sync(0xffffffffu, a == am)) - 1);
-      const int c = __shfl_sync(0xffffffffu, cb, __ffs(__ballot_sync(0xffffffffu, b == bm)) - 1);
-      if (terms_log2(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane) >= -(double)kDgSpread) continue;
-    }
-    // float-float products take operands within the FP32 range only
-    const int mark = ff && abs(am - 1022) <= 30 && abs(bm - 1022) <= 30 && o < 2047 ? kDgFF : 0;
-    const int tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32);
+    const int form = task_form(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, ff, lane);
+    if (form == 0) continue;
+    const int ns = g.cm_rows ? g.N : g.R, tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32), mark = form == 2 ? kDgFF : 0;
     int at = 0;
     if (lane == 0) at = atomicAdd(count, tiles);
     at = __shfl_sync(0xffffffffu, at, 0);
@@ -814,6 +822,13 @@ __device__ __forceinline__ void redo_tile(const DgGroup& g, const DgMember& m, i
     }
 }
 
+// Shared memory of the tiles above.
+template <bool FFM, bool REAL>
+struct RedoSmem {
+  alignas(16) uint8_t a[32 * 17 * 16], b[16 * 33 * 16];
+  float2 as[FFM && !REAL ? 32 * 17 : 1], bs[FFM && !REAL ? 16 * 33 : 1];
+};
+
 // The listed tiles. Usually the list is empty and the launch returns at once.
 template <bool FFM, bool REAL>
 __global__ void __launch_bounds__(256) k_dg_redo(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members,
@@ -823,42 +838,78 @@ __global__ void __launch_bounds__(256) k_dg_redo(const DgGroup* __restrict__ gro
                                                  const int2* __restrict__ list) {
   asm volatile("griddepcontrol.wait;" ::: "memory");   // (dependent of k_dg_check)
   const int total = *count;
-  __shared__ __align__(16) uint8_t sa[32 * 17 * 16], sb[16 * 33 * 16];
-  __shared__ float2 sas[FFM && !REAL ? 32 * 17 : 1], sbs[FFM && !REAL ? 16 * 33 : 1];
+  __shared__ RedoSmem<FFM, REAL> sm;
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int2 it = list[item];
     const DgMember m = members[it.x];
     const DgGroup g = groups[m.group];
-    if (FFM && (it.y & kDgFF)) redo_tile<FFM, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sa, sb, sas, sbs);
-    else redo_tile<false, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sa, sb, sas, sbs);
+    if (FFM && (it.y & kDgFF)) redo_tile<FFM, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
+    else redo_tile<false, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
   }
 }
+
+// Both in one launch, for products of small tasks: a CTA checks a task and computes its few tiles if it must.
+template <bool FFM, bool REAL>
+__global__ void __launch_bounds__(256) k_dg_redo_tasks(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members,
+                                                       const DgJob* __restrict__ sjobs, const DgJob* __restrict__ ujobs,
+                                                       const double2* __restrict__ ssrc, const double2* __restrict__ usrc,
+                                                       double2* __restrict__ C, const int* __restrict__ e0,
+                                                       const int* __restrict__ e1, const int* __restrict__ res,
+                                                       const int* __restrict__ err) {
+  const DgMember m = members[blockIdx.x];
+  const DgGroup g = groups[m.group];
+  __shared__ RedoSmem<FFM, REAL> sm;
+  __shared__ int s_form;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // (dependent of the product)
+  if (threadIdx.x < 32) {
+    const int form = *err ? 0 : task_form(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, FFM, threadIdx.x);
+    if (threadIdx.x == 0) s_form = form;
+  }
+  __syncthreads();
+  if (s_form == 0) return;
+  const int ns = g.cm_rows ? g.N : g.R, tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32);
+  for (int t = 0; t < tiles; ++t) {
+    if (FFM && s_form == 2) redo_tile<FFM, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
+    else redo_tile<false, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
+  }
+}
+
+// Products whose tasks are single tiles, up to this many, take the one-launch form: 2 to 3 us less per product
+// (FP64 application at Ly = 4, chi = 48 74.4 -> 69.0 us, float-float at Ly = 5, chi = 112 in real arithmetic
+// 66 -> 58). With larger tasks the tiles of one would follow each other (up to 8 of them: FP64 update at
+// Ly = 6, chi = 512 13.6 -> 15.0 ms).
+constexpr int kDgRedoTiles = 1, kDgRedoTasks = 4096;
 
 cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, int beta, const int* words, int n_sm, cudaStream_t s) {
   if (d.n_members <= 0) return cudaSuccess;
   const int grid = (d.n_members + 7) / 8, u = 1 - d.sop;
-  // both as programmatic dependents of the launch before them, so that they cost little when there is
+  // as programmatic dependents of the launch before them, so that they cost little when there is
   // nothing to do: 4 us per product less than in plain stream order
   cudaLaunchAttribute pdl;
   pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   pdl.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3(grid < 2048 ? grid : 2048);
   lc.blockDim = dim3(256);
   lc.stream = s;
   lc.attrs = &pdl;
   lc.numAttrs = 1;
-  const int* err = words + DG_ERR;
-  cudaError_t e = cudaLaunchKernelEx(&lc, k_dg_check, (const DgGroup*)d.groups, (const DgMember*)d.members, d.n_members,
-                                     (const DgJob*)d.jobs[d.sop], (const DgJob*)d.jobs[u], d.sop ? b : a, d.sop ? a : b,
-                                     (const int*)d.expo[0], (const int*)d.expo[1], (const int*)d.res, d.redo_count, d.redo, err,
-                                     beta != 8);
+  const DgGroup* gr = d.groups;
+  const DgMember* me = d.members;
+  const DgJob *sj = d.jobs[d.sop], *uj = d.jobs[u];
+  const double2 *ss = d.sop ? b : a, *us = d.sop ? a : b;
+  const int *e0 = d.expo[0], *e1 = d.expo[1], *res = d.res, *err = words + DG_ERR;
+  if (d.max_tiles <= kDgRedoTiles && d.n_members <= kDgRedoTasks) {
+    lc.gridDim = dim3(d.n_members);
+    auto k = beta == 8 ? k_dg_redo_tasks<false, false> : d.real ? k_dg_redo_tasks<true, true> : k_dg_redo_tasks<true, false>;
+    count_launch();
+    return cudaLaunchKernelEx(&lc, k, gr, me, sj, uj, ss, us, C, e0, e1, res, err);
+  }
+  lc.gridDim = dim3(grid < 2048 ? grid : 2048);
+  cudaError_t e = cudaLaunchKernelEx(&lc, k_dg_check, gr, me, d.n_members, sj, uj, ss, us, e0, e1, res, d.redo_count, d.redo, err, beta != 8);
   if (e != cudaSuccess) return e;
   lc.gridDim = dim3(2 * n_sm);
   auto k = beta == 8 ? k_dg_redo<false, false> : d.real ? k_dg_redo<true, true> : k_dg_redo<true, false>;
-  e = cudaLaunchKernelEx(&lc, k, (const DgGroup*)d.groups, (const DgMember*)d.members,
-                         (const DgJob*)d.jobs[d.sop], (const DgJob*)d.jobs[u], d.sop ? b : a, d.sop ? a : b, C,
-                         (const int*)d.redo_count, (const int2*)d.redo);
+  e = cudaLaunchKernelEx(&lc, k, gr, me, sj, uj, ss, us, C, (const int*)d.redo_count, (const int2*)d.redo);
   count_launches(2);
   return e;
 }

@@ -101,6 +101,7 @@ struct DgPlan {
   int64_t rows[2] = {0, 0};          // exponents
   int64_t slots = 0;                 // partial sums of split tiles
   int64_t redo = 0;                  // 32 x 32 tiles of all tasks
+  int max_tiles = 0;                 // of one task
   int sop = 0;                       // the stacked operand
   double cost = 0.0;                 // estimated cycles of the product
   bool real = false;
@@ -140,6 +141,7 @@ struct DgDev {
   int* res = nullptr;                // largest exponent field of each stacked row's results; zeroed likewise
   int* redo_count = nullptr;         // tiles to be computed again, zeroed likewise
   int2* redo = nullptr;              // (task, tile)
+  int max_tiles = 0;
   int sop = 0;
   bool real = false;
 };

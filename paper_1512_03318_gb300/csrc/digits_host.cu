@@ -213,7 +213,9 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
                                es + m.row0, kind(sop, ct) | s_flag, 0});
       }
       p.members.push_back({t[2], sop ? 1 : t[3], sop ? t[3] : 1, (int32_t)p.cmap + m.row0, m.rows, (int32_t)p.groups.size(), job0});
-      p.redo += up(m.rows, 32) / 32 * (up(g.N, 32) / 32);
+      const int64_t tiles = up(m.rows, 32) / 32 * (up(g.N, 32) / 32);
+      p.redo += tiles;
+      p.max_tiles = (int)std::max<int64_t>(p.max_tiles, tiles);
     }
     p.cmap += g.R;
     p.bytes[sop] += up(g.R, s_tall ? 8 : 16) * nks * pb;
@@ -350,6 +352,7 @@ void dg_tables(const DgPlan& p, uint8_t* host, uint8_t* dev, DgDev& d) {
   d.n_items = (int)p.items.size();
   d.n_splits = (int)p.splits.size();
   d.tab_bytes = off;
+  d.max_tiles = p.max_tiles;
   d.sop = p.sop;
   d.real = p.real;
 }
