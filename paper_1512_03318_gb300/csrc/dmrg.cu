@@ -110,6 +110,12 @@ struct Buf {
     bytes = 0;
     size_t nb = std::max<size_t>(b, 256);
     cudaError_t e = cudaMalloc(&p, nb);
+    if (e == cudaErrorMemoryAllocation) {   // what the library keeps cached may make the room
+      int dev = 0;
+      cudaGetLastError();
+      if (cudaGetDevice(&dev) == cudaSuccess) cache_trim(dev);
+      e = cudaMalloc(&p, nb);
+    }
     if (e == cudaSuccess) bytes = nb;
     return e;
   }
