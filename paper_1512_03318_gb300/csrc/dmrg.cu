@@ -385,8 +385,7 @@ struct mrd_dmrg {
   std::vector<double> schmidt_val;
   Buf schmidt_tab, schmidt_out;
   Buf ff_a, ff_b;   // float-float copies of the operands of a grouped GEMM
-  // digit-split grouped GEMMs: tables, panels, exponents and words of the last one
-  Buf dg_tab, dg_panel[2], dg_expo, dg_partial, dg_redo, dg_words;
+  Buf dg_words;          // of the digit-split grouped GEMMs
   bool dg_ran = false;   // since the last dg_check
   int last_iters = 0, last_refine = 0;
   bool timing = false;
@@ -415,31 +414,36 @@ int run_gemm_digits(mrd_dmrg* D, const GemmList& g, int64_t nt, const double2* A
   const double pass = (double)(p.bytes[0] + p.bytes[1]) * 2.0 / 5.0e12 * 1.9e9 + kSetup;
   if (p.items.empty() || p.cost + pass >= cores) return MRD_OK;
   const size_t tb = dg_table_bytes(p), nx = (size_t)(p.rows[0] + p.rows[1] + dg_state_words(p)) * 4;
-  const size_t need[6] = {dg_device_table_bytes(p), (size_t)p.bytes[0], (size_t)p.bytes[1], nx, (size_t)(p.slots * kDgSlotBytes),
-                          (size_t)p.redo * sizeof(int2)};
-  Buf* bufs[6] = {&D->dg_tab, &D->dg_panel[0], &D->dg_panel[1], &D->dg_expo, &D->dg_partial, &D->dg_redo};
-  for (int k = 0; k < 6; ++k) {
-    const cudaError_t e = bufs[k]->need(need[k]);
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      return MRD_OK;
-    }
-    if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "grouped GEMM: panels");
+  Arena A;   // back to the cache on return: later uses on this stream follow the launches below
+  A.stream = s;
+  uint8_t *tab = nullptr, *panel[2] = {nullptr, nullptr}, *partial = nullptr;
+  int* expo = nullptr;
+  int2* redo = nullptr;
+  cudaError_t e = A.alloc(&tab, dg_device_table_bytes(p));
+  if (e == cudaSuccess) e = A.alloc(&panel[0], (size_t)p.bytes[0]);
+  if (e == cudaSuccess) e = A.alloc(&panel[1], (size_t)p.bytes[1]);
+  if (e == cudaSuccess) e = A.alloc(&expo, nx / 4);
+  if (e == cudaSuccess) e = A.alloc(&partial, (size_t)(p.slots * kDgSlotBytes));
+  if (e == cudaSuccess) e = A.alloc(&redo, (size_t)p.redo);
+  if (e == cudaErrorMemoryAllocation) {   // the CUDA-core kernels need no panels
+    cudaGetLastError();
+    return MRD_OK;
   }
+  if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "grouped GEMM: panels");
   std::vector<uint8_t> host(tb);
   DgDev d;
-  dg_tables(p, host.data(), D->dg_tab.as<uint8_t>(), d);
-  MRD_CUDA(ctx, cudaMemcpyAsync(D->dg_tab.p, host.data(), tb, cudaMemcpyHostToDevice, s));   // pageable: consumed on return
+  dg_tables(p, host.data(), tab, d);
+  MRD_CUDA(ctx, cudaMemcpyAsync(tab, host.data(), tb, cudaMemcpyHostToDevice, s));   // pageable: consumed on return
   MRD_CUDA(ctx, dg_expand(d, s));
   MRD_CUDA(ctx, D->dg_words.need(DG_WORDS * 4));
   int* words = D->dg_words.as<int>();
-  d.panel[0] = D->dg_panel[0].as<uint8_t>();
-  d.panel[1] = D->dg_panel[1].as<uint8_t>();
-  d.partial = D->dg_partial.as<uint8_t>();
-  d.expo[0] = D->dg_expo.as<int>();
+  d.panel[0] = panel[0];
+  d.panel[1] = panel[1];
+  d.partial = partial;
+  d.expo[0] = expo;
   d.expo[1] = d.expo[0] + p.rows[0];
   dg_state(p, d.expo[1] + p.rows[1], d);
-  d.redo = D->dg_redo.as<int2>();
+  d.redo = redo;
   // the error flag (word DG_ERR) stays until dg_check reads it
   if (!D->dg_ran) MRD_CUDA(ctx, cudaMemsetAsync(words, 0, DG_WORDS * 4, s));
   MRD_CUDA(ctx, cudaMemsetAsync(d.expo[0], 0, nx, s));

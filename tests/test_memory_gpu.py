@@ -70,3 +70,19 @@ def test_cached_blocks_make_way_for_a_state(ctx):
         e, _ = d.update(16, +1, P.DMRG.params(800, 0.0, 2, 0.0, 0, 0, 1e-13))
         assert np.isfinite(e)
         d.close()
+
+
+def test_idle_state_keeps_no_panels(ctx):
+    """After an environment update the panels of its products are in the cache, which a program can give back."""
+    import paper_1512_03318_gb300 as P
+    d = _state(ctx, 800)
+    ctx.release_cached()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    size = 16 * d.env_len(16, 0)
+    d.env_update(15, +1, P.MRD_PREC_FF)
+    torch.cuda.synchronize()
+    ctx.release_cached()
+    # what stays: the state's own scratch (T, tables), a few times the environment's size at most
+    assert before - torch.cuda.mem_get_info()[0] <= 4 * size
+    d.close()
