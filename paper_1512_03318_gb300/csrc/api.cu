@@ -500,7 +500,7 @@ static int ensure_per_task(mrd_heff* h) {
 // tables and packed environments, float-float copies of the folded environments. Allocates
 // and may synchronise; a no-op once done (until the environments or the precision change).
 // h->gen counts the (re)allocations, which invalidate captured Lanczos steps.
-static int heff_prepare(mrd_heff* h, int32_t prec) {
+static int heff_prepare_once(mrd_heff* h, int32_t prec) {
   mrd_ctx* ctx = h->ctx;
   cudaStream_t s = ctx->stream;
   if (prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3) return tc_prepare(h, prec);
@@ -545,6 +545,11 @@ static int heff_prepare(mrd_heff* h, int32_t prec) {
     }
   }
   return MRD_OK;
+}
+
+static int heff_prepare(mrd_heff* h, int32_t prec) {
+  const int rc = heff_prepare_once(h, prec);
+  return rc == MRD_E_OOM && dg_release(h) ? heff_prepare_once(h, prec) : rc;
 }
 
 int mrd_heff_apply(mrd_heff* h, const double* theta_in_dev, double* theta_out_dev, int32_t prec) try {
@@ -723,6 +728,10 @@ static int replay_timing_cb(void* op) {
 static int ensure_lanczos(mrd_heff* h) {
   if (h->lz) return MRD_OK;
   cudaError_t e = lanczos_alloc(&h->lz, h->counts[C_THETA], h->ctx->stream);
+  if (e == cudaErrorMemoryAllocation && dg_release(h)) {   // digit panels make way
+    cudaGetLastError();
+    e = lanczos_alloc(&h->lz, h->counts[C_THETA], h->ctx->stream);
+  }
   if (e != cudaSuccess) return mrd_cuda_fail(h->ctx, e, "Lanczos workspace");
   return MRD_OK;
 }
@@ -749,7 +758,13 @@ int mrd_lanczos(mrd_heff* h, double* theta_dev, int32_t max_iter, double tol, in
       if (!ev) MRD_CUDA(ctx, cudaEventCreate(&ev));
   // with tensor-core matvecs (~1e-5 .. 1e-3 relative) the full reorthogonalisation pass runs
   // in FP32; FP64 and float-float runs keep it in FP64
-  MRD_CUDA(ctx, lanczos_set_fp32_full(h->lz, prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3));
+  const bool fp32 = prec == MRD_PREC_TF32 || prec == MRD_PREC_BF16X3;
+  cudaError_t e32 = lanczos_set_fp32_full(h->lz, fp32);
+  if (e32 == cudaErrorMemoryAllocation && dg_release(h)) {   // (these products do not use them)
+    cudaGetLastError();
+    e32 = lanczos_set_fp32_full(h->lz, fp32);
+  }
+  MRD_CUDA(ctx, e32);
   const uint64_t key =
       h->use_graph ? ((uint64_t)h->gen << 8 | (h->timing ? 0x80u : 0u) | (uint64_t)(prec + 1)) : 0;
   struct Run {   // every step's application is prepared

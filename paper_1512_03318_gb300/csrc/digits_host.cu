@@ -369,6 +369,8 @@ struct DgForm {
   int beta = 0;
   bool real = false, major = false;
   bool planned = false, use = false, built = false, env_dirty = true;
+  bool captured = false;   // a caller's graph reads the panels
+  bool no_room = false;    // the panels found no memory since the last environment load
   DgPlan p1, p2;
   DgDev d1, d2;
   int* words = nullptr;   // DG_WORDS, then the exponents of theta and Z and the products' states (zeroed
@@ -537,6 +539,10 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
   }
   *use = g->use;
   if (!g->use) return MRD_OK;
+  if (!g->built && g->no_room) {
+    *use = false;
+    return MRD_OK;
+  }
   if (!g->built) {
     Arena& A = g->mem;
     A.stream = s;
@@ -556,10 +562,12 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
     if (e == cudaSuccess) e = A.alloc(&g->d1.panel[1], (size_t)g->p1.bytes[1]);
     if (e == cudaSuccess) e = A.alloc(&g->d2.panel[0], (size_t)g->p2.bytes[0]);
     if (e == cudaSuccess) e = A.alloc(&g->d2.panel[1], (size_t)g->p2.bytes[1]);
-    if (e == cudaErrorMemoryAllocation) {   // no room for the panels: the CUDA-core kernels need none
+    if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
       A.release();
-      g->use = *use = false;
+      if (dg_release(h)) return dg_prepare(h, prec, use);   // another form's panels made way
+      g->no_room = true;   // the CUDA-core kernels need none
+      *use = false;
       return MRD_OK;
     }
     if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "digit-split products: buffers");
@@ -594,9 +602,27 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
   return MRD_OK;
 }
 
+// Panels of all forms back to the cache (but not those that a caller's graph reads); the next application
+// that needs them builds them again. Whether there were any.
+bool dg_release(mrd_heff* h) {
+  bool any = false;
+  if (h->dg)
+    for (auto& f : h->dg->forms) {
+      if (!f->built || f->captured) continue;
+      f->mem.release();
+      f->built = false;
+      any = true;
+    }
+  if (any) ++h->gen;   // captured Lanczos steps read them
+  return any;
+}
+
 void dg_env_changed(mrd_heff* h) {
   if (h->dg)
-    for (auto& f : h->dg->forms) f->env_dirty = true;
+    for (auto& f : h->dg->forms) {
+      f->env_dirty = true;
+      f->no_room = false;
+    }
 }
 
 // theta_out = H_eff theta_in; ev: timing events (or null) before step 1, between the steps and
@@ -606,6 +632,7 @@ int dg_apply(mrd_heff* h, const double2* in, double2* out, const cudaEvent_t ev[
   cudaStream_t s = ctx->stream;
   DgForm* g = h->dg->cur;
   const int beta = g->beta;
+  if (!h->in_lanczos && stream_capturing(s)) g->captured = true;
   // the error flag outlives a product; the exponents and the products' states do not
   MRD_CUDA(ctx, cudaMemsetAsync(g->words + DG_WORDS, 0, g->zero_bytes - DG_WORDS * 4, s));
   MRD_CUDA(ctx, dg_pack(g->d1, 1, in, beta, g->words, s));

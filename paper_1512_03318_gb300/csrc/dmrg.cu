@@ -1490,6 +1490,7 @@ int mrd_two_site_update(mrd_dmrg* D, int32_t i, int32_t direction, const mrd_dmr
       return rc;
     D->last_refine = it2;
   }
+  dg_release(h);   // no application follows: the panels' memory for the SVD and the environment
   collect(1);
   lap(2);
   // block SVD of theta by middle charge

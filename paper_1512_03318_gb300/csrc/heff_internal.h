@@ -28,6 +28,7 @@ void dg_prebuild(mrd_heff* h, int32_t prec);
 int dg_prepare(mrd_heff* h, int32_t prec, bool* use);
 int dg_apply(mrd_heff* h, const double2* in, double2* out, const cudaEvent_t ev[3], bool cap);
 void dg_env_changed(mrd_heff* h);
+bool dg_release(mrd_heff* h);
 int dg_status(mrd_heff* h);
 using mrd::Lanczos;
 using mrd::lanczos_free;

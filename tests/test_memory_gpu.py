@@ -54,6 +54,30 @@ def _state(ctx, chi):
     return P.DMRG(ctx, mpo, 16, 0, chi, seed=5, center=16, caps=caps)
 
 
+def test_panels_make_way_for_lanczos(ctx):
+    """FP64 applications hold panels of hundreds of MB; the Lanczos basis (65 MB here) that then finds no
+    memory gets theirs, and the applications go on."""
+    import paper_1512_03318_gb300 as P
+    case = _one_block_case(97, 160, 160, 40)
+    ref = _oracle(case)
+    h = P.Heff(ctx, **G.heff_args(case))
+    h.set_env(_dev(case["lflat"]), _dev(case["rflat"]))
+    T = _dev(case["tflat"])
+    out, v = torch.empty_like(T), T.clone()
+    ok = lambda: np.max(np.abs(out.cpu().numpy() - ref)) <= TOL[0] * np.max(np.abs(ref))
+    h.apply(T, out, 0)
+    assert ok()
+    with Hog(24 * MB):
+        e, steps = h.lanczos(v, 3, 0.0, 0)
+        assert steps == 3 and np.isfinite(e)
+        h.apply(T, out, 0)
+        assert ok()
+    h.set_env(_dev(case["lflat"]), _dev(case["rflat"]))
+    h.apply(T, out, 0)
+    assert ok()
+    h.close()
+
+
 def test_cached_blocks_make_way_for_a_state(ctx):
     """Blocks of a freed H_eff are cached; a DMRG state whose own buffers find no memory gets theirs."""
     import paper_1512_03318_gb300 as P
