@@ -117,6 +117,7 @@ struct Buf {
       e = cudaMalloc(&p, nb);
     }
     if (e == cudaSuccess) bytes = nb;
+    else cudaGetLastError();   // returned, so that the next launch's check does not see it
     return e;
   }
   template <class T>

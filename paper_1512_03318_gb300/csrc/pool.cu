@@ -73,7 +73,10 @@ cudaError_t cache_alloc(void** out, size_t bytes, cudaStream_t s) {
     trim_locked(c, dev);
     e = cudaMalloc(&p, want);
   }
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) {
+    cudaGetLastError();   // returned, so that the next launch's check does not see it
+    return e;
+  }
   c.live[p] = {want, dev};
   *out = p;
   return cudaSuccess;

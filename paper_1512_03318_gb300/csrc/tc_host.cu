@@ -478,7 +478,11 @@ int upload(mrd_heff* h, const TcTables& o) {
   TALLOC(T->j_lw, o.j_lw.size()); TALLOC(T->j_wr, o.j_wr.size()); TALLOC(T->j_th, o.j_th.size());
   TALLOC(T->words, 4);
 #undef TALLOC
-  if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "tc: device buffers");
+  if (e != cudaSuccess) {   // nothing half-built stays: the next application builds anew
+    delete h->tc;
+    h->tc = nullptr;
+    return mrd_cuda_fail(ctx, e, "tc: device buffers");
+  }
   T->n_it1 = (int)o.i1.size(); T->n_it2 = (int)o.i2.size();
   T->n_alt2 = (int)o.ia.size();
   T->task1 = o.task1; T->task2 = o.task2; T->taska = o.taska;
@@ -502,7 +506,11 @@ int upload(mrd_heff* h, const TcTables& o) {
   if (e == cudaSuccess && o.zero_z && T->z) e = cudaMemsetAsync(T->z, 0, (size_t)o.z_b, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(T->words, 0, 16, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host tables may be released after this
-  if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "tc: upload");
+  if (e != cudaSuccess) {
+    delete h->tc;
+    h->tc = nullptr;
+    return mrd_cuda_fail(ctx, e, "tc: upload");
+  }
   return MRD_OK;
 }
 
@@ -690,7 +698,7 @@ void tc_env_changed(mrd_heff* h) {
 }
 
 int tc_status(mrd_heff* h) {
-  if (!h->tc) return MRD_OK;
+  if (!h->tc || !h->tc->words) return MRD_OK;
   int herr = 0;
   MRD_CUDA(h->ctx, cudaMemcpyAsync(&herr, h->tc->err(), 4, cudaMemcpyDeviceToHost, h->ctx->stream));
   MRD_CUDA(h->ctx, cudaStreamSynchronize(h->ctx->stream));

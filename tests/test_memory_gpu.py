@@ -110,3 +110,25 @@ def test_idle_state_keeps_no_panels(ctx):
     # what stays: the state's own scratch (T, tables), a few times the environment's size at most
     assert before - torch.cuda.mem_get_info()[0] <= 4 * size
     d.close()
+
+
+@pytest.mark.parametrize("prec,tol", [(2, 1e-4), (3, TOL[3])])
+def test_application_after_one_that_found_no_memory(ctx, prec, tol):
+    """Split BF16 operands that find no memory: the application is refused, and the next one, with room, is
+    right (half-built tables are not taken for built). Float-float ones alike, whichever kernels run."""
+    import paper_1512_03318_gb300 as P
+    case = _one_block_case(103, 160, 160, 40)
+    ref = _oracle(case)
+    h = P.Heff(ctx, **G.heff_args(case))
+    h.set_env(_dev(case["lflat"]), _dev(case["rflat"]))
+    T = _dev(case["tflat"])
+    out = torch.empty_like(T)
+    with Hog(10 * MB):
+        with pytest.raises(P.MrdError) as ex:
+            h.apply(T, out, prec)
+        assert ex.value.code == -4
+        h.status()
+    h.apply(T, out, prec)
+    h.status()
+    assert np.max(np.abs(out.cpu().numpy() - ref)) <= tol * np.max(np.abs(ref))
+    h.close()
