@@ -915,14 +915,14 @@ cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2*
 }
 
 cudaError_t dg_init() {
-  static cudaError_t e = [] {
+  static DeviceOnce once;
+  return once.run([] {
     cudaError_t r = cudaSuccess;
     for (const void* f : {(const void*)k_dg_gemm<7, false>, (const void*)k_dg_gemm<7, true>,
                           (const void*)k_dg_gemm<8, false>, (const void*)k_dg_gemm<8, true>})
       if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kDgSmem);
     return r;
-  }();
-  return e;
+  });
 }
 
 cudaError_t dg_expand(const DgDev& d, cudaStream_t s) {

@@ -648,16 +648,14 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm(TcArgs g) {
 
 // Kernel attributes (dynamic shared memory above 48 KB); called before any capture.
 cudaError_t tc_gemm_init() {
-  static bool attr_set = false;
-  if (!attr_set) {
+  static DeviceOnce once;
+  return once.run([] {
+    cudaError_t e = cudaSuccess;
     for (const void* f : {(const void*)k_tc_gemm<TC_TF32>, (const void*)k_tc_gemm<TC_BF16X3>,
-                          (const void*)k_tc_gemm<TC_TF32_REAL>, (const void*)k_tc_gemm<TC_BF16X3_REAL>}) {
-      cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
-      if (e != cudaSuccess) return e;
-    }
-    attr_set = true;
-  }
-  return cudaSuccess;
+                          (const void*)k_tc_gemm<TC_TF32_REAL>, (const void*)k_tc_gemm<TC_BF16X3_REAL>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
+    return e;
+  });
 }
 
 cudaError_t tc_pack(const double2* src, uint8_t* dst, const int64_t* jobs, int njobs, int64_t npieces, int prec, int* ctr,

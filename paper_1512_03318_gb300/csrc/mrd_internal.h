@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <array>
+#include <atomic>
 #include <map>
 #include <string>
 #include <vector>
@@ -42,6 +43,25 @@ void cache_free(void* p, cudaStream_t s);
 void cache_trim(int device);
 cudaError_t cache_alloc_host(void** out, size_t bytes);   // pinned host memory, reused by size
 void cache_free_host(void* p);
+
+// Runs `set` once on every device of the process (kernel attributes belong to a device; up to 64 devices,
+// further ones every time); safe with several threads.
+class DeviceOnce {
+  std::atomic<uint64_t> done_{0};
+
+ public:
+  template <class F>
+  cudaError_t run(F set) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done_.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = set();
+    if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
 
 // A device buffer owned by the library.
 struct DevBuf {

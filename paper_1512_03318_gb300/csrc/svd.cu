@@ -890,13 +890,11 @@ static cudaError_t launch_bround(T2* work, const int64_t* blk, int xf, int vf, c
                                  unsigned long long* wctr, const int* prev_rotated, cudaStream_t s) {
   if (ncta == 0) return cudaSuccess;
   if (W < 2 || W > 16 || (W & 1)) return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_svd_bround<MODE, REAL, T, T2, T2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSvdMaxSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t ea = once.run([] {
+    return cudaFuncSetAttribute(k_svd_bround<MODE, REAL, T, T2, T2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdMaxSmem);
+  });
+  if (ea != cudaSuccess) return ea;
   // programmatic dependent launch: the round's CTAs are scheduled while the previous round
   // writes back, and wait (griddepcontrol.wait) before reading anything it wrote
   cudaLaunchConfig_t lc = {};
