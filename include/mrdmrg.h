@@ -329,6 +329,11 @@ int mrd_env_update(mrd_dmrg* d, int32_t site, int32_t direction, int32_t prec);
  *                           Columns are set aside before the final sweeps (mrd_dmrg_svd_stats)
  *                           only after at least 8 pre-sweeps or converged ones. */
 #define MRD_DMRG_OPT_SVD_PRESWEEPS 3
+/*   MRD_DMRG_OPT_WAIT_LIMIT_US  as MRD_OPT_WAIT_LIMIT_US, for the updates and environment updates
+ *                           that follow: their H_effs and the environments' own products. A wait
+ *                           that gives up ends the call with MRD_E_TIMEOUT; the environment that
+ *                           it was building is not usable, everything else is.               */
+#define MRD_DMRG_OPT_WAIT_LIMIT_US 4
 int mrd_dmrg_set_option(mrd_dmrg* d, int32_t option, int64_t value);
 /* Device memory of a DMRG state: out4 = {bytes of the stored environments, environments
  * built, bytes of the MPS tensors, 1 if environments are stored in complex64}. */

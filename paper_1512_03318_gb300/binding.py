@@ -30,6 +30,7 @@ MRD_SVD_F64 = 3
 MRD_DMRG_OPT_ENV_FP32 = 1
 MRD_DMRG_OPT_REAL = 2
 MRD_DMRG_OPT_SVD_PRESWEEPS = 3
+MRD_DMRG_OPT_WAIT_LIMIT_US = 4
 
 _LIB = None
 _LIVE = []        # weak references to open handles, closed in creation-reverse order at exit
@@ -340,7 +341,8 @@ class DMRG:
         return e.value
 
     def set_option(self, option, value):
-        """mrd_dmrg_set_option (MRD_DMRG_OPT_ENV_FP32, MRD_DMRG_OPT_REAL, MRD_DMRG_OPT_SVD_PRESWEEPS)."""
+        """mrd_dmrg_set_option (MRD_DMRG_OPT_ENV_FP32, MRD_DMRG_OPT_REAL, MRD_DMRG_OPT_SVD_PRESWEEPS,
+        MRD_DMRG_OPT_WAIT_LIMIT_US)."""
         self.ctx.check(lib().mrd_dmrg_set_option(self.h, option, int(value)))
 
     def memory(self):

@@ -388,6 +388,7 @@ struct mrd_dmrg {
   Buf ff_a, ff_b;   // float-float copies of the operands of a grouped GEMM
   Buf dg_words;          // of the digit-split grouped GEMMs
   bool dg_ran = false;   // since the last dg_check
+  uint64_t wait_ns = 1000000000ull;   // limit of each device-side wait (MRD_DMRG_OPT_WAIT_LIMIT_US)
   int last_iters = 0, last_refine = 0;
   bool timing = false;
   double kms[4] = {0, 0, 0, 0};   // accumulated GEMM ms: tensor-core step 1, step 2, FP64 step 1, step 2
@@ -451,7 +452,7 @@ int run_gemm_digits(mrd_dmrg* D, const GemmList& g, int64_t nt, const double2* A
   D->dg_ran = true;
   MRD_CUDA(ctx, dg_pack(d, 0, Aop, beta, words, s));
   MRD_CUDA(ctx, dg_pack(d, 1, Bop, beta, words, s));
-  MRD_CUDA(ctx, dg_gemm(d, C, beta, words, D->n_sm, 1000000000ull, s));
+  MRD_CUDA(ctx, dg_gemm(d, C, beta, words, D->n_sm, D->wait_ns, s));
   MRD_CUDA(ctx, dg_redo(d, Aop, Bop, C, beta, words, D->n_sm, s));
   *done = true;
   return MRD_OK;
@@ -631,6 +632,7 @@ int make_heff(mrd_dmrg* D, int i, const double2* lenv, const double2* renv, mrd_
   int rc = mrd_heff_create(D->ctx, &d, out);
   if (rc != MRD_OK) return rc;
   mrd_heff* h = *out;
+  h->wait_ns = D->wait_ns;
   rc = heff_fold(h, lenv, renv);   // an absent environment is not folded (nothing reads that side)
   if (rc != MRD_OK) { mrd_heff_free(h); *out = nullptr; }
   return rc;
@@ -1427,6 +1429,7 @@ int mrd_two_site_update(mrd_dmrg* D, int32_t i, int32_t direction, const mrd_dmr
   if (p->prec < MRD_PREC_FP64 || p->prec > MRD_PREC_FF)
     return mrd_fail(ctx, MRD_E_ARG, "mrd_two_site_update: unknown prec");
   D->gemm_ff = p->refine_prec == MRD_PREC_FF;
+  D->dg_ran = false;   // whatever a call that failed half-way has left
   if (!D->L[i].data.p || !D->R[i + 2].data.p)
     return mrd_fail(ctx, MRD_E_STATE, "mrd_two_site_update: environments of this bond are not available");
   Guard g(ctx->device);
@@ -1645,6 +1648,7 @@ int mrd_env_update(mrd_dmrg* D, int32_t site, int32_t direction, int32_t prec) t
   if (!src.data.p) return mrd_fail(ctx, MRD_E_STATE, "mrd_env_update: the input environment is not built");
   Guard g(ctx->device);
   D->gemm_ff = prec == MRD_PREC_FF;
+  D->dg_ran = false;   // whatever a call that failed half-way has left
   mrd_heff* h = nullptr;
   const int i = direction > 0 ? site : site - 1;
   const double2* ein = nullptr;
@@ -1732,6 +1736,11 @@ int mrd_dmrg_set_option(mrd_dmrg* D, int32_t option, int64_t value) try {
   if (option == MRD_DMRG_OPT_SVD_PRESWEEPS) {
     if (value < 0 || value > 64) return mrd_fail(ctx, MRD_E_ARG, "mrd_dmrg_set_option: pre-sweeps outside 0 .. 64");
     D->svd_presweeps = (int)value;
+    return MRD_OK;
+  }
+  if (option == MRD_DMRG_OPT_WAIT_LIMIT_US) {
+    if (value < 0 || value > 60000000) return mrd_fail(ctx, MRD_E_ARG, "mrd_dmrg_set_option: wait limit outside 0 .. 60 s");
+    D->wait_ns = (uint64_t)value * 1000ull;
     return MRD_OK;
   }
   if (option != MRD_DMRG_OPT_ENV_FP32) return mrd_fail(ctx, MRD_E_ARG, "mrd_dmrg_set_option: unknown option");

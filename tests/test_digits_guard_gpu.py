@@ -160,3 +160,28 @@ def test_graded_along_k(ctx, prec, decades):
                 e = np.abs(view(got) - view(ref))[ro:ro + da, co:co + db]
                 assert np.max(e) <= tol * np.max(view(bound)[ro:ro + da, co:co + db])
     h.close()
+
+
+@pytest.mark.parametrize("prec", [0, 3])
+def test_environment_wait_limit(ctx, prec):
+    """With no time to wait, an environment update's products give up before any copy or MMA and the call says
+    so, every time; with time, the next one is right."""
+    import paper_1512_03318_gb300 as P
+    ly, chi, lx = 8, 800, 4
+    mpo = P.MPO(None, lx, ly, 1, ly, 1.0, 1.0, P.MRD_BASIS_MIXED)
+    n, j = lx * ly, 15
+    caps = [[(q[0], q[1], m) for q, m in synth.bond_sectors(chi, ly, round(b / 2), synth.substream(97, 7, b), min_dim=1)]
+            if 2 <= b <= n - 2 else [] for b in range(n + 1)]
+    d = P.DMRG(ctx, mpo, n // 2, 0, chi, seed=3, center=16, caps=caps)
+    good = d.env(j + 1, 0)
+    d.set_option(P.MRD_DMRG_OPT_WAIT_LIMIT_US, 0)
+    for _ in range(2):
+        with pytest.raises(P.MrdError) as ex:
+            d.env_update(j, +1, prec)
+        assert ex.value.code == -7
+    with pytest.raises(P.MrdError):
+        d.set_option(P.MRD_DMRG_OPT_WAIT_LIMIT_US, -1)
+    d.set_option(P.MRD_DMRG_OPT_WAIT_LIMIT_US, 1000000)
+    d.env_update(j, +1, prec)
+    assert np.max(np.abs(d.env(j + 1, 0) - good)) <= TOL[prec] * np.max(np.abs(good))
+    d.close()
