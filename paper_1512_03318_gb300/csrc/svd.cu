@@ -20,6 +20,7 @@
 #include <cmath>
 
 #include "ff.cuh"
+#include "fp64_scalar.cuh"
 #include "mrd_internal.h"
 
 namespace mrd {
@@ -82,12 +83,12 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;"
 // is a numerical zero (rank deficiency): it is neither rotated nor counted as unconverged.
 // REAL: the columns are real (imaginary parts zero, the real-arithmetic mode): only the real
 // parts enter the dot products and the rotation, whose phase is a sign.
-template <class T, class T2, bool REAL>
-__device__ __forceinline__ bool jacobi_pair(T2* xi, T2* xj, int p, T2* vi, T2* vj, int r, T tol, double floor2,
+template <bool REAL>
+__device__ __forceinline__ bool jacobi_pair(float2* xi, float2* xj, int p, float2* vi, float2* vj, int r, float tol, double floor2,
                                             int lane) {
-  T a = 0, bb = 0, gr = 0, gi = 0;
+  float a = 0, bb = 0, gr = 0, gi = 0;
   for (int t = lane; t < p; t += 32) {
-    const T2 u = xi[t], v = xj[t];
+    const float2 u = xi[t], v = xj[t];
     if (REAL) {
       a = fma(u.x, u.x, a);
       bb = fma(v.x, v.x, bb);
@@ -106,39 +107,27 @@ __device__ __forceinline__ bool jacobi_pair(T2* xi, T2* xj, int p, T2* vi, T2* v
     gr += __shfl_xor_sync(0xffffffffu, gr, o);
     if (!REAL) gi += __shfl_xor_sync(0xffffffffu, gi, o);
   }
-  const T g = REAL ? fabs(gr) : sqrt(gr * gr + gi * gi);
+  const float g = REAL ? fabsf(gr) : sqrtf(gr * gr + gi * gi);
   if ((double)a <= floor2 || (double)bb <= floor2) return false;
-  if (!(g > tol * sqrt(a * bb))) return false;
+  if (!(g > tol * sqrtf(a * bb))) return false;
   // phase-free real rotation on (x_i, e^{-i phi} x_j), phi = arg(gamma)
-  T ph_r, ph_i, c, sn;
-  if constexpr (sizeof(T) == 4) {   // FP32 pre-sweeps: fast reciprocal and rsqrt (a few ulp)
-    const float ig = 1.f / g;
-    ph_r = gr * ig;
-    ph_i = -gi * ig;
-    const float zeta = 0.5f * (bb - a) * ig, q = 1.f + zeta * zeta;
-    // very different norms: t = 1 / (2 zeta), as zeta^2 would overflow
-    const float t = fabsf(zeta) > 1e4f ? __fdividef(0.5f, zeta)
-                                       : __fdividef(zeta >= 0.f ? 1.f : -1.f, fabsf(zeta) + q * rsqrtf(q));
-    c = rsqrtf(1.f + t * t);
-    sn = c * t;
-  } else {
-    ph_r = gr / g;
-    ph_i = -gi / g;                               // e^{-i phi}
-    const T zeta = (bb - a) / (T(2) * g);
-    const T t = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
-    c = T(1) / sqrt(T(1) + t * t);
-    sn = c * t;
-  }
-  auto rot = [&](T2* ci, T2* cj, int n) {
+  const float ig = 1.f / g;   // fast reciprocal and rsqrt below (a few ulp)
+  const float ph_r = gr * ig, ph_i = -gi * ig;
+  const float zeta = 0.5f * (bb - a) * ig, q = 1.f + zeta * zeta;
+  // very different norms: t = 1 / (2 zeta), as zeta^2 would overflow
+  const float t = fabsf(zeta) > 1e4f ? __fdividef(0.5f, zeta)
+                                     : __fdividef(zeta >= 0.f ? 1.f : -1.f, fabsf(zeta) + q * rsqrtf(q));
+  const float c = rsqrtf(1.f + t * t), sn = c * t;
+  auto rot = [&](float2* ci, float2* cj, int n) {
     for (int k = lane; k < n; k += 32) {
-      const T2 u = ci[k], v0 = cj[k];
-      T2 o1, o2;
+      const float2 u = ci[k], v0 = cj[k];
+      float2 o1, o2;
       if (REAL) {
-        const T vx = v0.x * ph_r;
-        o1.x = c * u.x - sn * vx; o1.y = T(0);
-        o2.x = sn * u.x + c * vx; o2.y = T(0);
+        const float vx = v0.x * ph_r;
+        o1.x = c * u.x - sn * vx; o1.y = 0.f;
+        o2.x = sn * u.x + c * vx; o2.y = 0.f;
       } else {
-        T2 v;
+        float2 v;
         v.x = v0.x * ph_r - v0.y * ph_i;
         v.y = v0.x * ph_i + v0.y * ph_r;
         o1.x = c * u.x - sn * v.x; o1.y = c * u.y - sn * v.y;
@@ -153,39 +142,11 @@ __device__ __forceinline__ bool jacobi_pair(T2* xi, T2* xj, int p, T2* vi, T2* v
   return true;
 }
 
-// FP64 version of jacobi_pair, with the columns' squared norms na, nb kept by the caller. An FP64
-// warp instruction occupies its quarter of an SM for 64 cycles whatever its lanes do (measured; a
-// division is 23 of them, a square root 13), and the first form spent more of them on the scalars of a
-// pair (3 divisions, 4 square roots, 20 shuffle additions: ~140) than on its elements (at p = 128, 80).
-// So square roots come from an FP32 seed and one third-order step, tests compare bits or squares,
-// the two sums share one shuffle tree, and the norms follow from the rotation: ~35 instructions. One sweep
-// at Ly = 6, chi = 512: 0.96 -> 0.57 ms, the update 18.5 -> 12.5.
-__device__ __forceinline__ bool bits_less_equal(double a, double b) {   // of non-negative numbers
-  return __double_as_longlong(a) <= __double_as_longlong(b);
-}
-
-// A float close to |x| (truncated mantissa; |x| within the FP32 exponent range), and a double from a normal
-// float, without the FP64 pipe.
-__device__ __forceinline__ float mag_f32(double x) {
-  const int hi = __double2hiint(x) & 0x7fffffff;
-  return __int_as_float(((hi >> 20) - 1023 + 127) << 23 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
-}
-__device__ __forceinline__ double from_f32(float x) {
-  const int i = __float_as_int(x);
-  return __hiloint2double((i & 0x80000000) | (((i >> 3) & 0x0fffffff) + ((1023 - 127) << 20)), i << 29);
-}
-
-// 1 / sqrt(x), x > 0 normal, to ~1 ulp: an FP32 seed y (error e = 1 - x y^2 ~ 2^-21) and y (1 + e / 2 + 3 e^2 / 8).
-__device__ __forceinline__ double rsqrt_fp64(double x) {
-  const int hi = __double2hiint(x);
-  const int k = ((hi >> 20) - 1023) & ~1;                                    // x = m 2^k, m in [1, 4)
-  const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
-  const double y = from_f32(rsqrtf(mag_f32(m)));
-  const double e = fma(-(m * y), y, 1.0);
-  const double r = fma(y * e, fma(0.375, e, 0.5), y);
-  return __hiloint2double(__double2hiint(r) - ((k / 2) << 20), __double2loint(r));
-}
-
+// FP64 version of jacobi_pair, with the columns' squared norms na, nb kept by the caller. The first form spent
+// more FP64 instructions on the scalars of a pair (3 divisions, 4 square roots, 20 shuffle additions: ~140)
+// than on its elements (at p = 128, 80). So square roots come from an FP32 seed (fp64_scalar.cuh), tests
+// compare bits or squares, the two sums share one shuffle tree, and the norms follow from the rotation: ~40
+// instructions. One sweep at Ly = 6, chi = 512: 0.96 -> 0.57 ms, the update 18.5 -> 12.5.
 template <bool REAL>
 __device__ __forceinline__ double norm2_fp64(const double2* x, int p, int lane) {
   double s = 0.0;
@@ -228,18 +189,8 @@ __device__ __forceinline__ bool jacobi_pair_fp64(double2* xi, double2* xj, int p
   const double ig = rsqrt_fp64(g2);
   const double ph_r = gr * ig, ph_i = -gi * ig;
   const double zeta = (b - a) * (0.5 * ig);
-  double tt;
-  {   // t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)): in FP32, then one Newton step for t^2 + 2 zeta t = 1
-    const int ex = ((__double2hiint(zeta) >> 20) & 0x7ff) - 1023;
-    const bool neg = __double2hiint(zeta) < 0;
-    if (ex > 120) return false;                   // no representable rotation
-    const float z = ex < -60 ? 0.f : mag_f32(zeta);
-    const float t0 = z > 1e9f ? 0.5f / z : 1.f / (z + sqrtf(1.f + z * z));
-    const float r0 = 0.5f / (t0 + z);             // 1 / f'
-    const double t1 = from_f32(t0), zz = neg ? -zeta : zeta;
-    tt = fma(-fma(t1, fma(2.0, zz, t1), -1.0), from_f32(r0), t1);
-    tt = neg ? -tt : tt;
-  }
+  if ((__double2hiint(zeta) & 0x7fffffff) >= (1023 + 120) << 20) return false;   // no representable rotation
+  const double tt = jacobi_tangent(zeta);
   const double c = rsqrt_fp64(fma(tt, tt, 1.0)), sn = c * tt;
   for (int k = lane; k < p; k += 32) {
     const double2 u = xi[k], v0 = xj[k];
@@ -534,7 +485,7 @@ __global__ void __launch_bounds__(512) k_svd_bround(T2* __restrict__ work, const
         s_norm2[j] = nb;
       }
     } else {
-      rot = jacobi_pair<T, T2, REAL>(sx + (int64_t)i * p, sx + (int64_t)j * p, p, V ? sv + (int64_t)i * r : nullptr,
+      rot = jacobi_pair<REAL>(sx + (int64_t)i * p, sx + (int64_t)j * p, p, V ? sv + (int64_t)i * r : nullptr,
                                V ? sv + (int64_t)j * r : nullptr, r, tol, floor2, lane);
     }
     my_tested += p;
