@@ -147,8 +147,10 @@ __device__ __forceinline__ bool jacobi_pair(float2* xi, float2* xj, int p, float
 // than on its elements (at p = 128, 80). So square roots come from an FP32 seed (fp64_scalar.cuh), tests
 // compare bits or squares, the two sums share one shuffle tree, and the norms follow from the rotation: ~40
 // instructions. One sweep at Ly = 6, chi = 512: 0.96 -> 0.57 ms, the update 18.5 -> 12.5.
+// Norms, floor2 and the sums are in units of the block's squared norm (2^-sc of it, an exact scale), so
+// that squares and products of them stay in range whatever the block's size.
 template <bool REAL>
-__device__ __forceinline__ double norm2_fp64(const double2* x, int p, int lane) {
+__device__ __forceinline__ double norm2_fp64(const double2* x, int p, int sc, int lane) {
   double s = 0.0;
   for (int t = lane; t < p; t += 32) {
     const double2 u = x[t];
@@ -156,11 +158,11 @@ __device__ __forceinline__ double norm2_fp64(const double2* x, int p, int lane) 
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
+  return scale2(s, sc);
 }
 
 template <bool REAL>
-__device__ __forceinline__ bool jacobi_pair_fp64(double2* xi, double2* xj, int p, double tol2, double floor2, double& na,
+__device__ __forceinline__ bool jacobi_pair_fp64(double2* xi, double2* xj, int p, double tol2, double floor2, int sc, double& na,
                                                  double& nb, int lane) {
   const double a = na, b = nb;
   if (bits_less_equal(a, floor2) || bits_less_equal(b, floor2)) return false;
@@ -179,6 +181,7 @@ __device__ __forceinline__ bool jacobi_pair_fp64(double2* xi, double2* xj, int p
     double s = REAL ? gr + __shfl_xor_sync(0xffffffffu, gr, 16) : (up ? gi : gr) + __shfl_xor_sync(0xffffffffu, up ? gr : gi, 16);
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    s = scale2(s, sc);
     gr = __shfl_sync(0xffffffffu, s, 0);
     gi = REAL ? 0.0 : __shfl_sync(0xffffffffu, s, 16);
   }
@@ -209,8 +212,8 @@ __device__ __forceinline__ bool jacobi_pair_fp64(double2* xi, double2* xj, int p
   na = a - tg;
   nb = b + tg;
   __syncwarp();
-  if (!bits_less_equal(0.125 * a, na) || __double2hiint(na) < 0) na = norm2_fp64<REAL>(xi, p, lane);
-  if (!bits_less_equal(0.125 * b, nb) || __double2hiint(nb) < 0) nb = norm2_fp64<REAL>(xj, p, lane);
+  if (!bits_less_equal(0.125 * a, na) || __double2hiint(na) < 0) na = norm2_fp64<REAL>(xi, p, sc, lane);
+  if (!bits_less_equal(0.125 * b, nb) || __double2hiint(nb) < 0) nb = norm2_fp64<REAL>(xj, p, sc, lane);
   return true;
 }
 
@@ -454,15 +457,16 @@ __global__ void __launch_bounds__(512) k_svd_bround(T2* __restrict__ work, const
     }
     __syncthreads();
   }
+  const int sc = MODE == 1 ? 1023 - ((__double2hiint(fro2[b]) >> 20) & 0x7ff) : 0;   // (MODE 1) units of norms: 2^-sc
   if constexpr (MODE == 1) {
     for (int cc = warp; cc < nI + nJ; cc += nwarp) {
       const int lc = cc < nI ? cc : W + cc - nI;
-      const double s = norm2_fp64<REAL>((const double2*)sx + (int64_t)lc * p, p, lane);
+      const double s = norm2_fp64<REAL>((const double2*)sx + (int64_t)lc * p, p, sc, lane);
       if (lane == 0) s_norm2[lc] = s;
     }
     __syncthreads();
   }
-  const double floor2 = zero_rel * fro2[b];
+  const double floor2 = MODE == 1 ? scale2(zero_rel * fro2[b], sc) : zero_rel * fro2[b];
   // A pair found orthogonal in the previous sweep stays orthogonal while neither column
   // rotates: pairs whose columns last rotated before the previous sweep are skipped (the
   // first two sweeps test every pair, last_rot starting at 0).
@@ -479,7 +483,7 @@ __global__ void __launch_bounds__(512) k_svd_bround(T2* __restrict__ work, const
       }
     } else if constexpr (MODE == 1) {
       double na = s_norm2[i], nb = s_norm2[j];
-      rot = jacobi_pair_fp64<REAL>(sx + (int64_t)i * p, sx + (int64_t)j * p, p, (double)tol * (double)tol, floor2, na, nb, lane);
+      rot = jacobi_pair_fp64<REAL>(sx + (int64_t)i * p, sx + (int64_t)j * p, p, (double)tol * (double)tol, floor2, sc, na, nb, lane);
       if (rot && lane == 0) {
         s_norm2[i] = na;
         s_norm2[j] = nb;

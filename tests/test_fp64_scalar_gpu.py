@@ -1,6 +1,8 @@
 """FP64 scalars of the Jacobi rotations (csrc/fp64_scalar.cuh) by themselves, against extended precision:
 the reciprocal square root to 2 ulp, next to CUDA's rsqrt, and the tangent of the rotation to 4 ulp (a last
-correction that is itself rounded, of a value whose residual is rounded against 1), over their ranges."""
+correction that is itself rounded, of a value whose residual is rounded against 1), over their ranges.
+
+And the SVD of a charge block far below the others: its singular vectors are as orthogonal as theirs."""
 import ctypes
 import os
 import subprocess
@@ -71,3 +73,39 @@ def test_tangent(lib):
     ref = 1.0 / (z + np.sqrt(1.0 + z * z))
     ref = np.where(np.signbit(x), -ref, ref)
     assert np.max(np.abs(t - ref) / np.spacing(np.abs(ref).astype(np.float64))) <= 4.0
+
+
+@pytest.mark.parametrize("power", [0, -60, -245, -400])
+def test_small_block_is_an_isometry(power):
+    """One middle sector of the two-site tensor scaled by 2^power (a single Lanczos step leaves the tensor as it
+    is): every kept singular vector, of that block too, is orthonormal to 1e-12 as elsewhere."""
+    import paper_1512_03318_gb300 as P
+    import synth
+    from tests.test_dmrg_gpu import _isometry_error
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ctx = P.Context(0, torch.cuda.current_stream())
+    lx, ly, chi = 6, 4, 130
+    n_sites = lx * ly
+    caps = [[(q[0], q[1], d) for q, d in synth.bond_sectors(chi, ly, round(j / ly), synth.substream(97, 7, j), min_dim=1)]
+            if 2 <= j <= n_sites - 2 else [] for j in range(n_sites + 1)]
+    i = (lx // 2) * ly + ly // 2 - 1
+    mpo = P.MPO(None, lx, ly, 1, 4, 1.0, 1.0, P.MRD_BASIS_MIXED)
+    d = P.DMRG(ctx, mpo, lx, 0, 100000, seed=5, center=i, caps=caps)
+    # tensor i + 1 is grouped by its left (the middle) sector: scale the largest group
+    mode, t = d.site(i + 1)
+    assert mode == 1
+    left, right = d.bond(i + 1), {(int(a), int(b)): int(c) for a, b, c in d.bond(i + 2)}
+    m2 = (i + 1) % ly
+    cols = [sum(right.get((int(n) + s, (int(k) + s * m2) % ly), 0) for s in (0, 1)) for n, k, _ in left]
+    size = [int(dim) * c for (_, _, dim), c in zip(left, cols)]
+    g = int(np.argmax(size))
+    x = t.copy()
+    x[sum(size[:g]):sum(size[:g + 1])] *= 2.0 ** power
+    host = np.ascontiguousarray(x)
+    d.set_site(i + 1, host.ctypes.data)
+    p = P.DMRG.params(100000, 0.0, 1, 0.0, P.MRD_PREC_FP64, 0, 1e-13, svd_mode=3)
+    e, _ = d.update(i, +1, p)
+    assert np.isfinite(e)
+    assert _isometry_error(d.site(i)[1], d.bond(i), d.bond(i + 1), i % ly, ly) < 1e-12
+    d.close()
