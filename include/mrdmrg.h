@@ -183,7 +183,8 @@ int mrd_heff_timing(mrd_heff* h, int32_t on);
  *                           replays it; 0: launches every kernel of every step.
  *   MRD_OPT_PER_TASK_LAUNCH 0 (default): each GEMM step of mrd_heff_apply is one grouped
  *                           persistent launch over all charge blocks; 1: one launch per task
- *                           (output block), the per-block baseline the grouped launch replaces.
+ *                           (output block; in digit products and split BF16 / TF32 one per stack
+ *                           of output blocks), the baseline the grouped launch replaces.
  *   MRD_OPT_AUTOTUNE        1 (default): the first tensor-core application of a problem
  *                           class (precision, size of theta, number of tasks) times every
  *                           candidate tile configuration (columns per tile, pipeline stages,
@@ -206,10 +207,16 @@ int mrd_heff_timing(mrd_heff* h, int32_t on);
  *                           be real, e.g. from MRD_BASIS_MIXED_REAL; environments; theta):
  *                           the tensor-core precisions drop the imaginary planes (TF32: one
  *                           MMA per K step instead of two, split BF16: two of half the width
- *                           instead of four) and write zero imaginary parts. The float-float and
- *                           FP64 paths are unchanged (their results are real for real inputs).
+ *                           instead of four) and write zero imaginary parts; so do the
+ *                           float-float products (real products only). The FP64 path is
+ *                           unchanged (its results are real for real inputs).
  *                           This is the real arithmetic the paper runs (Sec. IV.D, Eq. rot). */
 #define MRD_OPT_REAL 5
+/*   MRD_OPT_DIGITS          which arithmetic MRD_PREC_FP64 and MRD_PREC_FF applications take. 1 (default):
+ *                           fixed-point digit products on the tensor cores where they are cheaper,
+ *                           0: always FP64 / float-float arithmetic on the CUDA cores, 2: always digit
+ *                           products (while their panels find memory). MRD_E_ARG otherwise. */
+#define MRD_OPT_DIGITS 6
 int mrd_heff_set_option(mrd_heff* h, int32_t option, int64_t value);
 /* Wait for the context stream and report a device-side wait of a tensor-core GEMM that gave
  * up since the last check: MRD_E_TIMEOUT (the flag is then cleared), else 0. */
@@ -218,6 +225,10 @@ int mrd_heff_status(mrd_heff* h);
  * depth in tiles of 128 bytes of K, task order (0: charge order, 1: largest work first), source (0: default, 1: tuned on this
  * H_eff, 2: tuned earlier on the context)}; all -1 before the first tensor-core application. */
 int mrd_heff_tc_config(const mrd_heff* h, int32_t* cfg4);
+/* Arithmetic of the last MRD_PREC_FP64 or MRD_PREC_FF application: 0 FP64 / float-float on the CUDA
+ * cores, 1 digit products, 2 the CUDA cores because the panels of digit products found no memory
+ * (until environments are loaded again); -1 before the first. */
+int mrd_heff_form(const mrd_heff* h, int32_t* form);
 int mrd_heff_timing_collect(mrd_heff* h, double* ms_step1, double* ms_step2, int32_t* n_calls);
 
 /* ------------------------------------------------------------------ eigensolver */

@@ -23,6 +23,7 @@ MRD_OPT_PER_TASK_LAUNCH = 2
 MRD_OPT_AUTOTUNE = 3
 MRD_OPT_WAIT_LIMIT_US = 4
 MRD_OPT_REAL = 5
+MRD_OPT_DIGITS = 6
 MRD_SVD_F32_FF = 0
 MRD_SVD_FF = 1
 MRD_SVD_F32_F64 = 2
@@ -140,6 +141,7 @@ _SIGS = {
                                      C.POINTER(C.c_int32)]),
     "mrd_dmrg_schmidt": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int64), C.POINTER(C.c_int32),
                                    C.POINTER(C.c_double)]),
+    "mrd_heff_form": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32)]),
     "mrd_heff_timing_collect": (C.c_int, [C.c_void_p, C.POINTER(C.c_double), C.POINTER(C.c_double),
                                           C.POINTER(C.c_int32)]),
 }
@@ -504,12 +506,18 @@ class Heff:
 
     def set_option(self, option, value):
         """mrd_heff_set_option (MRD_OPT_GRAPH, MRD_OPT_PER_TASK_LAUNCH, MRD_OPT_AUTOTUNE,
-        MRD_OPT_WAIT_LIMIT_US)."""
+        MRD_OPT_WAIT_LIMIT_US, MRD_OPT_REAL, MRD_OPT_DIGITS)."""
         self.ctx.check(lib().mrd_heff_set_option(self.h, option, int(value)))
 
     def status(self):
         """mrd_heff_status: raises MrdError (MRD_E_TIMEOUT) if a tensor-core wait gave up."""
         self.ctx.check(lib().mrd_heff_status(self.h))
+
+    def form(self):
+        """Arithmetic of the last FP64 or float-float application (mrd_heff_form)."""
+        f = C.c_int32()
+        self.ctx.check(lib().mrd_heff_form(self.h, C.byref(f)))
+        return f.value
 
     def tc_config(self):
         """(columns per tile, stages, task order, source) of the tensor-core GEMM (mrd_heff_tc_config)."""

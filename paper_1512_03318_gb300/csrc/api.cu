@@ -831,6 +831,10 @@ int mrd_heff_set_option(mrd_heff* h, int32_t option, int64_t value) try {
       if (h->tc) { tc_free(h->tc); h->tc = nullptr; }   // panels of the other format
       ++h->gen;
     }
+  } else if (option == MRD_OPT_DIGITS) {
+    if (value < 0 || value > 2) return mrd_fail(h->ctx, MRD_E_ARG, "mrd_heff_set_option: MRD_OPT_DIGITS outside 0 .. 2");
+    h->dg_mode = (int)value;
+    ++h->gen;   // captured steps hold the products of the old choice
   } else if (option == MRD_OPT_WAIT_LIMIT_US) {
     if (value < 0 || value > 60000000) return mrd_fail(h->ctx, MRD_E_ARG, "mrd_heff_set_option: wait limit outside 0 .. 60 s");
     h->wait_ns = (uint64_t)value * 1000ull;
@@ -850,6 +854,14 @@ int mrd_heff_status(mrd_heff* h) try {
   const int rc = tc_status(h);
   const int rc2 = dg_status(h);   // both flags are read and cleared
   return rc != MRD_OK ? rc : rc2;
+} catch (...) {   // host memory or threads exhausted: no exception crosses the C ABI
+  return MRD_E_HOST;
+}
+
+int mrd_heff_form(const mrd_heff* h, int32_t* form) try {
+  if (!h || !form) return MRD_E_ARG;
+  *form = h->dg_form;
+  return MRD_OK;
 } catch (...) {   // host memory or threads exhausted: no exception crosses the C ABI
   return MRD_E_HOST;
 }

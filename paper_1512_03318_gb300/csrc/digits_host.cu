@@ -368,7 +368,9 @@ struct DgForm {
   int32_t prec = 0;
   int beta = 0;
   bool real = false, major = false;
-  bool planned = false, use = false, built = false, env_dirty = true;
+  bool decided = false, planned = false;   // whether digits are cheaper is known; the plans are made
+  bool refused = false;                    // dimensions beyond the tables' fields: there can be no plans
+  bool cheaper = false, built = false, env_dirty = true;
   bool captured = false;   // a caller's graph reads the panels
   bool no_room = false;    // the panels found no memory since the last environment load
   DgPlan p1, p2;
@@ -438,17 +440,17 @@ double k_padding(const mrd_heff* h) {
 // 280 / 191, 1.2 (Ly = 10, chi = 400) 717 / 183 | 699 / 520.
 constexpr double kMaxPadding = 1.55;
 
-// Plans of both products of a form, and whether they are the cheaper way (the same decision for
-// grouped and per-task launches, which give the same bits).
-void plan_both(const mrd_heff* h, DgForm* g) {
+// Decides whether the digit products of a form are the cheaper way (the same for grouped and per-task launches,
+// which give the same bits), with the plans of both unless it is plain without; force: the plans in any case.
+void plan_both(const mrd_heff* h, DgForm* g, bool force) {
   const int64_t n1 = h->counts[C_NT1], n2 = h->counts[C_NT2];
   const bool ff = g->prec == MRD_PREC_FF, real = g->real;
   const int beta = g->beta;
-  g->use = false;
-  g->planned = true;
   const double cores = cores_cost(h, ff, real);
-  if (cores * h->dg_uses < kSetupCycles) return;   // not worth planning
-  if (ff && k_padding(h) > kMaxPadding) return;
+  const bool worth = cores * h->dg_uses >= kSetupCycles && !(ff && k_padding(h) > kMaxPadding);
+  g->cheaper = false;
+  g->decided = true;
+  if (!worth && !force) return;
   std::vector<int32_t> ids((size_t)n2);   // step 2: the two row parts s1' of an output sector
   for (int64_t i = 0; i < n2; ++i) ids[(size_t)i] = (int32_t)(i >> 2 << 1 | (i & 1));   // share (nearly) all WR blocks
   // the two plans are independent: the second on a host thread of its own where that pays for starting
@@ -489,8 +491,11 @@ void plan_both(const mrd_heff* h, DgForm* g) {
   // the exponent and digit passes move ~80 bytes per element of theta and Z
   const double pass = (double)(h->counts[C_THETA] + h->counts[C_ZLEN]) * 80.0 / 5.0e12 * 1.9e9 + 25000.0;
   const double mine = g->p1.cost + g->p2.cost + pass;
-  g->use = !g->p1.items.empty() && !g->p2.items.empty() && mine * h->dg_uses + kSetupCycles < cores * h->dg_uses;
-  if (g->use && g->major) both(true);
+  const bool fits = !g->p1.items.empty() && !g->p2.items.empty();   // (else dimensions beyond the tables' fields)
+  g->cheaper = worth && fits && mine * h->dg_uses + kSetupCycles < cores * h->dg_uses;
+  if (fits && g->major) both(true);
+  g->planned = fits;
+  g->refused = !fits;
 }
 
 }  // namespace
@@ -499,7 +504,7 @@ void plan_both(const mrd_heff* h, DgForm* g) {
 // until h is freed); does nothing when no thread can be had.
 void dg_prebuild(mrd_heff* h, int32_t prec) {
   const bool ff = prec == MRD_PREC_FF;
-  if (h->dg || cores_cost(h, ff, h->real && ff) * h->dg_uses < 2 * kSetupCycles)
+  if (h->dg || h->dg_mode != 1 || cores_cost(h, ff, h->real && ff) * h->dg_uses < 2 * kSetupCycles)
     return;   // planned on demand (or not at all) where that is a matter of microseconds
   DgHeff* g = new DgHeff();
   h->dg = g;
@@ -507,9 +512,9 @@ void dg_prebuild(mrd_heff* h, int32_t prec) {
   try {
     g->th = std::thread([h, f] {
       try {
-        plan_both(h, f);
+        plan_both(h, f, false);
       } catch (...) {   // out of host memory: planned on demand instead
-        f->planned = false;
+        f->decided = f->planned = false;
       }
     });
   } catch (...) {
@@ -527,20 +532,21 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
   // themselves; float-float products run in the form that an earlier application has built.
   const bool cap = !h->in_lanczos && stream_capturing(s);
   *use = false;
-  if (cap && prec == MRD_PREC_FP64) return MRD_OK;
+  h->dg_form = 0;
+  if (h->dg_mode == 0 || (cap && prec == MRD_PREC_FP64)) return MRD_OK;
   if (!h->dg) h->dg = new DgHeff();
   if (h->dg->th.joinable()) h->dg->th.join();
   DgForm* g = h->dg->cur = h->dg->form(prec, h->real && prec == MRD_PREC_FF, h->per_task);
   const int beta = g->beta;
   if (cap && !g->built) return MRD_OK;
-  if (!g->planned) {
-    plan_both(h, g);
+  const bool force = h->dg_mode == 2;
+  if (!g->decided || (force && !g->planned && !g->refused)) {
+    plan_both(h, g, force);
     ++h->gen;
   }
-  *use = g->use;
-  if (!g->use) return MRD_OK;
+  if (!g->planned || !(g->cheaper || force)) return MRD_OK;
   if (!g->built && g->no_room) {
-    *use = false;
+    h->dg_form = 2;
     return MRD_OK;
   }
   if (!g->built) {
@@ -567,7 +573,7 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
       A.release();
       if (dg_release(h)) return dg_prepare(h, prec, use);   // another form's panels made way
       g->no_room = true;   // the CUDA-core kernels need none
-      *use = false;
+      h->dg_form = 2;
       return MRD_OK;
     }
     if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "digit-split products: buffers");
@@ -599,6 +605,8 @@ int dg_prepare(mrd_heff* h, int32_t prec, bool* use) {
     MRD_CUDA(ctx, dg_pack(g->d2, 1, h->wr, beta, g->words, s));
     g->env_dirty = cap;   // (packed by the replays, not now)
   }
+  h->dg_form = 1;
+  *use = true;
   return MRD_OK;
 }
 

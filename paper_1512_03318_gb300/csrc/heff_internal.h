@@ -115,6 +115,8 @@ struct mrd_heff {
   // digit-split products of the FP64 and float-float precisions (digits_host.cu)
   DgHeff* dg = nullptr;
   double dg_uses = 50.0;            // FP64 / float-float applications expected per environment load
+  int dg_mode = 1;                  // MRD_OPT_DIGITS
+  int dg_form = -1;                 // of the last FP64 / float-float application (mrd_heff_form)
   bool dg_use = false;              // the last prepared FP64 / float-float application runs on them
   bool in_lanczos = false;          // applications come from mrd_lanczos, which has prepared them
   bool env_captured = false;        // an environment load was captured: a replay may change LW and WR at any time

@@ -60,11 +60,13 @@ def test_non_finite_right_block_stays_with_its_part(ctx, prec, bad):
     fine = np.isfinite(ref)
     assert np.any(~fine) and np.any(fine)
     h = P.Heff(ctx, **G.heff_args(case))
+    h.set_option(P.MRD_OPT_DIGITS, 2)
     h.set_env(_dev(case["lflat"]), _dev(r))
     T = _dev(case["tflat"])
     out = torch.empty_like(T)
     h.apply(T, out, prec)
     h.status()
+    assert h.form() == 1
     got = out.cpu().numpy()
     assert np.all(np.isfinite(got[fine]))
     assert np.all(~np.isfinite(got[~fine]))
@@ -147,11 +149,13 @@ def test_graded_along_k(ctx, prec, decades):
     n = 4 * (dl + channels + channels * dr)
     tol = 2.0 * n * (2.0 ** -53 + (2.0 ** -53 if prec == 0 else 2.0 ** -46))
     h = P.Heff(ctx, **G.heff_args(case))
+    h.set_option(P.MRD_OPT_DIGITS, 2)
     h.set_env(_dev(l), _dev(r))
     T = _dev(t)
     out = torch.empty_like(T)
     h.apply(T, out, prec)
     h.status()
+    assert h.form() == 1
     got = out.cpu().numpy()
     for m in case["lay"]:
         view = lambda x: x[m["offset"]: m["offset"] + m["rowdim"] * m["coldim"]].reshape(m["rowdim"], m["coldim"])
