@@ -26,7 +26,7 @@ cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, co
                               int n_sm, cudaStream_t s);
 cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* rows, int64_t nrows,
                             const int64_t* env_map, int n_sec, const int32_t* perm, const int32_t* idx,
-                            const double* val, int chan_field, int64_t len, cudaStream_t s);
+                            const double* val, int chan_field, int64_t len, int n_sm, cudaStream_t s);
 struct Lanczos;
 void lanczos_free(Lanczos* L);
 cudaError_t lanczos_alloc(Lanczos** out, int64_t n, cudaStream_t stream);
@@ -438,10 +438,10 @@ int heff_fold(mrd_heff* h, const double2* lenv, const double2* renv) {
   cudaError_t e = cudaSuccess;
   if (lenv)
     e = launch_fold_env(lenv, h->lw, h->p.lw, h->counts[C_NLW], h->p.lmap, h->d.n_l, h->p.wi_perm, h->p.wi_idx,
-                        h->wi_val, 0, h->counts[C_LWLEN], ctx->stream);
+                        h->wi_val, 0, h->counts[C_LWLEN], h->n_sm, ctx->stream);
   if (renv && e == cudaSuccess)
     e = launch_fold_env(renv, h->wr, h->p.wr, h->counts[C_NWR], h->p.rmap, h->d.n_r, h->p.wj_perm, h->p.wj_idx,
-                        h->wj_val, 1, h->counts[C_WRLEN], ctx->stream);
+                        h->wj_val, 1, h->counts[C_WRLEN], h->n_sm, ctx->stream);
   if (e != cudaSuccess) return mrd_cuda_fail(ctx, e, "mrd_heff_set_env");
   h->env_loaded = (lenv || h->counts[C_LENV] == 0) && (renv || h->counts[C_RENV] == 0);
   h->env_captured = h->env_captured || stream_capturing(ctx->stream);

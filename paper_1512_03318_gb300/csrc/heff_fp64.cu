@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(256) k_cgemm_fp64(const double2* __restrict__ 
 // of four at once: 0.83 + 0.93.)
 constexpr int kFoldPer = 4, kFoldSub = kFoldPer * 256, kFoldTerms = 32;
 // Elements per CTA: 8192 where that gives four CTAs per SM, else fewer (down to one per thread).
-inline int64_t fold_chunk(int64_t len) {
-  const int64_t c = (len / 608 + 255) / 256 * 256;
+inline int64_t fold_chunk(int64_t len, int n_sm) {
+  const int64_t c = (len / (4 * n_sm) + 255) / 256 * 256;
   return c < 256 ? 256 : c > 8192 ? 8192 : c;
 }
 
@@ -294,7 +294,7 @@ cudaError_t launch_cgemm_fp64(const double2* A, const double2* B, double2* C, co
 
 cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* rows, int64_t nrows,
                             const int64_t* env_map, int n_sec, const int32_t* perm, const int32_t* idx,
-                            const double* val, int chan_field, int64_t len, cudaStream_t s) {
+                            const double* val, int chan_field, int64_t len, int n_sm, cudaStream_t s) {
   if (nrows <= 0 || len <= 0) return cudaSuccess;
   if (len <= kFoldSmall * nrows) {
     k_fold_small<<<(unsigned)(nrows < 65535 ? nrows : 65535), 256, 0, s>>>(env, out, rows, (int)nrows, env_map, n_sec, perm, idx, val,
@@ -302,7 +302,7 @@ cudaError_t launch_fold_env(const double2* env, double2* out, const int64_t* row
     mrd::count_launch();
     return cudaGetLastError();
   }
-  const int64_t chunk = fold_chunk(len);
+  const int64_t chunk = fold_chunk(len, n_sm);
   k_fold_env<<<(unsigned)((len + chunk - 1) / chunk), 256, 0, s>>>(env, out, rows, (int)nrows, len, env_map, n_sec, perm, idx, val,
                                                                    chan_field, (int)chunk);
   mrd::count_launch();

@@ -756,7 +756,7 @@ static int lanczos_step(Lanczos* L, mrd_ctx* ctx, int (*apply)(void*, const doub
   k_sub_combination<<<grid_for(n), 256, 0, s>>>(L->V, n, -2, L->st, L->c1, L->w, n, L->fp32_full ? L->w32 : nullptr);
   mrd::count_launch();
   if (L->fp32_full) {
-    k_multidot32<<<(unsigned)md32_blocks(n), md32_blocks(n) < 304 ? 512 : 256, 0, s>>>(L->V32, n, L->st, L->w32, n, L->partial32);
+    k_multidot32<<<(unsigned)md32_blocks(n), md32_blocks(n) < kRedBlocks ? 512 : 256, 0, s>>>(L->V32, n, L->st, L->w32, n, L->partial32);
     k_finish_dots<<<(MRD_LANCZOS_MAX_ITER + 1 + 3) / 4, 128, 0, s>>>(L->partial32, (int)md32_blocks(n), L->st, L->c2);
     k_sub_combination32<<<grid_for(n), 256, 0, s>>>(L->V32, n, L->st, L->c2, L->w, n);
     mrd::count_launches(3);
