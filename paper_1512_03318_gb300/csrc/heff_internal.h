@@ -158,7 +158,9 @@ inline const float4* heff_ff_wr(const mrd_heff* h) { return h->wr_ff && !h->ff_d
 
 inline bool stream_capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusActive;
+  const cudaError_t e = cudaStreamIsCapturing(s, &st);
+  if (e != cudaSuccess) cudaGetLastError();   // the legacy stream while another one is captured
+  return e == cudaSuccess && st == cudaStreamCaptureStatusActive;
 }
 
 inline cudaError_t record_event(cudaEvent_t e, cudaStream_t s, bool captured) {
