@@ -127,3 +127,41 @@ def test_lanczos_after_captured_loads(prec):
             assert h.lanczos(T.clone(), 3, 0.0, prec)[0] == fresh(L)
         h.close()
         del g
+
+
+def test_float_float_in_a_callers_graph_keeps_its_panels():
+    """A captured float-float application reads panels of the handle: they stay while other precisions, options
+    and a run that would release panels come and go, and a replay gives the same bits."""
+    import paper_1512_03318_gb300 as P
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    s = torch.cuda.Stream()
+    case = _one_block_case(107, 256, 200, 4)
+    with torch.cuda.stream(s):
+        ctx = P.Context(0, s)
+        h = P.Heff(ctx, **G.heff_args(case))
+        h.set_option(P.MRD_OPT_DIGITS, 2)
+        h.set_env(_dev(case["lflat"]), _dev(case["rflat"]))
+        T = _dev(case["tflat"])
+        out, out2 = torch.empty_like(T), torch.empty_like(T)
+        h.apply(T, out2, 3)
+        assert h.form() == 1
+        first = out2.cpu().numpy()
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            h.apply(T, out, 3)
+        for change in range(4):
+            if change == 1:
+                h.apply(T, out2, 0)
+            elif change == 2:
+                h.set_option(P.MRD_OPT_PER_TASK_LAUNCH, 1)
+                h.apply(T, out2, 3)
+                h.set_option(P.MRD_OPT_PER_TASK_LAUNCH, 0)
+            elif change == 3:
+                h.lanczos(T.clone(), 2, 0.0, 3)
+            out.fill_(0.0)
+            g.replay()
+            assert np.array_equal(out.cpu().numpy(), first)
+        h.close()
+        del g
