@@ -706,6 +706,122 @@ __device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, co
   return ff && abs(am - 1022) <= 30 && abs(bm - 1022) <= 30 ? 2 : 1;
 }
 
+// One listed tile: 8 stacked rows x 8 of the shared side, FP64 FMAs or float-float (REAL: imaginary parts taken
+// and returned as zeros). Few blocks are computed again, so what counts is the time of one: the FP64 pipe
+// has 2 lanes per SM, and a tile is small so that a block spreads over many SMs (32 x 32 tiles: 17 us
+// per 16 values of K, FP64 update at Ly = 8, chi = 1024 168 -> 208 ms for 12 blocks in 40 products). Four groups of 64
+// threads take the chunks of 16 values of K in turn, each with buffers and a barrier of its own, so that
+// their loads overlap; their sums are added in a fixed order.
+constexpr int kRedoTile = kDgRedoTile, kRedoK = 16, kRedoGroups = 4, kRedoJobs = 64;
+struct RedoJob {
+  int64_t so, uo, sl, ul;   // offsets and strides of the blocks; so < 0: a block this task does not multiply
+  int K, flags;             // flags: stacked operand's, shared operand's << 4
+};
+template <bool FFM, bool REAL>
+struct RedoSmem {
+  RedoJob jobs[kRedoJobs];
+  alignas(16) uint8_t a[kRedoGroups][kRedoTile * (kRedoK + 1) * 16], b[kRedoGroups][kRedoK * (kRedoTile + 1) * 16];
+  float2 as[kRedoGroups][FFM && !REAL ? kRedoTile * (kRedoK + 1) : 1], bs[kRedoGroups][FFM && !REAL ? kRedoK * (kRedoTile + 1) : 1];
+  double2 sum[kRedoGroups][kRedoTile * kRedoTile];
+};
+
+template <bool FFM, bool REAL, class Smem>
+__device__ __forceinline__ void redo_tile(const DgGroup& g, const DgMember& m, int tile, const DgJob* __restrict__ sjobs,
+                                          const DgJob* __restrict__ ujobs, const double2* __restrict__ ssrc,
+                                          const double2* __restrict__ usrc, double2* __restrict__ C, Smem& sm) {
+  const int tid = threadIdx.x, grp = tid >> 6, t = tid & 63, orow = t >> 3, ocol = t & 7;
+  const int ns = g.cm_rows ? g.N : g.R, tn = (ns + kRedoTile - 1) / kRedoTile;
+  const int r0 = tile / tn * kRedoTile, c0 = tile % tn * kRedoTile;
+  auto group_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory"); };
+  auto put = [&](uint8_t* s, float2* sum, int at, double2 v, bool conj) {   // stage one element
+    if (conj) v.y = -v.y;
+    if (REAL) v.y = 0.0;
+    if constexpr (FFM) {
+      const float4 x = cff_from(v);
+      ((float4*)s)[at] = x;
+      if (!REAL) sum[at] = cff_sum(x);
+    } else {
+      ((double2*)s)[at] = v;
+    }
+  };
+  double2 acc = make_double2(0.0, 0.0);
+  CAcc fac = {};
+  int chunk = 0;   // of the whole product
+  for (int f0 = 0; f0 < g.n_jobs; f0 += kRedoJobs) {
+    const int nf = g.n_jobs - f0 < kRedoJobs ? g.n_jobs - f0 : kRedoJobs;
+    __syncthreads();
+    if (tid < nf) {
+      const DgJob &x = sjobs[m.job + f0 + tid], &y = ujobs[g.job + f0 + tid];
+      sm.jobs[tid] = {x.off, y.off, x.ld, y.ld, y.K, x.flags | y.flags << 4};
+    }
+    __syncthreads();
+    for (int f = 0; f < nf; ++f) {
+      const RedoJob& j = sm.jobs[f];
+      if (j.so < 0) continue;
+      const int K = j.K, nc = (K + kRedoK - 1) / kRedoK;
+      const bool sk = j.flags & DGJ_KCONTIG, uk = (j.flags >> 4) & DGJ_KCONTIG;
+      for (int i = (grp - chunk) & (kRedoGroups - 1); i < nc; i += kRedoGroups) {
+        const int k0 = i * kRedoK;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int e = t + q * 64;
+          const int sr = sk ? e >> 4 : e & 7, sc = sk ? e & 15 : e >> 3;
+          double2 v = make_double2(0.0, 0.0), w = v;
+          if (r0 + sr < m.rows && k0 + sc < K) v = ssrc[j.so + (sk ? (r0 + sr) * j.sl + k0 + sc : (k0 + sc) * j.sl + r0 + sr)];
+          const int ur = uk ? e >> 4 : e & 7, uc = uk ? e & 15 : e >> 3;
+          if (c0 + ur < ns && k0 + uc < K) w = usrc[j.uo + (uk ? (c0 + ur) * j.ul + k0 + uc : (k0 + uc) * j.ul + c0 + ur)];
+          put(sm.a[grp], sm.as[grp], sr * (kRedoK + 1) + sc, v, j.flags & DGJ_CONJ);
+          put(sm.b[grp], sm.bs[grp], uc * (kRedoTile + 1) + ur, w, (j.flags >> 4) & DGJ_CONJ);
+        }
+        group_sync();
+        const int kn = K - k0 < kRedoK ? K - k0 : kRedoK;
+        for (int k = 0; k < kn; ++k) {
+          const int p = orow * (kRedoK + 1) + k, q = k * (kRedoTile + 1) + ocol;
+          if constexpr (FFM) {
+            const float4 x = ((const float4*)sm.a[grp])[p], y = ((const float4*)sm.b[grp])[q];
+            if (REAL) ff_mac(fac.rr, FF{x.x, x.z}, FF{y.x, y.z});
+            else cff_mac(fac, x, sm.as[grp][p], y, sm.bs[grp][q]);
+          } else {
+            const double2 x = ((const double2*)sm.a[grp])[p], y = ((const double2*)sm.b[grp])[q];
+            acc.x = fma(-x.y, y.y, fma(x.x, y.x, acc.x));
+            acc.y = fma(x.y, y.x, fma(x.x, y.y, acc.y));
+          }
+        }
+        if constexpr (FFM) {   // as the float-float GEMM: errors collected over 16 products at most
+          fac.rr = ff_renorm(fac.rr);
+          if (!REAL) {
+            fac.ii = ff_renorm(fac.ii);
+            fac.ss = ff_renorm(fac.ss);
+          }
+        }
+        group_sync();
+      }
+      chunk += nc;
+    }
+  }
+  if constexpr (FFM) {
+    FF re = ff_norm(fac.rr), im = {0.f, 0.f};
+    if (!REAL) cff_result(fac, re, im);
+    acc = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
+  }
+  sm.sum[grp][t] = acc;
+  __syncthreads();
+  if (grp == 0 && r0 + orow < m.rows && c0 + ocol < ns) {
+#pragma unroll
+    for (int q = 1; q < kRedoGroups; ++q) {
+      acc.x += sm.sum[q][t].x;
+      acc.y += sm.sum[q][t].y;
+    }
+    C[m.off + (r0 + orow) * m.step + (c0 + ocol) * m.other] = make_double2(acc.x, REAL ? 0.0 : acc.y);
+  }
+}
+
+// Tiles of a task.
+__device__ __forceinline__ int redo_tiles(const DgGroup& g, const DgMember& m) {
+  const int ns = g.cm_rows ? g.N : g.R;
+  return ((m.rows + kRedoTile - 1) / kRedoTile) * ((ns + kRedoTile - 1) / kRedoTile);
+}
+
 // One warp per task: the tiles of those to be computed again join the list. Not after a wait gave up, when
 // nothing is valid.
 __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members, int n,
@@ -724,110 +840,13 @@ __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ gr
   for (; i < n; i += gridDim.x * 8, m = members[min(i, n - 1)], g = groups[m.group]) {
     const int form = task_form(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, ff, lane);
     if (form == 0) continue;
-    const int ns = g.cm_rows ? g.N : g.R, tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32), mark = form == 2 ? kDgFF : 0;
+    const int tiles = redo_tiles(g, m), mark = form == 2 ? kDgFF : 0;
     int at = 0;
     if (lane == 0) at = atomicAdd(count, tiles);
     at = __shfl_sync(0xffffffffu, at, 0);
     for (int t = lane; t < tiles; t += 32) list[at + t] = make_int2(i, t | mark);
   }
 }
-
-// One listed tile: 32 stacked rows x 32 of the shared side, K in chunks of 16, blocks in the order of the job
-// lists. FP64 FMAs, or float-float (four times as fast: the FP64 pipe has 2 lanes per SM); REAL: imaginary
-// parts taken and returned as zeros.
-template <bool FFM, bool REAL>
-__device__ __forceinline__ void redo_tile(const DgGroup& g, const DgMember& m, int tile, const DgJob* __restrict__ sjobs,
-                                          const DgJob* __restrict__ ujobs, const double2* __restrict__ ssrc,
-                                          const double2* __restrict__ usrc, double2* __restrict__ C, void* sa, void* sb, float2* sas,
-                                          float2* sbs) {
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int ns = g.cm_rows ? g.N : g.R, tn = (ns + 31) / 32;
-  const int r0 = tile / tn * 32, c0 = tile % tn * 32;
-  auto put = [&](void* s, float2* sum, int at, double2 v, bool conj) {   // stage one element
-    if (conj) v.y = -v.y;
-    if (REAL) v.y = 0.0;
-    if constexpr (FFM) {
-      const float4 x = cff_from(v);
-      ((float4*)s)[at] = x;
-      if (!REAL) sum[at] = cff_sum(x);
-    } else {
-      ((double2*)s)[at] = v;
-    }
-  };
-  double2 acc[2][2] = {};
-  CAcc fac[2][2] = {};
-  for (int f = 0; f < g.n_jobs; ++f) {
-    const DgJob &sj = sjobs[m.job + f], &uj = ujobs[g.job + f];
-    if (sj.off < 0) continue;                            // a block this task does not multiply
-    const int K = uj.K;
-    const bool sk = sj.flags & DGJ_KCONTIG, uk = uj.flags & DGJ_KCONTIG;
-    for (int k0 = 0; k0 < K; k0 += 16) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int e = tid + q * 256;
-        const int sr = sk ? e >> 4 : e & 31, sc = sk ? e & 15 : e >> 5;
-        double2 v = make_double2(0.0, 0.0);
-        if (r0 + sr < m.rows && k0 + sc < K)
-          v = ssrc[sj.off + (sk ? (r0 + sr) * sj.ld + k0 + sc : (k0 + sc) * sj.ld + r0 + sr)];
-        put(sa, sas, sr * 17 + sc, v, sj.flags & DGJ_CONJ);
-        const int ur = uk ? e >> 4 : e & 31, uc = uk ? e & 15 : e >> 5;
-        v = make_double2(0.0, 0.0);
-        if (c0 + ur < ns && k0 + uc < K)
-          v = usrc[uj.off + (uk ? (c0 + ur) * uj.ld + k0 + uc : (k0 + uc) * uj.ld + c0 + ur)];
-        put(sb, sbs, uc * 33 + ur, v, uj.flags & DGJ_CONJ);
-      }
-      __syncthreads();
-      const int kn = K - k0 < 16 ? K - k0 : 16;
-      for (int k = 0; k < kn; ++k)
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int p = (2 * ty + i) * 17 + k, q = k * 33 + 2 * tx + j;
-            if constexpr (FFM) {
-              const float4 a = ((const float4*)sa)[p], b = ((const float4*)sb)[q];
-              if (REAL) ff_mac(fac[i][j].rr, FF{a.x, a.z}, FF{b.x, b.z});
-              else cff_mac(fac[i][j], a, sas[p], b, sbs[q]);
-            } else {
-              const double2 a = ((const double2*)sa)[p], b = ((const double2*)sb)[q];
-              acc[i][j].x = fma(-a.y, b.y, fma(a.x, b.x, acc[i][j].x));
-              acc[i][j].y = fma(a.y, b.x, fma(a.x, b.y, acc[i][j].y));
-            }
-          }
-      if constexpr (FFM) {   // as the float-float GEMM: errors collected over 16 products at most
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            CAcc& x = fac[i][j];
-            x.rr = ff_renorm(x.rr);
-            if (!REAL) { x.ii = ff_renorm(x.ii); x.ss = ff_renorm(x.ss); }
-          }
-      }
-      __syncthreads();
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int r = r0 + 2 * ty + i, c = c0 + 2 * tx + j;
-      double2 v = acc[i][j];
-      if constexpr (FFM) {
-        FF re = ff_norm(fac[i][j].rr), im = {0.f, 0.f};
-        if (!REAL) cff_result(fac[i][j], re, im);
-        v = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
-      }
-      if (r < m.rows && c < ns) C[m.off + r * m.step + c * m.other] = make_double2(v.x, REAL ? 0.0 : v.y);
-    }
-}
-
-// Shared memory of the tiles above.
-template <bool FFM, bool REAL>
-struct RedoSmem {
-  alignas(16) uint8_t a[32 * 17 * 16], b[16 * 33 * 16];
-  float2 as[FFM && !REAL ? 32 * 17 : 1], bs[FFM && !REAL ? 16 * 33 : 1];
-};
 
 // The listed tiles. Usually the list is empty and the launch returns at once.
 template <bool FFM, bool REAL>
@@ -843,8 +862,8 @@ __global__ void __launch_bounds__(256) k_dg_redo(const DgGroup* __restrict__ gro
     const int2 it = list[item];
     const DgMember m = members[it.x];
     const DgGroup g = groups[m.group];
-    if (FFM && (it.y & kDgFF)) redo_tile<FFM, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
-    else redo_tile<false, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
+    if (FFM && (it.y & kDgFF)) redo_tile<FFM, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sm);
+    else redo_tile<false, REAL>(g, m, it.y & ~kDgFF, sjobs, ujobs, ssrc, usrc, C, sm);
   }
 }
 
@@ -867,18 +886,16 @@ __global__ void __launch_bounds__(256) k_dg_redo_tasks(const DgGroup* __restrict
   }
   __syncthreads();
   if (s_form == 0) return;
-  const int ns = g.cm_rows ? g.N : g.R, tiles = ((m.rows + 31) / 32) * ((ns + 31) / 32);
-  for (int t = 0; t < tiles; ++t) {
-    if (FFM && s_form == 2) redo_tile<FFM, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
-    else redo_tile<false, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm.a, sm.b, sm.as, sm.bs);
+  for (int t = 0; t < redo_tiles(g, m); ++t) {
+    if (FFM && s_form == 2) redo_tile<FFM, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm);
+    else redo_tile<false, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm);
   }
 }
 
-// Products whose tasks are single tiles, up to this many, take the one-launch form: 2 to 3 us less per product
+// Products whose tasks have few tiles, up to this many tasks, take the one-launch form: 2 to 3 us less per product
 // (FP64 application at Ly = 4, chi = 48 74.4 -> 69.0 us, float-float at Ly = 5, chi = 112 in real arithmetic
-// 66 -> 58). With larger tasks the tiles of one would follow each other (up to 8 of them: FP64 update at
-// Ly = 6, chi = 512 13.6 -> 15.0 ms).
-constexpr int kDgRedoTiles = 1, kDgRedoTasks = 4096;
+// 66 -> 58). With larger tasks the tiles of one would follow each other.
+constexpr int kDgRedoTiles = 4, kDgRedoTasks = 4096;
 
 cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2* C, int beta, const int* words, int n_sm, cudaStream_t s) {
   if (d.n_members <= 0) return cudaSuccess;
@@ -907,7 +924,7 @@ cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2*
   lc.gridDim = dim3(grid < 2048 ? grid : 2048);
   cudaError_t e = cudaLaunchKernelEx(&lc, k_dg_check, gr, me, d.n_members, sj, uj, ss, us, e0, e1, res, d.redo_count, d.redo, err, beta != 8);
   if (e != cudaSuccess) return e;
-  lc.gridDim = dim3(2 * n_sm);
+  lc.gridDim = dim3(4 * n_sm);
   auto k = beta == 8 ? k_dg_redo<false, false> : d.real ? k_dg_redo<true, true> : k_dg_redo<true, false>;
   e = cudaLaunchKernelEx(&lc, k, gr, me, sj, uj, ss, us, C, (const int*)d.redo_count, (const int2*)d.redo);
   count_launches(2);

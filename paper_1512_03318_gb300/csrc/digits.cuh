@@ -46,6 +46,7 @@ constexpr int kDgRows = 128;      // rows of a left (tall) tile
 constexpr int kDgCols = 32;       // columns of a tile: 8 levels x 32 x (re, im) = 512 TMEM columns
 constexpr int kDgDigits = 8;
 constexpr int kDgStep = 16;       // K of one MMA, one panel step
+constexpr int kDgRedoTile = 8;    // tiles of blocks that are computed again
 constexpr int kDgSpread = 6;      // bits a block's largest result may lie below its operands' bounds
 __host__ __device__ inline int dg_planes(bool real) { return real ? kDgDigits : 2 * kDgDigits; }
 __host__ __device__ inline int dg_tbits(int beta) { return beta == 8 ? 62 : 55; }
@@ -100,7 +101,7 @@ struct DgPlan {
   int64_t bytes[2] = {0, 0};         // panels
   int64_t rows[2] = {0, 0};          // exponents
   int64_t slots = 0;                 // partial sums of split tiles
-  int64_t redo = 0;                  // 32 x 32 tiles of all tasks
+  int64_t redo = 0;                  // tiles of kDgRedoTile x kDgRedoTile of all tasks
   int max_tiles = 0;                 // of one task
   int sop = 0;                       // the stacked operand
   double cost = 0.0;                 // estimated cycles of the product

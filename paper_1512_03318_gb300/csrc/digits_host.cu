@@ -213,7 +213,7 @@ void dg_plan(DgPlan& p, const int64_t* tasks, const int64_t* segs, int64_t n_tas
                                es + m.row0, kind(sop, ct) | s_flag, 0});
       }
       p.members.push_back({t[2], sop ? 1 : t[3], sop ? t[3] : 1, (int32_t)p.cmap + m.row0, m.rows, (int32_t)p.groups.size(), job0});
-      const int64_t tiles = up(m.rows, 32) / 32 * (up(g.N, 32) / 32);
+      const int64_t tiles = up(m.rows, kDgRedoTile) / kDgRedoTile * (up(g.N, kDgRedoTile) / kDgRedoTile);
       p.redo += tiles;
       p.max_tiles = (int)std::max<int64_t>(p.max_tiles, tiles);
     }
