@@ -647,22 +647,29 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
 
 constexpr int kDgFF = 1 << 30;   // mark of a listed tile that float-float arithmetic can do
 
-// log2 of sum_k |s_rk| |u_ck| over the bounds of row r and column c, in the part (real or imaginary) where
-// it is larger; one warp, 8 lanes per block, the lanes along K.
-__device__ __forceinline__ double terms_log2(const DgJob* sj, const DgJob* uj, int n, const double2* ssrc, const double2* usrc, int r,
-                                             int c, int er, int ec, int lane) {
-  const double sr = ldexp(1.0, 1022 - er), sc = ldexp(1.0, 1022 - ec);
-  double re = 0.0, im = 0.0;
+// sum_k |s_rk| |u_ck| over the bounds 2^(er - 1022) of row r and 2^(ec - 1022) of column c, in the part (real or
+// imaginary) where it is larger; one warp, 8 lanes per block, the lanes along K. In FP32 from truncated
+// magnitudes, so that the FP64 pipe has no part in it: low by 2^-20 at most, and right to 2^-10 in a sum
+// of 10^4 terms. FP64 application at Ly = 4, chi = 48 70.1 -> 68.0 us, at Ly = 8, chi = 1024 488 -> 485.
+__device__ __forceinline__ float mag_over(double x, int e) {   // |x| / 2^(e - 1022), truncated, below 1
+  const int hi = __double2hiint(x) & 0x7fffffff, f = (hi >> 20) - e + 126;
+  return f <= 0 ? 0.f : __int_as_float(f << 23 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ float terms_sum(const DgJob* sj, const DgJob* uj, int n, const double2* ssrc, const double2* usrc, int r,
+                                           int c, int er, int ec, int lane) {
+  float re = 0.f, im = 0.f;
   for (int f = lane >> 3; f < n; f += 4) {
     const DgJob &x = sj[f], &y = uj[f];
     if (x.off < 0) continue;
     const int64_t x0 = x.off + (x.flags & DGJ_KCONTIG ? r * x.ld : r), xs = x.flags & DGJ_KCONTIG ? 1 : x.ld;
     const int64_t y0 = y.off + (y.flags & DGJ_KCONTIG ? c * y.ld : c), ys = y.flags & DGJ_KCONTIG ? 1 : y.ld;
-    for (int k = lane & 7; k < y.K; k += 8) {
+    const int K = y.K;
+#pragma unroll 4
+    for (int k = lane & 7; k < K; k += 8) {
       const double2 p = ssrc[x0 + k * xs], q = usrc[y0 + k * ys];
-      const double px = fabs(p.x * sr), py = fabs(p.y * sr), qx = fabs(q.x * sc), qy = fabs(q.y * sc);
-      re = fma(px, qx, fma(py, qy, re));
-      im = fma(px, qy, fma(py, qx, im));
+      const float px = mag_over(p.x, er), py = mag_over(p.y, er), qx = mag_over(q.x, ec), qy = mag_over(q.y, ec);
+      re = fmaf(px, qx, fmaf(py, qy, re));
+      im = fmaf(px, qy, fmaf(py, qx, im));
     }
   }
 #pragma unroll
@@ -670,7 +677,7 @@ __device__ __forceinline__ double terms_log2(const DgJob* sj, const DgJob* uj, i
     re += __shfl_xor_sync(0xffffffffu, re, o);
     im += __shfl_xor_sync(0xffffffffu, im, o);
   }
-  return log2(fmax(re, im));
+  return fmaxf(re, im);
 }
 
 // Whether a task has to be computed again (0: no, 1: in FP64, 2: in float-float): a row or column of its
@@ -701,7 +708,8 @@ __device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, co
   if (am == 0 || bm == 0 || am + bm - o <= 1021 + kDgSpread) return 0;
   const int r = __shfl_sync(0xffffffffu, ra, __ffs(__ballot_sync(0xffffffffu, a == am)) - 1);
   const int c = __shfl_sync(0xffffffffu, cb, __ffs(__ballot_sync(0xffffffffu, b == bm)) - 1);
-  if (terms_log2(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane) >= -(double)kDgSpread) return 0;
+  constexpr float kLine = 1.01f / (1 << kDgSpread);   // (with room for the sum's rounding)
+  if (terms_sum(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane) >= kLine) return 0;
   // float-float products take operands within the FP32 range only
   return ff && abs(am - 1022) <= 30 && abs(bm - 1022) <= 30 ? 2 : 1;
 }
@@ -709,7 +717,7 @@ __device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, co
 // One listed tile: 8 stacked rows x 8 of the shared side, FP64 FMAs or float-float (REAL: imaginary parts taken
 // and returned as zeros). Few blocks are computed again, so what counts is the time of one: the FP64 pipe
 // has 2 lanes per SM, and a tile is small so that a block spreads over many SMs (32 x 32 tiles: 17 us
-// per 16 values of K, FP64 update at Ly = 8, chi = 1024 168 -> 208 ms for 12 blocks in 40 products). Four groups of 64
+// per 16 values of K, FP64 update at Ly = 8, chi = 1024 208 ms, with these 181, for 12 blocks in 40 products). Four groups of 64
 // threads take the chunks of 16 values of K in turn, each with buffers and a barrier of its own, so that
 // their loads overlap; their sums are added in a fixed order.
 constexpr int kRedoTile = kDgRedoTile, kRedoK = 16, kRedoGroups = 4, kRedoJobs = 64;

@@ -30,7 +30,7 @@
 //
 // Measured on H_eff applications (Hofstadter cylinder, mid-ring sites, random operands): FP64 at
 // Ly = 8, chi = 1024 0.49 ms (CUDA cores 11.2 ms); loading environments and one float-float
-// application at Ly = 10, chi = 3200 7.5 ms (31.9 ms). The product kernel is bound by the tensor
+// application at Ly = 10, chi = 3200 7.6 ms (31.9 ms). The product kernel is bound by the tensor
 // pipe: 26 complex multiply-adds per cycle and SM at full tiles, against 0.21 for FP64 FMAs.
 #pragma once
 #include <cuda_runtime.h>
