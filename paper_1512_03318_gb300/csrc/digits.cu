@@ -648,17 +648,18 @@ __global__ void __launch_bounds__(320, 1) k_dg_gemm(DgArgs g) {
 constexpr int kDgFF = 1 << 30;   // mark of a listed tile that float-float arithmetic can do
 
 // sum_k |s_rk| |u_ck| over the bounds 2^(er - 1022) of row r and 2^(ec - 1022) of column c, in the part (real or
-// imaginary) where it is larger; one warp, 8 lanes per block, the lanes along K. In FP32 from truncated
+// imaginary) where it is larger; NW warps, 8 lanes per block, the lanes along K. In FP32 from truncated
 // magnitudes, so that the FP64 pipe has no part in it: low by 2^-20 at most, and right to 2^-10 in a sum
 // of 10^4 terms. FP64 application at Ly = 4, chi = 48 70.1 -> 68.0 us, at Ly = 8, chi = 1024 488 -> 485.
 __device__ __forceinline__ float mag_over(double x, int e) {   // |x| / 2^(e - 1022), truncated, below 1
   const int hi = __double2hiint(x) & 0x7fffffff, f = (hi >> 20) - e + 126;
   return f <= 0 ? 0.f : __int_as_float(f << 23 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(x) >> 29));
 }
+template <int NW>
 __device__ __forceinline__ float terms_sum(const DgJob* sj, const DgJob* uj, int n, const double2* ssrc, const double2* usrc, int r,
-                                           int c, int er, int ec, int lane) {
+                                           int c, int er, int ec, int lane, int warp) {
   float re = 0.f, im = 0.f;
-  for (int f = lane >> 3; f < n; f += 4) {
+  for (int f = warp * 4 + (lane >> 3); f < n; f += 4 * NW) {
     const DgJob &x = sj[f], &y = uj[f];
     if (x.off < 0) continue;
     const int64_t x0 = x.off + (x.flags & DGJ_KCONTIG ? r * x.ld : r), xs = x.flags & DGJ_KCONTIG ? 1 : x.ld;
@@ -677,6 +678,17 @@ __device__ __forceinline__ float terms_sum(const DgJob* sj, const DgJob* uj, int
     re += __shfl_xor_sync(0xffffffffu, re, o);
     im += __shfl_xor_sync(0xffffffffu, im, o);
   }
+  if constexpr (NW > 1) {
+    __shared__ float2 part[NW];
+    if (lane == 0) part[warp] = make_float2(re, im);
+    __syncthreads();
+    re = im = 0.f;
+    for (int w = 0; w < NW; ++w) {
+      re += part[w].x;
+      im += part[w].y;
+    }
+    __syncthreads();
+  }
   return fmaxf(re, im);
 }
 
@@ -684,9 +696,10 @@ __device__ __forceinline__ float terms_sum(const DgJob* sj, const DgJob* uj, int
 // operands is not finite (exponent field 2047), a result is outside the normal range (marked likewise), or
 // the fixed point was too coarse: no result within 2^kDgSpread of the largest row times the largest
 // column, and not for want of large terms (sums that cancel are as inexact in FMAs): the terms of the
-// largest row and column tell. One warp.
+// largest row and column tell. NW warps, all with the same answer.
+template <int NW>
 __device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, const DgJob* sjobs, const DgJob* ujobs, const double2* ssrc,
-                                         const double2* usrc, const int* e0, const int* e1, const int* res, bool ff, int lane) {
+                                         const double2* usrc, const int* e0, const int* e1, const int* res, bool ff, int lane, int warp) {
   const int *tall = g.tall_op ? e1 : e0, *flat = g.tall_op ? e0 : e1;
   const int* stacked = (g.cm_rows ? tall + g.ea : flat + g.eb) + (m.first - g.cm);
   const int* shared = g.cm_rows ? flat + g.eb : tall + g.ea;
@@ -708,8 +721,8 @@ __device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, co
   if (am == 0 || bm == 0 || am + bm - o <= 1021 + kDgSpread) return 0;
   const int r = __shfl_sync(0xffffffffu, ra, __ffs(__ballot_sync(0xffffffffu, a == am)) - 1);
   const int c = __shfl_sync(0xffffffffu, cb, __ffs(__ballot_sync(0xffffffffu, b == bm)) - 1);
-  constexpr float kLine = 1.01f / (1 << kDgSpread);   // (with room for the sum's rounding)
-  if (terms_sum(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane) >= kLine) return 0;
+  const float line = ff ? kDgLineFF : kDgLine64;
+  if (terms_sum<NW>(sjobs + m.job, ujobs + g.job, g.n_jobs, ssrc, usrc, r, c, am, bm, lane, warp) >= line) return 0;
   // float-float products take operands within the FP32 range only
   return ff && abs(am - 1022) <= 30 && abs(bm - 1022) <= 30 ? 2 : 1;
 }
@@ -719,7 +732,9 @@ __device__ __forceinline__ int task_form(const DgGroup& g, const DgMember& m, co
 // has 2 lanes per SM, and a tile is small so that a block spreads over many SMs (32 x 32 tiles: 17 us
 // per 16 values of K, FP64 update at Ly = 8, chi = 1024 208 ms, with these 181, for 12 blocks in 40 products). Four groups of 64
 // threads take the chunks of 16 values of K in turn, each with buffers and a barrier of its own, so that
-// their loads overlap; their sums are added in a fixed order.
+// their loads overlap; their sums are added in a fixed order. Float-float operands are split from
+// their bits, which the FP64 pipe has no part in: step 2 of the refinement in the update that repeats most
+// (Ly = 10, chi = 3200) 6.2 -> 5.3 ms.
 constexpr int kRedoTile = kDgRedoTile, kRedoK = 16, kRedoGroups = 4, kRedoJobs = 64;
 struct RedoJob {
   int64_t so, uo, sl, ul;   // offsets and strides of the blocks; so < 0: a block this task does not multiply
@@ -745,7 +760,8 @@ __device__ __forceinline__ void redo_tile(const DgGroup& g, const DgMember& m, i
     if (conj) v.y = -v.y;
     if (REAL) v.y = 0.0;
     if constexpr (FFM) {
-      const float4 x = cff_from(v);
+      const FF re = ff_from_bits(v.x), im = ff_from_bits(v.y);
+      const float4 x = make_float4(re.hi, im.hi, re.lo, im.lo);
       ((float4*)s)[at] = x;
       if (!REAL) sum[at] = cff_sum(x);
     } else {
@@ -830,24 +846,27 @@ __device__ __forceinline__ int redo_tiles(const DgGroup& g, const DgMember& m) {
   return ((m.rows + kRedoTile - 1) / kRedoTile) * ((ns + kRedoTile - 1) / kRedoTile);
 }
 
-// One warp per task: the tiles of those to be computed again join the list. Not after a wait gave up, when
-// nothing is valid.
+// NW warps per task: the tiles of those to be computed again join the list. Not after a wait gave up, when
+// nothing is valid. A CTA per task where there are few: adding up the terms of a task's largest row and column
+// is a chain of loads along K (step 2 at Ly = 10, chi = 3200, 260 tasks: a warp each
+// 322 us, a CTA each 74).
+template <int NW>
 __global__ void __launch_bounds__(256) k_dg_check(const DgGroup* __restrict__ groups, const DgMember* __restrict__ members, int n,
                                                   const DgJob* __restrict__ sjobs, const DgJob* __restrict__ ujobs,
                                                   const double2* __restrict__ ssrc, const double2* __restrict__ usrc,
                                                   const int* __restrict__ e0, const int* __restrict__ e1,
                                                   const int* __restrict__ res, int* __restrict__ count, int2* __restrict__ list,
                                                   const int* __restrict__ err, bool ff) {
-  const int lane = threadIdx.x & 31;
-  int i = (blockIdx.x * 256 + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31, warp = NW > 1 ? threadIdx.x >> 5 : 0;
+  int i = NW > 1 ? (int)blockIdx.x : (int)(blockIdx.x * 256 + threadIdx.x) >> 5;
   DgMember m = members[min(i, n - 1)];
   DgGroup g = groups[m.group];
   // launched as a programmatic dependent of the product: above are tables, below its results
   asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
   if (*err) return;
-  for (; i < n; i += gridDim.x * 8, m = members[min(i, n - 1)], g = groups[m.group]) {
-    const int form = task_form(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, ff, lane);
-    if (form == 0) continue;
+  for (; i < n; i += gridDim.x * (8 / NW), m = members[min(i, n - 1)], g = groups[m.group]) {
+    const int form = task_form<NW>(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, ff, lane, warp);
+    if (form == 0 || warp > 0) continue;
     const int tiles = redo_tiles(g, m), mark = form == 2 ? kDgFF : 0;
     int at = 0;
     if (lane == 0) at = atomicAdd(count, tiles);
@@ -886,16 +905,12 @@ __global__ void __launch_bounds__(256) k_dg_redo_tasks(const DgGroup* __restrict
   const DgMember m = members[blockIdx.x];
   const DgGroup g = groups[m.group];
   __shared__ RedoSmem<FFM, REAL> sm;
-  __shared__ int s_form;
   asm volatile("griddepcontrol.wait;" ::: "memory");   // (dependent of the product)
-  if (threadIdx.x < 32) {
-    const int form = *err ? 0 : task_form(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, FFM, threadIdx.x);
-    if (threadIdx.x == 0) s_form = form;
-  }
-  __syncthreads();
-  if (s_form == 0) return;
+  if (*err) return;
+  const int form = task_form<8>(g, m, sjobs, ujobs, ssrc, usrc, e0, e1, res, FFM, threadIdx.x & 31, threadIdx.x >> 5);
+  if (form == 0) return;
   for (int t = 0; t < redo_tiles(g, m); ++t) {
-    if (FFM && s_form == 2) redo_tile<FFM, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm);
+    if (FFM && form == 2) redo_tile<FFM, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm);
     else redo_tile<false, REAL>(g, m, t, sjobs, ujobs, ssrc, usrc, C, sm);
   }
 }
@@ -929,8 +944,9 @@ cudaError_t dg_redo(const DgDev& d, const double2* a, const double2* b, double2*
     count_launch();
     return cudaLaunchKernelEx(&lc, k, gr, me, sj, uj, ss, us, C, e0, e1, res, err);
   }
-  lc.gridDim = dim3(grid < 2048 ? grid : 2048);
-  cudaError_t e = cudaLaunchKernelEx(&lc, k_dg_check, gr, me, d.n_members, sj, uj, ss, us, e0, e1, res, d.redo_count, d.redo, err, beta != 8);
+  const bool wide = d.n_members <= 4 * n_sm;   // (that many CTAs run at once)
+  lc.gridDim = dim3(wide ? d.n_members : grid < 2048 ? grid : 2048);
+  cudaError_t e = cudaLaunchKernelEx(&lc, wide ? k_dg_check<8> : k_dg_check<1>, gr, me, d.n_members, sj, uj, ss, us, e0, e1, res, d.redo_count, d.redo, err, beta != 8);
   if (e != cudaSuccess) return e;
   lc.gridDim = dim3(4 * n_sm);
   auto k = beta == 8 ? k_dg_redo<false, false> : d.real ? k_dg_redo<true, true> : k_dg_redo<true, false>;

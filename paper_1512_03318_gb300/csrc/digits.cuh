@@ -21,8 +21,8 @@
 // times its column's bound: two roundings of 2^-63 (2^-56), seven dropped digit pairs of 2^-62 (2^-56)
 // on the first level, and twice that in a complex product. K FMAs in FP64 may be off by
 // 2 K 2^-53 (float-float: 2 K 2^-46) of the sum of the terms' magnitudes, so a result block is kept when
-// that sum reaches 2^-kDgSpread of the largest row times the largest column somewhere in it: the error is
-// then below what FMAs may be off in the block. The largest result is a lower bound of the sum and costs
+// that sum reaches 2^-6 (float-float: 2^-6.8) of the largest row times the largest column somewhere in it: the
+// error is then below what FMAs may be off in the block. The largest result is a lower bound of the sum and costs
 // nothing; where it is too small, the terms of the largest row and column are added up. The other blocks
 // (operands graded against each other along K) are computed again in FP64, or in float-float for the
 // float-float products. On states of the cylinders
@@ -48,6 +48,9 @@ constexpr int kDgDigits = 8;
 constexpr int kDgStep = 16;       // K of one MMA, one panel step
 constexpr int kDgRedoTile = 8;    // tiles of blocks that are computed again
 constexpr int kDgSpread = 6;      // bits a block's largest result may lie below its operands' bounds
+// the same of the sum of the terms' magnitudes: 2^-6 (FP64), 2^-6.8 (float-float), with 1% for its rounding.
+// With 2^-6 for both step 2 of the refinement that repeats most (Ly = 10, chi = 3200) took 5.3 instead of 4.0 ms (repeats and their check together).
+constexpr float kDgLine64 = 1.01f / 64.f, kDgLineFF = 1.01f / 111.4f;
 __host__ __device__ inline int dg_planes(bool real) { return real ? kDgDigits : 2 * kDgDigits; }
 __host__ __device__ inline int dg_tbits(int beta) { return beta == 8 ? 62 : 55; }
 // K steps between flushes. Level l sums 2 (l + 1) digit products of at most 2^(2 beta - 2) per
